@@ -145,7 +145,9 @@ ssj_status ssj_collection_info(ssj_ctx* ctx, ssj_coll coll, uint32_t* n_sets, ui
 #define SSJ_EMIT_ALL 0x8u       /* diagnostic: emit every listed pair (except self pairs of a
                                    self-join) with its exact overlap, no threshold test and no
                                    early termination */
-#define SSJ_FORCE_THREAD 0x10u  /* verify every pair with one thread (Alternative A/B style) */
+#define SSJ_FORCE_THREAD 0x10u  /* verify every pair with one thread (Alternative A/B style); a
+                                   forced granularity verifies every pair that the length filter
+                                   leaves, without the signature test */
 #define SSJ_FORCE_WARP 0x20u    /* verify every pair with one warp (merge path over 32 lanes) */
 #define SSJ_FORCE_BLOCK 0x40u   /* verify every pair with one thread block (Alternative C) */
 #define SSJ_FORCE_LANE 0x80u    /* verify every pair with one lane, the probe set held in the
@@ -507,7 +509,9 @@ ssj_status ssj_set_granularity(ssj_ctx* ctx, uint32_t thread_max_key, uint32_t l
 
 /* Index items of later launches of the context (prepared launches take the
  * value at ssj_multi_create; ssj_multi_autotune tunes it per launch): a probe
- * with at least min_cands candidates is verified by a whole thread block
+ * with at least min_cands candidates left by the signature test (among those
+ * that one warp of the plan kernel tests, about a thousand; values above 480
+ * count as 480) is verified by a whole thread block
  * that holds the probe set r as a bitmap over the token values in shared
  * memory (one bit per value: the launch's token values must stay below
  * 786,432, which frequency renumbering gives for vocabularies of that size;

@@ -78,6 +78,9 @@ struct Collection {
     uint64_t n_chunks = 0;
     uint32_t* d_toks = nullptr;  // n_chunks * 4 tokens
     uint2* d_desc = nullptr;
+    uint4* d_rec[kRecClasses] = {};  // records of class 0 .. rec_classes - 1
+    uint32_t rec_classes = 0;        // 0: no records (sets too long for a signature, or no memory)
+    double typical_len = 0;          // size-weighted mean set size
     bool renumbered = false;
     uint32_t max_len = 0;        // longest set
     uint32_t vocab = 0;          // largest token on the device + 1
@@ -365,6 +368,17 @@ uint32_t vflags(uint32_t f) {
     return v;
 }
 
+// Signature bits per token of a set of typical size (the size-weighted mean:
+// long sets have the most candidates) wanted of the two levels.
+constexpr double kFirstBits = 1.0, kSecondBits = 3.0;
+
+// The smallest record class with that many bits (the largest if none has).
+uint32_t record_class(double bits) {
+    uint32_t c = 0;
+    while (c + 1 < kRecClasses && rec_bits(c) < bits) ++c;
+    return c;
+}
+
 // The instance of one batch (arrays, output and count are filled by the caller).
 Instance make_instance(const ssj_batch* b, const Collection& R, const Collection& S, uint64_t n_cands) {
     Instance I;
@@ -377,6 +391,22 @@ Instance make_instance(const ssj_batch* b, const Collection& R, const Collection
     I.s_n_sets = S.n_sets;
     I.r_n_chunks = R.n_chunks;
     I.s_n_chunks = S.n_chunks;
+    // pairs are dropped by their records unless every pair is asked for, or a granularity is forced
+    // (which means every pair that the length filter leaves)
+    const uint32_t classes = std::min(R.rec_classes, S.rec_classes);
+    const uint32_t every = SSJ_EMIT_ALL | SSJ_FORCE_THREAD | SSJ_FORCE_WARP | SSJ_FORCE_BLOCK | SSJ_FORCE_LANE |
+                           SSJ_FORCE_INDEX;
+    if (classes && !(b->flags & every)) {
+        const double len = std::min(R.typical_len, S.typical_len);
+        const uint32_t c[2] = {std::min(record_class(kFirstBits * len), classes - 1),
+                               std::min(record_class(kSecondBits * len), classes - 1)};
+        for (int l = 0; l < 2; ++l) {
+            if (l == 1 && c[1] <= c[0]) break;  // the first level is as good
+            I.r_rec[l] = R.d_rec[c[l]];
+            I.s_rec[l] = S.d_rec[c[l]];
+            I.rec_sectors[l] = rec_sectors(c[l]);
+        }
+    }
     I.p = b->p;
     I.sim = (b->flags & SSJ_SIM_MASK) >> 8;
     switch (I.sim) {
@@ -391,6 +421,16 @@ Instance make_instance(const ssj_batch* b, const Collection& R, const Collection
     I.n_cands = n_cands;
     I.tile_base = 0;
     return I;
+}
+
+// Chunk partition of a launch's instances (t: sh.n_inst of them), once their total is known.
+void set_chunks(Instance* t, LaunchShape& sh, int num_sms) {
+    const uint32_t chunk = plan_chunk(sh.total_cands, num_sms);
+    sh.n_chunks = 0;
+    for (uint32_t i = 0; i < sh.n_inst; ++i) {
+        t[i].chunk_base = sh.n_chunks;
+        sh.n_chunks += chunks_of(t[i].n_probes, t[i].n_cands, chunk);
+    }
 }
 
 // The context's granularity policy for a launch whose collections' token
@@ -438,6 +478,12 @@ cudaEvent_t* profile_events(ssj_ctx* ctx) {
     cudaEvent_t* evs = &ctx->prof_ev[3 * ctx->prof_used];
     ctx->prof_used++;
     return evs;
+}
+
+void free_collection(Collection& c) {
+    cudaFree(c.d_toks);
+    cudaFree(c.d_desc);
+    for (uint4* r : c.d_rec) cudaFree(r);
 }
 
 bool triple_less(const ssj_triple& x, const ssj_triple& y) { return x.r != y.r ? x.r < y.r : x.s < y.s; }
@@ -536,10 +582,7 @@ extern "C" void ssj_destroy(ssj_ctx* ctx) {
             cudaStreamSynchronize(kv.second->stream);
         }
     if (ctx->n_pinned) release_l2(ctx);
-    for (auto& kv : ctx->colls) {
-        cudaFree(kv.second.d_toks);
-        cudaFree(kv.second.d_desc);
-    }
+    for (auto& kv : ctx->colls) free_collection(kv.second);
     cudaFree(ctx->ws);
     cudaFree(ctx->io);
     cudaFreeHost(ctx->h_count);
@@ -626,8 +669,12 @@ extern "C" ssj_status ssj_load_collection(ssj_ctx* ctx, const uint64_t* offsets,
     c.n_sets = n_sets;
     c.n_tokens = total;
     c.renumbered = (flags & SSJ_RENUMBER_BY_FREQ) != 0;
-    for (uint32_t i = 0; i < n_sets; ++i)
-        c.max_len = std::max<uint32_t>(c.max_len, (uint32_t)std::min<uint64_t>(offsets[i + 1] - offsets[i], 0xFFFFFFFFu));
+    double sum_sq = 0;
+    for (uint32_t i = 0; i < n_sets; ++i) {
+        const uint64_t len = offsets[i + 1] - offsets[i];
+        c.max_len = std::max<uint32_t>(c.max_len, (uint32_t)std::min<uint64_t>(len, 0xFFFFFFFFu));
+        sum_sq += (double)len * (double)len;
+    }
     for (uint64_t t = 0; t < total; ++t) c.vocab = std::max<uint32_t>(c.vocab, src[t] == 0xFFFFFFFFu ? src[t] : src[t] + 1);
     auto cleanup = [&]() {
         cudaFree(d_offs);
@@ -670,11 +717,24 @@ extern "C" ssj_status ssj_load_collection(ssj_ctx* ctx, const uint64_t* offsets,
         return fail(ctx, SSJ_ENOMEM, "collection: %s", cudaGetErrorString(e));
     }
     e = layout_scatter(d_offs, d_raw, n_sets, d_scratch, c.d_toks, c.d_desc, st, ctx->num_sms);
+    // records up to the class that the second level wants; none when even the largest has less than
+    // half a bit per token
+    c.typical_len = total ? sum_sq / (double)total : 0.0;
+    const uint32_t classes = n_sets && rec_bits(kRecClasses - 1) >= 0.5 * c.typical_len
+                                 ? record_class(kSecondBits * c.typical_len) + 1 : 0u;
+    for (uint32_t k = 0; k < classes && e == cudaSuccess; ++k) {
+        if (cudaMalloc(&c.d_rec[k], 32ull * rec_sectors(k) * n_sets) != cudaSuccess) {
+            cudaGetLastError();  // no memory: pairs are verified without this class
+            c.d_rec[k] = nullptr;
+            break;
+        }
+        e = build_records(reinterpret_cast<const uint4*>(c.d_toks), c.d_desc, n_sets, k, c.d_rec[k], st, ctx->num_sms);
+        c.rec_classes = k + 1;
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cleanup();
     if (e != cudaSuccess) {
-        cudaFree(c.d_toks);
-        cudaFree(c.d_desc);
+        free_collection(c);
         return cuda_fail(ctx, e, "layout_scatter");
     }
     if (flags & SSJ_PIN_L2) {
@@ -716,8 +776,7 @@ extern "C" ssj_status ssj_unload_collection(ssj_ctx* ctx, ssj_coll coll) {
     if (it->second.busy) return fail(ctx, SSJ_EBUSY, "collection %u is used by submitted batches", coll);
     DeviceGuard g(ctx->device);
     cudaStreamSynchronize(ctx->stream);
-    cudaFree(it->second.d_toks);
-    cudaFree(it->second.d_desc);
+    free_collection(it->second);
     if (it->second.l2_window && --ctx->n_pinned == 0) release_l2(ctx);
     ctx->colls.erase(it);
     return SSJ_OK;
@@ -893,6 +952,7 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
     sh.n_tiles = 0;
     sh.total_probes = 0;
     sh.total_cands = 0;
+    sh.n_chunks = 0;
     size_t off = align256(sizeof(uint64_t) * n_batches);  // counts first
     uint64_t launch_vocab = 1;
     bool launch_force_index = false;
@@ -950,6 +1010,7 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
         q.n_tiles = 0;
         q.total_probes = 0;
         q.total_cands = 0;
+        q.n_chunks = 0;
         for (uint32_t i = gstart[gi]; i < gstart[gi + 1]; ++i) {
             table[i].tile_base = q.n_tiles;
             q.n_inst += 1;
@@ -957,6 +1018,7 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
             q.total_probes += batches[i].n_probes;
             q.total_cands += n_cands[i];
         }
+        set_chunks(table.data() + gstart[gi], q, ctx->num_sms);
         ws_off[gi + 1] = ws_off[gi] + align256(workspace_bytes(q, ctx->num_sms));
     }
     const size_t ws_total = ws_off[groups];
@@ -1814,6 +1876,7 @@ extern "C" ssj_status ssj_multi_create(ssj_ctx* ctx, const ssj_batch* batches, u
     sh.n_tiles = 0;
     sh.total_probes = 0;
     sh.total_cands = 0;
+    sh.n_chunks = 0;
     std::unique_ptr<ssj_multi> m(new ssj_multi());
     uint64_t vocab = 1;
     const Collection* pinned = nullptr;  // the first pinned collection: its L2 window
@@ -1848,6 +1911,7 @@ extern "C" ssj_status ssj_multi_create(ssj_ctx* ctx, const ssj_batch* batches, u
         m->force_index = m->force_index || (b->flags & SSJ_FORCE_INDEX) != 0;
         if (!pinned) pinned = R->l2_window ? R : (S->l2_window ? S : nullptr);
     }
+    set_chunks(table.data(), sh, ctx->num_sms);
     DeviceGuard g(ctx->device);
     const size_t bytes = workspace_bytes(sh, ctx->num_sms);
     cudaError_t e = cudaMalloc(&m->ws, bytes);

@@ -1,0 +1,19 @@
+// Index checks of the checked build (SSJ_CHECKED), shared by the kernels.
+#pragma once
+
+#include <cstdint>
+
+#include "ssj_internal.h"
+
+namespace ssj {
+
+// Checked build: false, and ERR_BOUNDS set, when idx is not below n.
+__device__ __forceinline__ bool in_bounds(uint64_t idx, uint64_t n, uint32_t* err) {
+    if (kChecked && idx >= n) {
+        atomicOr(err, ERR_BOUNDS);
+        return false;
+    }
+    return true;
+}
+
+}  // namespace ssj

@@ -11,6 +11,7 @@
 //   1. len_kernel   - per set: length, 16-byte chunk count, sortedness check
 //   2. scan         - exclusive prefix sum of chunk counts (three kernels)
 //   3. scatter_kernel - one warp per set copies its tokens and the padding
+//   4. record_kernel  - one warp per set: its length, signature and loss
 #include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -119,7 +120,47 @@ __global__ void scatter_kernel(const uint64_t* __restrict__ offs, const uint32_t
     }
 }
 
+// One warp per set: the signature (a bit per token, at a multiplicative hash of
+// its value scaled to the bitmap) collected in shared memory, then the record
+// in whole 16-byte words.
+constexpr int kRecWarps = 8;
+__global__ void __launch_bounds__(kRecWarps * 32) record_kernel(const uint4* __restrict__ toks4,
+                                                                const uint2* __restrict__ desc, uint32_t n,
+                                                                uint32_t sectors, uint4* __restrict__ rec) {
+    __shared__ uint4 s_rec[kRecWarps][2 * rec_sectors(kRecClasses - 1)];
+    const uint32_t warps = gridDim.x * kRecWarps;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t* w = reinterpret_cast<uint32_t*>(s_rec[warp]);
+    const uint32_t words = 8 * sectors, bits = 32 * (words - 1);
+    for (uint32_t i = blockIdx.x * kRecWarps + warp; i < n; i += warps) {
+        const uint2 d = desc[i];
+        const uint32_t* t = reinterpret_cast<const uint32_t*>(toks4 + d.x);
+        for (uint32_t k = lane; k < words; k += 32) w[k] = 0u;
+        __syncwarp();
+        for (uint32_t k = lane; k < d.y; k += 32) {
+            const uint32_t b = __umulhi(t[k] * 0x9E3779B1u, bits);
+            atomicOr(w + 1 + (b >> 5), 1u << (b & 31u));
+        }
+        __syncwarp();
+        uint32_t set = 0;
+        for (uint32_t k = 1 + lane; k < words; k += 32) set += __popc(w[k]);
+        set = __reduce_add_sync(0xFFFFFFFFu, set);
+        if (lane == 0) w[0] = d.y >= 0xFFFFu ? 0xFFFF0000u : (d.y << 16) | (d.y - set);
+        __syncwarp();
+        if (lane < 2 * sectors) rec[(uint64_t)i * 2 * sectors + lane] = s_rec[warp][lane];
+        __syncwarp();
+    }
+}
+
 }  // namespace
+
+cudaError_t build_records(const uint4* toks4, const uint2* desc, uint32_t n, uint32_t c, uint4* rec, cudaStream_t st,
+                          int num_sms) {
+    if (n == 0) return cudaSuccess;
+    const unsigned blocks = (unsigned)std::min<uint64_t>(((uint64_t)n + kRecWarps - 1) / kRecWarps, (uint64_t)num_sms * 8);
+    record_kernel<<<blocks, kRecWarps * 32, 0, st>>>(toks4, desc, n, rec_sectors(c), rec);
+    return cudaGetLastError();
+}
 
 // Build the padded device layout from raw device copies of offsets/tokens.
 // Returns the number of 16-byte chunks via *n_chunks (host), after a sync.

@@ -33,6 +33,8 @@ enum : uint32_t {
 // threshold and output.  A launch verifies any number of instances; the
 // table of them lives in device memory (the workspace).
 struct Instance {
+    const uint4* r_rec[2];      // records of R and S for the two levels of the signature test
+    const uint4* s_rec[2];
     const uint4* r_toks4;
     const uint2* r_desc;
     const uint4* s_toks4;
@@ -45,6 +47,7 @@ struct Instance {
     uint64_t magic;             // div_magic(den) for Jaccard and Dice
     uint64_t n_cands;
     uint64_t cap;
+    uint64_t chunk_base;        // first candidate chunk of this instance in the launch (VerifyArgs::chunk)
     uint64_t r_n_chunks, s_n_chunks;  // 16-byte blocks of the token arrays (bounds of the checked build)
     uint32_t r_n_sets, s_n_sets;
     uint32_t p, den;            // t = p / q; den: see SIM_*
@@ -52,7 +55,19 @@ struct Instance {
     uint32_t tile_base;         // first plan tile (32 probes) of this instance
     uint32_t flags;             // VF_*
     uint32_t sim;               // SIM_*
+    uint32_t rec_sectors[2];    // their sizes in 32-byte sectors; 0: no such level (no first: the length filter alone)
 };
+
+// A set's record: a header word (length in the upper 16 bits, loss in the
+// lower: tokens that share a signature bit with another token of the set,
+// |x| - popcount), and a bitmap of hash values of its tokens in the remaining
+// bits.  A set of 65,535 tokens or more has length 65,535 and loss 0 there.
+// Records of class c take 1 << c sectors of 32 bytes; a collection has the
+// classes from 0 up to what its set sizes want, so that any two collections
+// share some.
+constexpr uint32_t kRecClasses = 4;
+constexpr uint32_t rec_sectors(uint32_t c) { return 1u << c; }
+constexpr uint32_t rec_bits(uint32_t c) { return rec_sectors(c) * 256u - 32u; }
 
 // Similarity function of an instance, and what den / magic hold for it.
 enum : uint32_t {
@@ -62,12 +77,12 @@ enum : uint32_t {
     SIM_OVERLAP = 3,  // den = ceil(p / q), the required overlap itself
 };
 
-// Work item for warp-, lane- or block-per-pair verification: n candidates of
-// probe set r starting at candidate index c0, in instance inst.  In the warp
-// list, mode 0 is one warp per pair, mode 1 one lane per pair (r in shared
-// memory).  In the block list, mode 0 is one thread block per pair, mode 1
-// an index item: the whole block holds r as a bitmap over the token values
-// and every thread verifies one candidate at a time against it.
+// Work item for lane- or block-per-pair verification: n queued pairs of
+// probe set r starting at pair list index c0, in instance inst.  The warp
+// list holds lane items (one lane per pair, r in shared memory).  In the
+// block list, mode 0 is one thread block per pair, mode 1 an index item: the
+// whole block holds r as a bitmap over the token values and every thread
+// verifies one candidate at a time against it.
 struct WorkItem {
     uint32_t r;
     uint32_t n;
@@ -76,22 +91,24 @@ struct WorkItem {
     uint32_t pad;  // mode
 };
 
-// One short pair of the compacted list: probe slot k (index into the
-// launch's per-probe arrays) and candidate set id s.  k == kNoProbe marks a
-// padding slot.
+// One queued pair: probe slot k (32 * its instance's tile_base + the probe's
+// index) and candidate set id s.  Short pairs grow from the front of the pair
+// list, the others from its back.
 struct PairRef {
     uint32_t k;
     uint32_t s;
 };
-constexpr uint32_t kNoProbe = 0xFFFFFFFFu;
+constexpr uint32_t kInItem = 0x80000000u;  // in s (set ids are below 2^31): a work item covers the pair
 
 // Per-call counters, cleared by one memset before the plan kernel.
 struct Counters {
-    unsigned long long thread_pairs;  // slots of the compacted short-pair list (multiple of 32)
-    unsigned long long warp_items;    // warp work items written by the plan kernel
+    unsigned long long thread_pairs;  // short pairs queued at the front of the pair list
+    unsigned long long long_pairs;    // other pairs, queued at its back
+    unsigned long long warp_items;    // lane work items written by the plan kernel
     unsigned long long block_items;   // block work items written by the plan kernel
     uint32_t block_cursor;            // dynamic cursors of the verify kernel
     uint32_t warp_cursor;
+    uint32_t long_cursor;
     uint32_t chunk_cursor;
     uint32_t err;                     // device-side check bits (see ssj_device_error)
 };
@@ -114,10 +131,12 @@ constexpr bool kChecked = true;
 constexpr bool kChecked = false;
 #endif
 
-constexpr uint32_t kWarpItemCands = 8;   // most candidates per warp work item
+constexpr uint32_t kWarpItemCands = 8;   // candidates per entry that the warp list's capacity allows for
 constexpr uint32_t kBlockItemCands = 16; // most candidates per block work item
 constexpr uint32_t kLaneItemCands = 128; // most candidates per lane work item
 constexpr uint32_t kLaneMinCands = 16;   // fewest candidates of a probe sent to the lane bin
+constexpr uint32_t kWarpRCap = 1024;     // r kept whole in a warp's shared memory up to this
+constexpr uint32_t kPlanFlush = 480;     // pairs left that a plan warp queues at once
 constexpr uint32_t kIndexMaxWords = 24576;  // largest probe bitmap (32-bit words, 96 KiB): token values below 786,432
 constexpr uint32_t kIndexItemCands = 8192;  // most candidates per index item
 
@@ -129,17 +148,16 @@ struct VerifyArgs {
     uint32_t n_inst;
     uint32_t n_tiles;             // plan tiles over all instances
     uint32_t total_probes;        // probe slots over all instances (instance-major)
+    uint32_t chunk;               // candidates per plan chunk (a warp's unit of work)
+    uint64_t n_chunks;            // over all instances
     uint64_t total_cands;
     Counters* ctr;
-    uint2* rdesc;                 // per probe slot: descriptor of its set r
-    uint32_t* rid;                // per probe slot: id of its set r
-    uint32_t* chunk_inst;         // per 32-slot chunk of the pair list: its instance
-    PairRef* pairs;               // compacted short pairs
+    PairRef* pairs;               // pairs left to verify: short ones from the front, others from the back
     WorkItem* warp_items;
     WorkItem* block_items;
     uint64_t pair_cap;
     uint32_t warp_item_cap, block_item_cap;
-    uint32_t warp_item_cands, block_item_cands;  // candidates per work item
+    uint32_t block_item_cands;    // candidates per work item
     uint32_t lane_item_cands;
     uint32_t thread_max_key;      // 2|r| <= this: one thread per pair
     uint32_t lane_max_key;        // 2|r| <= this (and r fits, >= kLaneMinCands candidates): one lane per pair
@@ -169,12 +187,19 @@ struct LaunchShape {
     uint32_t n_tiles;
     uint32_t total_probes;
     uint64_t total_cands;
+    uint64_t n_chunks;  // plan chunks over all instances (plan_chunk, chunks_of)
 };
+
+// Candidates per plan chunk of a launch, and the chunks of one instance.
+uint32_t plan_chunk(uint64_t total_cands, int num_sms);
+inline uint64_t chunks_of(uint64_t n_probes, uint64_t n_cands, uint32_t chunk) {
+    return n_probes ? (n_cands + chunk - 1) / chunk : 0;
+}
 
 // Scratch a launch of this shape needs, in bytes, on a device with num_sms SMs.
 size_t workspace_bytes(const LaunchShape& sh, int num_sms);
 // Shape of a one-batch launch.
-LaunchShape single_shape(uint32_t n_probes, uint64_t n_cands);
+LaunchShape single_shape(uint32_t n_probes, uint64_t n_cands, int num_sms);
 size_t workspace_bytes(uint32_t n_probes, uint64_t n_cands, int num_sms);
 
 // Carve the workspace and fill the scratch pointers of a.
@@ -196,6 +221,11 @@ cudaError_t prepare_verify(uint32_t block_threads, uint32_t index_words = 0);
 // verify, and after the verify kernel, on st.
 cudaError_t launch_verify(const VerifyArgs& a, cudaStream_t st, int num_sms, uint32_t block_threads,
                           cudaEvent_t* ev = nullptr);
+cudaError_t launch_plan(const VerifyArgs& a, cudaStream_t st, int num_sms);
+
+// Records of class c (rec_bits) of a laid-out collection, on st.
+cudaError_t build_records(const uint4* toks4, const uint2* desc, uint32_t n, uint32_t c, uint4* rec, cudaStream_t st,
+                          int num_sms);
 
 // Exclusive prefix sum of n 64-bit values in place on st; *total (device)
 // receives the sum.  scratch holds scan_scratch_words(n) values.

@@ -8,11 +8,12 @@
 //
 // How the work is laid out (the paper's Alternatives A-C of Section 3.3.2,
 // re-designed for one GB300):
-//   * plan_kernel, one thread per probe: validates the grouped candidate
-//     list and bins each probe by |r|+|s| (estimated as 2|r|; the length
-//     filter keeps |s| within [t|r|, |r|/t]).  Short probes append their
-//     pairs to a compacted (probe, candidate) list; longer probes become
-//     warp or block work items.  Space is reserved with one atomic per warp.
+//   * plan_kernel (plan.cu): validates the grouped candidate list, drops
+//     the pairs that their sets' signatures prove dissimilar and bins the
+//     others by their probe's |r|+|s| (estimated as 2|r|; the length filter
+//     keeps |s| within [t|r|, |r|/t]): pairs of short probes go to the front
+//     of one pair list, the others to its back, where a probe with several
+//     pairs left may become lane, block or index work items.
 //   * verify_kernel, persistent (one wave of CTAs over the SMs):
 //       phase 1 - block items: one CTA per pair, Intersect Path across the
 //                 whole CTA (Alternative C, Sections 4.2.2-4.2.3), r kept in
@@ -25,18 +26,16 @@
 //                 pair (Alternative B with the probe in shared memory,
 //                 Section 3.3.2; the s-side positional bound of Section
 //                 2.2.3 after every 16-byte block);
-//       phase 2 - warp items: one warp per pair, 32-lane merge path, r kept
-//                 in the warp's shared memory for the item's candidates;
-//       phase 3 - short pairs, one pair per thread (Alternatives A/B), 32
-//                 consecutive pairs of the compacted list per warp step.
+//       phase 2 - lane items: one candidate per lane, r in the warp's shared
+//                 memory; and long pairs: one warp per pair, 32-lane merge
+//                 path, r kept in the warp's shared memory while the next
+//                 pair has the same probe;
+//       phase 3 - short pairs, one pair per thread (Alternatives A/B).
 //                 The merge compares 16-byte blocks (4 tokens of r against
 //                 4 of s, 16 compares; the block with the smaller last token
-//                 advances).  Pass 1: every lane loads the first three blocks
-//                 of both sets and runs exactly three block steps, unrolled
-//                 and predicated, which decides most pairs (the positional
-//                 bound rejects them early).  Pass 2: undecided pairs are
-//                 parked with their merge state in a per-warp shared buffer
-//                 and finished 32 at a time by a loop.
+//                 advances).  Pairs wait with their merge state in a per-warp
+//                 shared buffer and are merged 32 at a time; a warp with too
+//                 few lanes still merging parks them again and refills.
 //     Heavy work goes first so that short pairs fill the tail.  The first
 //     unit of each phase is assigned statically (CTA / warp index), later
 //     ones through one atomic per unit, so small batches need no atomics.
@@ -46,12 +45,14 @@
 //   Survivors are compacted into (r, s, o) triples with warp-aggregated
 //   atomics on one global cursor (output select, Section 3.3.2), or only
 //   counted (output count).
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 #include <cstring>
 #include <cuda_runtime.h>
 
 #include "arith.h"
+#include "checked.cuh"
 #include "ssj_internal.h"
 
 namespace ssj {
@@ -61,14 +62,13 @@ namespace {
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr int kWarpD = 8;                          // merge steps per lane per window (warp)
 constexpr uint32_t kWarpWin = 32 * kWarpD;         // merge steps per window (warp)
-constexpr uint32_t kWarpRCap = 1024;               // r kept whole in a warp's shared memory up to this
 constexpr uint32_t kWarpABuf = kWarpRCap + 16;     // r buffer (whole r, or one window of it)
 constexpr uint32_t kWarpBBuf = kWarpWin + 16;      // s window buffer
 constexpr int kBlockD = 8;                         // merge steps per thread per window (block)
 constexpr uint32_t kBlockRCap = 4096;              // r kept whole in shared memory up to this
-constexpr uint32_t kFlatGrab = 4;                  // 32-pair chunks taken per dynamic grab in phase 3
+constexpr uint32_t kFlatGrab = 4;                  // most 32-pair chunks taken per dynamic grab in phase 3
+constexpr uint32_t kLongGrab = 8;                  // most long pairs taken per dynamic grab in phase 2
 constexpr uint32_t kCont = 64;                     // parked pairs per warp in phase 3
-constexpr int kPlanThreads = 256;                  // plan kernel block size
 
 // Checked build (SSJ_CHECKED): the functions that are not inlined take the
 // token arrays' remaining extents and the error word as extra arguments;
@@ -90,15 +90,6 @@ constexpr int kPlanThreads = 256;                  // plan kernel block size
 #define CHK_SLIM (~0ull)
 #define CHK_ERR (static_cast<uint32_t*>(nullptr))
 #endif
-
-// Checked build: false, and ERR_BOUNDS set, when idx is not below n.
-__device__ __forceinline__ bool in_bounds(uint64_t idx, uint64_t n, uint32_t* err) {
-    if (kChecked && idx >= n) {
-        atomicOr(err, ERR_BOUNDS);
-        return false;
-    }
-    return true;
-}
 
 // Block idx of a token array with lim blocks from base on (the checked
 // build reads zeros past the end).
@@ -176,7 +167,7 @@ __device__ __forceinline__ void bulk_stage(uint32_t* dst, const uint4* set4, uin
 
 // A parked pair with its merge state.
 struct ContEntry {
-    uint4 m0;  // probe slot (its r id is rid[slot]), s id, current 16-byte block of r, of s (token array indices)
+    uint4 m0;  // r id, s id, current 16-byte block of r, of s (token array indices)
     uint4 m1;  // tokens of r and of s from the current blocks on, required overlap, overlap so far
     uint4 m2;  // instance, unused, unused, unused
 };
@@ -439,7 +430,7 @@ __device__ uint32_t block_merge(const uint4* __restrict__ r4, uint32_t nr, const
     return o;
 }
 
-// Block step of pass 2 on a (block cursor, tokens remaining) state; the same
+// Block step of the short-pair phase on a (block cursor, tokens remaining) state; the same
 // step as block_step: positional bound, 16 compares between the current
 // blocks, then the block with the smaller last valid token advances (both on
 // a tie), predicated like block_step.  rn / sn hold the next block of each
@@ -471,22 +462,19 @@ __device__ __forceinline__ void lean_step(uint4& rc, uint4& rn, uint4& sc, uint4
     fin = fin || bad || remr == 0 || rems == 0;
 }
 
-// Pass 2 of the short-pair phase: the parked pairs [n_cont - m, n_cont) are
+// One step of the short-pair phase: the parked pairs [n_cont - m, n_cont) are
 // taken one per lane (lanes may belong to different instances) and merged
 // while at least min_live lanes are still undecided; decided pairs are
 // emitted, undecided ones parked again, compacted, so that lanes are refilled
 // from later pairs instead of idling behind the longest merge of the warp.
-// min_live = 1 finishes every pair.  A parked pair carries its probe slot;
-// the r id is read from it only for a survivor.  Returns the new number of
-// parked pairs.
+// min_live = 1 finishes every pair.  Returns the new number of parked pairs.
 __device__ __noinline__ uint32_t drain_parked(ContEntry* cont, uint32_t n_cont, uint32_t m, uint32_t min_live,
-                                              const Instance* table, const uint32_t* rid_of_slot,
-                                              int lane CHK_ERR_PARAM) {
+                                              const Instance* table, int lane CHK_ERR_PARAM) {
     const unsigned lt_mask = (1u << lane) - 1u;
     const uint4 zero4 = make_uint4(0, 0, 0, 0);
     const uint32_t base = n_cont - m;
     const bool have = (uint32_t)lane < m && in_bounds(base + lane, kCont, CHK_ERR);
-    uint32_t slot = 0, sid = 0, rcur = 0, scur = 0, remr = 0, rems = 0, req = 0, o = 0, inst = 0;
+    uint32_t rid = 0, sid = 0, rcur = 0, scur = 0, remr = 0, rems = 0, req = 0, o = 0, inst = 0;
     const uint4* rb = nullptr;
     const uint4* sb = nullptr;
     uint64_t rlim = 0, slim = 0;
@@ -495,7 +483,7 @@ __device__ __noinline__ uint32_t drain_parked(ContEntry* cont, uint32_t n_cont, 
     if (have) {
         const ContEntry* ce = cont + base + lane;
         const uint4 m0 = ce->m0, m1 = ce->m1, m2 = ce->m2;
-        slot = m0.x;
+        rid = m0.x;
         sid = m0.y;
         rcur = m0.z;
         scur = m0.w;
@@ -511,9 +499,9 @@ __device__ __noinline__ uint32_t drain_parked(ContEntry* cont, uint32_t n_cont, 
         slim = I.s_n_chunks;
         early = !(I.flags & VF_EMIT_ALL);
         fin = remr == 0 || rems == 0;
-        rc = ld_block(rb, rcur, rlim, CHK_ERR);
+        if (remr > 0) rc = ld_block(rb, rcur, rlim, CHK_ERR);
         if (remr > 4) rn = ld_block(rb, rcur + 1, rlim, CHK_ERR);
-        sc = ld_block(sb, scur, slim, CHK_ERR);
+        if (rems > 0) sc = ld_block(sb, scur, slim, CHK_ERR);
         if (rems > 4) sn = ld_block(sb, scur + 1, slim, CHK_ERR);
     }
     __syncwarp();  // every entry is read before any is written again
@@ -533,15 +521,14 @@ __device__ __noinline__ uint32_t drain_parked(ContEntry* cont, uint32_t n_cont, 
             if (lane == leader) b0 = atomicAdd(I.count, (unsigned long long)__popc(grp));
             b0 = __shfl_sync(grp, b0, leader);
             if (!(I.flags & VF_COUNT_ONLY))
-                emit_triple(I.out, I.cap, (I.flags & VF_SELF_JOIN) != 0, b0 + __popc(grp & lt_mask),
-                            rid_of_slot[slot], sid, o);
+                emit_triple(I.out, I.cap, (I.flags & VF_SELF_JOIN) != 0, b0 + __popc(grp & lt_mask), rid, sid, o);
         }
     }
     const bool again = have && !fin;
     const uint32_t amask = __ballot_sync(kFull, again);
     if (again) {
         ContEntry* ce = cont + base + __popc(amask & lt_mask);
-        ce->m0 = make_uint4(slot, sid, rcur, scur);
+        ce->m0 = make_uint4(rid, sid, rcur, scur);
         ce->m1 = make_uint4(remr, rems, req, o);
         ce->m2 = make_uint4(inst, 0u, 0u, 0u);
     }
@@ -571,12 +558,12 @@ struct WarpOut {
 
 // One lane item (Alternative B): the item's probe r is staged whole in the
 // warp's shared memory (rsm, 16-byte blocks), each lane verifies one of the
-// item's candidates at a time with the block merge, reading r's blocks from
+// item's pairs (run) at a time with the block merge, reading r's blocks from
 // shared memory and s's from global memory one block ahead; a lane that
 // finishes takes the item's next candidate.  Survivors are emitted with one
 // atomic per warp step.
-__device__ __noinline__ void lane_item(const Instance& I, const WorkItem& wi, uint32_t nr, const uint4* rsm, int lane,
-                          uint32_t* err) {
+__device__ __noinline__ void lane_item(const Instance& I, const WorkItem& wi, const PairRef* run, uint32_t nr,
+                                       const uint4* rsm, int lane, uint32_t* err) {
     const uint32_t flags = I.flags;
     const bool emit_all = (flags & VF_EMIT_ALL) != 0, early = !emit_all;
     const bool self_join = (flags & VF_SELF_JOIN) != 0;
@@ -598,28 +585,21 @@ __device__ __noinline__ void lane_item(const Instance& I, const WorkItem& wi, ui
         if (idle && cursor < wi.n) {
             const uint32_t my = cursor + __popc(idle & lt_mask);
             if (!active && my < wi.n) {
-                const uint32_t s = in_bounds(wi.c0 + my, I.n_cands, err) ? I.cand_ids[wi.c0 + my] : ~0u;
-                if (s >= I.s_n_sets) {
-                    atomicOr(err, ERR_CAND_ID);
-                } else if (!(self_join && s == wi.r)) {
-                    const uint2 ds = I.s_desc[s];
-                    const uint32_t q = required_overlap(I.sim, I.p, I.den, I.magic, nr, ds.y);
-                    if (emit_all || (nr + ds.y > 0 && q <= min(nr, ds.y))) {  // length filter
-                        active = true;
-                        s_id = s;
-                        ns = ds.y;
-                        req = q;
-                        sq = (ns + 3) >> 2;
-                        s4 = I.s_toks4 + ds.x;
-                        slim = I.s_n_chunks - ds.x;
-                        st.qi = st.qj = st.o = 0;
-                        st.rej = false;
-                        st.fin = nr == 0 || ns == 0;
-                        rc = rq ? rsm[0] : zero4;
-                        sc = sq ? ld_block(s4, 0, slim, err) : zero4;
-                        sn = sq > 1 ? ld_block(s4, 1, slim, err) : zero4;
-                    }
-                }
+                const uint32_t s = run[my].s & ~kInItem;
+                const uint2 ds = I.s_desc[s];
+                active = true;
+                s_id = s;
+                ns = ds.y;
+                req = required_overlap(I.sim, I.p, I.den, I.magic, nr, ns);
+                sq = (ns + 3) >> 2;
+                s4 = I.s_toks4 + ds.x;
+                slim = I.s_n_chunks - ds.x;
+                st.qi = st.qj = st.o = 0;
+                st.rej = false;
+                st.fin = nr == 0 || ns == 0;
+                rc = rq ? rsm[0] : zero4;
+                sc = sq ? ld_block(s4, 0, slim, err) : zero4;
+                sn = sq > 1 ? ld_block(s4, 1, slim, err) : zero4;
             }
             cursor += __popc(idle);
         }
@@ -680,7 +660,7 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// One index item: candidates [c0, c0 + n) of probe r, verified by every
+// One index item: wi.n queued pairs (run) of probe r, verified by every
 // thread of the CTA, one candidate per thread at a time.  r is held as a
 // bitmap over the token values (bm, all zero on entry and on return).  A
 // candidate s is merged against r from the s side: block by block (16
@@ -696,9 +676,9 @@ __device__ __forceinline__ void cp_async_wait() {
 // The walk is software-pipelined so that no thread waits on a load it has
 // just issued, and its common path is short.  Each warp prepares its
 // candidates 32 at a time: their ids are loaded, one round later their
-// descriptors, one round later again the required overlap and the length
-// filter decide which enter the warp's queue (shared memory), and the next
-// batch's ids are loaded in that same step.  A round is
+// descriptors, one round later again they enter the warp's queue (shared
+// memory) with their required overlap, and the next batch's ids are loaded
+// in that same step.  A round is
 // kIndexSteps walk steps followed by one maintenance step (preparation,
 // survivors out, idle lanes refilled from the queue).  In a walk step a lane
 // asks for one more block of s (cp.async into its own ring of kIndexRing
@@ -718,8 +698,8 @@ __device__ __forceinline__ uint32_t bm_test(const uint32_t* bm, uint32_t x, uint
 }
 
 template <int BT>
-__device__ __noinline__ void index_item(const Instance& I, const WorkItem& wi, uint32_t nr, const uint4* r4,
-                                        uint64_t rlim, uint32_t* bm, uint32_t n_words, uint4* rings,
+__device__ __noinline__ void index_item(const Instance& I, const WorkItem& wi, const PairRef* run, uint32_t nr,
+                                        const uint4* r4, uint64_t rlim, uint32_t* bm, uint32_t n_words, uint4* rings,
                                         uint4* queues, BlockSmem<BT>* sm, uint32_t* err) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const unsigned lt_mask = (1u << lane) - 1u;
@@ -729,26 +709,21 @@ __device__ __noinline__ void index_item(const Instance& I, const WorkItem& wi, u
     uint4* ring = rings + (size_t)tid * kIndexRing;
     uint4* queue = queues + (size_t)warp * kIndexQueue;
     // candidate preparation (warp-uniform stage: 0 takes 32 candidates, 1 loads descriptors,
-    // 2 filters and queues); queue cursors are free-running.  Warp w's first batch is
+    // 2 queues); queue cursors are free-running.  Warp w's first batch is
     // candidates [32w, 32w + 32): its ids and descriptors are loaded while r's bits are set,
     // so the walk starts one round after the item does; later batches are taken from the
     // item's cursor, which starts after the first batches.
     uint32_t pstage = 0, qhead = 0, qtail = 0;
     bool pdone = 32u * (BT / 32) >= wi.n;  // warp-uniform: no candidates left to take
     const uint32_t my0 = 32u * (uint32_t)warp + (uint32_t)lane;
-    bool p_ok = my0 < wi.n && in_bounds(wi.c0 + my0, I.n_cands, err);
-    uint32_t p_id = p_ok ? I.cand_ids[wi.c0 + my0] : 0u;
+    bool p_ok = my0 < wi.n;
+    uint32_t p_id = p_ok ? run[my0].s & ~kInItem : 0u;
     uint2 p_desc = make_uint2(0u, 0u);
     if (tid == 0) sm->next = 32u * (BT / 32);
     bm_mark<BT>(bm, r4, nr, rlim, n_words, false, tid, err);
     // r's last token (the padding repeats it in the last block's last lane)
     const uint32_t rmax = nr ? ld_block(r4, (nr - 1) >> 2, rlim, err).w : 0u;
     if (32u * (uint32_t)warp < wi.n) {  // warp-uniform: the first batch's descriptors
-        if (p_ok && p_id >= I.s_n_sets) {
-            atomicOr(err, ERR_CAND_ID);
-            p_ok = false;
-        }
-        if (p_ok && self_join && p_id == wi.r) p_ok = false;
         if (p_ok) p_desc = I.s_desc[p_id];
         pstage = 2;
     }
@@ -806,20 +781,11 @@ __device__ __noinline__ void index_item(const Instance& I, const WorkItem& wi, u
         // ---- preparation (a batch queued here makes room for the next one to be taken in the
         // same step, so a batch is taken every second round)
         if (pstage == 1) {
-            if (p_ok && p_id >= I.s_n_sets) {
-                atomicOr(err, ERR_CAND_ID);
-                p_ok = false;
-            }
-            if (p_ok && self_join && p_id == wi.r) p_ok = false;
             if (p_ok) p_desc = I.s_desc[p_id];
             pstage = 2;
         } else {
             if (pstage == 2) {
-                uint32_t q = 0;
-                if (p_ok) {
-                    q = required_overlap(I.sim, I.p, I.den, I.magic, nr, p_desc.y);
-                    p_ok = emit_all || (nr + p_desc.y > 0 && q <= min(nr, p_desc.y));  // length filter
-                }
+                const uint32_t q = p_ok ? required_overlap(I.sim, I.p, I.den, I.magic, nr, p_desc.y) : 0u;
                 const uint32_t m = __ballot_sync(kFull, p_ok);
                 if (p_ok) queue[(qtail + __popc(m & lt_mask)) % kIndexQueue] = make_uint4(p_id, p_desc.x, p_desc.y, q);
                 qtail += __popc(m);
@@ -833,8 +799,8 @@ __device__ __noinline__ void index_item(const Instance& I, const WorkItem& wi, u
                     base = __shfl_sync(kFull, base, 0);
                     if (base + 32 >= wi.n) pdone = true;
                     const uint32_t my = base + (uint32_t)lane;
-                    p_ok = my < wi.n && in_bounds(wi.c0 + my, I.n_cands, err);
-                    if (p_ok) p_id = I.cand_ids[wi.c0 + my];
+                    p_ok = my < wi.n;
+                    if (p_ok) p_id = run[my].s & ~kInItem;
                     if (base < wi.n) pstage = 1;
                 }
             }
@@ -872,289 +838,22 @@ __device__ __noinline__ void index_item(const Instance& I, const WorkItem& wi, u
     __syncthreads();
 }
 
-// Granularity of a probe with |r| = nr and n candidates: 0 thread per pair,
-// 1 warp per pair, 2 block per pair, 3 lane per pair with r in the warp's
-// shared memory (Alternative B; needs r to fit and enough candidates to
-// occupy the lanes), 4 index items (probes with many candidates, when the
-// launch's token values fit the probe bitmap).
-__device__ __forceinline__ uint32_t probe_bin(const VerifyArgs& a, uint32_t flags, uint32_t nr, uint64_t n) {
-    const bool lane_ok = nr + 4 <= kWarpRCap;
-    if (flags & VF_FORCE_INDEX) return a.index_words ? 4u : (lane_ok ? 3u : 1u);
-    if (flags & VF_FORCE_BLOCK) return 2;
-    if (flags & VF_FORCE_WARP) return 1;
-    if (flags & VF_FORCE_THREAD) return 0;
-    if (flags & VF_FORCE_LANE) return lane_ok ? 3u : 1u;
-    if (a.index_words && a.index_min_cands && n >= a.index_min_cands) return 4;
-    const uint64_t key = 2ull * nr;  // |r|+|s| at |s| = |r|
-    if (key <= a.thread_max_key) return 0;
-    if (key <= a.lane_max_key && lane_ok && n >= kLaneMinCands) return 3;
-    return key <= a.warp_max_key ? 1u : 2u;
-}
-
-// Instance fields read by the plan kernel (from the kernel parameters for a
-// one-batch launch, else from the device table).
-struct PlanInst {
-    const uint32_t* probe_ids;
-    const uint64_t* cand_offsets;
-    const uint32_t* cand_ids;
-    const uint2* r_desc;
-    uint64_t n_cands;
-    uint32_t r_n_sets, n_probes, tile_base, flags;
-};
-
-__device__ __forceinline__ PlanInst plan_inst(const VerifyArgs& a, uint32_t i) {
-    PlanInst q;
-    if (a.table) {
-        const Instance* I = a.table + i;
-        q.probe_ids = I->probe_ids;
-        q.cand_offsets = I->cand_offsets;
-        q.cand_ids = I->cand_ids;
-        q.r_desc = I->r_desc;
-        q.n_cands = I->n_cands;
-        q.r_n_sets = I->r_n_sets;
-        q.n_probes = I->n_probes;
-        q.tile_base = I->tile_base;
-        q.flags = I->flags;
-    } else {
-        q.probe_ids = a.single.probe_ids;
-        q.cand_offsets = a.single.cand_offsets;
-        q.cand_ids = a.single.cand_ids;
-        q.r_desc = a.single.r_desc;
-        q.n_cands = a.single.n_cands;
-        q.r_n_sets = a.single.r_n_sets;
-        q.n_probes = a.single.n_probes;
-        q.tile_base = a.single.tile_base;
-        q.flags = a.single.flags;
+// Instance of a probe slot: the last one whose first tile is not past it.
+__device__ __forceinline__ uint32_t instance_of(const Instance* table, uint32_t n_inst, uint32_t slot) {
+    uint32_t lo = 0, hi = n_inst - 1;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (table[mid].tile_base <= slot >> 5) lo = mid; else hi = mid - 1;
     }
-    return q;
+    return lo;
 }
 
 }  // namespace
 
 // -------------------------------------------------------------------------
-// Plan.  The probes of every instance are cut into tiles of 32; warp w takes
-// tiles w, w + n_warps, ...  Lane l of tile t of an instance with T tiles
-// takes probe t + l*T, so a warp's 32 probes are spread over the instance and
-// warps get similar amounts of copying even when probes come in size order.
-// Each probe is validated and binned; short probes append their pairs to
-// the compacted list (a warp's range is padded to whole 32-slot chunks, so
-// a chunk never mixes instances), longer probes become work items.
-// -------------------------------------------------------------------------
-__global__ void __launch_bounds__(kPlanThreads) plan_kernel(VerifyArgs a) {
-    constexpr int kPlanWarps = kPlanThreads / 32;
-    // per-warp list sizes and the CTA's list bases, double-buffered by round
-    // parity so that a warp one round ahead never overwrites what others read
-    __shared__ unsigned long long s_tot[2][3][kPlanWarps];
-    __shared__ unsigned long long s_base[2][3];
-    // each warp's tile, for the copy of the short pairs by the whole CTA
-    __shared__ unsigned long long s_incl[2][kPlanWarps][32];  // inclusive prefix of the lanes' short pairs
-    __shared__ unsigned long long s_c0[2][kPlanWarps][32];    // the lanes' first candidates
-    __shared__ uint32_t s_slot[2][kPlanWarps][32];            // the lanes' probe slots
-    __shared__ unsigned long long s_pre[2][kPlanWarps + 1];   // exclusive prefix of the tiles' padded ranges
-    __shared__ const uint32_t* s_cand[2][kPlanWarps];         // the tiles' candidate arrays
-    __shared__ unsigned long long s_ncand[2][kPlanWarps];     // their lengths (checked build)
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    if (blockIdx.x == 0) {
-        if (!a.table && threadIdx.x == 0) a.table_out[0] = a.single;
-        for (uint32_t i = threadIdx.x; i < a.n_inst; i += blockDim.x)
-            *(a.table ? a.table[i].count : a.single.count) = 0ull;
-    }
-    // Rounds are uniform over the CTA: warp w of the CTA takes tile g0 + w.
-    // The three lists (short pairs, warp/lane items, block items) are
-    // reserved with one atomic per CTA and round, not per warp.
-    // With few tiles a CTA takes fewer than one per warp, so that more CTAs
-    // share the copying.
-    const uint32_t per_round =
-        a.n_tiles >= gridDim.x * (uint32_t)kPlanWarps ? kPlanWarps : max(1u, (a.n_tiles + gridDim.x - 1) / gridDim.x);
-    uint32_t par = 0;
-    for (uint32_t g0 = blockIdx.x * per_round; g0 < a.n_tiles; g0 += gridDim.x * per_round, par ^= 1u) {
-        const uint32_t g = g0 + (uint32_t)warp;
-        const bool tile_ok = (uint32_t)warp < per_round && g < a.n_tiles;
-        // instance owning tile g: the last one whose tile_base <= g
-        uint32_t inst = 0;
-        if (a.table) {
-            uint32_t lo = 0, hi = a.n_inst - 1;
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi + 1) >> 1;
-                if (a.table[mid].tile_base <= g) lo = mid; else hi = mid - 1;
-            }
-            inst = lo;
-        }
-        const PlanInst I = plan_inst(a, inst);
-        const uint32_t T = (I.n_probes + 31) >> 5;
-        const uint32_t t = g - I.tile_base;
-        const uint32_t k = t + (uint32_t)lane * T;           // local probe index
-        const uint32_t slot = I.tile_base * 32u + (uint32_t)lane * T + t;  // probe slot, unique per launch
-        uint64_t c0 = 0, n = 0;
-        uint32_t r = 0, bin = 0;
-        uint2 rdesc = make_uint2(0, 0);
-        if (tile_ok && k < I.n_probes) {
-            c0 = I.cand_offsets[k];
-            const uint64_t c1 = I.cand_offsets[k + 1];
-            if ((k == 0 && c0 != 0) || (k + 1 == I.n_probes && c1 != I.n_cands) || c1 < c0 || c1 > I.n_cands) {
-                atomicOr(&a.ctr->err, ERR_OFFSETS);
-            } else {
-                r = I.probe_ids[k];
-                if (r >= I.r_n_sets) {
-                    if (c1 > c0) atomicOr(&a.ctr->err, ERR_PROBE_ID);
-                } else {
-                    rdesc = I.r_desc[r];
-                    if (in_bounds(slot, 32ull * a.n_tiles + 1, &a.ctr->err)) {
-                        a.rdesc[slot] = rdesc;
-                        a.rid[slot] = r;
-                    }
-                    n = c1 - c0;
-                    bin = probe_bin(a, I.flags, rdesc.y, n);
-                }
-            }
-        }
-        // short probes: the warp's pairs form one contiguous, chunk-aligned range
-        // of the list; it is copied flat and coalesced, each slot finding its probe
-        // by a search over the lanes' prefix sums
-        const unsigned long long tn = (bin == 0) ? n : 0;
-        unsigned long long tincl = tn;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned long long y = __shfl_up_sync(kFull, tincl, off);
-            if (lane >= off) tincl += y;
-        }
-        const unsigned long long ttotal = __shfl_sync(kFull, tincl, 31);
-        const unsigned long long tpadded = (ttotal + 31) & ~31ull;
-        // work item counts (lane items share the warp item list, marked by mode 1)
-        const uint32_t wc = bin == 3 ? a.lane_item_cands : a.warp_item_cands;
-        const uint32_t bc = bin == 4 ? a.index_item_cands : a.block_item_cands;
-        const unsigned long long wn = (bin == 1 || bin == 3) ? (n + wc - 1) / wc : 0;
-        const unsigned long long bn = (bin == 2 || bin == 4) ? (n + bc - 1) / bc : 0;
-        unsigned long long wincl = wn, bincl = bn;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const unsigned long long yw = __shfl_up_sync(kFull, wincl, off);
-            const unsigned long long yb = __shfl_up_sync(kFull, bincl, off);
-            if (lane >= off) { wincl += yw; bincl += yb; }
-        }
-        if (lane == 31) {
-            s_tot[par][0][warp] = tpadded;
-            s_tot[par][1][warp] = wincl;
-            s_tot[par][2][warp] = bincl;
-        }
-        __syncthreads();
-        if (threadIdx.x < 3) {
-            unsigned long long sum = 0;
-#pragma unroll
-            for (int w = 0; w < kPlanWarps; ++w) sum += s_tot[par][threadIdx.x][w];
-            unsigned long long* ctr = threadIdx.x == 0 ? &a.ctr->thread_pairs
-                                                       : (threadIdx.x == 1 ? &a.ctr->warp_items : &a.ctr->block_items);
-            s_base[par][threadIdx.x] = sum ? atomicAdd(ctr, sum) : 0ull;
-        }
-        __syncthreads();
-        unsigned long long tbase0 = s_base[par][0], wbase = s_base[par][1], bbase = s_base[par][2];
-        for (int w = 0; w < warp; ++w) {
-            tbase0 += s_tot[par][0][w];
-            wbase += s_tot[par][1][w];
-            bbase += s_tot[par][2][w];
-        }
-        wbase += wincl - wn;  // this lane's first item
-        bbase += bincl - bn;
-        // short pairs: the CTA's tiles have one contiguous, chunk-aligned range of
-        // the list (warp order); all its threads copy it flat and coalesced, each
-        // slot finding its tile by the prefix of the tiles' ranges and its probe
-        // by a search over that tile's lane prefix sums
-        s_incl[par][warp][lane] = tincl;
-        s_c0[par][warp][lane] = c0;
-        s_slot[par][warp][lane] = slot;
-        if (lane == 0) s_cand[par][warp] = I.cand_ids;
-        if (kChecked && lane == 0) s_ncand[par][warp] = I.n_cands;
-        if (threadIdx.x == 0) {
-            unsigned long long acc = 0;
-            for (int w = 0; w < kPlanWarps; ++w) {
-                s_pre[par][w] = acc;
-                acc += s_tot[par][0][w];
-            }
-            s_pre[par][kPlanWarps] = acc;
-        }
-        if (tpadded && tbase0 + tpadded > a.pair_cap) {  // cannot happen with a sized workspace
-            if (lane == 0) atomicOr(&a.ctr->err, ERR_GUARD);
-        } else {
-            for (unsigned long long c = lane; c < tpadded / 32; c += 32) a.chunk_inst[tbase0 / 32 + c] = inst;
-        }
-        __syncthreads();
-        {
-            const unsigned long long cta_base = s_base[par][0], cta_total = s_pre[par][kPlanWarps];
-            if (cta_base + cta_total <= a.pair_cap) {
-                // each thread writes 4 consecutive slots (cta_total is a multiple of
-                // 32, so all 4 exist): it locates the first by binary search and
-                // follows the tile and probe boundaries for the other three
-                for (unsigned long long f0 = 4ull * threadIdx.x; f0 < cta_total; f0 += 4ull * kPlanThreads) {
-                    int w = 0;
-#pragma unroll
-                    for (int step = kPlanWarps / 2; step >= 1; step >>= 1)
-                        if (s_pre[par][w + step] <= f0) w += step;
-                    uint32_t pos = 0, out[8];
-                    bool located = false;
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const unsigned long long f = f0 + e;
-                        while (f >= s_pre[par][w + 1]) {  // into the next tile with slots
-                            ++w;
-                            located = false;
-                        }
-                        const unsigned long long fl = f - s_pre[par][w];
-                        out[2 * e] = kNoProbe;
-                        out[2 * e + 1] = 0u;
-                        if (fl < s_incl[par][w][31]) {
-                            if (!located) {
-                                pos = 0;
-#pragma unroll
-                                for (int step = 16; step >= 1; step >>= 1)
-                                    if (s_incl[par][w][pos + step - 1] <= fl) pos += step;
-                                located = true;
-                            } else {
-                                while (s_incl[par][w][pos] <= fl) ++pos;  // past probes that end before fl
-                            }
-                            const unsigned long long ex = pos ? s_incl[par][w][pos - 1] : 0ull;
-                            const unsigned long long ci = s_c0[par][w][pos] + (fl - ex);
-                            out[2 * e] = s_slot[par][w][pos];
-                            out[2 * e + 1] =
-                                in_bounds(ci, kChecked ? s_ncand[par][w] : 0ull, &a.ctr->err) ? s_cand[par][w][ci] : 0u;
-                        }
-                    }
-                    uint4* dst = reinterpret_cast<uint4*>(a.pairs + cta_base + f0);
-                    dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
-                    dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
-                }
-            }
-        }
-        // longer probes: work items of up to warp_item_cands / lane_item_cands /
-        // block_item_cands candidates
-        for (unsigned long long it = 0; it < wn; ++it) {
-            if (wbase + it >= a.warp_item_cap) { atomicOr(&a.ctr->err, ERR_GUARD); break; }
-            const uint64_t s0 = c0 + it * wc;
-            WorkItem wi;
-            wi.r = r;
-            wi.n = (uint32_t)min((uint64_t)wc, c0 + n - s0);
-            wi.c0 = s0;
-            wi.inst = inst;
-            wi.pad = bin == 3 ? 1u : 0u;
-            a.warp_items[wbase + it] = wi;
-        }
-        for (unsigned long long it = 0; it < bn; ++it) {
-            if (bbase + it >= a.block_item_cap) { atomicOr(&a.ctr->err, ERR_GUARD); break; }
-            const uint64_t s0 = c0 + it * bc;
-            WorkItem bi;
-            bi.r = r;
-            bi.n = (uint32_t)min((uint64_t)bc, c0 + n - s0);
-            bi.c0 = s0;
-            bi.inst = inst;
-            bi.pad = bin == 4 ? 1u : 0u;
-            a.block_items[bbase + it] = bi;
-        }
-    }
-}
-
-// -------------------------------------------------------------------------
 // Persistent verification kernel.  Instance fields come from the device table
-// (table_out), loaded once per work item or per 32-pair chunk.
+// (table_out).  The queued pairs' ids are valid and no pair is a set with
+// itself (the plan kernel's checks).
 // -------------------------------------------------------------------------
 // MINB: CTAs per SM the registers are budgeted for (1024 / BT: 64 registers
 // per thread; fewer CTAs leave more registers per thread).
@@ -1175,15 +874,22 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
 
     if (a.ctr->err & (ERR_OFFSETS | ERR_GUARD)) return;  // the plan is not trustworthy
 
-    // Static first-round assignment: phase 1 takes CTAs [0, n_bs); phase 2 starts
-    // on the warps after those, phase 3 on the warps after phase 2's, so a small
-    // batch spreads over idle warps at once.  Later rounds are dynamic.
+    // Static first-round assignment: phase 1 takes CTAs [0, n_bs); lane items start
+    // on the warps after those, long pairs on the warps after these, short pairs on the
+    // rest, so a small batch spreads over idle warps at once.  Later rounds are dynamic.
     const unsigned long long n_block = min(a.ctr->block_items, (unsigned long long)a.block_item_cap);
     const unsigned long long n_warp = min(a.ctr->warp_items, (unsigned long long)a.warp_item_cap);
+    const unsigned long long n_long = min(a.ctr->long_pairs, (unsigned long long)a.pair_cap);
+    const unsigned long long n_pairs = min(a.ctr->thread_pairs, (unsigned long long)a.pair_cap);
     const uint32_t n_bs = (uint32_t)min(n_block, (unsigned long long)gridDim.x);
     const uint32_t free2 = n_bs * kWarps;
     const uint32_t slots2 = n_warps_total - free2;
-    const uint32_t free3 = free2 + (uint32_t)min(n_warp, (unsigned long long)slots2);
+    // units of the pair lists: few pairs spread over the warps, many go several to a grab
+    const uint32_t long_grab = (uint32_t)max(1ull, min(n_long / (4ull * n_warps_total), (unsigned long long)kLongGrab));
+    const unsigned long long long_units = (n_long + long_grab - 1) / long_grab;
+    const uint32_t freel = free2 + (uint32_t)min(n_warp, (unsigned long long)slots2);
+    const uint32_t slotsl = n_warps_total - freel;
+    const uint32_t free3 = freel + (uint32_t)min(long_units, (unsigned long long)slotsl);
     const uint32_t slots3 = n_warps_total - free3;
 
     // ---------------- phase 1: block-per-pair items ----------------------
@@ -1224,7 +930,8 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
                     bm_zero = true;
                 }
                 uint4* rings = reinterpret_cast<uint4*>(bm + a.index_words);
-                index_item<BT>(I, bi, nr, r4, I.r_n_chunks - dr.x, bm, a.index_words, rings, rings + BT * kIndexRing,
+                if (!in_bounds(bi.c0 + bi.n - 1, a.pair_cap, &a.ctr->err)) continue;
+                index_item<BT>(I, bi, a.pairs + bi.c0, nr, r4, I.r_n_chunks - dr.x, bm, a.index_words, rings, rings + BT * kIndexRing,
                                &bsm, &a.ctr->err);
                 continue;
             }
@@ -1235,14 +942,10 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
             // copy into buffer m & 1 (wr / ws), issued while the previous candidate merges
             const bool bulk = a.bulk_stage && r_staged;
             uint32_t* sbuf[2] = {wr, ws};
-            // thread 0: stage candidate m's s if it will be merged and fits a buffer
+            // thread 0: stage candidate m's s if it fits a buffer
             auto prefetch = [&](uint32_t m) -> uint32_t {
-                if (m >= bi.n || !in_bounds(bi.c0 + m, I.n_cands, &a.ctr->err)) return 0u;
-                const uint32_t sx = I.cand_ids[bi.c0 + m];
-                if (sx >= I.s_n_sets || (self_join && sx == bi.r)) return 0u;
-                const uint2 dx = I.s_desc[sx];
-                const uint32_t rq = required_overlap(I.sim, I.p, I.den, I.magic, nr, dx.y);
-                if (!emit_all && (nr + dx.y == 0 || rq > min(nr, dx.y))) return 0u;
+                if (m >= bi.n || !in_bounds(bi.c0 + m, a.pair_cap, &a.ctr->err)) return 0u;
+                const uint2 dx = I.s_desc[a.pairs[bi.c0 + m].s & ~kInItem];
                 if (dx.y == 0 || dx.y + 4 > kBlockWin + 16) return 0u;
                 bulk_stage(sbuf[m & 1], I.s_toks4 + dx.x, 0u, (dx.y + 3) >> 2, I.s_n_chunks - dx.x,
                            (kBlockWin + 16) / 4, &bsm.bar[1 + (m & 1)], &a.ctr->err);
@@ -1282,17 +985,11 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
                     __syncthreads();
                     if (s_whole && !bsm.ok) return;  // (uniform) reported, the CTA stops
                 }
-                if (!in_bounds(bi.c0 + m, I.n_cands, &a.ctr->err)) break;
-                const uint32_t s = I.cand_ids[bi.c0 + m];
-                if (s >= I.s_n_sets) {
-                    if (tid == 0) atomicOr(&a.ctr->err, ERR_CAND_ID);
-                    continue;
-                }
-                if (self_join && s == bi.r) continue;
+                if (!in_bounds(bi.c0 + m, a.pair_cap, &a.ctr->err)) break;
+                const uint32_t s = a.pairs[bi.c0 + m].s & ~kInItem;
                 const uint2 ds = I.s_desc[s];
                 const uint32_t ns = ds.y;
                 const uint32_t req = required_overlap(I.sim, I.p, I.den, I.magic, nr, ns);
-                if (!emit_all && (nr + ns == 0 || req > min(nr, ns))) continue;  // length filter
                 bool rej;
                 const uint32_t o = block_merge<BT>(r4, nr, I.s_toks4 + ds.x, ns, req, early, rbuf, r_staged, wr,
                                                    bulk ? sbuf[m & 1] : ws, s_whole, &bsm, &rej
@@ -1319,8 +1016,8 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
         }
     }
 
-    // ---------------- phase 2: warp-per-pair items -----------------------
-    if (n_warp) {
+    // ---------------- phase 2: lane items, then long pairs, one per warp --
+    if (n_warp || n_long) {
         WarpOut wout;
         uint32_t* abuf = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(smem) + warp * kWarpSliceBytes);
         uint32_t* bbuf = abuf + kWarpABuf;
@@ -1331,7 +1028,25 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
             if (lane == 0) mbar_init(wbar, 1);
             __syncwarp();
         }
-        for (uint32_t round = 0;; ++round) {
+        // r whole into abuf: by one bulk copy that lane 0 waits for, or by the lanes; false if the copy
+        // did not complete (reported)
+        auto stage_r = [&](const uint4* r4, uint32_t nr, uint64_t rlim) -> bool {
+            __syncwarp();  // abuf reuse
+            if (wbar) {
+                uint32_t ok = 1;
+                if (lane == 0) {
+                    bulk_stage(abuf, r4, 0u, (nr + 3) >> 2, rlim, kWarpABuf / 4, wbar, &a.ctr->err);
+                    ok = mbar_wait(wbar, wph, &a.ctr->err) ? 1u : 0u;
+                }
+                wph ^= 1u;
+                if (!__shfl_sync(kFull, ok, 0)) return false;
+            } else {
+                stage<32>(r4, 0, nr, abuf, lane, rlim, kWarpABuf / 4, &a.ctr->err);
+            }
+            __syncwarp();
+            return true;
+        };
+        for (uint32_t round = 0; n_warp; ++round) {
             uint32_t it = 0;
             if (lane == 0) {
                 if (round == 0 && gwarp >= free2) it = gwarp - free2;
@@ -1342,77 +1057,74 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
             const WorkItem wi = a.warp_items[it];
             if (!in_bounds(wi.inst, a.n_inst, &a.ctr->err)) continue;  // (uniform over the warp)
             const Instance& I = table[wi.inst];
-            const uint32_t flags = I.flags;
-            const bool emit_all = (flags & VF_EMIT_ALL) != 0, early = !emit_all;
-            const bool self_join = (flags & VF_SELF_JOIN) != 0;
             if (!in_bounds(wi.r, I.r_n_sets, &a.ctr->err)) continue;
-            const uint2 dr = I.r_desc[wi.r];
-            const uint32_t nr = dr.y;
-            const uint4* r4 = I.r_toks4 + dr.x;
-            const bool r_staged = nr + 4 <= kWarpRCap;
-            if (r_staged && wbar) {  // r by one bulk copy, lane 0 waits
-                uint32_t ok = 1;
-                if (lane == 0) {
-                    bulk_stage(abuf, r4, 0u, (nr + 3) >> 2, I.r_n_chunks - dr.x, kWarpABuf / 4, wbar, &a.ctr->err);
-                    ok = mbar_wait(wbar, wph, &a.ctr->err) ? 1u : 0u;
-                }
-                wph ^= 1u;
-                if (!__shfl_sync(kFull, ok, 0)) return;  // reported; the warp stops
-                __syncwarp();
-            } else if (r_staged) {
-                stage<32>(r4, 0, nr, abuf, lane, I.r_n_chunks - dr.x, kWarpABuf / 4, &a.ctr->err);
-                __syncwarp();
+            if (!in_bounds(wi.c0 + wi.n - 1, a.pair_cap, &a.ctr->err)) continue;
+            const uint2 dr = I.r_desc[wi.r];  // (lane items are made of probes that fit abuf)
+            if (!stage_r(I.r_toks4 + dr.x, dr.y, I.r_n_chunks - dr.x)) return;  // the warp stops
+            lane_item(I, wi, a.pairs + wi.c0, dr.y, reinterpret_cast<const uint4*>(abuf), lane, &a.ctr->err);
+        }
+        for (uint32_t round = 0; n_long; ++round) {
+            uint32_t u = 0;
+            if (lane == 0) {
+                if (round == 0 && gwarp >= freel) u = gwarp - freel;
+                else u = slotsl + atomicAdd(&a.ctr->long_cursor, 1u);
             }
-            if (wi.pad == 1 && r_staged) {
-                lane_item(I, wi, nr, reinterpret_cast<const uint4*>(abuf), lane, &a.ctr->err);
-                __syncwarp();  // abuf reuse
-                continue;
-            }
-            for (uint32_t m = 0; m < wi.n; ++m) {
-                if (!in_bounds(wi.c0 + m, I.n_cands, &a.ctr->err)) break;
-                const uint32_t s = I.cand_ids[wi.c0 + m];
-                if (s >= I.s_n_sets) {
-                    if (lane == 0) atomicOr(&a.ctr->err, ERR_CAND_ID);
-                    continue;
+            u = __shfl_sync(kFull, u, 0);
+            if (u >= long_units) break;
+            const unsigned long long first = a.pair_cap - n_long + (unsigned long long)u * long_grab;
+            const unsigned long long end = min(first + long_grab, (unsigned long long)a.pair_cap);
+            uint32_t held = 0, inst = 0;  // slot + 1 of the r in abuf
+            for (unsigned long long m = first; m < end; ++m) {
+                const PairRef pr = a.pairs[m];
+                if (pr.s & kInItem) continue;
+                const uint32_t i = a.n_inst > 1 ? instance_of(table, a.n_inst, pr.k) : 0u;
+                if (wout.n && i != inst) wout.flush(table[inst], lane);
+                inst = i;
+                const Instance& I = table[inst];
+                const bool early = !(I.flags & VF_EMIT_ALL);
+                const uint32_t r = I.probe_ids[pr.k - 32u * I.tile_base];
+                if (!in_bounds(r, I.r_n_sets, &a.ctr->err)) continue;
+                const uint2 dr = I.r_desc[r], ds = I.s_desc[pr.s];
+                const uint32_t nr = dr.y, ns = ds.y;
+                const uint4* r4 = I.r_toks4 + dr.x;
+                const bool r_staged = nr + 4 <= kWarpRCap;
+                if (r_staged && held != pr.k + 1) {
+                    if (!stage_r(r4, nr, I.r_n_chunks - dr.x)) return;  // the warp stops
+                    held = pr.k + 1;
                 }
-                if (self_join && s == wi.r) continue;
-                const uint2 ds = I.s_desc[s];
-                const uint32_t ns = ds.y;
+                if (!r_staged) held = 0;  // (abuf becomes a window buffer)
                 const uint32_t req = required_overlap(I.sim, I.p, I.den, I.magic, nr, ns);
-                if (!emit_all && (nr + ns == 0 || req > min(nr, ns))) continue;  // length filter
                 bool rej, failed;
                 const uint32_t o =
                     warp_merge(r4, nr, I.s_toks4 + ds.x, ns, req, early, r_staged, abuf, bbuf, lane, wbar, &wph,
                                I.s_n_chunks - ds.x, &a.ctr->err, &failed,
                                &rej CHK_ARGS(I.r_n_chunks - dr.x, I.s_n_chunks - ds.x, &a.ctr->err));
                 if (failed) return;  // (warp-uniform) reported; the warp stops
-                const bool pass = emit_all || (!rej && o >= req);
-                if (pass) {
-                    if (flags & VF_COUNT_ONLY) {
+                if (!early || (!rej && o >= req)) {
+                    if (I.flags & VF_COUNT_ONLY) {
                         if (lane == 0) atomicAdd(I.count, 1ull);
                     } else {
-                        wout.push(I, lane, wi.r, s, o);
+                        wout.push(I, lane, r, pr.s, o);
                     }
                 }
             }
-            wout.flush(I, lane);
-            __syncwarp();  // abuf reuse
+            if (wout.n) wout.flush(table[inst], lane);
         }
+        __syncwarp();  // the slice is phase 3's now
     }
 
     // ---------------- phase 3: short pairs, one per thread ----------------
     {
         ContEntry* cont = reinterpret_cast<ContEntry*>(reinterpret_cast<char*>(smem) + warp * kWarpSliceBytes);
         uint32_t n_cont = 0;  // warp-uniform
-        const unsigned long long n_pairs = min(a.ctr->thread_pairs, (unsigned long long)a.pair_cap);
-        const unsigned long long n_units = (n_pairs + 32 * kFlatGrab - 1) / (32 * kFlatGrab);
+        const uint32_t grab = n_pairs > 4ull * 32 * n_warps_total ? kFlatGrab : 1u;
+        const unsigned long long n_units = (n_pairs + 32 * grab - 1) / (32 * grab);
         const unsigned lt_mask = (1u << lane) - 1u;
-        const uint4 zero4 = make_uint4(0, 0, 0, 0);
 
-        // Pass 2 (drain_parked): the last m parked pairs, one per lane, merged
-        // while at least min_live lanes still work; the rest are parked again.
+        // drain_parked: the last m parked pairs, one per lane, merged while at
+        // least min_live lanes still work; the rest are parked again.
         auto drain = [&](uint32_t m, uint32_t live) {
-            n_cont = drain_parked(cont, n_cont, m, live, table, a.rid, lane CHK_ERR_ARG(&a.ctr->err));
+            n_cont = drain_parked(cont, n_cont, m, live, table, lane CHK_ERR_ARG(&a.ctr->err));
         };
         const uint32_t min_live = a.drain_min_live ? min(max(a.drain_min_live, 1u), 24u) : kDrainMinLive;
 
@@ -1424,102 +1136,39 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
             }
             u = __shfl_sync(kFull, u, 0);
             if (u >= n_units) break;
-            for (uint32_t sub = 0; sub < kFlatGrab; ++sub) {
-                const unsigned long long first = ((unsigned long long)u * kFlatGrab + sub) * 32;
+            for (uint32_t sub = 0; sub < grab; ++sub) {
+                const unsigned long long first = ((unsigned long long)u * grab + sub) * 32;
                 if (first >= n_pairs) break;  // warp-uniform
-                // the chunk's instance (uniform)
-                if (!in_bounds(first / 32, a.pair_cap / 32 + 1, &a.ctr->err)) break;
-                const uint32_t inst = a.chunk_inst[first / 32];
-                if (!in_bounds(inst, a.n_inst, &a.ctr->err)) continue;
-                const Instance& I = table[inst];
-                const uint32_t flags = I.flags;
-                const bool emit_all = (flags & VF_EMIT_ALL) != 0, early = !emit_all;
-                const bool self_join = (flags & VF_SELF_JOIN) != 0;
-                const uint32_t s_n_sets = I.s_n_sets, p = I.p, den = I.den, sim = I.sim;
-                const uint64_t magic = I.magic;
-                const uint4* r_toks4 = I.r_toks4;
-                const uint4* s_toks4 = I.s_toks4;
-                // ---- pass 1
-                bool live = false;
-                uint32_t pr_k = 0, ps_id = 0, nr = 0, ns = 0, req = 0;
+                // the next 32 pairs, parked at their start
+                bool live = first + lane < n_pairs;
+                uint32_t r = 0, inst = 0, req = 0;
                 uint2 dr = make_uint2(0, 0), ds = make_uint2(0, 0);
-                {
-                    PairRef pr;
-                    pr.k = kNoProbe;
-                    pr.s = 0;
-                    if (in_bounds(first + lane, a.pair_cap, &a.ctr->err)) pr = a.pairs[first + lane];
-                    if (pr.k != kNoProbe && !in_bounds(pr.k, 32ull * a.n_tiles + 1, &a.ctr->err)) pr.k = kNoProbe;
-                    if (pr.k != kNoProbe) {
-                        ps_id = pr.s;
-                        if (ps_id >= s_n_sets) {
-                            atomicOr(&a.ctr->err, ERR_CAND_ID);
-                        } else {
-                            pr_k = pr.k;
-                            dr = a.rdesc[pr_k];
-                            ds = I.s_desc[ps_id];
-                            nr = dr.y;
-                            ns = ds.y;
-                            // (r, r) of a self-join: non-empty sets have disjoint blocks, so
-                            // equal descriptors name the same set; empty ones need the id
-                            const bool same = self_join && dr.x == ds.x && nr == ns && (nr > 0 || a.rid[pr_k] == ps_id);
-                            if (!same) {
-                                req = required_overlap(sim, p, den, magic, nr, ns);
-                                live = emit_all || (nr + ns > 0 && req <= min(nr, ns));  // length filter
-                            }
-                        }
-                    }
-                }
-                uint4 r0 = zero4, r1 = zero4, r2 = zero4, s0 = zero4, s1 = zero4, s2 = zero4;
+                PairRef pr;
+                pr.k = pr.s = 0;
                 if (live) {
-                    const uint4* r4 = r_toks4 + dr.x;
-                    const uint4* s4 = s_toks4 + ds.x;
-                    const uint64_t rlim = I.r_n_chunks - dr.x, slim = I.s_n_chunks - ds.x;
-                    if (nr > 0) r0 = ld_block(r4, 0, rlim, &a.ctr->err);
-                    if (nr > 4) r1 = ld_block(r4, 1, rlim, &a.ctr->err);
-                    if (nr > 8) r2 = ld_block(r4, 2, rlim, &a.ctr->err);
-                    if (ns > 0) s0 = ld_block(s4, 0, slim, &a.ctr->err);
-                    if (ns > 4) s1 = ld_block(s4, 1, slim, &a.ctr->err);
-                    if (ns > 8) s2 = ld_block(s4, 2, slim, &a.ctr->err);
-                }
-                BlockState st;
-                st.qi = st.qj = st.o = 0;
-                st.rej = false;
-                st.fin = !live || nr == 0 || ns == 0;
-#pragma unroll
-                for (int step = 0; step < 3; ++step) {
-                    bool ar, as;
-                    block_step(r0, s0, nr, ns, req, early, st, ar, as);
-                    if (ar) { r0 = r1; r1 = r2; }
-                    if (as) { s0 = s1; s1 = s2; }
-                }
-                // decided pairs
-                const bool pass = live && st.fin && (emit_all || (!st.rej && st.o >= req));
-                const uint32_t pmask = __ballot_sync(kFull, pass);
-                if (pmask) {
-                    unsigned long long b0 = 0;
-                    if (lane == 0) b0 = atomicAdd(I.count, (unsigned long long)__popc(pmask));
-                    if (!(flags & VF_COUNT_ONLY)) {
-                        b0 = __shfl_sync(kFull, b0, 0);
-                        if (pass)
-                            emit_triple(I.out, I.cap, self_join, b0 + __popc(pmask & lt_mask), a.rid[pr_k], ps_id,
-                                        st.o);
+                    pr = a.pairs[first + lane];
+                    if (a.n_inst > 1) inst = instance_of(table, a.n_inst, pr.k);
+                    const Instance& I = table[inst];
+                    live = in_bounds(pr.k - 32u * I.tile_base, I.n_probes, &a.ctr->err);
+                    if (live) r = I.probe_ids[pr.k - 32u * I.tile_base];
+                    live = live && in_bounds(r, I.r_n_sets, &a.ctr->err) && in_bounds(pr.s, I.s_n_sets, &a.ctr->err);
+                    if (live) {
+                        dr = I.r_desc[r];
+                        ds = I.s_desc[pr.s];
+                        req = required_overlap(I.sim, I.p, I.den, I.magic, dr.y, ds.y);
                     }
                 }
-                // undecided pairs: park them with their merge state
-                const bool park = live && !st.fin;
-                const uint32_t kmask = __ballot_sync(kFull, park);
-                if (kmask) {
-                    while (n_cont + 32 > kCont) drain(32, min_live);  // room for a full warp of parked pairs
-                    if (park && in_bounds(n_cont + __popc(kmask & lt_mask), kCont, &a.ctr->err)) {
-                        ContEntry* ce = cont + n_cont + __popc(kmask & lt_mask);
-                        ce->m0 = make_uint4(pr_k, ps_id, dr.x + st.qi, ds.x + st.qj);
-                        ce->m1 = make_uint4(nr - 4 * st.qi, ns - 4 * st.qj, req, st.o);
-                        ce->m2 = make_uint4(inst, 0u, 0u, 0u);
-                    }
-                    n_cont += __popc(kmask);
-                    __syncwarp();
-                    if (n_cont >= 32) drain(32, min_live);
+                const uint32_t kmask = __ballot_sync(kFull, live);
+                while (n_cont + 32 > kCont) drain(32, min_live);  // room for a full warp of parked pairs
+                if (live && in_bounds(n_cont + __popc(kmask & lt_mask), kCont, &a.ctr->err)) {
+                    ContEntry* ce = cont + n_cont + __popc(kmask & lt_mask);
+                    ce->m0 = make_uint4(r, pr.s, dr.x, ds.x);
+                    ce->m1 = make_uint4(dr.y, ds.y, req, 0u);
+                    ce->m2 = make_uint4(inst, 0u, 0u, 0u);
                 }
+                n_cont += __popc(kmask);
+                __syncwarp();
+                if (n_cont >= 32) drain(32, min_live);
             }
         }
         // the tail: keep refilling lanes while more than a warp is parked, then finish
@@ -1560,12 +1209,27 @@ static void item_sizes(uint64_t n_cands, int num_sms, uint32_t* per_warp_item, u
 
 static uint64_t pair_cap(const LaunchShape& sh) { return sh.total_cands + 32ull * sh.n_tiles + 32; }
 
-LaunchShape single_shape(uint32_t n_probes, uint64_t n_cands) {
+// Small chunks for small batches, so that a wave of warps shares the work;
+// at least 256 candidates once block items hold several pairs, so that the
+// runs of pairs that chunk borders cut (one more work item each) fit the
+// block list (see bind_workspace).
+uint32_t plan_chunk(uint64_t total_cands, int num_sms) {
+    uint32_t wc, bc, lc, ic;
+    item_sizes(total_cands, num_sms, &wc, &bc, &lc, &ic);
+    // whole rounds of a wave's warps (plan kernel: 32 per SM), of chunks of at most about 1024
+    const uint64_t warps = 32ull * (uint64_t)num_sms, rounds = (total_cands + 1024 * warps - 1) / (1024 * warps);
+    const uint64_t per = (total_cands + warps * std::max<uint64_t>(rounds, 1) - 1) / (warps * std::max<uint64_t>(rounds, 1));
+    const uint32_t c = std::max<uint32_t>((uint32_t)((per + 31) & ~31ull), 32u);
+    return bc > 1 && c < 256 ? 256u : c;
+}
+
+LaunchShape single_shape(uint32_t n_probes, uint64_t n_cands, int num_sms) {
     LaunchShape sh;
     sh.n_inst = 1;
     sh.n_tiles = (n_probes + 31) / 32;
     sh.total_probes = n_probes;
     sh.total_cands = n_cands;
+    sh.n_chunks = chunks_of(n_probes, n_cands, plan_chunk(n_cands, num_sms));
     return sh;
 }
 
@@ -1573,6 +1237,7 @@ size_t workspace_bytes(const LaunchShape& sh, int num_sms) {
     uint32_t wc, bc, lc, ic;
     item_sizes(sh.total_cands, num_sms, &wc, &bc, &lc, &ic);
     const uint64_t slots = 32ull * sh.n_tiles + 1, pc = pair_cap(sh);
+    // slots * 12 + pc / 8 bytes: extra work items, see bind_workspace
     return align256(sizeof(Counters)) + align256(sizeof(Instance) * ((size_t)sh.n_inst + 1)) +
            align256(sizeof(uint2) * slots) + align256(sizeof(uint32_t) * slots) +
            align256(sizeof(uint32_t) * (pc / 32 + 1)) + align256(sizeof(PairRef) * pc) +
@@ -1581,40 +1246,42 @@ size_t workspace_bytes(const LaunchShape& sh, int num_sms) {
 }
 
 size_t workspace_bytes(uint32_t n_probes, uint64_t n_cands, int num_sms) {
-    return workspace_bytes(single_shape(n_probes, n_cands), num_sms);
+    return workspace_bytes(single_shape(n_probes, n_cands, num_sms), num_sms);
 }
 
 void bind_workspace(VerifyArgs& a, void* ws, const LaunchShape& sh, int num_sms) {
     char* p = static_cast<char*>(ws);
-    item_sizes(sh.total_cands, num_sms, &a.warp_item_cands, &a.block_item_cands, &a.lane_item_cands,
-               &a.index_item_cands);
-    const uint64_t slots = 32ull * sh.n_tiles + 1;
+    uint32_t wc;
+    item_sizes(sh.total_cands, num_sms, &wc, &a.block_item_cands, &a.lane_item_cands, &a.index_item_cands);
     a.n_inst = sh.n_inst;
     a.n_tiles = sh.n_tiles;
     a.total_probes = sh.total_probes;
     a.total_cands = sh.total_cands;
+    a.chunk = plan_chunk(sh.total_cands, num_sms);
+    a.n_chunks = sh.n_chunks;
     a.ctr = reinterpret_cast<Counters*>(p);
     p += align256(sizeof(Counters));
     a.table_out = reinterpret_cast<Instance*>(p);
     p += align256(sizeof(Instance) * ((size_t)sh.n_inst + 1));
-    a.rdesc = reinterpret_cast<uint2*>(p);
-    p += align256(sizeof(uint2) * slots);
-    a.rid = reinterpret_cast<uint32_t*>(p);
-    p += align256(sizeof(uint32_t) * slots);
     a.pair_cap = pair_cap(sh);
-    a.chunk_inst = reinterpret_cast<uint32_t*>(p);
-    p += align256(sizeof(uint32_t) * (a.pair_cap / 32 + 1));
     a.pairs = reinterpret_cast<PairRef*>(p);
     p += align256(sizeof(PairRef) * a.pair_cap);
     a.warp_items = reinterpret_cast<WorkItem*>(p);
-    a.warp_item_cap = (uint32_t)item_cap(sh.total_probes, sh.total_cands, a.warp_item_cands);
+    a.warp_item_cap = (uint32_t)item_cap(sh.total_probes, sh.total_cands, wc);
     p += align256(sizeof(WorkItem) * ((size_t)a.warp_item_cap + 1));
+    // Block items take the rest: n_probes + n_cands / block_item_cands, and 12 bytes per probe slot
+    // and 1/8 byte per candidate beyond that, one item per 192 candidates: runs cut at chunk borders
+    // (chunks of 256 or more) and by early flushes (every kPlanFlush pairs of chunks above that size)
+    // are at most one per 256 candidates, or one per 480 and one per 512.  Chunks below 256 come with
+    // one pair per block item and one index item per run, at most n_cands items.  Lane items, at
+    // least one pair and up to 32 of a run, fit n_probes + n_cands / 8 the same way.
     a.block_items = reinterpret_cast<WorkItem*>(p);
-    a.block_item_cap = (uint32_t)item_cap(sh.total_probes, sh.total_cands, a.block_item_cands);
+    const size_t left = static_cast<char*>(ws) + workspace_bytes(sh, num_sms) - p;
+    a.block_item_cap = (uint32_t)(left / sizeof(WorkItem) > 0xFFFFFFF0ull ? 0xFFFFFFF0ull : left / sizeof(WorkItem));
 }
 
 void bind_workspace(VerifyArgs& a, void* ws, uint32_t n_probes, uint64_t n_cands, int num_sms) {
-    bind_workspace(a, ws, single_shape(n_probes, n_cands), num_sms);
+    bind_workspace(a, ws, single_shape(n_probes, n_cands, num_sms), num_sms);
 }
 
 // Dynamic shared memory of the verify kernel: the largest of the block
@@ -1748,26 +1415,8 @@ cudaError_t launch_verify(const VerifyArgs& a, cudaStream_t st, int num_sms, uin
         return cudaSuccess;
     }
     // the plan kernel also runs for empty batches: it clears the instances' counts
-    {
-        // at most one wave of CTAs; a CTA takes up to kPlanThreads / 32 tiles per round
-        static int plan_ctas_per_sm = 0;  // resident CTAs per SM (same value from every thread)
-        if (plan_ctas_per_sm == 0) {
-            int n = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, plan_kernel, kPlanThreads, 0) != cudaSuccess || n < 1)
-                n = 4;
-            plan_ctas_per_sm = n;
-        }
-        // one tile per CTA while tiles are fewer than a wave of CTAs (a tile's candidates are copied
-        // by the whole CTA, so few tiles still fill the GPU), else a wave with several tiles each
-        const int threads = kPlanThreads;
-        uint64_t blocks = a.n_tiles;
-        const uint64_t max_blocks = (uint64_t)num_sms * (uint64_t)plan_ctas_per_sm;
-        if (blocks > max_blocks) blocks = max_blocks;
-        if (blocks < 1) blocks = 1;
-        plan_kernel<<<(unsigned)blocks, threads, 0, st>>>(a);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-    }
+    e = launch_plan(a, st, num_sms);
+    if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[1], st);
     VerifyArgs va = a;
     va.bulk_stage = (block_threads & kBulkStaging) ? 1u : 0u;
