@@ -299,8 +299,9 @@ ssj_status ssj_verify_batch_noalloc(ssj_ctx* ctx, const ssj_batch* batch, ssj_tr
  * on the device (sets ordered by size; each set's prefix indexed; each
  * probe matched against the earlier sets' prefix entries that pass the
  * length filter, SSJ_JOIN_POSITIONAL adding the positional bound;
- * candidates deduplicated), then the candidates are verified by the same
- * launch as ssj_verify_batch, without a host round trip.  The candidates
+ * candidates deduplicated), each candidate's signatures are tested as it is
+ * found, and the pairs left are verified by the verify kernel of
+ * ssj_verify_batch.  The candidates
  * are those of the CPU feeder (ssj_feeder.h) for the same function and
  * threshold.  Results as for ssj_verify_batch of a self-join: (min id, max
  * id, overlap) triples in the caller's ids, to out (host memory, or device
@@ -309,8 +310,9 @@ ssj_status ssj_verify_batch_noalloc(ssj_ctx* ctx, const ssj_batch* batch, ssj_tr
  * of candidates verified.  Flags: SSJ_SIM_*, SSJ_JOIN_POSITIONAL,
  * SSJ_COUNT_ONLY, SSJ_SORTED, SSJ_DEVICE_PTRS, SSJ_FORCE_*.  Token values
  * must stay below 2^30 (load with SSJ_RENUMBER_BY_FREQ, which the prefix
- * filter wants anyway).  Allocates its scratch (the prefix index, a hash
- * set of candidate pairs and the candidate list) for the call.
+ * filter wants anyway).  The prefix index comes from the context's memory
+ * pool, the queue of pairs is the context's workspace; a join that leaves
+ * more pairs than the queue holds is probed a second time with a larger one.
  * Errors: SSJ_EINVAL, SSJ_ENOTFOUND, SSJ_ENOMEM, SSJ_EDEVICE.
  */
 ssj_status ssj_self_join(ssj_ctx* ctx, ssj_coll coll, uint32_t p, uint32_t q, uint32_t flags, ssj_triple* out,

@@ -169,6 +169,7 @@ struct ssj_ctx {
     size_t io_bytes = 0;
     uint64_t* h_count = nullptr;  // pinned
     uint32_t* h_err = nullptr;    // pinned, kMaxGroups words
+    Counters* h_ctr = nullptr;    // pinned
     // ssj_verify_batches: the stream and event that carry the second group's input copies
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t copy_done[kMaxGroups] = {};
@@ -486,6 +487,37 @@ void free_collection(Collection& c) {
     for (uint4* r : c.d_rec) cudaFree(r);
 }
 
+// Device memory of one call, from the context's pool in the order of its
+// stream: it stays in the pool (up to the pool's release threshold, the
+// serving budget) instead of being mapped and unmapped by every call (a dozen
+// cudaMalloc and cudaFree took about 1 ms), and goes back with the context.
+class CallMemory {
+public:
+    explicit CallMemory(ssj_ctx* c) : ctx_(c) {}
+    ~CallMemory() {
+        for (void* m : mem_) cudaFreeAsync(m, ctx_->stream);
+    }
+    CallMemory(const CallMemory&) = delete;
+    CallMemory& operator=(const CallMemory&) = delete;
+    template <class T>
+    T* get(uint64_t n) {
+        void* m = nullptr;
+        if (cudaMallocFromPoolAsync(&m, std::max<size_t>(n * sizeof(T), 16), ctx_->pool, ctx_->stream) != cudaSuccess) {
+            cudaGetLastError();
+            failed_ = true;
+            return nullptr;
+        }
+        mem_.push_back(m);
+        return static_cast<T*>(m);
+    }
+    bool ok() const { return !failed_; }
+
+private:
+    ssj_ctx* ctx_;
+    std::vector<void*> mem_;
+    bool failed_ = false;
+};
+
 bool triple_less(const ssj_triple& x, const ssj_triple& y) { return x.r != y.r ? x.r < y.r : x.s < y.s; }
 
 void completion_loop(ssj_ctx* ctx, int slot);
@@ -518,6 +550,7 @@ extern "C" ssj_status ssj_create(const ssj_config* config, ssj_ctx** out) {
     if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_count), sizeof(uint64_t)) != cudaSuccess) return SSJ_EDEVICE;
     if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_err), kMaxGroups * sizeof(uint32_t)) != cudaSuccess)
         return SSJ_EDEVICE;
+    if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_ctr), sizeof(Counters)) != cudaSuccess) return SSJ_EDEVICE;
     cudaMemPoolProps props;
     memset(&props, 0, sizeof(props));
     props.allocType = cudaMemAllocationTypePinned;
@@ -587,6 +620,7 @@ extern "C" void ssj_destroy(ssj_ctx* ctx) {
     cudaFree(ctx->io);
     cudaFreeHost(ctx->h_count);
     cudaFreeHost(ctx->h_err);
+    cudaFreeHost(ctx->h_ctr);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     for (cudaEvent_t ev : ctx->copy_done)
         if (ev) cudaEventDestroy(ev);
@@ -1144,32 +1178,18 @@ extern "C" ssj_status ssj_self_join(ssj_ctx* ctx, ssj_coll coll, uint32_t p, uin
     DeviceGuard g(ctx->device);
     cudaStream_t s = ctx->stream;
     const uint32_t n = C.n_sets;
-    std::vector<void*> mem;
-    auto release = [&]() {
-        for (void* m : mem) cudaFree(m);
-        mem.clear();
-    };
-    auto alloc = [&](size_t bytes) -> void* {
-        void* m = nullptr;
-        if (cudaMalloc(&m, std::max<size_t>(bytes, 16)) != cudaSuccess) return nullptr;
-        mem.push_back(m);
-        return m;
-    };
+    CallMemory mem(ctx);
     CandgenIndex ix;
     const uint64_t scan_n = std::max<uint64_t>((uint64_t)C.max_len + 2, (uint64_t)C.vocab + 1);
-    ix.size_hist = static_cast<uint64_t*>(alloc(8ull * (C.max_len + 2)));
-    ix.order = static_cast<uint32_t*>(alloc(4ull * n));
-    ix.rank = static_cast<uint32_t*>(alloc(4ull * n));
-    ix.tcnt = static_cast<uint64_t*>(alloc(8ull * (C.vocab + 1)));
-    ix.toff = static_cast<uint64_t*>(alloc(8ull * (C.vocab + 1)));
-    ix.scan_scratch = static_cast<uint64_t*>(alloc(8ull * scan_scratch_words(scan_n)));
-    ix.total = static_cast<uint64_t*>(alloc(8));
-    ix.post = nullptr;
-    uint32_t* d_err = static_cast<uint32_t*>(alloc(4));
-    if (!ix.size_hist || !ix.order || !ix.rank || !ix.tcnt || !ix.toff || !ix.scan_scratch || !ix.total || !d_err) {
-        release();
-        return fail(ctx, SSJ_ENOMEM, "candidate generation index");
-    }
+    ix.size_hist = mem.get<uint64_t>((uint64_t)C.max_len + 2);
+    ix.probes = mem.get<uint32_t>(n);
+    ix.rank = mem.get<uint32_t>(n);
+    ix.tcnt = mem.get<uint64_t>((uint64_t)C.vocab + 1);
+    ix.toff = mem.get<uint64_t>((uint64_t)C.vocab + 1);
+    ix.scan_scratch = mem.get<uint64_t>(scan_scratch_words(scan_n));
+    ix.total = mem.get<uint64_t>(1);
+    uint64_t* d_count = mem.get<uint64_t>(1);
+    if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "candidate generation index");
     CandgenInput in;
     memset(&in, 0, sizeof(in));
     in.toks4 = reinterpret_cast<const uint4*>(C.d_toks);
@@ -1181,124 +1201,78 @@ extern "C" ssj_status ssj_self_join(ssj_ctx* ctx, ssj_coll coll, uint32_t p, uin
     in.p = p;
     in.q = q;
     in.positional = (flags & SSJ_JOIN_POSITIONAL) ? 1u : 0u;
-    cudaError_t e = cudaMemsetAsync(d_err, 0, 4, s);
     in.stage = 0;
-    if (e == cudaSuccess) e = candgen_run(in, s, ctx->num_sms, &ix, ctx->h_count);
-    if (e != cudaSuccess) {
-        release();
-        return cuda_fail(ctx, e, "candidate generation (index)");
-    }
+    cudaError_t e = candgen_run(in, s, ctx->num_sms, &ix, ctx->h_count);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "candidate generation (index)");
     const uint64_t entries = *ctx->h_count;
-    ix.post = static_cast<uint4*>(alloc(16ull * entries));
-    if (!ix.post) {
-        release();
-        return fail(ctx, SSJ_ENOMEM, "prefix index of %llu entries", (unsigned long long)entries);
-    }
+    ix.post = mem.get<uint4>(entries);
+    if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "prefix index of %llu entries", (unsigned long long)entries);
     in.stage = 1;
     e = candgen_run(in, s, ctx->num_sms, &ix, ctx->h_count);
-    if (e != cudaSuccess) {
-        release();
-        return cuda_fail(ctx, e, "candidate generation (count)");
-    }
-    const uint64_t bound = *ctx->h_count;  // entries that can yield a candidate
-    uint64_t tsize = 1024;
-    while (tsize < 2 * bound) tsize <<= 1;
-    const uint64_t group_cap = (uint64_t)n + bound / 224 + 1;
-    in.table = static_cast<unsigned long long*>(alloc(8ull * tsize));
-    in.table_mask = tsize - 1;
-    in.out.probe_ids = static_cast<uint32_t*>(alloc(4ull * group_cap));
-    in.out.cand_offsets = static_cast<uint64_t*>(alloc(8ull * (group_cap + 1)));
-    in.out.cand_ids = static_cast<uint32_t*>(alloc(4ull * std::max<uint64_t>(bound, 1)));
-    in.out.packed = static_cast<unsigned long long*>(alloc(8));
-    in.out.group_cap = group_cap;
-    in.out.cand_cap = bound;
-    in.out.err = d_err;
-    if (!in.table || !in.out.probe_ids || !in.out.cand_offsets || !in.out.cand_ids || !in.out.packed) {
-        release();
-        return fail(ctx, SSJ_ENOMEM, "candidate generation output (%llu entries)", (unsigned long long)bound);
-    }
-    in.stage = 2;
-    e = candgen_run(in, s, ctx->num_sms, &ix, ctx->h_count);
-    uint32_t derr = 0;
-    if (e == cudaSuccess) e = cudaMemcpy(&derr, d_err, 4, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) {
-        release();
-        return cuda_fail(ctx, e, "candidate generation (probe)");
-    }
-    if (derr) {
-        release();
-        return fail(ctx, SSJ_EDEVICE, "candidate generation: an output capacity was exceeded or the candidate hash set was full (code %u)", derr);
-    }
-    const uint64_t packed = *ctx->h_count;
-    const uint64_t groups = packed >> 40, total = packed & ((1ull << 40) - 1);
-    if (n_candidates) *n_candidates = total;
-    e = cudaMemcpy(in.out.cand_offsets + groups, &total, 8, cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-        release();
-        return cuda_fail(ctx, e, "candidate offsets");
-    }
-    // index and hash table are no longer needed; verify the generated batch
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "candidate generation (lists)");
+    // probe, test and verify; the queue is sized for the pairs that joins usually leave, and once
+    // more from the counted pairs if they were more
+    const bool count_only = (flags & SSJ_COUNT_ONLY) != 0;
+    const bool dev_out = (flags & SSJ_DEVICE_PTRS) != 0;
     ssj_batch b;
     memset(&b, 0, sizeof(b));
     b.R = b.S = coll;
     b.p = p;
     b.q = q;
-    b.n_probes = (uint32_t)groups;
-    b.probe_ids = in.out.probe_ids;
-    b.cand_offsets = in.out.cand_offsets;
-    b.cand_ids = in.out.cand_ids;
-    b.n_cands = total;
-    b.flags = (flags & ~(SSJ_JOIN_POSITIONAL | SSJ_DEVICE_PTRS | SSJ_SORTED)) | SSJ_DEVICE_PTRS;
-    if (groups > 0xFFFFFFFFull) {
-        release();
-        return fail(ctx, SSJ_EINVAL, "too many candidate groups");
-    }
-    const bool count_only = (flags & SSJ_COUNT_ONLY) != 0;
-    const bool dev_out = (flags & SSJ_DEVICE_PTRS) != 0;
+    b.n_probes = n;
+    b.flags = flags & ~(SSJ_JOIN_POSITIONAL | SSJ_DEVICE_PTRS | SSJ_SORTED);
+    uint64_t room = std::min<uint64_t>(std::max<uint64_t>(8ull * n, 1u << 18), 1u << 22);
     ssj_triple* d_out = nullptr;
-    uint64_t d_cap = 0;
-    if (!count_only) {
-        if (dev_out) {
-            d_out = out;
-            d_cap = cap;
-        } else {
-            d_cap = std::min<uint64_t>(cap, total);
-            d_out = static_cast<ssj_triple*>(alloc(sizeof(ssj_triple) * std::max<uint64_t>(d_cap, 1)));
-            if (!d_out) {
-                release();
-                return fail(ctx, SSJ_ENOMEM, "join output");
-            }
+    for (;;) {
+        VerifyArgs a = make_args(ctx, &b, *R, *S, 0);
+        a.single.probe_ids = ix.probes;
+        a.single.count = reinterpret_cast<unsigned long long*>(d_count);
+        if (!count_only) {
+            // no more results than queued pairs
+            const uint64_t d_cap = dev_out ? cap : std::min<uint64_t>(cap, room);
+            d_out = dev_out ? out : mem.get<ssj_triple>(std::max<uint64_t>(d_cap, 1));
+            if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "join output");
+            a.single.out = d_out;
+            a.single.cap = d_cap;
         }
+        st = ensure_device_buffer(ctx, &ctx->ws, &ctx->ws_bytes, join_workspace_bytes(n, room, ctx->num_sms));
+        if (st != SSJ_OK) return st;
+        const JoinQueue queue = bind_join_workspace(a, ctx->ws, n, room, ctx->num_sms);
+        ctx->last_ctr = a.ctr;
+        cudaEvent_t* ev = profile_events(ctx);
+        if (ev) cudaEventRecord(ev[0], s);
+        e = join_probe(in, ix, a, queue, s, ctx->num_sms);
+        if (ev) cudaEventRecord(ev[1], s);
+        if (e == cudaSuccess) e = launch_merge(a, s, ctx->num_sms, ctx->block_threads);
+        if (ev) cudaEventRecord(ev[2], s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->h_ctr, a.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->h_count, d_count, sizeof(uint64_t), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "candidate generation (probe)");
+        if (ctx->h_ctr->join_pairs <= room) break;
+        room = ctx->h_ctr->join_pairs;
     }
-    uint64_t count = 0;
-    st = ssj_verify_batch(ctx, &b, d_out, d_cap, &count);
+    if (n_candidates) *n_candidates = ctx->h_ctr->candidates;
+    if (ctx->h_ctr->err) return device_check_status(ctx, ctx->h_ctr->err);
+    const uint64_t count = *ctx->h_count;
     *n_out = count;
-    if (st != SSJ_OK && st != SSJ_ENOMEM) {
-        release();
-        return st;
-    }
-    if (!count_only) {
-        const uint64_t n_copy = std::min(count, cap);
-        if (dev_out) {
-            if ((flags & SSJ_SORTED) && n_copy) {
-                std::vector<ssj_triple> h(n_copy);
-                e = cudaMemcpy(h.data(), out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost);
-                std::sort(h.begin(), h.end(), triple_less);
-                if (e == cudaSuccess) e = cudaMemcpy(out, h.data(), sizeof(ssj_triple) * n_copy, cudaMemcpyHostToDevice);
-            }
-        } else if (n_copy) {
-            e = cudaMemcpy(out, d_out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost);
-            if (e == cudaSuccess && (flags & SSJ_SORTED)) std::sort(out, out + n_copy, triple_less);
+    if (count_only) return SSJ_OK;
+    const uint64_t n_copy = std::min(count, cap);
+    if (dev_out) {
+        if ((flags & SSJ_SORTED) && n_copy) {
+            std::vector<ssj_triple> h(n_copy);
+            e = cudaMemcpy(h.data(), out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost);
+            std::sort(h.begin(), h.end(), triple_less);
+            if (e == cudaSuccess) e = cudaMemcpy(out, h.data(), sizeof(ssj_triple) * n_copy, cudaMemcpyHostToDevice);
         }
-        if (e != cudaSuccess) {
-            release();
-            return cuda_fail(ctx, e, "join results");
-        }
+    } else if (n_copy) {
+        e = cudaMemcpyAsync(out, d_out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e == cudaSuccess && (flags & SSJ_SORTED)) std::sort(out, out + n_copy, triple_less);
     }
-    release();
-    if (count > cap && !count_only)
-        return fail(ctx, SSJ_ENOMEM, "%llu result pairs, room for %llu", (unsigned long long)count,
-                    (unsigned long long)cap);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "join results");
+    if (count > cap) return fail(ctx, SSJ_ENOMEM, "%llu result pairs, room for %llu", (unsigned long long)count,
+                                 (unsigned long long)cap);
     return SSJ_OK;
 }
 
@@ -1347,17 +1321,7 @@ extern "C" ssj_status ssj_verify_groups(ssj_ctx* ctx, const ssj_group_batch* gb,
         if (gb->cand_groups[c] >= gb->n_groups) return fail(ctx, SSJ_EINVAL, "candidate group id out of range");
     DeviceGuard g(ctx->device);
     cudaStream_t s = ctx->stream;
-    std::vector<void*> mem;
-    auto release = [&]() {
-        for (void* m : mem) cudaFree(m);
-        mem.clear();
-    };
-    auto alloc = [&](size_t bytes) -> void* {
-        void* m = nullptr;
-        if (cudaMalloc(&m, std::max<size_t>(bytes, 16)) != cudaSuccess) return nullptr;
-        mem.push_back(m);
-        return m;
-    };
+    CallMemory mem(ctx);
     const uint64_t n_entries = (uint64_t)gb->n_groups + gb->n_probe_groups;
     GroupExpand x;
     memset(&x, 0, sizeof(x));
@@ -1368,21 +1332,17 @@ extern "C" ssj_status ssj_verify_groups(ssj_ctx* ctx, const ssj_group_batch* gb,
     x.q = gb->q;
     x.n_groups = gb->n_groups;
     x.n_probe_groups = gb->n_probe_groups;
-    uint64_t* d_goff = static_cast<uint64_t*>(alloc(8ull * (gb->n_groups + 1)));
-    uint32_t* d_mem = static_cast<uint32_t*>(alloc(4ull * n_members));
-    uint32_t* d_pg = static_cast<uint32_t*>(alloc(4ull * gb->n_probe_groups));
-    uint64_t* d_coff = static_cast<uint64_t*>(alloc(8ull * (gb->n_probe_groups + 1)));
-    uint32_t* d_cg = static_cast<uint32_t*>(alloc(4ull * n_cg));
-    x.probe_off = static_cast<uint64_t*>(alloc(8ull * (n_entries + 1)));
-    x.pair_off = static_cast<uint64_t*>(alloc(8ull * (n_entries + 1)));
-    x.per_probe = static_cast<uint64_t*>(alloc(8ull * (n_entries + 1)));
-    x.scan_scratch = static_cast<uint64_t*>(alloc(8ull * scan_scratch_words(n_entries + 1)));
-    x.total = static_cast<uint64_t*>(alloc(8));
-    if (!d_goff || !d_mem || !d_pg || !d_coff || !d_cg || !x.probe_off || !x.pair_off || !x.per_probe ||
-        !x.scan_scratch || !x.total) {
-        release();
-        return fail(ctx, SSJ_ENOMEM, "group expansion");
-    }
+    uint64_t* d_goff = mem.get<uint64_t>((uint64_t)gb->n_groups + 1);
+    uint32_t* d_mem = mem.get<uint32_t>(n_members);
+    uint32_t* d_pg = mem.get<uint32_t>(gb->n_probe_groups);
+    uint64_t* d_coff = mem.get<uint64_t>((uint64_t)gb->n_probe_groups + 1);
+    uint32_t* d_cg = mem.get<uint32_t>(n_cg);
+    x.probe_off = mem.get<uint64_t>(n_entries + 1);
+    x.pair_off = mem.get<uint64_t>(n_entries + 1);
+    x.per_probe = mem.get<uint64_t>(n_entries + 1);
+    x.scan_scratch = mem.get<uint64_t>(scan_scratch_words(n_entries + 1));
+    x.total = mem.get<uint64_t>(1);
+    if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "group expansion");
     cudaError_t e = cudaMemcpyAsync(d_goff, gb->group_offsets, 8ull * (gb->n_groups + 1), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && n_members) e = cudaMemcpyAsync(d_mem, gb->members, 4ull * n_members, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && gb->n_probe_groups) {
@@ -1399,29 +1359,17 @@ extern "C" ssj_status ssj_verify_groups(ssj_ctx* ctx, const ssj_group_batch* gb,
     uint64_t words[2] = {0, 0};
     x.stage = 0;
     if (e == cudaSuccess) e = expand_groups(x, s, ctx->num_sms, words);
-    if (e != cudaSuccess) {
-        release();
-        return cuda_fail(ctx, e, "group expansion (count)");
-    }
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "group expansion (count)");
     const uint64_t probes = words[0], pairs = words[1];
     if (n_pairs) *n_pairs = pairs;
-    if (probes > 0xFFFFFFFFull) {
-        release();
-        return fail(ctx, SSJ_EINVAL, "too many expanded probes");
-    }
-    x.probe_ids = static_cast<uint32_t*>(alloc(4ull * probes));
-    x.cand_offsets_out = static_cast<uint64_t*>(alloc(8ull * (probes + 1)));
-    x.cand_ids = static_cast<uint32_t*>(alloc(4ull * pairs));
-    if (!x.probe_ids || !x.cand_offsets_out || !x.cand_ids) {
-        release();
-        return fail(ctx, SSJ_ENOMEM, "expanded candidates (%llu pairs)", (unsigned long long)pairs);
-    }
+    if (probes > 0xFFFFFFFFull) return fail(ctx, SSJ_EINVAL, "too many expanded probes");
+    x.probe_ids = mem.get<uint32_t>(probes);
+    x.cand_offsets_out = mem.get<uint64_t>(probes + 1);
+    x.cand_ids = mem.get<uint32_t>(pairs);
+    if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "expanded candidates (%llu pairs)", (unsigned long long)pairs);
     x.stage = 1;
     e = expand_groups(x, s, ctx->num_sms, words);
-    if (e != cudaSuccess) {
-        release();
-        return cuda_fail(ctx, e, "group expansion (write)");
-    }
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "group expansion (write)");
     ssj_batch b;
     memset(&b, 0, sizeof(b));
     b.R = b.S = gb->coll;
@@ -1443,20 +1391,14 @@ extern "C" ssj_status ssj_verify_groups(ssj_ctx* ctx, const ssj_group_batch* gb,
             d_cap = cap;
         } else {
             d_cap = std::min<uint64_t>(cap, pairs);
-            d_out = static_cast<ssj_triple*>(alloc(sizeof(ssj_triple) * std::max<uint64_t>(d_cap, 1)));
-            if (!d_out) {
-                release();
-                return fail(ctx, SSJ_ENOMEM, "group join output");
-            }
+            d_out = mem.get<ssj_triple>(std::max<uint64_t>(d_cap, 1));
+            if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "group join output");
         }
     }
     uint64_t count = 0;
     st = ssj_verify_batch(ctx, &b, d_out, d_cap, &count);
     *n_out = count;
-    if (st != SSJ_OK && st != SSJ_ENOMEM) {
-        release();
-        return st;
-    }
+    if (st != SSJ_OK && st != SSJ_ENOMEM) return st;
     if (!count_only) {
         const uint64_t n_copy = std::min(count, cap);
         if (dev_out) {
@@ -1470,12 +1412,8 @@ extern "C" ssj_status ssj_verify_groups(ssj_ctx* ctx, const ssj_group_batch* gb,
             e = cudaMemcpy(out, d_out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost);
             if (e == cudaSuccess && (gb->flags & SSJ_SORTED)) std::sort(out, out + n_copy, triple_less);
         }
-        if (e != cudaSuccess) {
-            release();
-            return cuda_fail(ctx, e, "group join results");
-        }
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "group join results");
     }
-    release();
     if (count > cap && !count_only)
         return fail(ctx, SSJ_ENOMEM, "%llu result pairs, room for %llu", (unsigned long long)count,
                     (unsigned long long)cap);

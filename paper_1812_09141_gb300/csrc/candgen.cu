@@ -1,8 +1,8 @@
-// Candidate generation on the device for a self-join: the prefix filter and
-// inverted-index probing of algorithm ALL (Sections 2.2.3, 2.2.4, 3.1),
-// which the paper leaves on the CPU and names as future work (Section 6).
-// The candidates come out in the grouped (probe ids, offsets, candidate ids)
-// layout of a device batch, so verification follows without a host round trip.
+// Self-join on the device: the prefix filter and inverted-index probing of
+// algorithm ALL (Sections 2.2.3, 2.2.4, 3.1), which the paper leaves on the
+// CPU and names as future work (Section 6), and the signature test of every
+// candidate as it is found; the pairs left go straight to the verify
+// kernel's lists.
 //
 // Steps, on one stream:
 //   1. order the sets by size (counting sort; ties in any order: the set of
@@ -10,31 +10,32 @@
 //   2. index every set's prefix: per token, the entries (position in that
 //      order, position of the token in the set, set size, set id), by a
 //      count / scan / scatter over the prefix tokens;
-//   3. count, per probe, the index entries that can yield a candidate (an
-//      earlier set in the order, passing the length filter), to size a hash
-//      table and the output;
-//   4. one warp per probe walks its prefix tokens' entries, keeps those of
-//      earlier sets that pass the length filter (and optionally the
-//      positional bound of the matching token, PPJoin-style), deduplicates
-//      (probe, candidate) with a hash set of 64-bit keys, and appends the new
-//      candidates to the output through a per-warp buffer; one atomic on a
-//      packed (groups, candidates) counter reserves a group and its range, so
-//      the group offsets are contiguous in group order.
+//   3. one warp per probe walks its prefix tokens' entries, keeps those of
+//      earlier sets that pass the length filter (positions [lo, its own), and
+//      optionally the positional bound of the matching token, PPJoin-style),
+//      drops repeated ones by a set in shared memory, and tests the others'
+//      short records 32 at a time;
+//   4. a warp per run of pairs left tests their long records and queues what
+//      remains for the verify kernel (signature.cuh).
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
 #include <cuda_runtime.h>
 
 #include "arith.h"
+#include "signature.cuh"
 #include "ssj_internal.h"
 
 namespace ssj {
 namespace {
 
-constexpr int kGenWarps = 8;             // warps per CTA of the probing kernel
-constexpr uint32_t kGenBuf = 256;        // candidates buffered per warp before a flush
+constexpr int kJoinWarps = 8;             // warps per CTA of the join kernel
+constexpr uint32_t kSeenWords = 1024;    // a warp's set of candidates seen: a bitmap of 32,768 positions, or a
+constexpr uint32_t kSeenBits = 32 * kSeenWords;  // hash set of up to half as many as it has words
+constexpr uint32_t kJoinFlush = kJoinRun - 32;  // pairs left that a warp hands over at once (room for 32 more)
+constexpr uint32_t kLongList = 64;       // index entries of a token that a whole warp reads as one list
 constexpr unsigned kAll = 0xFFFFFFFFu;
-constexpr uint64_t kEmpty = ~0ull;
+constexpr uint32_t kFree = 0xFFFFFFFFu;
 
 struct Params {
     const uint4* toks4;
@@ -83,16 +84,48 @@ __device__ __forceinline__ uint32_t pair_required(const Params& P, uint32_t nr, 
     }
 }
 
-__global__ void size_hist_kernel(Params P, uint64_t* hist) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n; i += gridDim.x * blockDim.x)
-        atomicAdd(reinterpret_cast<unsigned long long*>(hist + P.desc[i].y), 1ull);
+// Counting sort by size.  A CTA takes one run of sets and counts them in shared
+// memory first, so that the global counters see one atomic per size and CTA
+// (200,000 sets of about 100 sizes: 54 + 56 us with one atomic per set).
+constexpr uint32_t kSizeBins = 4096;  // sizes counted in shared memory; longer sets one by one
+constexpr int kSizeThreads = 256;
+
+__global__ void __launch_bounds__(kSizeThreads) size_hist_kernel(Params P, uint32_t per_cta, uint64_t* hist) {
+    __shared__ uint32_t cnt[kSizeBins];
+    for (uint32_t b = threadIdx.x; b < kSizeBins; b += kSizeThreads) cnt[b] = 0;
+    __syncthreads();
+    const uint32_t lo = blockIdx.x * per_cta, hi = min(lo + per_cta, P.n);
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += kSizeThreads) {
+        const uint32_t L = P.desc[i].y;
+        if (L < kSizeBins) atomicAdd(cnt + L, 1u);
+        else atomicAdd(reinterpret_cast<unsigned long long*>(hist + L), 1ull);
+    }
+    __syncthreads();
+    for (uint32_t b = threadIdx.x; b < kSizeBins; b += kSizeThreads)
+        if (cnt[b]) atomicAdd(reinterpret_cast<unsigned long long*>(hist + b), (unsigned long long)cnt[b]);
 }
 
-__global__ void place_kernel(Params P, uint64_t* cursor, uint32_t* order, uint32_t* rank) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < P.n; i += gridDim.x * blockDim.x) {
-        const uint32_t pos =
-            (uint32_t)atomicAdd(reinterpret_cast<unsigned long long*>(cursor + P.desc[i].y), 1ull);
-        order[pos] = i;
+// cursor: the sizes' first positions; afterwards the positions after their
+// last.  probes: the sets from the last position down.
+__global__ void __launch_bounds__(kSizeThreads) place_kernel(Params P, uint32_t per_cta, uint64_t* cursor,
+                                                             uint32_t* probes, uint32_t* rank) {
+    __shared__ uint32_t cnt[kSizeBins], at[kSizeBins];
+    for (uint32_t b = threadIdx.x; b < kSizeBins; b += kSizeThreads) cnt[b] = 0;
+    __syncthreads();
+    const uint32_t lo = blockIdx.x * per_cta, hi = min(lo + per_cta, P.n);
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += kSizeThreads) {
+        const uint32_t L = P.desc[i].y;
+        if (L < kSizeBins) atomicAdd(cnt + L, 1u);
+    }
+    __syncthreads();
+    for (uint32_t b = threadIdx.x; b < kSizeBins; b += kSizeThreads)
+        if (cnt[b]) at[b] = (uint32_t)atomicAdd(reinterpret_cast<unsigned long long*>(cursor + b), (unsigned long long)cnt[b]);
+    __syncthreads();
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += kSizeThreads) {
+        const uint32_t L = P.desc[i].y;
+        const uint32_t pos = L < kSizeBins ? atomicAdd(at + L, 1u)
+                                           : (uint32_t)atomicAdd(reinterpret_cast<unsigned long long*>(cursor + L), 1ull);
+        probes[P.n - 1 - pos] = i;
         rank[i] = pos;
     }
 }
@@ -125,133 +158,233 @@ __global__ void postings_kernel(Params P, const uint32_t* rank, uint64_t* tcur, 
     }
 }
 
-// Does index entry e (a set at position e.x, token position e.y, size e.z)
-// matched at probe token position a yield a candidate of the probe at
-// position rpos with size L?
-__device__ __forceinline__ bool entry_ok(const Params& P, uint4 e, uint32_t rpos, uint32_t L, uint64_t min_size,
-                                         uint32_t a) {
-    if (e.x >= rpos || e.z < min_size) return false;  // earlier sets only; length filter
-    if (P.positional) {
-        // at most min(a, j) matches before this one, one here, min(|r|-a-1, |s|-j-1) after
-        const uint32_t ub = min(a, e.y) + 1 + min(L - a - 1, e.z - e.y - 1);
-        if (ub < pair_required(P, L, e.z)) return false;
-    }
-    return true;
+// Positional bound of index entry e (a set of size e.z, the token at e.y)
+// matched at probe token position a: at most min(a, j) matches before this
+// one, one here, min(|r|-a-1, |s|-j-1) after.
+__device__ __forceinline__ bool position_ok(const Params& P, uint4 e, uint32_t L, uint32_t a) {
+    const uint32_t ub = min(a, e.y) + 1 + min(L - a - 1, e.z - e.y - 1);
+    return ub >= pair_required(P, L, e.z);
 }
 
-// one warp per probe position: entries that pass entry_ok, summed per warp
-__global__ void precount_kernel(Params P, const uint32_t* order, const uint64_t* toff, const uint4* post,
-                                unsigned long long* total) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-    unsigned long long mine = 0;
-    for (uint32_t rpos = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; rpos < P.n; rpos += warps) {
-        const uint32_t r = order[rpos];
-        const uint2 d = P.desc[r];
-        const uint32_t* t = set_tokens(P, d);
-        const uint32_t L = d.y, pl = prefix_len(P, L);
-        const uint64_t min_size = min_overlap(P, L);
-        for (uint32_t a = 0; a < pl; ++a) {
-            const uint32_t tok = t[a];
-            for (uint64_t e = toff[tok] + lane; e < toff[tok + 1]; e += 32)
-                mine += entry_ok(P, post[e], rpos, L, min_size, a) ? 1 : 0;
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(kAll, mine, o);
-    if (lane == 0 && mine) atomicAdd(total, mine);
-}
-
-__device__ __forceinline__ uint64_t mix64(uint64_t x) {
-    x ^= x >> 33;
-    x *= 0xff51afd7ed558ccdull;
-    x ^= x >> 33;
-    x *= 0xc4ceb9fe1a85ec53ull;
-    x ^= x >> 33;
+__device__ __forceinline__ uint32_t mix32(uint32_t x) {
+    x ^= x >> 16;
+    x *= 0x85ebca6bu;
+    x ^= x >> 13;
+    x *= 0xc2b2ae35u;
+    x ^= x >> 16;
     return x;
 }
 
-// Insert key; true if it was not there.  The table has a power-of-two size
-// at least twice the number of keys ever inserted, so a free slot is always
-// found within the table.  Should the probe loop ever run through the whole
-// table (a sizing bug), the key cannot be stored: ERR_GUARD is set, so the
-// call fails with SSJ_EDEVICE instead of losing the candidate silently.
-__device__ __forceinline__ bool hash_insert(unsigned long long* table, uint64_t mask, uint64_t key, uint32_t* err) {
-    uint64_t h = mix64(key) & mask;
-    for (uint64_t probe = 0; probe <= mask; ++probe) {
-        const unsigned long long prev = atomicCAS(table + h, (unsigned long long)kEmpty, (unsigned long long)key);
-        if (prev == kEmpty) return true;
-        if (prev == key) return false;
-        h = (h + 1) & mask;
-    }
-    atomicOr(err, ERR_GUARD);
-    return false;
-}
-
-struct GenOut {
-    uint32_t* probe_ids;           // per group: probe set id
-    uint64_t* cand_offsets;        // per group: first candidate (the final entry is written last)
-    uint32_t* cand_ids;
-    unsigned long long* packed;    // groups << 40 | candidates
-    uint64_t group_cap, cand_cap;
-    uint32_t* err;
+struct JoinArgs {
+    const uint32_t* probes;    // the sets in the order in which they probe: from the last position down
+    const uint64_t* size_end;  // size -> position after its last set
+    const uint64_t* toff;      // token -> first index entry (n_tokens + 1)
+    const uint4* post;         // index entries
+    uint32_t* cursor;          // next probe (from the last position down)
+    uint32_t grab;             // probes per grab
+    JoinQueue out;             // pairs left
 };
 
-__global__ void __launch_bounds__(kGenWarps * 32) generate_kernel(Params P, const uint32_t* order,
-                                                                  const uint64_t* toff, const uint4* post,
-                                                                  unsigned long long* table, uint64_t mask,
-                                                                  GenOut O) {
-    __shared__ uint32_t buf[kGenWarps][kGenBuf];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+struct JoinWarp {
+    uint32_t seen[kSeenWords];
+    uint2 buf[kJoinRun];
+    uint32_t fresh[64];  // candidates to be tested
+};
+
+// The join of the sets in size order: a warp takes a probe at a time, the
+// largest first (they have the most candidates).  The tokens' index entries
+// are read flat, 32 at a time, lists of kLongList entries or more one by one.
+// A candidate found through several tokens is kept once, by a bitmap over the
+// positions that the length filter admits; when these are more than the
+// bitmap holds, by a hash set if there are few entries, else window by window
+// of positions.  G: sectors per record of the first level of the signature
+// test, 0: every candidate is handed over.
+// Bound by latency (index entries and records from L2, shared-memory atomics).
+// All kernels up to the queue take 0.28 ms on 5.7e6 candidates of short sets
+// and 0.64 ms on 1.4e7 of long sets; with a hash set of all the join's pairs in
+// device memory, a sizing pass for it and the candidate lists written and
+// read, they took 1.75 and 3.65 ms.
+template <int G>
+__global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_constant__ VerifyArgs a, Params P,
+                                                                  JoinArgs J) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ PlanInst s_inst;
+    constexpr int kG = G > 0 ? G : 1;
+    const int lane = threadIdx.x & 31;
+    JoinWarp& W = reinterpret_cast<JoinWarp*>(smem)[threadIdx.x >> 5];
     const unsigned lt = (1u << lane) - 1u;
-    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-    uint32_t* b = buf[warp];
-    for (uint32_t rpos = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; rpos < P.n; rpos += warps) {
-        const uint32_t r = order[rpos];
-        const uint2 d = P.desc[r];
-        const uint32_t* t = set_tokens(P, d);
-        const uint32_t L = d.y, pl = prefix_len(P, L);
-        const uint64_t min_size = min_overlap(P, L);
-        uint32_t nb = 0;  // buffered candidates (warp-uniform)
-        auto flush = [&]() {
-            unsigned long long old = 0;
-            if (lane == 0) old = atomicAdd(O.packed, (1ull << 40) | (unsigned long long)nb);
-            old = __shfl_sync(kAll, old, 0);
-            const uint64_t g = old >> 40, start = old & ((1ull << 40) - 1);
-            if (g >= O.group_cap || start + nb > O.cand_cap) {  // cannot happen with sized outputs
-                if (lane == 0) atomicOr(O.err, ERR_GUARD);
-            } else {
-                if (lane == 0) {
-                    O.probe_ids[g] = r;
-                    O.cand_offsets[g] = start;
-                }
-                for (uint32_t k = lane; k < nb; k += 32) O.cand_ids[start + k] = b[k];
+    if (threadIdx.x == 0) {
+        s_inst = plan_inst(a.single);
+        if (blockIdx.x == 0) {
+            a.table_out[0] = a.single;
+            *a.single.count = 0ull;
+        }
+    }
+    __syncthreads();
+    const PlanInst& I = s_inst;
+    unsigned long long found = 0;  // candidates (warp-uniform)
+    uint32_t n = 0;                // pairs in buf (warp-uniform)
+    auto hand_over = [&]() {       // buf as one run
+        unsigned long long at = 0, run = 0;
+        if (lane == 0) {
+            at = atomicAdd(&a.ctr->join_pairs, (unsigned long long)n);
+            if (at + n <= J.out.pair_cap) run = atomicAdd(&a.ctr->join_runs, 1ull);
+        }
+        at = __shfl_sync(kAll, at, 0);
+        if (at + n <= J.out.pair_cap) {  // (else the host sees the count and asks again with more room)
+            if (lane == 0) {
+                if (run < J.out.run_cap) J.out.runs[run] = make_ulonglong2(at, n);
+                else atomicOr(&a.ctr->err, ERR_GUARD);  // cannot happen with a sized workspace
             }
-            __syncwarp();
-            nb = 0;
-        };
-        for (uint32_t a = 0; a < pl; ++a) {
-            const uint32_t tok = t[a];
-            const uint64_t e0 = toff[tok], e1 = toff[tok + 1];
-            for (uint64_t base = e0; base < e1; base += 32) {
-                const uint64_t e = base + lane;
-                bool fresh = false;
-                uint32_t sid = 0;
-                if (e < e1) {
-                    const uint4 en = post[e];
-                    if (entry_ok(P, en, rpos, L, min_size, a)) {
-                        fresh = hash_insert(table, mask, ((uint64_t)rpos << 32) | en.x, O.err);
-                        sid = en.w;
+            for (uint32_t k = lane; k < n; k += 32) J.out.pairs[at + k] = W.buf[k];
+        }
+        __syncwarp();
+        n = 0;
+    };
+    for (;;) {
+        uint32_t g0 = 0;
+        if (lane == 0) g0 = atomicAdd(J.cursor, J.grab);
+        g0 = __shfl_sync(kAll, g0, 0);
+        if (g0 >= P.n) break;
+        for (uint32_t g = g0; g < min(g0 + J.grab, P.n); ++g) {
+            const uint32_t rpos = P.n - 1 - g, r = J.probes[g];
+            const uint2 d = P.desc[r];
+            const uint32_t* t = set_tokens(P, d);
+            const uint32_t L = d.y, pl = prefix_len(P, L);
+            if (pl == 0) continue;
+            const uint64_t min_size = min_overlap(P, L);  // at least 1, at most L
+            const uint32_t lo = (uint32_t)J.size_end[min_size - 1];
+            if (lo >= rpos) continue;
+            Sector rs;
+            uint32_t nr = 0, q = 0;  // q: candidates waiting for the test
+            if (G > 0) {
+                rs = ld_sector(I.r_rec[0] + ((uint64_t)r * kG + lane % kG) * 2);
+                nr = __ldg(&I.r_rec[0][(uint64_t)r * kG * 2].x) >> 16;
+            }
+            auto test = [&](uint32_t m) {
+                const uint32_t s = W.fresh[(uint32_t)lane < m ? lane : 0];
+                bool pass = (uint32_t)lane < m;
+                if (G > 0) {
+                    const uint32_t v = bound_of_pair<kG, true>(I.s_rec[0], nullptr, s, 0u, rs, lane);
+                    pass = pass && bound_passes(I, v, nr);
+                }
+                const uint32_t pm = __ballot_sync(kAll, pass);
+                if (pass) W.buf[n + __popc(pm & lt)] = make_uint2(g, s);
+                n += __popc(pm);
+                __syncwarp();
+            };
+            // entries in all, if the positions are more than the bitmap holds
+            uint32_t hash_mask = 0;
+            if (rpos - lo > kSeenBits) {
+                uint64_t e = 0;
+                for (uint32_t k = lane; k < pl; k += 32) e += J.toff[t[k] + 1] - J.toff[t[k]];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(kAll, e, o);
+                if (e <= kSeenWords / 2) hash_mask = e <= 32 ? 63u : (2u << (31 - __clz((uint32_t)e * 2 - 1))) - 1;
+            }
+            const uint32_t window = hash_mask ? rpos - lo : kSeenBits;
+            for (uint32_t w0 = lo; w0 < rpos; w0 += min(window, rpos - w0)) {
+                const uint32_t w1 = w0 + min(window, rpos - w0);
+                const uint32_t words = hash_mask ? hash_mask + 1 : (w1 - w0 + 31) / 32;
+                for (uint32_t k = lane; k < words; k += 32) W.seen[k] = hash_mask ? kFree : 0u;
+                __syncwarp();
+                // one index entry per lane (if have), found at the probe's token k
+                auto take = [&](bool have, uint64_t e, uint32_t k) {
+                    bool is_new = false;
+                    uint4 en = make_uint4(0u, 0u, 0u, 0u);
+                    if (have) {
+                        en = __ldg(J.post + e);
+                        if (en.x >= w0 && en.x < w1 && !(P.positional && !position_ok(P, en, L, k))) {
+                            if (hash_mask) {
+                                uint32_t h = mix32(en.x) & hash_mask;
+                                for (;;) {  // (at most half of the slots are ever taken)
+                                    const uint32_t old = atomicCAS(W.seen + h, kFree, en.x);
+                                    is_new = old == kFree;
+                                    if (is_new || old == en.x) break;
+                                    h = (h + 1) & hash_mask;
+                                }
+                            } else {
+                                const uint32_t b = en.x - w0, bit = 1u << (b & 31u);
+                                is_new = (atomicOr(W.seen + (b >> 5), bit) & bit) == 0;
+                            }
+                        }
+                    }
+                    const uint32_t m = __ballot_sync(kAll, is_new);
+                    if (is_new) W.fresh[q + __popc(m & lt)] = en.w;
+                    q += __popc(m);
+                    found += __popc(m);
+                    __syncwarp();
+                    if (q >= 32) {
+                        if (n >= kJoinFlush) hand_over();
+                        test(32);
+                        q -= 32;
+                        const uint32_t keep = W.fresh[32 + lane];
+                        __syncwarp();
+                        if ((uint32_t)lane < q) W.fresh[lane] = keep;
+                        __syncwarp();
+                    }
+                };
+                for (uint32_t k0 = 0; k0 < pl; k0 += 32) {
+                    uint64_t start = 0, len = 0;
+                    if (k0 + lane < pl) {
+                        const uint32_t tok = t[k0 + lane];
+                        start = J.toff[tok];
+                        len = J.toff[tok + 1] - start;
+                    }
+                    uint32_t longs = __ballot_sync(kAll, len >= kLongList);
+                    while (longs) {
+                        const int src = __ffs(longs) - 1;
+                        longs &= longs - 1;
+                        const uint64_t e0 = __shfl_sync(kAll, start, src), e1 = e0 + __shfl_sync(kAll, len, src);
+                        for (uint64_t e = e0; e < e1; e += 32) take(e + lane < e1, e + lane, k0 + src);
+                    }
+                    const uint32_t mine = len >= kLongList ? 0u : (uint32_t)len;
+                    uint32_t incl = mine;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t y = __shfl_up_sync(kAll, incl, o);
+                        if (lane >= o) incl += y;
+                    }
+                    const uint32_t total = __shfl_sync(kAll, incl, 31);
+                    const uint64_t base = start - (incl - mine);  // entry e of the flat list is base + e of its token
+                    for (uint32_t e0 = 0; e0 < total; e0 += 32) {
+                        const uint32_t e = e0 + lane;
+                        uint32_t k = 0;  // tokens whose entries end by e
+#pragma unroll
+                        for (int step = 16; step >= 1; step >>= 1) {
+                            const uint32_t v = __shfl_sync(kAll, incl, k + step - 1);
+                            if (v <= e) k += step;
+                        }
+                        const uint64_t at = __shfl_sync(kAll, base, k) + e;
+                        take(e < total, at, k0 + k);
                     }
                 }
-                const unsigned fm = __ballot_sync(kAll, fresh);
-                if (fresh) b[nb + __popc(fm & lt)] = sid;
-                nb += __popc(fm);
-                __syncwarp();
-                if (nb > kGenBuf - 32) flush();
             }
+            if (n >= kJoinFlush) hand_over();
+            if (q) test(q);
         }
-        if (nb) flush();
+    }
+    if (n) hand_over();
+    if (lane == 0 && found) atomicAdd(&a.ctr->candidates, found);
+}
+
+// The runs' second level and queueing (a kernel of its own: a function call in
+// the join kernel's loops would cost them their registers).
+__global__ void __launch_bounds__(kJoinWarps * 32) queue_kernel(const __grid_constant__ VerifyArgs a, JoinQueue Q) {
+    __shared__ PlanInst s_inst;
+    __shared__ uint2 s_buf[kJoinWarps][kJoinRun];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_inst = plan_inst(a.single);
+    __syncthreads();
+    if (a.ctr->join_pairs > Q.pair_cap) return;  // not all of them are here: the host asks again
+    const unsigned long long runs = min(a.ctr->join_runs, (unsigned long long)Q.run_cap);
+    for (unsigned long long b = blockIdx.x * kJoinWarps + warp; b < runs; b += gridDim.x * kJoinWarps) {
+        const ulonglong2 run = Q.runs[b];
+        const uint32_t n = min((uint32_t)run.y, kJoinRun);
+        for (uint32_t k = lane; k < n; k += 32) s_buf[warp][k] = Q.pairs[run.x + k];
+        __syncwarp();
+        flush_survivors(a, s_inst, 0, s_buf[warp], n, lane);
+        __syncwarp();
     }
 }
 
@@ -370,10 +503,12 @@ cudaError_t candgen_run(const CandgenInput& in, cudaStream_t st, int num_sms, Ca
         if (e == cudaSuccess) e = cudaMemsetAsync(ix->tcnt, 0, 8ull * (in.vocab + 1), st);
         if (e != cudaSuccess) return e;
         if (in.n) {
-            size_hist_kernel<<<grid_for(in.n, tb, num_sms, 8), tb, 0, st>>>(P, ix->size_hist);
+            const uint32_t per = std::max<uint32_t>((in.n + 2 * (uint32_t)num_sms - 1) / (2 * (uint32_t)num_sms), 1024u);
+            const unsigned blocks = (in.n + per - 1) / per;
+            size_hist_kernel<<<blocks, kSizeThreads, 0, st>>>(P, per, ix->size_hist);
             e = exclusive_scan_u64(ix->size_hist, in.max_len + 2, ix->scan_scratch, ix->total, st);
             if (e != cudaSuccess) return e;
-            place_kernel<<<grid_for(in.n, tb, num_sms, 8), tb, 0, st>>>(P, ix->size_hist, ix->order, ix->rank);
+            place_kernel<<<blocks, kSizeThreads, 0, st>>>(P, per, ix->size_hist, ix->probes, ix->rank);
             token_count_kernel<<<grid_for(32ull * in.n, tb, num_sms, 8), tb, 0, st>>>(P, ix->tcnt);
         }
         e = cudaMemcpyAsync(ix->toff, ix->tcnt, 8ull * (in.vocab + 1), cudaMemcpyDeviceToDevice, st);
@@ -382,39 +517,57 @@ cudaError_t candgen_run(const CandgenInput& in, cudaStream_t st, int num_sms, Ca
         if (e != cudaSuccess) return e;
         return cudaStreamSynchronize(st);  // *host_word: index entries
     }
-    if (in.stage == 1) {
-        // fill the token lists, then count the entries that can yield candidates
-        e = cudaMemcpyAsync(ix->tcnt, ix->toff, 8ull * (in.vocab + 1), cudaMemcpyDeviceToDevice, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(ix->total, 0, 8, st);
-        if (e != cudaSuccess) return e;
-        if (in.n) {
-            postings_kernel<<<grid_for(32ull * in.n, tb, num_sms, 8), tb, 0, st>>>(P, ix->rank, ix->tcnt, ix->post);
-            precount_kernel<<<grid_for(32ull * in.n, tb, num_sms, 8), tb, 0, st>>>(
-                P, ix->order, ix->toff, ix->post, reinterpret_cast<unsigned long long*>(ix->total));
-        }
-        e = cudaMemcpyAsync(host_word, ix->total, 8, cudaMemcpyDeviceToHost, st);
-        if (e != cudaSuccess) return e;
-        return cudaStreamSynchronize(st);  // *host_word: entries passing the filters
-    }
-    // stage 2: probe, deduplicate and emit
-    e = cudaMemsetAsync(in.table, 0xFF, 8ull * (in.table_mask + 1), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(in.out.packed, 0, 8, st);
-    if (e != cudaSuccess) return e;
+    // fill the token lists
     if (in.n) {
-        GenOut O;
-        O.probe_ids = in.out.probe_ids;
-        O.cand_offsets = in.out.cand_offsets;
-        O.cand_ids = in.out.cand_ids;
-        O.packed = in.out.packed;
-        O.group_cap = in.out.group_cap;
-        O.cand_cap = in.out.cand_cap;
-        O.err = in.out.err;
-        generate_kernel<<<grid_for(32ull * in.n, kGenWarps * 32, num_sms, 4), kGenWarps * 32, 0, st>>>(
-            P, ix->order, ix->toff, ix->post, in.table, in.table_mask, O);
+        e = cudaMemcpyAsync(ix->tcnt, ix->toff, 8ull * (in.vocab + 1), cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) return e;
+        postings_kernel<<<grid_for(32ull * in.n, tb, num_sms, 8), tb, 0, st>>>(P, ix->rank, ix->tcnt, ix->post);
     }
-    e = cudaMemcpyAsync(host_word, in.out.packed, 8, cudaMemcpyDeviceToHost, st);
+    return cudaGetLastError();
+}
+
+template <int G>
+static cudaError_t launch_join(const VerifyArgs& a, const Params& P, JoinArgs J, int num_sms, cudaStream_t st) {
+    constexpr size_t smem = kJoinWarps * sizeof(JoinWarp);
+    cudaError_t e = cudaFuncSetAttribute(join_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    return cudaStreamSynchronize(st);  // *host_word: groups << 40 | candidates
+    const unsigned blocks = (unsigned)std::max<uint64_t>(
+        1, std::min<uint64_t>(((uint64_t)P.n + kJoinWarps - 1) / kJoinWarps, 4ull * num_sms));
+    J.grab = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(8, P.n / (16ull * blocks * kJoinWarps)));
+    join_kernel<G><<<blocks, kJoinWarps * 32, smem, st>>>(a, P, J);
+    return cudaGetLastError();
+}
+
+cudaError_t join_probe(const CandgenInput& in, const CandgenIndex& ix, const VerifyArgs& a, const JoinQueue& out,
+                       cudaStream_t st, int num_sms) {
+    Params P;
+    P.toks4 = in.toks4;
+    P.desc = in.desc;
+    P.n = in.n;
+    P.sim = in.sim;
+    P.p = in.p;
+    P.q = in.q;
+    P.positional = in.positional;
+    JoinArgs J;
+    J.probes = ix.probes;
+    J.size_end = ix.size_hist;
+    J.toff = ix.toff;
+    J.post = ix.post;
+    J.cursor = &a.ctr->probe_cursor;
+    J.grab = 1;
+    J.out = out;
+    cudaError_t e = cudaMemsetAsync(a.ctr, 0, sizeof(Counters), st);
+    if (e != cudaSuccess) return e;
+    switch (a.single.rec_sectors[0]) {
+        case 1: e = launch_join<1>(a, P, J, num_sms, st); break;
+        case 2: e = launch_join<2>(a, P, J, num_sms, st); break;
+        case 4: e = launch_join<4>(a, P, J, num_sms, st); break;
+        case 8: e = launch_join<8>(a, P, J, num_sms, st); break;
+        default: e = launch_join<0>(a, P, J, num_sms, st); break;
+    }
+    if (e != cudaSuccess) return e;
+    queue_kernel<<<(unsigned)(2 * num_sms), kJoinWarps * 32, 0, st>>>(a, out);
+    return cudaGetLastError();
 }
 
 cudaError_t expand_groups(const GroupExpand& x, cudaStream_t st, int num_sms, uint64_t* host_words) {

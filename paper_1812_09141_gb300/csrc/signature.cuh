@@ -1,0 +1,329 @@
+// The signature test of candidate pairs and the queueing of the pairs that it
+// leaves, shared by the plan kernel (plan.cu) and the join kernel
+// (candgen.cu).
+//
+// The signature test is the bitmap filter of Sandes, Teodoro and Melo
+// ("Bitmap filter: speeding up exact set similarity joins with bitwise
+// operations", 2020): a set's record (layout.cu) holds its length, a bitmap
+// of its tokens' hash values, and its loss, the number of tokens that share
+// a bit with another token of the set.  With a the common bits of two
+// bitmaps, |r n s| <= a + min(loss_r, loss_s): every common token sets a
+// common bit, and of the tokens of x on common bits at most loss_x are not
+// the first on their bit.  The bound is tested with the exact integer form of
+// the similarity function, which is monotone in the overlap, so a pair that
+// passes the join is never dropped.  (The bound never exceeds min(|r|, |s|),
+// so the test includes the length filter of Section 2.2.3.)
+//
+// Two levels: a short record first (about one bit per token), and for the
+// pairs that it leaves, a few percent, a long one.
+#pragma once
+
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "arith.h"
+#include "checked.cuh"
+#include "ssj_internal.h"
+
+namespace ssj {
+
+namespace {
+
+constexpr uint32_t kFull = 0xFFFFFFFFu;
+constexpr uint32_t kPlanBuf = kPlanFlush + 32;  // pairs buffered per warp
+constexpr int kSectors = 2;                     // 32-byte record loads in flight per lane, at most (4: 2% slower)
+
+// Instance fields read by the plan kernel (from the kernel parameters for a
+// one-batch launch, else from the device table).
+struct PlanInst {
+    const uint32_t* probe_ids;
+    const uint64_t* cand_offsets;
+    const uint32_t* cand_ids;
+    const uint4* r_rec[2];
+    const uint4* s_rec[2];
+    const uint2* r_desc;
+    const uint2* s_desc;
+    uint64_t n_cands, chunk_base;
+    uint32_t r_n_sets, s_n_sets, n_probes, tile_base, flags, sim, p, den;
+    uint32_t rec_sectors[2];
+};
+
+__device__ __forceinline__ PlanInst plan_inst(const Instance& I) {
+    PlanInst q;
+    q.probe_ids = I.probe_ids;
+    q.cand_offsets = I.cand_offsets;
+    q.cand_ids = I.cand_ids;
+    q.r_desc = I.r_desc;
+    q.s_desc = I.s_desc;
+    q.n_cands = I.n_cands;
+    q.chunk_base = I.chunk_base;
+    q.r_n_sets = I.r_n_sets;
+    q.s_n_sets = I.s_n_sets;
+    q.n_probes = I.n_probes;
+    q.tile_base = I.tile_base;
+    q.flags = I.flags;
+    q.sim = I.sim;
+    q.p = I.p;
+    q.den = I.den;
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+        q.r_rec[l] = I.r_rec[l];
+        q.s_rec[l] = I.s_rec[l];
+        q.rec_sectors[l] = I.rec_sectors[l];
+    }
+    return q;
+}
+
+// Does overlap o reach the threshold (Table "Similarity Functions", exact
+// integer forms)?  Empty sets never match.
+__device__ __forceinline__ bool overlap_passes(const PlanInst& I, uint32_t o, uint32_t nr, uint32_t ns) {
+    if (nr == 0 || ns == 0) return false;
+    if (I.sim == SIM_COSINE) return cosine_pass(o, I.p, I.den, nr, ns);
+    if (I.sim == SIM_OVERLAP) return o >= I.den;
+    return (uint64_t)o * I.den >= (uint64_t)I.p * ((uint64_t)nr + ns);  // Jaccard: den = p + q, Dice: 2q
+}
+
+// One 32-byte sector of a record.
+struct Sector {
+    uint32_t w[8];
+};
+
+__device__ __forceinline__ Sector ld_sector(const uint4* p) {
+    Sector x;
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(x.w[0]), "=r"(x.w[1]), "=r"(x.w[2]), "=r"(x.w[3]), "=r"(x.w[4]), "=r"(x.w[5]), "=r"(x.w[6]), "=r"(x.w[7])
+        : "l"(p));
+    return x;
+}
+
+// Common bits of two sectors, the first word only where `first` has bits:
+// full adders (a sum and a carry of three words, one logic operation each)
+// turn eight words into four to count, since counting runs at a fraction of
+// the rate of logic.
+__device__ __forceinline__ uint32_t common_bits(const Sector& x, const Sector& y, uint32_t first) {
+    uint32_t v[8];
+    v[0] = x.w[0] & y.w[0] & first;
+#pragma unroll
+    for (int i = 1; i < 8; ++i) v[i] = x.w[i] & y.w[i];
+    auto sum = [](uint32_t p, uint32_t q, uint32_t r) { return p ^ q ^ r; };
+    auto carry = [](uint32_t p, uint32_t q, uint32_t r) { return (p & q) | (p & r) | (q & r); };
+    const uint32_t s1 = sum(v[0], v[1], v[2]), c1 = carry(v[0], v[1], v[2]);
+    const uint32_t s2 = sum(v[3], v[4], v[5]), c2 = carry(v[3], v[4], v[5]);
+    const uint32_t s3 = sum(s1, s2, v[6]), c3 = carry(s1, s2, v[6]);
+    const uint32_t s4 = sum(c1, c2, c3), c4 = carry(c1, c2, c3);
+    return __popc(s3) + __popc(v[7]) + 2 * __popc(s4) + 4 * __popc(c4);
+}
+
+// Sum over the G lanes of a group of their part[i], i the lane's place in the
+// group: a butterfly that halves the values at each step.
+template <int G>
+__device__ __forceinline__ uint32_t sum_of_group(uint32_t (&part)[G], uint32_t sub) {
+#pragma unroll
+    for (int m = G / 2; m > 0; m /= 2) {
+#pragma unroll
+        for (int i = 0; i < m; ++i) {
+            const bool up = (sub & m) != 0;
+            const uint32_t give = up ? part[i] : part[i + m], keep = up ? part[i + m] : part[i];
+            part[i] = keep + __shfl_xor_sync(kFull, give, m);
+        }
+    }
+    return part[0];
+}
+
+// For the lane's own pair (any valid ids s, r): |s| in the upper half, the
+// bound on the overlap in the lower half (see the record header, rec_bits).
+// G lanes read a record, a sector each, so that a load takes whole lines (a
+// lane reading its own record 16 bytes at a time costs one L1 wavefront per
+// lane and load: with 128-byte records 90% of the L1's wavefronts and twice
+// the time); the partial counts of the group's G pairs are then summed across
+// it.  kSame: every lane's probe is the one whose sector of this lane is rs.
+template <int G, bool kSame>
+__device__ __forceinline__ uint32_t bound_of_pair(const uint4* s_rec, const uint4* r_rec, uint32_t s, uint32_t r,
+                                                  const Sector& rs, int lane, uint32_t* r_head = nullptr) {
+    const uint32_t sub = lane % G;
+    const uint32_t first = sub == 0 ? 0u : kFull;  // the first sector's first word is the header
+    constexpr int kBatch = G < kSectors ? G : kSectors;  // loads in flight
+    uint32_t part[G];
+#pragma unroll
+    for (int b = 0; b < G; b += kBatch) {
+        Sector x[kBatch];
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+            const uint32_t sj = G == 1 ? s : __shfl_sync(kFull, s, b + i, G);
+            x[i] = ld_sector(s_rec + ((uint64_t)sj * G + sub) * 2);
+        }
+#pragma unroll
+        for (int i = 0; i < kBatch; ++i) {
+            uint32_t hr;
+            if (kSame) {
+                part[b + i] = common_bits(x[i], rs, first);
+                hr = rs.w[0];
+            } else {
+                const uint32_t rj = G == 1 ? r : __shfl_sync(kFull, r, b + i, G);
+                const Sector y = ld_sector(r_rec + ((uint64_t)rj * G + sub) * 2);
+                part[b + i] = common_bits(x[i], y, first);
+                hr = y.w[0];
+                if (G == 1) *r_head = hr;
+            }
+            if (G == 1 || sub == 0) part[b + i] += (x[i].w[0] & 0xFFFF0000u) + min(x[i].w[0] & 0xFFFFu, hr & 0xFFFFu);
+        }
+    }
+    return sum_of_group<G>(part, sub);
+}
+
+// The signature test of a pair from its bound_of_pair value and |r| (65535 in
+// a header: 65535 tokens or more, not tested).
+__device__ __forceinline__ bool bound_passes(const PlanInst& I, uint32_t v, uint32_t nr) {
+    const uint32_t ns = v >> 16;
+    return ns == 0xFFFFu || nr == 0xFFFFu || overlap_passes(I, v & 0xFFFFu, nr, ns);
+}
+
+// Second level: the n buffered pairs tested with the long records; the ones
+// left stay in the buffer, in order.  Returns their number.
+template <int G>
+__device__ __noinline__ uint32_t second_level(const PlanInst& I, uint2* buf, uint32_t n, int lane) {
+    const unsigned lt_mask = (1u << lane) - 1u;
+    uint32_t left = 0;
+    for (uint32_t t = 0; t < n; t += 32) {
+        const bool have = t + lane < n;
+        const uint2 e = buf[have ? t + lane : t];
+        const uint32_t r = __ldg(I.probe_ids + (e.x - 32u * I.tile_base));
+        const uint32_t r_head = __ldg(&I.r_rec[1][(uint64_t)r * G * 2].x);
+        const uint32_t v = bound_of_pair<G, false>(I.s_rec[1], I.r_rec[1], e.y, r, Sector(), lane);
+        const bool pass = have && bound_passes(I, v, r_head >> 16);
+        const uint32_t m = __ballot_sync(kFull, pass);  // (every lane has read its entry)
+        if (pass) buf[left + __popc(m & lt_mask)] = e;
+        left += __popc(m);
+        __syncwarp();
+    }
+    return left;
+}
+
+// Granularity of a probe with |r| = nr and n candidates left: 0 thread per
+// pair, 1 warp per pair, 2 block per pair, 3 lane per pair with r in the
+// warp's shared memory (Alternative B; needs r to fit and enough candidates
+// to occupy the lanes), 4 index items (many candidates, when the launch's
+// token values fit the probe bitmap).
+__device__ __forceinline__ uint32_t probe_bin(const VerifyArgs& a, uint32_t flags, uint32_t nr, uint32_t n) {
+    const bool lane_ok = nr + 4 <= kWarpRCap;
+    if (flags & VF_FORCE_INDEX) return a.index_words ? 4u : (lane_ok ? 3u : 1u);
+    if (flags & VF_FORCE_BLOCK) return 2;
+    if (flags & VF_FORCE_WARP) return 1;
+    if (flags & VF_FORCE_THREAD) return 0;
+    if (flags & VF_FORCE_LANE) return lane_ok ? 3u : 1u;
+    if (a.index_words && a.index_min_cands && n >= min(a.index_min_cands, kPlanFlush)) return 4;
+    const uint64_t key = 2ull * nr;  // |r|+|s| at |s| = |r|
+    if (key <= a.thread_max_key) return 0;
+    if (key <= a.lane_max_key && lane_ok && n >= kLaneMinCands) return 3;
+    return key <= a.warp_max_key ? 1u : 2u;
+}
+
+// Queue the pairs that the second level leaves of the warp's n buffered ones
+// (probe slot, candidate id), in candidate order (slots ascending).  Short pairs go to the front of the pair list, the others
+// to its back, a probe's pairs side by side; lane, block and index items
+// refer to such a run, and its pairs are marked (kInItem) so that the
+// warp-per-pair phase passes over them.
+__device__ __noinline__ void flush_survivors(const VerifyArgs& a, const PlanInst& I, uint32_t inst, uint2* buf,
+                                             uint32_t n, int lane) {
+    const unsigned lt_mask = (1u << lane) - 1u;
+    switch (I.rec_sectors[1]) {
+        case 2: n = second_level<2>(I, buf, n, lane); break;
+        case 4: n = second_level<4>(I, buf, n, lane); break;
+        case 8: n = second_level<8>(I, buf, n, lane); break;
+        default: break;
+    }
+    if (n == 0) return;
+    uint32_t* err = &a.ctr->err;
+    // bin of entry i and the run [h, e) of its probe's entries
+    auto classify = [&](uint32_t i, uint32_t* h, uint32_t* e, uint32_t* r) -> uint32_t {
+        const uint32_t slot = buf[i].x;
+        uint32_t lo = 0, hi = i;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (buf[mid].x < slot) lo = mid + 1; else hi = mid;
+        }
+        *h = lo;
+        lo = i + 1;
+        hi = n;
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi) >> 1;
+            if (buf[mid].x <= slot) lo = mid + 1; else hi = mid;
+        }
+        *e = lo;
+        *r = I.probe_ids[slot - 32u * I.tile_base];
+        return probe_bin(a, I.flags, I.r_desc[*r].y, *e - *h);
+    };
+    uint32_t n_long = 0;
+    for (uint32_t t = 0; t < n; t += 32) {
+        uint32_t h, e, r;
+        const bool is_long = t + lane < n && classify(t + lane, &h, &e, &r) != 0;
+        n_long += __popc(__ballot_sync(kFull, is_long));
+    }
+    unsigned long long base_s = 0, base_l = 0;
+    if (lane == 0) {
+        if (n > n_long) base_s = atomicAdd(&a.ctr->thread_pairs, (unsigned long long)(n - n_long));
+        if (n_long) base_l = atomicAdd(&a.ctr->long_pairs, (unsigned long long)n_long);
+    }
+    base_s = __shfl_sync(kFull, base_s, 0);
+    base_l = __shfl_sync(kFull, base_l, 0);
+    // every candidate is queued at most once, so the lists never meet
+    if (base_s + (n - n_long) > a.pair_cap || base_l + n_long > a.pair_cap) {
+        if (lane == 0) atomicOr(err, ERR_GUARD);
+        return;
+    }
+    unsigned long long at_s = base_s, at_l = a.pair_cap - base_l - n_long;
+    for (uint32_t t = 0; t < n; t += 32) {
+        const uint32_t i = t + lane;
+        uint32_t h = 0, e = 0, r = 0, bin = 5;
+        if (i < n) bin = classify(i, &h, &e, &r);
+        const uint32_t ms = __ballot_sync(kFull, bin == 0), ml = __ballot_sync(kFull, bin >= 1 && bin <= 4);
+        const unsigned long long pos = bin == 0 ? at_s + __popc(ms & lt_mask) : at_l + __popc(ml & lt_mask);
+        at_s += __popc(ms);
+        at_l += __popc(ml);
+        if (bin <= 4 && in_bounds(pos, a.pair_cap, err)) {
+            PairRef pr;
+            pr.k = buf[i].x;
+            pr.s = buf[i].y | (bin >= 2 ? kInItem : 0u);
+            a.pairs[pos] = pr;
+        }
+        // items, by the first entry of a run
+        const bool head = i < n && i == h;
+        const uint32_t per = bin == 3 ? a.lane_item_cands : (bin == 4 ? a.index_item_cands : a.block_item_cands);
+        const uint32_t items = head && bin >= 2 ? (e - h + per - 1) / per : 0u;
+        uint32_t wn = bin == 3 ? items : 0u, bn = bin == 3 ? 0u : items;
+        if (__any_sync(kFull, items != 0)) {
+            uint32_t wincl = wn, bincl = bn;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t yw = __shfl_up_sync(kFull, wincl, off), yb = __shfl_up_sync(kFull, bincl, off);
+                if (lane >= off) { wincl += yw; bincl += yb; }
+            }
+            unsigned long long wbase = 0, bbase = 0;
+            if (lane == 31) {
+                if (wincl) wbase = atomicAdd(&a.ctr->warp_items, (unsigned long long)wincl);
+                if (bincl) bbase = atomicAdd(&a.ctr->block_items, (unsigned long long)bincl);
+            }
+            wbase = __shfl_sync(kFull, wbase, 31) + (wincl - wn);
+            bbase = __shfl_sync(kFull, bbase, 31) + (bincl - bn);
+            for (uint32_t it = 0; it < items; ++it) {
+                WorkItem wi;
+                wi.r = r;
+                wi.n = min(per, e - h - it * per);
+                wi.c0 = pos + (uint64_t)it * per;
+                wi.inst = inst;
+                wi.pad = bin >= 3 ? 1u : 0u;
+                const unsigned long long q = (bin == 3 ? wbase : bbase) + it;
+                if (q >= (bin == 3 ? a.warp_item_cap : a.block_item_cap)) {
+                    atomicOr(err, ERR_GUARD);
+                    break;
+                }
+                (bin == 3 ? a.warp_items : a.block_items)[q] = wi;
+            }
+        }
+    }
+    __syncwarp();
+}
+
+}  // namespace
+
+}  // namespace ssj

@@ -110,6 +110,9 @@ struct Counters {
     uint32_t warp_cursor;
     uint32_t long_cursor;
     uint32_t chunk_cursor;
+    uint32_t probe_cursor;            // join kernel: probes taken
+    unsigned long long candidates;    // join kernel: candidates found
+    unsigned long long join_pairs, join_runs;  // and pairs and runs handed over
     uint32_t err;                     // device-side check bits (see ssj_device_error)
 };
 
@@ -222,6 +225,7 @@ cudaError_t prepare_verify(uint32_t block_threads, uint32_t index_words = 0);
 cudaError_t launch_verify(const VerifyArgs& a, cudaStream_t st, int num_sms, uint32_t block_threads,
                           cudaEvent_t* ev = nullptr);
 cudaError_t launch_plan(const VerifyArgs& a, cudaStream_t st, int num_sms);
+cudaError_t launch_merge(const VerifyArgs& a, cudaStream_t st, int num_sms, uint32_t block_threads);
 
 // Records of class c (rec_bits) of a laid-out collection, on st.
 cudaError_t build_records(const uint4* toks4, const uint2* desc, uint32_t n, uint32_t c, uint4* rec, cudaStream_t st,
@@ -232,14 +236,14 @@ cudaError_t build_records(const uint4* toks4, const uint2* desc, uint32_t n, uin
 size_t scan_scratch_words(uint64_t n);
 cudaError_t exclusive_scan_u64(uint64_t* data, uint64_t n, uint64_t* scratch, uint64_t* total, cudaStream_t st);
 
-// Device candidate generation of a self-join (candgen.cu).  Scratch of the
-// prefix index, sized by the caller: size_hist max_len + 2 words, order and
-// rank n each, tcnt and toff vocab + 1 words each, scan_scratch
+// Self-join on the device (candgen.cu).  Scratch of the prefix index, sized by
+// the caller: size_hist max_len + 2 words, probes and rank n each, tcnt and
+// toff vocab + 1 words each, scan_scratch
 // scan_scratch_words(max(max_len + 2, vocab + 1)), total 1 word, post one
 // uint4 per index entry (known after stage 0).
 struct CandgenIndex {
-    uint64_t* size_hist;
-    uint32_t* order;
+    uint64_t* size_hist;          // after stage 0: per size, the position after its last set
+    uint32_t* probes;             // the sets from the largest down
     uint32_t* rank;
     uint64_t* tcnt;
     uint64_t* toff;
@@ -248,32 +252,40 @@ struct CandgenIndex {
     uint4* post;
 };
 
-struct CandgenOutput {
-    uint32_t* probe_ids;          // group -> probe set id
-    uint64_t* cand_offsets;       // group -> first candidate
-    uint32_t* cand_ids;
-    unsigned long long* packed;   // groups << 40 | candidates
-    uint64_t group_cap, cand_cap;
-    uint32_t* err;                // ERR_GUARD if a capacity was exceeded
-};
-
 struct CandgenInput {
     const uint4* toks4;
     const uint2* desc;
     uint32_t n, max_len, vocab;   // vocab: largest token + 1
     uint32_t sim, p, q;           // SIM_*, t = p/q
     uint32_t positional;          // positional bound at the matching prefix token
-    int stage;                    // 0: order + token counts; 1: lists + filtered count; 2: probe and emit
-    unsigned long long* table;    // stage 2: hash set of (probe position, candidate position)
-    uint64_t table_mask;          // its size - 1 (a power of two minus one)
-    CandgenOutput out;
+    int stage;                    // 0: order + token counts; 1: token lists
 };
 
-// Run one stage on st and wait for it; *host_word (pinned) receives stage
-// 0: index entries, stage 1: entries passing the filters (an upper bound of
-// the candidates), stage 2: the packed group / candidate counter.
+// Run one stage on st.  Stage 0 waits for it and leaves the number of index
+// entries in *host_word (pinned).
 cudaError_t candgen_run(const CandgenInput& in, cudaStream_t st, int num_sms, CandgenIndex* ix,
                         uint64_t* host_word);
+
+// Pairs that the join kernel hands over to the queue kernel, in runs of up to
+// kJoinRun in probe order: (first pair, pairs).
+constexpr uint32_t kJoinRun = 288;
+struct JoinQueue {
+    uint2* pairs;  // (index of the probe, candidate set)
+    ulonglong2* runs;
+    uint64_t pair_cap, run_cap;
+};
+
+// Clear the counters and probe the index (after stage 1): candidates left by
+// the signature test are queued in a's lists for launch_merge, a.single being
+// the self-join with ix.probes as its probes.  If Counters::join_pairs
+// exceeds out.pair_cap, nothing is queued.
+cudaError_t join_probe(const CandgenInput& in, const CandgenIndex& ix, const VerifyArgs& a, const JoinQueue& out,
+                       cudaStream_t st, int num_sms);
+
+// Room for a self-join's queues of up to `pairs` pairs over n probes, and its
+// carving.
+size_t join_workspace_bytes(uint32_t n_probes, uint64_t pairs, int num_sms);
+JoinQueue bind_join_workspace(VerifyArgs& a, void* ws, uint32_t n_probes, uint64_t pairs, int num_sms);
 
 // GroupJoin expansion on the device (candgen.cu).  Entries: the probe
 // groups, then every group (pairs inside it).  probe_off / pair_off /

@@ -1418,11 +1418,60 @@ cudaError_t launch_verify(const VerifyArgs& a, cudaStream_t st, int num_sms, uin
     e = launch_plan(a, st, num_sms);
     if (e != cudaSuccess) return e;
     if (ev) cudaEventRecord(ev[1], st);
-    VerifyArgs va = a;
-    va.bulk_stage = (block_threads & kBulkStaging) ? 1u : 0u;
-    e = dispatch_variant(block_threads, LaunchVariant{va, st, num_sms});
+    e = launch_merge(a, st, num_sms, block_threads);
     if (ev) cudaEventRecord(ev[2], st);
     return e;
+}
+
+// The verify kernel on the pairs and items that a's lists hold.
+cudaError_t launch_merge(const VerifyArgs& a, cudaStream_t st, int num_sms, uint32_t block_threads) {
+    VerifyArgs va = a;
+    va.bulk_stage = (block_threads & kBulkStaging) ? 1u : 0u;
+    return dispatch_variant(block_threads, LaunchVariant{va, st, num_sms});
+}
+
+// Items: at most one per probe's run and per kJoinBlockCands pairs, and one more wherever a run is
+// cut (every kJoinRun - 32 pairs).  Runs: full ones, and one per warp of the join kernel.
+constexpr uint32_t kJoinBlockCands = 8;
+static uint64_t join_items(uint32_t n_probes, uint64_t pairs) {
+    return std::min<uint64_t>(pairs, (uint64_t)n_probes + pairs / 4) + 1;
+}
+static uint64_t join_runs(uint64_t pairs, int num_sms) { return pairs / (kJoinRun - 32) + 64ull * num_sms + 1; }
+
+size_t join_workspace_bytes(uint32_t n_probes, uint64_t pairs, int num_sms) {
+    return align256(sizeof(Counters)) + align256(2 * sizeof(Instance)) + align256(sizeof(PairRef) * pairs) +
+           2 * align256(sizeof(WorkItem) * join_items(n_probes, pairs)) + align256(sizeof(uint2) * pairs) +
+           align256(sizeof(ulonglong2) * join_runs(pairs, num_sms));
+}
+
+JoinQueue bind_join_workspace(VerifyArgs& a, void* ws, uint32_t n_probes, uint64_t pairs, int num_sms) {
+    char* p = static_cast<char*>(ws);
+    auto take = [&](size_t bytes) {
+        char* at = p;
+        p += align256(bytes);
+        return at;
+    };
+    a.block_item_cands = kJoinBlockCands;
+    a.lane_item_cands = 32;
+    a.index_item_cands = kIndexItemCands;
+    a.n_inst = 1;
+    a.n_tiles = (n_probes + 31) / 32;
+    a.total_probes = n_probes;
+    a.total_cands = pairs;
+    a.ctr = reinterpret_cast<Counters*>(take(sizeof(Counters)));
+    a.table_out = reinterpret_cast<Instance*>(take(2 * sizeof(Instance)));
+    a.pair_cap = pairs;
+    a.pairs = reinterpret_cast<PairRef*>(take(sizeof(PairRef) * pairs));
+    const uint64_t items = join_items(n_probes, pairs);
+    a.warp_item_cap = a.block_item_cap = (uint32_t)std::min<uint64_t>(items, 0xFFFFFFF0ull);
+    a.warp_items = reinterpret_cast<WorkItem*>(take(sizeof(WorkItem) * items));
+    a.block_items = reinterpret_cast<WorkItem*>(take(sizeof(WorkItem) * items));
+    JoinQueue q;
+    q.pairs = reinterpret_cast<uint2*>(take(sizeof(uint2) * pairs));
+    q.run_cap = join_runs(pairs, num_sms);
+    q.runs = reinterpret_cast<ulonglong2*>(take(sizeof(ulonglong2) * q.run_cap));
+    q.pair_cap = pairs;
+    return q;
 }
 
 }  // namespace ssj
