@@ -26,7 +26,7 @@ LIB_CHECKED = os.path.join(HERE, "libssj_checked.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O3",
               "--expt-relaxed-constexpr", "-I", INCLUDE]
-SOURCES = ["api.cu", "verify.cu", "plan.cu", "layout.cu", "noalloc.cu", "probe.cu", "candgen.cu", "feeder.cpp", "groups.cpp", "renumber.cpp", "serve_driver.cpp"]
+SOURCES = ["api.cu", "verify.cu", "plan.cu", "sort.cu", "layout.cu", "noalloc.cu", "probe.cu", "candgen.cu", "feeder.cpp", "groups.cpp", "renumber.cpp", "serve_driver.cpp"]
 
 
 def _nvcc() -> str:

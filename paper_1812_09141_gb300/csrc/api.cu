@@ -71,6 +71,11 @@ constexpr uint64_t kDirectCands = 1ull << 25;
 // Candidates of one batch, and of one call or prepared launch: 2^40 ids are 4 TiB, beyond any
 // device's memory, and keep every workspace size computed from the count far from 64-bit wrap.
 constexpr uint64_t kMaxCands = 1ull << 40;
+// Results copied to pinned memory along with their count, before the host knows it, so that calls
+// with up to that many wait for the device once (48 KiB take about 2 us; a second wait and copy
+// take about 15): of one batch, and of a group of ssj_verify_batches.
+constexpr uint64_t kFirstResults = 4096;
+constexpr uint64_t kPackResults = 16384;
 
 struct Collection {
     uint32_t n_sets = 0;
@@ -108,9 +113,10 @@ struct Ticket {
     uint64_t bytes = 0;              // charged to the budget
     ssj_triple* d_out = nullptr;
     uint64_t out_cap = 0;
-    uint64_t* h_count = nullptr;     // pinned
-    uint32_t* h_err = nullptr;       // pinned
+    ssj_triple* d_tmp = nullptr;     // the workspace behind the counters, free once the kernels are done
+    uint64_t tmp_cap = 0;            // triples it holds
     ssj_triple* h_out = nullptr;     // pinned, grown as needed
+    bool sorted = false;             // h_out is sorted
     uint64_t count = 0;
     TicketState state = TicketState::kRunning;
     std::string error;
@@ -129,8 +135,7 @@ struct Slot {
     uint64_t h_probe_cap = 0, h_offs_cap = 0, h_cand_cap = 0;
     ssj_triple* h_out = nullptr;
     uint64_t h_out_cap = 0;
-    uint64_t* h_count = nullptr;
-    uint32_t* h_err = nullptr;
+    Counters* h_ctr = nullptr;
     bool busy = false;          // reserved by a ticket until ssj_results collects it
     struct Ticket* pending = nullptr;  // launched, waiting for the completion thread
     std::thread completer;
@@ -170,6 +175,14 @@ struct ssj_ctx {
     uint64_t* h_count = nullptr;  // pinned
     uint32_t* h_err = nullptr;    // pinned, kMaxGroups words
     Counters* h_ctr = nullptr;    // pinned
+    // pinned: results that come back with their count (kFirstResults; ssj_verify_batches: kPackResults
+    // a group), and ssj_verify_batches' counts and instance table
+    ssj_triple* h_first = nullptr;
+    uint64_t h_first_cap = 0;
+    uint64_t* h_counts = nullptr;
+    uint64_t h_counts_cap = 0;
+    Instance* h_table = nullptr;
+    uint64_t h_table_cap = 0;
     // ssj_verify_batches: the stream and event that carry the second group's input copies
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t copy_done[kMaxGroups] = {};
@@ -366,6 +379,7 @@ uint32_t vflags(uint32_t f) {
     if (f & SSJ_FORCE_BLOCK) v |= VF_FORCE_BLOCK;
     if (f & SSJ_FORCE_LANE) v |= VF_FORCE_LANE;
     if (f & SSJ_FORCE_INDEX) v |= VF_FORCE_INDEX;
+    if ((f & SSJ_SORTED) && !(f & SSJ_COUNT_ONLY)) v |= VF_SORTED;
     return v;
 }
 
@@ -518,7 +532,69 @@ private:
     bool failed_ = false;
 };
 
+// Queue, after the verify kernel of a one-batch launch on the context's
+// stream, the sort of the results and their way back: the counters (with the
+// count), and with `host` the first results.
+ssj_status queue_results(ssj_ctx* ctx, const VerifyArgs& a, bool host) {
+    cudaStream_t s = ctx->stream;
+    if (a.single.flags & VF_SORTED) CUDA_TRY(ctx, sort_results(a.table_out, 1, s));
+    CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_ctr, a.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
+    if (host && a.single.cap) {
+        const ssj_status st = ensure_pinned(ctx, &ctx->h_first, &ctx->h_first_cap, kFirstResults);
+        if (st != SSJ_OK) return st;
+        CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_first, a.single.out,
+                                      sizeof(ssj_triple) * std::min<uint64_t>(a.single.cap, kFirstResults),
+                                      cudaMemcpyDeviceToHost, s));
+    }
+    return SSJ_OK;
+}
+
+ssj_status device_check_status(ssj_ctx* ctx, uint32_t derr);
+
 bool triple_less(const ssj_triple& x, const ssj_triple& y) { return x.r != y.r ? x.r < y.r : x.s < y.s; }
+
+// n triples in device memory sorted on the context's stream (on the host if
+// there is no memory for the passes).
+cudaError_t sort_in_place(ssj_ctx* ctx, ssj_triple* t, uint64_t n) {
+    CallMemory mem(ctx);
+    ssj_triple* tmp = mem.get<ssj_triple>(n);
+    if (mem.ok()) return sort_triples(t, n, tmp, ctx->stream);
+    std::vector<ssj_triple> h(n);
+    cudaError_t e = cudaMemcpyAsync(h.data(), t, sizeof(ssj_triple) * n, cudaMemcpyDeviceToHost, ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    std::sort(h.begin(), h.end(), triple_less);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(t, h.data(), sizeof(ssj_triple) * n, cudaMemcpyHostToDevice, ctx->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+    return e;
+}
+
+// After a wait for what queue_results queued: the count, and the results to
+// `out` (host; NULL: they stay where the launch wrote them), sorted if asked for.
+ssj_status collect_results(ssj_ctx* ctx, const VerifyArgs& a, ssj_triple* out, uint64_t cap, uint64_t* n_out) {
+    const uint64_t count = ctx->h_ctr->results;
+    *n_out = count;
+    if (ctx->h_ctr->err) return device_check_status(ctx, ctx->h_ctr->err);
+    if (a.single.flags & VF_COUNT_ONLY) return SSJ_OK;
+    const uint64_t n = std::min(count, a.single.cap);
+    const bool sort = (a.single.flags & VF_SORTED) && n > kSortTile;
+    cudaStream_t s = ctx->stream;
+    if (sort) {
+        CUDA_TRY(ctx, sort_in_place(ctx, a.single.out, n));
+        if (!out) CUDA_TRY(ctx, cudaStreamSynchronize(s));
+    }
+    if (out && n) {
+        if (n <= kFirstResults && !sort) {
+            memcpy(out, ctx->h_first, sizeof(ssj_triple) * n);
+        } else {
+            CUDA_TRY(ctx, cudaMemcpyAsync(out, a.single.out, sizeof(ssj_triple) * n, cudaMemcpyDeviceToHost, s));
+            CUDA_TRY(ctx, cudaStreamSynchronize(s));
+        }
+    }
+    if (count > cap) return fail(ctx, SSJ_ENOMEM, "%llu result pairs, room for %llu", (unsigned long long)count,
+                                 (unsigned long long)cap);
+    return SSJ_OK;
+}
+
 
 void completion_loop(ssj_ctx* ctx, int slot);
 
@@ -567,8 +643,7 @@ extern "C" ssj_status ssj_create(const ssj_config* config, ssj_ctx** out) {
         if (cudaEventCreateWithFlags(&s.ev, cudaEventDisableTiming | cudaEventBlockingSync) != cudaSuccess)
             return SSJ_EDEVICE;
         if (cudaEventCreateWithFlags(&s.copied, cudaEventDisableTiming) != cudaSuccess) return SSJ_EDEVICE;
-        if (cudaMallocHost(reinterpret_cast<void**>(&s.h_count), sizeof(uint64_t)) != cudaSuccess) return SSJ_EDEVICE;
-        if (cudaMallocHost(reinterpret_cast<void**>(&s.h_err), sizeof(uint32_t)) != cudaSuccess) return SSJ_EDEVICE;
+        if (cudaMallocHost(reinterpret_cast<void**>(&s.h_ctr), sizeof(Counters)) != cudaSuccess) return SSJ_EDEVICE;
     }
     ssj_ctx* raw = ctx.release();
     for (size_t i = 0; i < raw->slots.size(); ++i) raw->slots[i].completer = std::thread(completion_loop, raw, (int)i);
@@ -606,8 +681,7 @@ extern "C" void ssj_destroy(ssj_ctx* ctx) {
         cudaFreeHost(s.h_offs);
         cudaFreeHost(s.h_cand);
         cudaFreeHost(s.h_out);
-        cudaFreeHost(s.h_count);
-        cudaFreeHost(s.h_err);
+        cudaFreeHost(s.h_ctr);
     }
     for (auto& kv : ctx->tickets)
         if (kv.second->d_mem) {
@@ -621,6 +695,9 @@ extern "C" void ssj_destroy(ssj_ctx* ctx) {
     cudaFreeHost(ctx->h_count);
     cudaFreeHost(ctx->h_err);
     cudaFreeHost(ctx->h_ctr);
+    cudaFreeHost(ctx->h_first);
+    cudaFreeHost(ctx->h_counts);
+    cudaFreeHost(ctx->h_table);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     for (cudaEvent_t ev : ctx->copy_done)
         if (ev) cudaEventDestroy(ev);
@@ -880,6 +957,28 @@ extern "C" ssj_status ssj_device_error(ssj_ctx* ctx, uint32_t* code) {
     return SSJ_OK;
 }
 
+namespace {
+
+// Launch one batch (a: everything but the workspace and the count) on the
+// context's stream and wait for its results; host_out: where they go, NULL if
+// they stay in a.single.out.
+ssj_status run_batch(ssj_ctx* ctx, VerifyArgs& a, uint32_t n_probes, uint64_t n_cands, ssj_triple* host_out,
+                     uint64_t cap, uint64_t* n_out) {
+    ssj_status st = ensure_device_buffer(ctx, &ctx->ws, &ctx->ws_bytes, workspace_bytes(n_probes, n_cands, ctx->num_sms));
+    if (st != SSJ_OK) return st;
+    bind_workspace(a, ctx->ws, n_probes, n_cands, ctx->num_sms);
+    a.single.count = &a.ctr->results;
+    ctx->last_ctr = a.ctr;
+    const cudaError_t e = launch_verify(a, ctx->stream, ctx->num_sms, ctx->block_threads, profile_events(ctx));
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "launch_verify");
+    st = queue_results(ctx, a, host_out != nullptr);
+    if (st != SSJ_OK) return st;
+    CUDA_TRY(ctx, cudaStreamSynchronize(ctx->stream));
+    return collect_results(ctx, a, host_out, cap, n_out);
+}
+
+}  // namespace
+
 extern "C" ssj_status ssj_verify_batch(ssj_ctx* ctx, const ssj_batch* batch, ssj_triple* out, uint64_t cap,
                                        uint64_t* n_out) {
     NvtxScope nvtx_scope("ssj_verify_batch");
@@ -894,7 +993,6 @@ extern "C" ssj_status ssj_verify_batch(ssj_ctx* ctx, const ssj_batch* batch, ssj
     cudaStream_t s = ctx->stream;
     uint64_t n_cands = 0;
     VerifyArgs a;
-    uint64_t* d_count = nullptr;
     if (!dev) {
         st = validate_host_batch(ctx, batch, &n_cands);
         if (st != SSJ_OK) return st;
@@ -905,7 +1003,6 @@ extern "C" ssj_status ssj_verify_batch(ssj_ctx* ctx, const ssj_batch* batch, ssj
         const size_t o_probe = off; off += align256(4ull * std::max<uint32_t>(batch->n_probes, 1));
         const size_t o_offs = off;  off += align256(8ull * (batch->n_probes + 1));
         const size_t o_cand = off;  off += align256(4ull * std::max<uint64_t>(n_cands, 1));
-        const size_t o_cnt = off;   off += 256;
         const size_t o_out = off;   off += align256(sizeof(ssj_triple) * std::max<uint64_t>(out_cap, 1));
         st = ensure_device_buffer(ctx, &ctx->io, &ctx->io_bytes, off);
         if (st != SSJ_OK) return st;
@@ -913,7 +1010,6 @@ extern "C" ssj_status ssj_verify_batch(ssj_ctx* ctx, const ssj_batch* batch, ssj
         uint32_t* d_probe = reinterpret_cast<uint32_t*>(base + o_probe);
         uint64_t* d_offs = reinterpret_cast<uint64_t*>(base + o_offs);
         uint32_t* d_cand = reinterpret_cast<uint32_t*>(base + o_cand);
-        d_count = reinterpret_cast<uint64_t*>(base + o_cnt);
         ssj_triple* d_out = reinterpret_cast<ssj_triple*>(base + o_out);
         if (batch->n_probes) {
             CUDA_TRY(ctx, cudaMemcpyAsync(d_probe, batch->probe_ids, 4ull * batch->n_probes, cudaMemcpyHostToDevice, s));
@@ -940,38 +1036,8 @@ extern "C" ssj_status ssj_verify_batch(ssj_ctx* ctx, const ssj_batch* batch, ssj
         a.single.cand_ids = batch->cand_ids;
         a.single.out = out;
         a.single.cap = count_only ? 0 : cap;
-        st = ensure_device_buffer(ctx, &ctx->io, &ctx->io_bytes, 256);
-        if (st != SSJ_OK) return st;
-        d_count = static_cast<uint64_t*>(ctx->io);
     }
-    st = ensure_device_buffer(ctx, &ctx->ws, &ctx->ws_bytes, workspace_bytes(batch->n_probes, n_cands, ctx->num_sms));
-    if (st != SSJ_OK) return st;
-    a.single.count = reinterpret_cast<unsigned long long*>(d_count);
-    bind_workspace(a, ctx->ws, batch->n_probes, n_cands, ctx->num_sms);
-    ctx->last_ctr = a.ctr;
-    cudaError_t e = launch_verify(a, s, ctx->num_sms, ctx->block_threads, profile_events(ctx));
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "launch_verify");
-    CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_count, d_count, sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_err, &a.ctr->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(ctx, cudaStreamSynchronize(s));
-    const uint64_t count = *ctx->h_count;
-    const uint32_t derr = *ctx->h_err;
-    *n_out = count;
-    if (derr) return device_check_status(ctx, derr);
-    if (count_only) return SSJ_OK;
-    const uint64_t n_copy = std::min(count, cap);
-    if (!dev) {
-        if (n_copy) CUDA_TRY(ctx, cudaMemcpy(out, a.single.out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost));
-        if (batch->flags & SSJ_SORTED) std::sort(out, out + n_copy, triple_less);
-    } else if ((batch->flags & SSJ_SORTED) && n_copy) {
-        std::vector<ssj_triple> h(n_copy);
-        CUDA_TRY(ctx, cudaMemcpy(h.data(), out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost));
-        std::sort(h.begin(), h.end(), triple_less);
-        CUDA_TRY(ctx, cudaMemcpy(out, h.data(), sizeof(ssj_triple) * n_copy, cudaMemcpyHostToDevice));
-    }
-    if (count > cap) return fail(ctx, SSJ_ENOMEM, "%llu result pairs, room for %llu", (unsigned long long)count,
-                                 (unsigned long long)cap);
-    return SSJ_OK;
+    return run_batch(ctx, a, batch->n_probes, n_cands, dev ? nullptr : out, cap, n_out);
 }
 
 extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches, uint32_t n_batches,
@@ -987,7 +1053,8 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
     sh.total_probes = 0;
     sh.total_cands = 0;
     sh.n_chunks = 0;
-    size_t off = align256(sizeof(uint64_t) * n_batches);  // counts first
+    const size_t packed_bytes = sizeof(ssj_triple) * kPackResults;  // a group's results for one copy
+    size_t off = align256(sizeof(uint64_t) * n_batches) + kMaxGroups * align256(packed_bytes);  // counts and these first
     uint64_t launch_vocab = 1;
     bool launch_force_index = false;
     const Collection* pinned = nullptr;  // the first pinned collection: its L2 window
@@ -1061,6 +1128,10 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
     if (st != SSJ_OK) return st;
     st = ensure_device_buffer(ctx, &ctx->ws, &ctx->ws_bytes, ws_total);
     if (st != SSJ_OK) return st;
+    if ((st = ensure_pinned(ctx, &ctx->h_counts, &ctx->h_counts_cap, n_batches)) != SSJ_OK ||
+        (st = ensure_pinned(ctx, &ctx->h_table, &ctx->h_table_cap, n_batches)) != SSJ_OK ||
+        (st = ensure_pinned(ctx, &ctx->h_first, &ctx->h_first_cap, kMaxGroups * kPackResults)) != SSJ_OK)
+        return st;
     cudaStream_t s = ctx->stream;
     cudaStream_t cs = s;  // the later groups' copies
     if (groups > 1) {
@@ -1075,6 +1146,7 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
     }
     char* base = static_cast<char*>(ctx->io);
     uint64_t* d_counts = reinterpret_cast<uint64_t*>(base);
+    char* d_packed = base + align256(sizeof(uint64_t) * n_batches);
     for (uint32_t i = 0, gi = 0; i < n_batches; ++i) {
         if (i == gstart[gi + 1]) {  // group gi's copies are all queued
             if (gi > 0) CUDA_TRY(ctx, cudaEventRecord(ctx->copy_done[gi], cs));
@@ -1109,6 +1181,7 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
         I.count = reinterpret_cast<unsigned long long*>(d_counts + i);
     }
     if (groups > 1) CUDA_TRY(ctx, cudaEventRecord(ctx->copy_done[groups - 1], cs));
+    memcpy(ctx->h_table, table.data(), sizeof(Instance) * n_batches);
     for (uint32_t gi = 0; gi < groups; ++gi) {
         const uint32_t lo = gstart[gi], hi = gstart[gi + 1];
         VerifyArgs a;
@@ -1118,32 +1191,56 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
         bind_workspace(a, static_cast<char*>(ctx->ws) + ws_off[gi], shp[gi], ctx->num_sms);
         a.table = a.table_out;
         if (gi > 0) CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->copy_done[gi], 0));  // the group's inputs are in
-        CUDA_TRY(ctx, cudaMemcpyAsync(a.table_out, table.data() + lo, sizeof(Instance) * (hi - lo),
+        CUDA_TRY(ctx, cudaMemcpyAsync(a.table_out, ctx->h_table + lo, sizeof(Instance) * (hi - lo),
                                       cudaMemcpyHostToDevice, s));
         ctx->last_ctr = a.ctr;
         cudaError_t e = launch_verify(a, s, ctx->num_sms, ctx->block_threads, profile_events(ctx));
         if (e != cudaSuccess) return cuda_fail(ctx, e, "launch_verify");
+        // sorted where asked for, and the group's results packed, so that they come back in one copy
+        bool any_sorted = false, any_results = false;
+        for (uint32_t i = lo; i < hi; ++i) {
+            any_sorted = any_sorted || (table[i].flags & VF_SORTED);
+            any_results = any_results || table[i].cap;
+        }
+        ssj_triple* packed = reinterpret_cast<ssj_triple*>(d_packed + gi * align256(packed_bytes));
+        if (any_sorted) CUDA_TRY(ctx, sort_results(a.table_out, hi - lo, s));
+        if (any_results) {
+            CUDA_TRY(ctx, pack_results(a.table_out, hi - lo, packed, kPackResults, s));
+            CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_first + gi * kPackResults, packed, packed_bytes, cudaMemcpyDeviceToHost, s));
+        }
         CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_err + gi, &a.ctr->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     }
-    std::vector<uint64_t> counts(n_batches);
-    CUDA_TRY(ctx, cudaMemcpyAsync(counts.data(), d_counts, sizeof(uint64_t) * n_batches, cudaMemcpyDeviceToHost, s));
+    const uint64_t* counts = ctx->h_counts;
+    CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_counts, d_counts, sizeof(uint64_t) * n_batches, cudaMemcpyDeviceToHost, s));
     CUDA_TRY(ctx, cudaStreamSynchronize(s));
     uint32_t derr = 0;
     for (uint32_t gi = 0; gi < groups; ++gi) derr |= ctx->h_err[gi];
     if (derr) return device_check_status(ctx, derr);
-    bool short_cap = false;
-    for (uint32_t i = 0; i < n_batches; ++i) {
-        n_outs[i] = counts[i];
-        if (batches[i].flags & SSJ_COUNT_ONLY) continue;
-        const uint64_t n_copy = std::min(counts[i], caps[i]);
-        if (n_copy)
-            CUDA_TRY(ctx, cudaMemcpyAsync(outs[i], table[i].out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost, s));
-        short_cap |= counts[i] > caps[i];
+    bool short_cap = false, waiting = false;
+    for (uint32_t gi = 0; gi < groups; ++gi) {
+        uint64_t total = 0;
+        for (uint32_t i = gstart[gi]; i < gstart[gi + 1]; ++i) {
+            n_outs[i] = counts[i];
+            if (batches[i].flags & SSJ_COUNT_ONLY) continue;
+            total += std::min(counts[i], table[i].cap);
+            short_cap = short_cap || counts[i] > caps[i];
+        }
+        const ssj_triple* from = ctx->h_first + gi * kPackResults;
+        for (uint32_t i = gstart[gi]; i < gstart[gi + 1]; ++i) {
+            if (batches[i].flags & SSJ_COUNT_ONLY) continue;
+            const uint64_t n = std::min(counts[i], table[i].cap);
+            const bool sort = (table[i].flags & VF_SORTED) && n > kSortTile;
+            if (total <= kPackResults && !sort) {
+                if (n) memcpy(outs[i], from, sizeof(ssj_triple) * n);
+            } else if (n) {
+                if (sort) CUDA_TRY(ctx, sort_in_place(ctx, table[i].out, n));
+                CUDA_TRY(ctx, cudaMemcpyAsync(outs[i], table[i].out, sizeof(ssj_triple) * n, cudaMemcpyDeviceToHost, s));
+                waiting = true;
+            }
+            from += n;
+        }
     }
-    CUDA_TRY(ctx, cudaStreamSynchronize(s));
-    for (uint32_t i = 0; i < n_batches; ++i)
-        if ((batches[i].flags & SSJ_SORTED) && !(batches[i].flags & SSJ_COUNT_ONLY))
-            std::sort(outs[i], outs[i] + std::min(counts[i], caps[i]), triple_less);
+    if (waiting) CUDA_TRY(ctx, cudaStreamSynchronize(s));
     if (short_cap) return fail(ctx, SSJ_ENOMEM, "a batch has more result pairs than its capacity (see n_outs)");
     return SSJ_OK;
 }
@@ -1188,7 +1285,6 @@ extern "C" ssj_status ssj_self_join(ssj_ctx* ctx, ssj_coll coll, uint32_t p, uin
     ix.toff = mem.get<uint64_t>((uint64_t)C.vocab + 1);
     ix.scan_scratch = mem.get<uint64_t>(scan_scratch_words(scan_n));
     ix.total = mem.get<uint64_t>(1);
-    uint64_t* d_count = mem.get<uint64_t>(1);
     if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "candidate generation index");
     CandgenInput in;
     memset(&in, 0, sizeof(in));
@@ -1220,13 +1316,13 @@ extern "C" ssj_status ssj_self_join(ssj_ctx* ctx, ssj_coll coll, uint32_t p, uin
     b.p = p;
     b.q = q;
     b.n_probes = n;
-    b.flags = flags & ~(SSJ_JOIN_POSITIONAL | SSJ_DEVICE_PTRS | SSJ_SORTED);
+    b.flags = flags & ~(SSJ_JOIN_POSITIONAL | SSJ_DEVICE_PTRS);
+    VerifyArgs a;
     uint64_t room = std::min<uint64_t>(std::max<uint64_t>(8ull * n, 1u << 18), 1u << 22);
     ssj_triple* d_out = nullptr;
     for (;;) {
-        VerifyArgs a = make_args(ctx, &b, *R, *S, 0);
+        a = make_args(ctx, &b, *R, *S, 0);
         a.single.probe_ids = ix.probes;
-        a.single.count = reinterpret_cast<unsigned long long*>(d_count);
         if (!count_only) {
             // no more results than queued pairs
             const uint64_t d_cap = dev_out ? cap : std::min<uint64_t>(cap, room);
@@ -1238,6 +1334,7 @@ extern "C" ssj_status ssj_self_join(ssj_ctx* ctx, ssj_coll coll, uint32_t p, uin
         st = ensure_device_buffer(ctx, &ctx->ws, &ctx->ws_bytes, join_workspace_bytes(n, room, ctx->num_sms));
         if (st != SSJ_OK) return st;
         const JoinQueue queue = bind_join_workspace(a, ctx->ws, n, room, ctx->num_sms);
+        a.single.count = &a.ctr->results;
         ctx->last_ctr = a.ctr;
         cudaEvent_t* ev = profile_events(ctx);
         if (ev) cudaEventRecord(ev[0], s);
@@ -1245,35 +1342,15 @@ extern "C" ssj_status ssj_self_join(ssj_ctx* ctx, ssj_coll coll, uint32_t p, uin
         if (ev) cudaEventRecord(ev[1], s);
         if (e == cudaSuccess) e = launch_merge(a, s, ctx->num_sms, ctx->block_threads);
         if (ev) cudaEventRecord(ev[2], s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->h_ctr, a.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->h_count, d_count, sizeof(uint64_t), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "candidate generation (probe)");
+        st = queue_results(ctx, a, !dev_out);
+        if (st != SSJ_OK) return st;
+        CUDA_TRY(ctx, cudaStreamSynchronize(s));
         if (ctx->h_ctr->join_pairs <= room) break;
         room = ctx->h_ctr->join_pairs;
     }
     if (n_candidates) *n_candidates = ctx->h_ctr->candidates;
-    if (ctx->h_ctr->err) return device_check_status(ctx, ctx->h_ctr->err);
-    const uint64_t count = *ctx->h_count;
-    *n_out = count;
-    if (count_only) return SSJ_OK;
-    const uint64_t n_copy = std::min(count, cap);
-    if (dev_out) {
-        if ((flags & SSJ_SORTED) && n_copy) {
-            std::vector<ssj_triple> h(n_copy);
-            e = cudaMemcpy(h.data(), out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost);
-            std::sort(h.begin(), h.end(), triple_less);
-            if (e == cudaSuccess) e = cudaMemcpy(out, h.data(), sizeof(ssj_triple) * n_copy, cudaMemcpyHostToDevice);
-        }
-    } else if (n_copy) {
-        e = cudaMemcpyAsync(out, d_out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess && (flags & SSJ_SORTED)) std::sort(out, out + n_copy, triple_less);
-    }
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "join results");
-    if (count > cap) return fail(ctx, SSJ_ENOMEM, "%llu result pairs, room for %llu", (unsigned long long)count,
-                                 (unsigned long long)cap);
-    return SSJ_OK;
+    return collect_results(ctx, a, dev_out ? nullptr : out, cap, n_out);
 }
 
 // ===========================================================================
@@ -1376,48 +1453,20 @@ extern "C" ssj_status ssj_verify_groups(ssj_ctx* ctx, const ssj_group_batch* gb,
     b.p = gb->p;
     b.q = gb->q;
     b.n_probes = (uint32_t)probes;
-    b.probe_ids = x.probe_ids;
-    b.cand_offsets = x.cand_offsets_out;
-    b.cand_ids = x.cand_ids;
-    b.n_cands = pairs;
-    b.flags = (gb->flags & ~(SSJ_DEVICE_PTRS | SSJ_SORTED)) | SSJ_DEVICE_PTRS;
+    b.flags = gb->flags & ~SSJ_DEVICE_PTRS;
     const bool count_only = (gb->flags & SSJ_COUNT_ONLY) != 0;
     const bool dev_out = (gb->flags & SSJ_DEVICE_PTRS) != 0;
-    ssj_triple* d_out = nullptr;
-    uint64_t d_cap = 0;
+    if (probes >= (1u << 31) || pairs >= kMaxCands) return fail(ctx, SSJ_EINVAL, "too many expanded pairs");
+    VerifyArgs a = make_args(ctx, &b, *R, *S, pairs);
+    a.single.probe_ids = x.probe_ids;
+    a.single.cand_offsets = x.cand_offsets_out;
+    a.single.cand_ids = x.cand_ids;
     if (!count_only) {
-        if (dev_out) {
-            d_out = out;
-            d_cap = cap;
-        } else {
-            d_cap = std::min<uint64_t>(cap, pairs);
-            d_out = mem.get<ssj_triple>(std::max<uint64_t>(d_cap, 1));
-            if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "group join output");
-        }
+        a.single.cap = dev_out ? cap : std::min<uint64_t>(cap, pairs);
+        a.single.out = dev_out ? out : mem.get<ssj_triple>(std::max<uint64_t>(a.single.cap, 1));
+        if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "group join output");
     }
-    uint64_t count = 0;
-    st = ssj_verify_batch(ctx, &b, d_out, d_cap, &count);
-    *n_out = count;
-    if (st != SSJ_OK && st != SSJ_ENOMEM) return st;
-    if (!count_only) {
-        const uint64_t n_copy = std::min(count, cap);
-        if (dev_out) {
-            if ((gb->flags & SSJ_SORTED) && n_copy) {
-                std::vector<ssj_triple> h(n_copy);
-                e = cudaMemcpy(h.data(), out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost);
-                std::sort(h.begin(), h.end(), triple_less);
-                if (e == cudaSuccess) e = cudaMemcpy(out, h.data(), sizeof(ssj_triple) * n_copy, cudaMemcpyHostToDevice);
-            }
-        } else if (n_copy) {
-            e = cudaMemcpy(out, d_out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost);
-            if (e == cudaSuccess && (gb->flags & SSJ_SORTED)) std::sort(out, out + n_copy, triple_less);
-        }
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "group join results");
-    }
-    if (count > cap && !count_only)
-        return fail(ctx, SSJ_ENOMEM, "%llu result pairs, room for %llu", (unsigned long long)count,
-                    (unsigned long long)cap);
-    return SSJ_OK;
+    return run_batch(ctx, a, (uint32_t)probes, pairs, dev_out || count_only ? nullptr : out, cap, n_out);
 }
 
 // ===========================================================================
@@ -1489,17 +1538,24 @@ void completion_loop(ssj_ctx* ctx, int slot) {
         cudaError_t e = cudaEventSynchronize(t->kernel_done);
         uint64_t count = 0;
         if (e == cudaSuccess) {
-            count = *sl.h_count;
-            if (*sl.h_err) {
+            count = sl.h_ctr->results;
+            if (sl.h_ctr->err) {
                 err = "device-side batch check failed";
-                t->derr = *sl.h_err;
+                t->derr = sl.h_ctr->err;
             }
         } else {
             err = std::string("batch failed: ") + cudaGetErrorString(e);
         }
         if (err.empty() && !(t->flags & SSJ_COUNT_ONLY)) {
+            // the first results came with the counters; more are sorted if asked for and copied now
             const uint64_t n_copy = std::min(count, t->out_cap);
-            if (n_copy) {
+            const bool sort = (t->flags & SSJ_SORTED) && n_copy > kSortTile;
+            t->sorted = !sort || n_copy <= t->tmp_cap;
+            if (sort && t->sorted) {
+                e = sort_triples(t->d_out, n_copy, t->d_tmp, sl.stream);
+                if (e != cudaSuccess) err = std::string("result sort: ") + cudaGetErrorString(e);
+            }
+            if (err.empty() && (n_copy > kFirstResults || sort)) {
                 if (ensure_pinned(nullptr, &sl.h_out, &sl.h_out_cap, n_copy) != SSJ_OK) err = "pinned output";
                 if (err.empty()) {
                     e = cudaMemcpyAsync(sl.h_out, t->d_out, sizeof(ssj_triple) * n_copy, cudaMemcpyDeviceToHost,
@@ -1653,16 +1709,26 @@ extern "C" ssj_status ssj_submit(ssj_ctx* ctx, const ssj_batch* batch, uint64_t*
         a.single.cand_offsets = batch->cand_offsets;
         a.single.cand_ids = batch->cand_ids;
     }
-    uint64_t* d_count = reinterpret_cast<uint64_t*>(base + off); off += 256;
-    void* ws = base + off; off += align256(workspace_bytes(batch->n_probes, n_cands, ctx->num_sms));
+    off += 256;
+    void* ws = base + off;
+    const size_t ws_bytes = align256(workspace_bytes(batch->n_probes, n_cands, ctx->num_sms));
+    off += ws_bytes;
     ssj_triple* d_out = count_only ? nullptr : reinterpret_cast<ssj_triple*>(base + off);
     a.single.out = d_out;
     a.single.cap = count_only ? 0 : n_cands;
-    a.single.count = reinterpret_cast<unsigned long long*>(d_count);
     bind_workspace(a, ws, batch->n_probes, n_cands, ctx->num_sms);
+    a.single.count = &a.ctr->results;
+    t->d_tmp = reinterpret_cast<ssj_triple*>(static_cast<char*>(ws) + align256(sizeof(Counters)));
+    t->tmp_cap = (ws_bytes - align256(sizeof(Counters))) / sizeof(ssj_triple);
     e = launch_verify(a, s, ctx->num_sms, ctx->block_threads, nullptr);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sl.h_count, d_count, sizeof(uint64_t), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sl.h_err, &a.ctr->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess && (a.single.flags & VF_SORTED)) e = sort_results(a.table_out, 1, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(sl.h_ctr, a.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess && a.single.cap) {
+        if (ensure_pinned(ctx, &sl.h_out, &sl.h_out_cap, kFirstResults) != SSJ_OK) e = cudaErrorMemoryAllocation;
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(sl.h_out, d_out, sizeof(ssj_triple) * std::min<uint64_t>(a.single.cap, kFirstResults),
+                                cudaMemcpyDeviceToHost, s);
+    }
     if (e == cudaSuccess) e = cudaEventRecord(sl.ev, s);
     // pinned inputs: wait for their copies unless the caller keeps them until the ticket is done
     if (e == cudaSuccess && direct_copy && !(batch->flags & SSJ_KEEP_INPUTS)) e = cudaEventSynchronize(sl.copied);
@@ -1719,7 +1785,7 @@ extern "C" ssj_status ssj_results(ssj_ctx* ctx, uint64_t ticket, ssj_triple* out
         if (cap < t->count) return fail(ctx, SSJ_ENOMEM, "%llu result pairs, room for %llu",
                                         (unsigned long long)t->count, (unsigned long long)cap);
         if (t->count) memcpy(out, t->h_out, sizeof(ssj_triple) * t->count);
-        if (t->flags & SSJ_SORTED) std::sort(out, out + t->count, triple_less);
+        if ((t->flags & SSJ_SORTED) && !t->sorted) std::sort(out, out + t->count, triple_less);
     }
     ctx->slots[t->slot].busy = false;
     auto ir = ctx->colls.find(t->R);

@@ -1,0 +1,172 @@
+// Result triples sorted by (r, s) on the device (SSJ_SORTED), and the results of
+// a launch's instances packed for one copy to the host.
+//
+// The number of results is known on the device only, so the sort of up to
+// kSortTile triples an instance is queued right after the verify kernel, one
+// CTA per instance, and the host reads count and triples back at once (2,034
+// results: std::sort between two copies took about 100 us, the kernel takes
+// 6).  More results are sorted after the count has come back: tiles by the
+// same code, then passes that merge two runs each.
+#include <algorithm>
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "ssj_internal.h"
+
+namespace ssj {
+
+namespace {
+
+constexpr int kSortThreads = 1024;
+constexpr int kMergeThreads = 256;
+constexpr uint32_t kMergeTile = 1024;  // triples written by one CTA of a merge pass
+
+__device__ __forceinline__ unsigned long long key_of(const ssj_triple& t) {
+    return ((unsigned long long)t.r << 32) | t.s;
+}
+
+// n <= kSortTile triples from src to dst (may be the same), by one CTA:
+// bitonic network over the next power of two in shared memory.  (Set ids are
+// below 2^31, so the padding goes last.)
+__device__ void sort_tile(const ssj_triple* src, ssj_triple* dst, uint32_t n, unsigned long long* key, uint32_t* val) {
+    uint32_t size = 2;
+    while (size < n) size <<= 1;
+    for (uint32_t i = threadIdx.x; i < size; i += blockDim.x) {
+        key[i] = i < n ? key_of(src[i]) : ~0ull;
+        val[i] = i < n ? src[i].overlap : ~0u;
+    }
+    __syncthreads();
+    for (uint32_t k = 2; k <= size; k <<= 1) {
+        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
+            for (uint32_t x = threadIdx.x; x < size / 2; x += blockDim.x) {
+                const uint32_t lo = 2 * x - (x & (j - 1)), hi = lo + j;
+                const unsigned long long a = key[lo], b = key[hi];
+                if ((a > b) == ((lo & k) == 0)) {
+                    key[lo] = b;
+                    key[hi] = a;
+                    const uint32_t v = val[lo];
+                    val[lo] = val[hi];
+                    val[hi] = v;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        ssj_triple t;
+        t.r = (uint32_t)(key[i] >> 32);
+        t.s = (uint32_t)key[i];
+        t.overlap = val[i];
+        dst[i] = t;
+    }
+}
+
+__global__ void __launch_bounds__(kSortThreads) sort_results_kernel(const Instance* table) {
+    __shared__ unsigned long long key[kSortTile];
+    __shared__ uint32_t val[kSortTile];
+    const Instance& I = table[blockIdx.x];
+    if (!(I.flags & VF_SORTED)) return;
+    const unsigned long long n = min(*I.count, (unsigned long long)I.cap);
+    if (n >= 2 && n <= kSortTile) sort_tile(I.out, I.out, (uint32_t)n, key, val);
+}
+
+__global__ void __launch_bounds__(kSortThreads) sort_tiles_kernel(const ssj_triple* src, ssj_triple* dst, uint64_t n) {
+    __shared__ unsigned long long key[kSortTile];
+    __shared__ uint32_t val[kSortTile];
+    const uint64_t at = (uint64_t)blockIdx.x * kSortTile;
+    sort_tile(src + at, dst + at, (uint32_t)min((uint64_t)kSortTile, n - at), key, val);
+}
+
+// Runs of `run` sorted triples merged two by two from src to dst.  A CTA writes
+// kMergeTile of them: it finds the tile's part of both runs by the merge-path
+// search of its two diagonals, and each triple its place by a search of the
+// other part.
+__global__ void __launch_bounds__(kMergeThreads) merge_runs_kernel(const ssj_triple* src, ssj_triple* dst, uint64_t n,
+                                                                   uint64_t run) {
+    __shared__ unsigned long long key[kMergeTile];
+    __shared__ uint32_t val[kMergeTile];
+    __shared__ uint64_t s_split[2];
+    const uint64_t tile0 = (uint64_t)blockIdx.x * kMergeTile;  // (runs are multiples of the tile)
+    const uint64_t base = tile0 / (2 * run) * (2 * run);
+    const uint64_t na = min(run, n - base), nb = min(2 * run, n - base) - na;
+    const uint64_t d0 = tile0 - base, d1 = min(d0 + kMergeTile, na + nb);
+    const ssj_triple *A = src + base, *B = A + na;
+    if (threadIdx.x < 2) {  // taken from A by diagonal d (A first on equal keys)
+        const uint64_t d = threadIdx.x ? d1 : d0;
+        uint64_t lo = d > nb ? d - nb : 0, hi = min(d, na);
+        while (lo < hi) {
+            const uint64_t mid = (lo + hi) >> 1;
+            if (key_of(A[mid]) <= key_of(B[d - 1 - mid])) lo = mid + 1; else hi = mid;
+        }
+        s_split[threadIdx.x] = lo;
+    }
+    __syncthreads();
+    const uint64_t a0 = s_split[0], b0 = d0 - a0;
+    const uint32_t ca = (uint32_t)(s_split[1] - a0), c = (uint32_t)(d1 - d0);
+    for (uint32_t i = threadIdx.x; i < c; i += kMergeThreads) {
+        const ssj_triple t = i < ca ? A[a0 + i] : B[b0 + (i - ca)];
+        key[i] = key_of(t);
+        val[i] = t.overlap;
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < c; i += kMergeThreads) {
+        const unsigned long long k = key[i];
+        uint32_t lo = i < ca ? ca : 0u, hi = i < ca ? c : ca;  // the other part
+        while (lo < hi) {  // its triples that go before: smaller ones, and for B's also A's equal ones
+            const uint32_t mid = (lo + hi) >> 1;
+            if (i < ca ? key[mid] < k : key[mid] <= k) lo = mid + 1; else hi = mid;
+        }
+        ssj_triple t;
+        t.r = (uint32_t)(k >> 32);
+        t.s = (uint32_t)k;
+        t.overlap = val[i];
+        dst[base + d0 + (i < ca ? i + (lo - ca) : (i - ca) + lo)] = t;
+    }
+}
+
+// The instances' triples side by side, as far as there is room; one CTA each.
+__global__ void __launch_bounds__(256) pack_results_kernel(const Instance* table, ssj_triple* packed, uint64_t room) {
+    __shared__ unsigned long long s_at;
+    if (threadIdx.x == 0) s_at = 0;
+    __syncthreads();
+    unsigned long long mine = 0;
+    for (uint32_t i = threadIdx.x; i < blockIdx.x; i += blockDim.x) mine += min(*table[i].count, (unsigned long long)table[i].cap);
+    if (mine) atomicAdd(&s_at, mine);
+    __syncthreads();
+    const Instance& I = table[blockIdx.x];
+    const unsigned long long at = s_at, n = min(*I.count, (unsigned long long)I.cap);
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(I.out);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(packed + at);
+    if (at + n <= room)
+        for (unsigned long long k = threadIdx.x; k < 3 * n; k += blockDim.x) dst[k] = src[k];
+}
+
+}  // namespace
+
+cudaError_t sort_results(const Instance* table, uint32_t n_inst, cudaStream_t st) {
+    if (n_inst == 0) return cudaSuccess;
+    sort_results_kernel<<<n_inst, kSortThreads, 0, st>>>(table);
+    return cudaGetLastError();
+}
+
+cudaError_t pack_results(const Instance* table, uint32_t n_inst, ssj_triple* packed, uint64_t room, cudaStream_t st) {
+    if (n_inst == 0) return cudaSuccess;
+    pack_results_kernel<<<n_inst, 256, 0, st>>>(table, packed, room);
+    return cudaGetLastError();
+}
+
+cudaError_t sort_triples(ssj_triple* t, uint64_t n, ssj_triple* tmp, cudaStream_t st) {
+    if (n < 2) return cudaSuccess;
+    uint32_t passes = 0;
+    for (uint64_t run = kSortTile; run < n; run *= 2) ++passes;
+    ssj_triple* from = (passes & 1) ? tmp : t;  // the last pass ends in t
+    ssj_triple* to = (passes & 1) ? t : tmp;
+    sort_tiles_kernel<<<(unsigned)((n + kSortTile - 1) / kSortTile), kSortThreads, 0, st>>>(t, from, n);
+    for (uint64_t run = kSortTile; run < n; run *= 2) {
+        merge_runs_kernel<<<(unsigned)((n + kMergeTile - 1) / kMergeTile), kMergeThreads, 0, st>>>(from, to, n, run);
+        std::swap(from, to);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace ssj

@@ -27,6 +27,7 @@ enum : uint32_t {
     VF_SELF_JOIN = 32u,
     VF_FORCE_LANE = 64u,
     VF_FORCE_INDEX = 128u,
+    VF_SORTED = 256u,
 };
 
 // One join instance of a launch: its collections, grouped candidate list,
@@ -113,6 +114,7 @@ struct Counters {
     uint32_t probe_cursor;            // join kernel: probes taken
     unsigned long long candidates;    // join kernel: candidates found
     unsigned long long join_pairs, join_runs;  // and pairs and runs handed over
+    unsigned long long results;       // result count of a synchronous call, read back with the rest
     uint32_t err;                     // device-side check bits (see ssj_device_error)
 };
 
@@ -226,6 +228,15 @@ cudaError_t launch_verify(const VerifyArgs& a, cudaStream_t st, int num_sms, uin
                           cudaEvent_t* ev = nullptr);
 cudaError_t launch_plan(const VerifyArgs& a, cudaStream_t st, int num_sms);
 cudaError_t launch_merge(const VerifyArgs& a, cudaStream_t st, int num_sms, uint32_t block_threads);
+
+// Sort the triples of the instances that ask for it (VF_SORTED) and have at
+// most kSortTile of them, on st.
+constexpr uint32_t kSortTile = 4096;
+cudaError_t sort_results(const Instance* table, uint32_t n_inst, cudaStream_t st);
+// The instances' triples side by side in packed, complete if they all fit.
+cudaError_t pack_results(const Instance* table, uint32_t n_inst, ssj_triple* packed, uint64_t room, cudaStream_t st);
+// Sort n triples by (r, s) with room for n more at tmp.
+cudaError_t sort_triples(ssj_triple* t, uint64_t n, ssj_triple* tmp, cudaStream_t st);
 
 // Records of class c (rec_bits) of a laid-out collection, on st.
 cudaError_t build_records(const uint4* toks4, const uint2* desc, uint32_t n, uint32_t c, uint4* rec, cudaStream_t st,
