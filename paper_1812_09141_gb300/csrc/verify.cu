@@ -27,9 +27,10 @@
 //                 Section 3.3.2; the s-side positional bound of Section
 //                 2.2.3 after every 16-byte block);
 //       phase 2 - lane items: one candidate per lane, r in the warp's shared
-//                 memory; and long pairs: one warp per pair, 32-lane merge
-//                 path, r kept in the warp's shared memory while the next
-//                 pair has the same probe;
+//                 memory; and long pairs, or all pairs when they are few: one
+//                 warp per pair, s's tokens looked up in r, which stays in the
+//                 warp's shared memory while the next pair has the same probe
+//                 (longer probes: 32-lane merge path in windows);
 //       phase 3 - short pairs, one pair per thread (Alternatives A/B).
 //                 The merge compares 16-byte blocks (4 tokens of r against
 //                 4 of s, 16 compares; the block with the smaller last token
@@ -68,6 +69,11 @@ constexpr int kBlockD = 8;                         // merge steps per thread per
 constexpr uint32_t kBlockRCap = 4096;              // r kept whole in shared memory up to this
 constexpr uint32_t kFlatGrab = 4;                  // most 32-pair chunks taken per dynamic grab in phase 3
 constexpr uint32_t kLongGrab = 8;                  // most long pairs taken per dynamic grab in phase 2
+// Up to this many queued pairs per warp of the grid, short ones too are verified one per warp, dealt
+// out statically: a thread takes about 10 us of dependent loads however few pairs there are (2,034
+// results of short sets: 10 us instead of 17 for the kernel; 48 of the tiny collection: 9 instead of
+// 14).  At 8, 48 uneven joins take 84 us instead of 71 (long and short pairs dealt out alike).
+constexpr uint32_t kFewPairs = 2;
 constexpr uint32_t kCont = 64;                     // parked pairs per warp in phase 3
 
 // Checked build (SSJ_CHECKED): the functions that are not inlined take the
@@ -302,6 +308,38 @@ __device__ __forceinline__ void lane_merge(const uint32_t* A, uint32_t rw, const
     *c_out = c;
     *i_out = i;
     *j_out = j;
+}
+
+// -------------------------------------------------------------------------
+// Overlap of one pair by a warp, r whole in its shared memory (R): the lanes
+// read s's blocks side by side and look each token up in r by binary search,
+// a block's four tokens in step.  One memory wait and about log2|r| waits on
+// shared memory per 128 tokens of s; a merge in windows waits for both in each
+// window, which costs the pairs that the signature test leaves more than its
+// early termination saves them (they mostly pass).
+// -------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t warp_lookup(const uint32_t* R, uint32_t nr, const uint4* __restrict__ s4,
+                                                uint32_t ns, int lane, uint64_t slim, uint32_t* err) {
+    uint32_t c = 0;
+    if (nr) {
+        for (uint32_t b = lane; b < (ns + 3) >> 2; b += 32) {
+            const uint4 x = ld_block(s4, b, slim, err);
+            uint32_t p0 = 0, p1 = 0, p2 = 0, p3 = 0;  // first token of r not below x's, among the last n
+            for (uint32_t n = nr; n > 1;) {
+                const uint32_t half = n >> 1;
+                const uint32_t* m = R + half - 1;
+                p0 += m[p0] < x.x ? half : 0u;
+                p1 += m[p1] < x.y ? half : 0u;
+                p2 += m[p2] < x.z ? half : 0u;
+                p3 += m[p3] < x.w ? half : 0u;
+                n -= half;
+            }
+            const uint32_t valid = ns - 4 * b;  // (the tokens past s's end repeat its last one)
+            c += (R[p0] == x.x ? 1u : 0u) + (valid > 1 && R[p1] == x.y ? 1u : 0u) +
+                 (valid > 2 && R[p2] == x.z ? 1u : 0u) + (valid > 3 && R[p3] == x.w ? 1u : 0u);
+        }
+    }
+    return __reduce_add_sync(kFull, c);
 }
 
 // -------------------------------------------------------------------------
@@ -1017,7 +1055,8 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
     }
 
     // ---------------- phase 2: lane items, then long pairs, one per warp --
-    if (n_warp || n_long) {
+    const bool few = n_long + n_pairs <= (unsigned long long)kFewPairs * n_warps_total;
+    if (n_warp || n_long || (few && n_pairs)) {
         WarpOut wout;
         uint32_t* abuf = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(smem) + warp * kWarpSliceBytes);
         uint32_t* bbuf = abuf + kWarpABuf;
@@ -1050,7 +1089,7 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
             uint32_t it = 0;
             if (lane == 0) {
                 if (round == 0 && gwarp >= free2) it = gwarp - free2;
-                else it = slots2 + atomicAdd(&a.ctr->warp_cursor, 1u);
+                else it = n_warp > slots2 ? slots2 + atomicAdd(&a.ctr->warp_cursor, 1u) : slots2;
             }
             it = __shfl_sync(kFull, it, 0);
             if (it >= n_warp) break;
@@ -1063,58 +1102,76 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
             if (!stage_r(I.r_toks4 + dr.x, dr.y, I.r_n_chunks - dr.x)) return;  // the warp stops
             lane_item(I, wi, a.pairs + wi.c0, dr.y, reinterpret_cast<const uint4*>(abuf), lane, &a.ctr->err);
         }
-        for (uint32_t round = 0; n_long; ++round) {
-            uint32_t u = 0;
-            if (lane == 0) {
-                if (round == 0 && gwarp >= freel) u = gwarp - freel;
-                else u = slotsl + atomicAdd(&a.ctr->long_cursor, 1u);
-            }
-            u = __shfl_sync(kFull, u, 0);
-            if (u >= long_units) break;
-            const unsigned long long first = a.pair_cap - n_long + (unsigned long long)u * long_grab;
-            const unsigned long long end = min(first + long_grab, (unsigned long long)a.pair_cap);
-            uint32_t held = 0, inst = 0;  // slot + 1 of the r in abuf
-            for (unsigned long long m = first; m < end; ++m) {
-                const PairRef pr = a.pairs[m];
-                if (pr.s & kInItem) continue;
-                const uint32_t i = a.n_inst > 1 ? instance_of(table, a.n_inst, pr.k) : 0u;
-                if (wout.n && i != inst) wout.flush(table[inst], lane);
-                inst = i;
-                const Instance& I = table[inst];
-                const bool early = !(I.flags & VF_EMIT_ALL);
-                const uint32_t r = I.probe_ids[pr.k - 32u * I.tile_base];
-                if (!in_bounds(r, I.r_n_sets, &a.ctr->err)) continue;
-                const uint2 dr = I.r_desc[r], ds = I.s_desc[pr.s];
-                const uint32_t nr = dr.y, ns = ds.y;
-                const uint4* r4 = I.r_toks4 + dr.x;
-                const bool r_staged = nr + 4 <= kWarpRCap;
-                if (r_staged && held != pr.k + 1) {
-                    if (!stage_r(r4, nr, I.r_n_chunks - dr.x)) return;  // the warp stops
+        uint32_t held = 0, inst = 0;  // slot + 1 of the r in abuf, instance of the buffered survivors
+        uint32_t counted = 0;         // results of that instance that are only counted
+        auto flush = [&]() {
+            wout.flush(table[inst], lane);
+            if (counted && lane == 0) atomicAdd(table[inst].count, (unsigned long long)counted);
+            counted = 0;
+        };
+        // one queued pair; false if a copy did not complete (reported)
+        auto verify_pair = [&](const PairRef pr) -> bool {
+            const uint32_t i = a.n_inst > 1 ? instance_of(table, a.n_inst, pr.k) : 0u;
+            if (i != inst) flush();
+            inst = i;
+            const Instance& I = table[inst];
+            const bool early = !(I.flags & VF_EMIT_ALL);
+            if (!in_bounds(pr.k - 32u * I.tile_base, I.n_probes, &a.ctr->err)) return true;
+            const uint32_t r = I.probe_ids[pr.k - 32u * I.tile_base];
+            if (!in_bounds(r, I.r_n_sets, &a.ctr->err) || !in_bounds(pr.s, I.s_n_sets, &a.ctr->err)) return true;
+            const uint2 dr = I.r_desc[r], ds = I.s_desc[pr.s];
+            const uint32_t nr = dr.y, ns = ds.y;
+            const uint4 *r4 = I.r_toks4 + dr.x, *s4 = I.s_toks4 + ds.x;
+            const uint32_t req = required_overlap(I.sim, I.p, I.den, I.magic, nr, ns);
+            uint32_t o;
+            bool rej = false, failed;
+            if (nr + 4 <= kWarpRCap) {
+                if (held != pr.k + 1) {
+                    if (!stage_r(r4, nr, I.r_n_chunks - dr.x)) return false;
                     held = pr.k + 1;
                 }
-                if (!r_staged) held = 0;  // (abuf becomes a window buffer)
-                const uint32_t req = required_overlap(I.sim, I.p, I.den, I.magic, nr, ns);
-                bool rej, failed;
-                const uint32_t o =
-                    warp_merge(r4, nr, I.s_toks4 + ds.x, ns, req, early, r_staged, abuf, bbuf, lane, wbar, &wph,
-                               I.s_n_chunks - ds.x, &a.ctr->err, &failed,
-                               &rej CHK_ARGS(I.r_n_chunks - dr.x, I.s_n_chunks - ds.x, &a.ctr->err));
-                if (failed) return;  // (warp-uniform) reported; the warp stops
-                if (!early || (!rej && o >= req)) {
-                    if (I.flags & VF_COUNT_ONLY) {
-                        if (lane == 0) atomicAdd(I.count, 1ull);
-                    } else {
-                        wout.push(I, lane, r, pr.s, o);
-                    }
+                o = warp_lookup(abuf, nr, s4, ns, lane, I.s_n_chunks - ds.x, &a.ctr->err);
+            } else {
+                held = 0;  // (abuf becomes a window buffer)
+                o = warp_merge(r4, nr, s4, ns, req, early, false, abuf, bbuf, lane, wbar, &wph, I.s_n_chunks - ds.x,
+                               &a.ctr->err, &failed, &rej CHK_ARGS(I.r_n_chunks - dr.x, I.s_n_chunks - ds.x, &a.ctr->err));
+                if (failed) return false;
+            }
+            if (!early || (!rej && o >= req)) {
+                if (I.flags & VF_COUNT_ONLY) ++counted;
+                else wout.push(I, lane, r, pr.s, o);
+            }
+            return true;
+        };
+        if (few) {  // neighbouring pairs on different SMs
+            for (unsigned long long u = (unsigned long long)warp * gridDim.x + blockIdx.x; u < n_long + n_pairs;
+                 u += n_warps_total) {
+                const PairRef pr = a.pairs[u < n_long ? a.pair_cap - n_long + u : u - n_long];
+                if (!(pr.s & kInItem) && !verify_pair(pr)) return;  // the warp stops
+            }
+        } else {
+            for (uint32_t round = 0; n_long; ++round) {
+                uint32_t u = 0;
+                if (lane == 0) {
+                    if (round == 0 && gwarp >= freel) u = gwarp - freel;
+                    else u = long_units > slotsl ? slotsl + atomicAdd(&a.ctr->long_cursor, 1u) : slotsl;
+                }
+                u = __shfl_sync(kFull, u, 0);
+                if (u >= long_units) break;
+                const unsigned long long first = a.pair_cap - n_long + (unsigned long long)u * long_grab;
+                const unsigned long long end = min(first + long_grab, (unsigned long long)a.pair_cap);
+                for (unsigned long long m = first; m < end; ++m) {
+                    const PairRef pr = a.pairs[m];
+                    if (!(pr.s & kInItem) && !verify_pair(pr)) return;  // the warp stops
                 }
             }
-            if (wout.n) wout.flush(table[inst], lane);
         }
+        flush();
         __syncwarp();  // the slice is phase 3's now
     }
 
     // ---------------- phase 3: short pairs, one per thread ----------------
-    {
+    if (!few) {
         ContEntry* cont = reinterpret_cast<ContEntry*>(reinterpret_cast<char*>(smem) + warp * kWarpSliceBytes);
         uint32_t n_cont = 0;  // warp-uniform
         const uint32_t grab = n_pairs > 4ull * 32 * n_warps_total ? kFlatGrab : 1u;
@@ -1132,7 +1189,7 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
             uint32_t u = 0;
             if (lane == 0) {
                 if (round == 0 && gwarp >= free3) u = gwarp - free3;
-                else u = slots3 + atomicAdd(&a.ctr->chunk_cursor, 1u);
+                else u = n_units > slots3 ? slots3 + atomicAdd(&a.ctr->chunk_cursor, 1u) : slots3;
             }
             u = __shfl_sync(kFull, u, 0);
             if (u >= n_units) break;
