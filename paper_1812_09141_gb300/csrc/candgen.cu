@@ -8,8 +8,9 @@
 //   1. order the sets by size (counting sort; ties in any order: the set of
 //      unordered candidate pairs does not depend on it);
 //   2. index every set's prefix: per token, the entries (position in that
-//      order, position of the token in the set, set size, set id), by a
-//      count / scan / scatter over the prefix tokens;
+//      order, set id; for the positional bound also the token's position in
+//      the set and the set's size), by a count / scan / scatter over the
+//      prefix tokens;
 //   3. one warp per probe walks its prefix tokens' entries, keeps those of
 //      earlier sets that pass the length filter (positions [lo, its own), and
 //      optionally the positional bound of the matching token, PPJoin-style),
@@ -33,7 +34,7 @@ constexpr int kJoinWarps = 8;             // warps per CTA of the join kernel
 constexpr uint32_t kSeenWords = 1024;    // a warp's set of candidates seen: a bitmap of 32,768 positions, or a
 constexpr uint32_t kSeenBits = 32 * kSeenWords;  // hash set of up to half as many as it has words
 constexpr uint32_t kJoinFlush = kJoinRun - 32;  // pairs left that a warp hands over at once (room for 32 more)
-constexpr uint32_t kLongList = 64;       // index entries of a token that a whole warp reads as one list
+constexpr uint64_t kLongList = 1u << 26;  // 32 lists below this add up in 32 bits
 constexpr unsigned kAll = 0xFFFFFFFFu;
 constexpr uint32_t kFree = 0xFFFFFFFFu;
 
@@ -130,40 +131,63 @@ __global__ void __launch_bounds__(kSizeThreads) place_kernel(Params P, uint32_t 
     }
 }
 
-// one warp per set: count its prefix tokens per token
+// Prefix tokens of every set, by kSetLanes lanes a set (prefixes are mostly
+// shorter than a warp): f(set, its size, token's position, token).
+constexpr uint32_t kSetLanes = 8;
+template <class F>
+__device__ __forceinline__ void for_prefix_tokens(const Params& P, F&& f) {
+    const uint32_t sub = threadIdx.x % kSetLanes;
+    const uint32_t groups = (gridDim.x * blockDim.x) / kSetLanes;
+    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) / kSetLanes; i < P.n; i += groups) {
+        const uint2 d = P.desc[i];
+        const uint32_t* t = set_tokens(P, d);
+        const uint32_t pl = prefix_len(P, d.y);
+        for (uint32_t a = sub; a < pl; a += kSetLanes) f(i, d.y, a, t[a]);
+    }
+}
+
 __global__ void token_count_kernel(Params P, uint64_t* tcnt) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < P.n; i += warps) {
-        const uint2 d = P.desc[i];
-        const uint32_t* t = set_tokens(P, d);
-        const uint32_t pl = prefix_len(P, d.y);
-        for (uint32_t a = lane; a < pl; a += 32) atomicAdd(reinterpret_cast<unsigned long long*>(tcnt + t[a]), 1ull);
-    }
+    for_prefix_tokens(P, [&](uint32_t, uint32_t, uint32_t, uint32_t tok) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(tcnt + tok), 1ull);
+    });
 }
 
-// one warp per set: its prefix entries into the token lists
-__global__ void postings_kernel(Params P, const uint32_t* rank, uint64_t* tcur, uint4* post) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < P.n; i += warps) {
-        const uint2 d = P.desc[i];
-        const uint32_t* t = set_tokens(P, d);
-        const uint32_t pl = prefix_len(P, d.y);
-        const uint32_t pos = rank[i];
-        for (uint32_t a = lane; a < pl; a += 32) {
-            const uint64_t slot = atomicAdd(reinterpret_cast<unsigned long long*>(tcur + t[a]), 1ull);
-            post[slot] = make_uint4(pos, a, d.y, i);
-        }
-    }
+// An index entry: position and id of the set; with the positional bound also
+// the token's position in the set and the set's size.
+template <bool POS>
+struct Entry {
+    uint32_t rank, id;
+};
+template <>
+struct Entry<true> {
+    uint32_t rank, id, at, size;
+};
+__device__ __forceinline__ Entry<false> ld_entry(const Entry<false>* e) {
+    const uint2 x = __ldg(reinterpret_cast<const uint2*>(e));
+    return {x.x, x.y};
+}
+__device__ __forceinline__ Entry<true> ld_entry(const Entry<true>* e) {
+    const uint4 x = __ldg(reinterpret_cast<const uint4*>(e));
+    return {x.x, x.y, x.z, x.w};
 }
 
-// Positional bound of index entry e (a set of size e.z, the token at e.y)
-// matched at probe token position a: at most min(a, j) matches before this
-// one, one here, min(|r|-a-1, |s|-j-1) after.
-__device__ __forceinline__ bool position_ok(const Params& P, uint4 e, uint32_t L, uint32_t a) {
-    const uint32_t ub = min(a, e.y) + 1 + min(L - a - 1, e.z - e.y - 1);
-    return ub >= pair_required(P, L, e.z);
+// every set's prefix entries into the token lists
+template <bool POS>
+__global__ void postings_kernel(Params P, const uint32_t* rank, uint64_t* tcur, void* post) {
+    for_prefix_tokens(P, [&](uint32_t i, uint32_t size, uint32_t a, uint32_t tok) {
+        const uint64_t slot = atomicAdd(reinterpret_cast<unsigned long long*>(tcur + tok), 1ull);
+        if constexpr (POS) reinterpret_cast<uint4*>(post)[slot] = make_uint4(rank[i], i, a, size);
+        else reinterpret_cast<uint2*>(post)[slot] = make_uint2(rank[i], i);
+    });
+}
+
+// Positional bound of an index entry matched at probe token position a: at
+// most min(a, j) matches before this one, one here, min(|r|-a-1, |s|-j-1)
+// after.
+__device__ __forceinline__ bool position_ok(const Params&, const Entry<false>&, uint32_t, uint32_t) { return true; }
+__device__ __forceinline__ bool position_ok(const Params& P, const Entry<true>& e, uint32_t L, uint32_t a) {
+    const uint32_t ub = min(a, e.at) + 1 + min(L - a - 1, e.size - e.at - 1);
+    return ub >= pair_required(P, L, e.size);
 }
 
 __device__ __forceinline__ uint32_t mix32(uint32_t x) {
@@ -179,7 +203,7 @@ struct JoinArgs {
     const uint32_t* probes;    // the sets in the order in which they probe: from the last position down
     const uint64_t* size_end;  // size -> position after its last set
     const uint64_t* toff;      // token -> first index entry (n_tokens + 1)
-    const uint4* post;         // index entries
+    const void* post;          // index entries (Entry<POS>)
     uint32_t* cursor;          // next probe (from the last position down)
     uint32_t grab;             // probes per grab
     JoinQueue out;             // pairs left
@@ -188,23 +212,25 @@ struct JoinArgs {
 struct JoinWarp {
     uint32_t seen[kSeenWords];
     uint2 buf[kJoinRun];
-    uint32_t fresh[64];  // candidates to be tested
+    uint2 fresh[64];  // candidates to be tested: index of the probe, set
 };
 
-// The join of the sets in size order: a warp takes a probe at a time, the
-// largest first (they have the most candidates).  The tokens' index entries
-// are read flat, 32 at a time, lists of kLongList entries or more one by one.
+// The join of the sets in size order: a warp takes a few probes at a time, the
+// largest first (they have the most candidates).  The index entries of 32
+// tokens are read as one list, 32 at a time.
 // A candidate found through several tokens is kept once, by a bitmap over the
 // positions that the length filter admits; when these are more than the
 // bitmap holds, by a hash set if there are few entries, else window by window
 // of positions.  G: sectors per record of the first level of the signature
-// test, 0: every candidate is handed over.
-// Bound by latency (index entries and records from L2, shared-memory atomics).
-// All kernels up to the queue take 0.28 ms on 5.7e6 candidates of short sets
-// and 0.64 ms on 1.4e7 of long sets; with a hash set of all the join's pairs in
-// device memory, a sizing pass for it and the candidate lists written and
-// read, they took 1.75 and 3.65 ms.
-template <int G>
+// test, 0: every candidate is handed over.  POS: the positional bound.
+//
+// Bound by latency: a probe is a chain of dependent loads (set, size, tokens,
+// list bounds, entries, records).  The sets and sizes are therefore loaded for
+// all probes of a grab at once, the tokens and list bounds of the next 32
+// tokens while the entries of these are read, the next entries before these
+// are taken, and with one-sector records the candidates of several probes are
+// tested together.
+template <int G, bool POS>
 __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_constant__ VerifyArgs a, Params P,
                                                                   JoinArgs J) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -222,8 +248,9 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
     }
     __syncthreads();
     const PlanInst& I = s_inst;
+    const Entry<POS>* post = static_cast<const Entry<POS>*>(J.post);
     unsigned long long found = 0;  // candidates (warp-uniform)
-    uint32_t n = 0;                // pairs in buf (warp-uniform)
+    uint32_t n = 0, q = 0;         // pairs in buf, candidates waiting for the test (warp-uniform)
     auto hand_over = [&]() {       // buf as one run
         unsigned long long at = 0, run = 0;
         if (lane == 0) {
@@ -241,43 +268,76 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
         __syncwarp();
         n = 0;
     };
+    Sector rs;        // G > 1: the probe's record
+    uint32_t nr = 0;
+    auto test = [&](uint32_t m) {  // the first m waiting candidates
+        if (n >= kJoinFlush) hand_over();
+        const uint2 e = W.fresh[(uint32_t)lane < m ? lane : 0];
+        bool pass = (uint32_t)lane < m;
+        if (G == 1) {
+            uint32_t r_head;
+            const uint32_t r = __ldg(J.probes + e.x);
+            const uint32_t v = bound_of_pair<1, false>(I.s_rec[0], I.r_rec[0], e.y, r, rs, lane, &r_head);
+            pass = pass && bound_passes(I, v, r_head >> 16);
+        } else if (G > 1) {
+            const uint32_t v = bound_of_pair<kG, true>(I.s_rec[0], nullptr, e.y, 0u, rs, lane);
+            pass = pass && bound_passes(I, v, nr);
+        }
+        const uint32_t pm = __ballot_sync(kAll, pass);
+        if (pass) W.buf[n + __popc(pm & lt)] = e;
+        n += __popc(pm);
+        __syncwarp();
+    };
     for (;;) {
         uint32_t g0 = 0;
         if (lane == 0) g0 = atomicAdd(J.cursor, J.grab);
         g0 = __shfl_sync(kAll, g0, 0);
         if (g0 >= P.n) break;
-        for (uint32_t g = g0; g < min(g0 + J.grab, P.n); ++g) {
-            const uint32_t rpos = P.n - 1 - g, r = J.probes[g];
-            const uint2 d = P.desc[r];
-            const uint32_t* t = set_tokens(P, d);
-            const uint32_t L = d.y, pl = prefix_len(P, L);
-            if (pl == 0) continue;
-            const uint64_t min_size = min_overlap(P, L);  // at least 1, at most L
-            const uint32_t lo = (uint32_t)J.size_end[min_size - 1];
-            if (lo >= rpos) continue;
-            Sector rs;
-            uint32_t nr = 0, q = 0;  // q: candidates waiting for the test
-            if (G > 0) {
+        const uint32_t probes = min(J.grab, P.n - g0);  // (at most 32)
+        // lane i: probe g0 + i, its set, prefix length (0: no candidates) and the first position admitted
+        uint32_t my_r = 0, my_pl = 0, my_lo = 0;
+        uint2 my_d = make_uint2(0u, 0u);
+        if ((uint32_t)lane < probes) {
+            my_r = J.probes[g0 + lane];
+            my_d = P.desc[my_r];
+            my_pl = prefix_len(P, my_d.y);
+            if (my_pl) {
+                my_lo = (uint32_t)J.size_end[min_overlap(P, my_d.y) - 1];  // (at least 1, at most the size)
+                if (my_lo >= P.n - 1 - (g0 + lane)) my_pl = 0;
+            }
+        }
+        uint32_t left = __ballot_sync(kAll, my_pl != 0);
+        // bounds of the lists of tokens k .. k + 31 of a probe, asked for ahead of their use
+        uint64_t next_start = 0, next_end = 0;
+        auto bounds = [&](uint32_t tok, bool have) {
+            next_start = have ? J.toff[tok] : 0;
+            next_end = have ? J.toff[tok + 1] : 0;
+        };
+        if (left) {
+            const int p = __ffs(left) - 1;
+            const uint32_t* t = reinterpret_cast<const uint32_t*>(P.toks4 + __shfl_sync(kAll, my_d.x, p));
+            const bool have = (uint32_t)lane < __shfl_sync(kAll, my_pl, p);
+            bounds(have ? t[lane] : 0u, have);
+        }
+        while (left) {
+            const int p = __ffs(left) - 1;
+            left &= left - 1;
+            const int p2 = left ? __ffs(left) - 1 : p;  // the probe after this
+            const uint32_t g = g0 + p, rpos = P.n - 1 - g, lo = __shfl_sync(kAll, my_lo, p);
+            const uint32_t L = __shfl_sync(kAll, my_d.y, p), pl = __shfl_sync(kAll, my_pl, p);
+            const uint32_t pl2 = left ? __shfl_sync(kAll, my_pl, p2) : 0u;
+            const uint32_t* t = reinterpret_cast<const uint32_t*>(P.toks4 + __shfl_sync(kAll, my_d.x, p));
+            const uint32_t* t2 = reinterpret_cast<const uint32_t*>(P.toks4 + __shfl_sync(kAll, my_d.x, p2));
+            if (G > 1) {
+                const uint32_t r = __shfl_sync(kAll, my_r, p);
                 rs = ld_sector(I.r_rec[0] + ((uint64_t)r * kG + lane % kG) * 2);
                 nr = __ldg(&I.r_rec[0][(uint64_t)r * kG * 2].x) >> 16;
             }
-            auto test = [&](uint32_t m) {
-                const uint32_t s = W.fresh[(uint32_t)lane < m ? lane : 0];
-                bool pass = (uint32_t)lane < m;
-                if (G > 0) {
-                    const uint32_t v = bound_of_pair<kG, true>(I.s_rec[0], nullptr, s, 0u, rs, lane);
-                    pass = pass && bound_passes(I, v, nr);
-                }
-                const uint32_t pm = __ballot_sync(kAll, pass);
-                if (pass) W.buf[n + __popc(pm & lt)] = make_uint2(g, s);
-                n += __popc(pm);
-                __syncwarp();
-            };
             // entries in all, if the positions are more than the bitmap holds
             uint32_t hash_mask = 0;
             if (rpos - lo > kSeenBits) {
-                uint64_t e = 0;
-                for (uint32_t k = lane; k < pl; k += 32) e += J.toff[t[k] + 1] - J.toff[t[k]];
+                uint64_t e = next_end - next_start;
+                for (uint32_t k = 32 + lane; k < pl; k += 32) e += J.toff[t[k] + 1] - J.toff[t[k]];
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(kAll, e, o);
                 if (e <= kSeenWords / 2) hash_mask = e <= 32 ? 63u : (2u << (31 - __clz((uint32_t)e * 2 - 1))) - 1;
@@ -289,54 +349,54 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
                 for (uint32_t k = lane; k < words; k += 32) W.seen[k] = hash_mask ? kFree : 0u;
                 __syncwarp();
                 // one index entry per lane (if have), found at the probe's token k
-                auto take = [&](bool have, uint64_t e, uint32_t k) {
+                auto take = [&](bool have, const Entry<POS>& en, uint32_t k) {
                     bool is_new = false;
-                    uint4 en = make_uint4(0u, 0u, 0u, 0u);
-                    if (have) {
-                        en = __ldg(J.post + e);
-                        if (en.x >= w0 && en.x < w1 && !(P.positional && !position_ok(P, en, L, k))) {
-                            if (hash_mask) {
-                                uint32_t h = mix32(en.x) & hash_mask;
-                                for (;;) {  // (at most half of the slots are ever taken)
-                                    const uint32_t old = atomicCAS(W.seen + h, kFree, en.x);
-                                    is_new = old == kFree;
-                                    if (is_new || old == en.x) break;
-                                    h = (h + 1) & hash_mask;
-                                }
-                            } else {
-                                const uint32_t b = en.x - w0, bit = 1u << (b & 31u);
-                                is_new = (atomicOr(W.seen + (b >> 5), bit) & bit) == 0;
+                    if (have && en.rank >= w0 && en.rank < w1 && position_ok(P, en, L, k)) {
+                        if (hash_mask) {
+                            uint32_t h = mix32(en.rank) & hash_mask;
+                            for (;;) {  // (at most half of the slots are ever taken)
+                                const uint32_t old = atomicCAS(W.seen + h, kFree, en.rank);
+                                is_new = old == kFree;
+                                if (is_new || old == en.rank) break;
+                                h = (h + 1) & hash_mask;
                             }
+                        } else {
+                            const uint32_t b = en.rank - w0, bit = 1u << (b & 31u);
+                            is_new = (atomicOr(W.seen + (b >> 5), bit) & bit) == 0;
                         }
                     }
                     const uint32_t m = __ballot_sync(kAll, is_new);
-                    if (is_new) W.fresh[q + __popc(m & lt)] = en.w;
+                    if (m == 0) return;
+                    if (is_new) W.fresh[q + __popc(m & lt)] = make_uint2(g, en.id);
                     q += __popc(m);
                     found += __popc(m);
                     __syncwarp();
                     if (q >= 32) {
-                        if (n >= kJoinFlush) hand_over();
                         test(32);
                         q -= 32;
-                        const uint32_t keep = W.fresh[32 + lane];
+                        const uint2 keep = W.fresh[32 + lane];
                         __syncwarp();
                         if ((uint32_t)lane < q) W.fresh[lane] = keep;
                         __syncwarp();
                     }
                 };
                 for (uint32_t k0 = 0; k0 < pl; k0 += 32) {
-                    uint64_t start = 0, len = 0;
-                    if (k0 + lane < pl) {
-                        const uint32_t tok = t[k0 + lane];
-                        start = J.toff[tok];
-                        len = J.toff[tok + 1] - start;
-                    }
+                    const uint64_t start = next_start, len = next_end - next_start;
+                    // the tokens after these: this probe's, its first again (another window), or the next probe's
+                    const bool more = k0 + 32 < pl, again = !more && w1 < rpos;
+                    const uint32_t kn = more ? k0 + 32 + lane : (uint32_t)lane;
+                    const bool have_n = kn < (more || again ? pl : pl2);
+                    const uint32_t tok_n = have_n ? (more || again ? t : t2)[kn] : 0u;
+                    // lists that do not add up in 32 bits, one by one
                     uint32_t longs = __ballot_sync(kAll, len >= kLongList);
                     while (longs) {
                         const int src = __ffs(longs) - 1;
                         longs &= longs - 1;
                         const uint64_t e0 = __shfl_sync(kAll, start, src), e1 = e0 + __shfl_sync(kAll, len, src);
-                        for (uint64_t e = e0; e < e1; e += 32) take(e + lane < e1, e + lane, k0 + src);
+                        for (uint64_t e = e0; e < e1; e += 32) {
+                            const bool have = e + lane < e1;
+                            take(have, ld_entry(post + (have ? e + lane : e)), k0 + src);
+                        }
                     }
                     const uint32_t mine = len >= kLongList ? 0u : (uint32_t)len;
                     uint32_t incl = mine;
@@ -346,24 +406,43 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
                         if (lane >= o) incl += y;
                     }
                     const uint32_t total = __shfl_sync(kAll, incl, 31);
-                    const uint64_t base = start - (incl - mine);  // entry e of the flat list is base + e of its token
-                    for (uint32_t e0 = 0; e0 < total; e0 += 32) {
-                        const uint32_t e = e0 + lane;
-                        uint32_t k = 0;  // tokens whose entries end by e
+                    const uint64_t base = start - (incl - mine);  // entry e of the one list is base + e of its token
+                    auto locate = [&](uint32_t e, uint32_t* k) -> const Entry<POS>* {
+                        uint32_t x = 0;  // tokens whose entries end by e
 #pragma unroll
                         for (int step = 16; step >= 1; step >>= 1) {
-                            const uint32_t v = __shfl_sync(kAll, incl, k + step - 1);
-                            if (v <= e) k += step;
+                            const uint32_t v = __shfl_sync(kAll, incl, x + step - 1);
+                            if (v <= e) x += step;
                         }
-                        const uint64_t at = __shfl_sync(kAll, base, k) + e;
-                        take(e < total, at, k0 + k);
+                        *k = x;
+                        return post + (__shfl_sync(kAll, base, x) + e);
+                    };
+                    Entry<POS> en_n = {};
+                    uint32_t k_n = 0;
+                    if (total) {
+                        const Entry<POS>* at = locate(lane, &k_n);
+                        if ((uint32_t)lane < total) en_n = ld_entry(at);
+                    }
+                    bounds(tok_n, have_n);
+                    for (uint32_t e0 = 0; e0 < total; e0 += 32) {
+                        const Entry<POS> en = en_n;
+                        const uint32_t k = k_n;
+                        if (e0 + 32 < total) {
+                            const uint32_t e = e0 + 32 + lane;
+                            const Entry<POS>* at = locate(e, &k_n);
+                            if (e < total) en_n = ld_entry(at);
+                        }
+                        take(e0 + lane < total, en, k0 + k);
                     }
                 }
             }
-            if (n >= kJoinFlush) hand_over();
-            if (q) test(q);
+            if (G > 1 && q) {  // (the record is this probe's)
+                test(q);
+                q = 0;
+            }
         }
     }
+    if (q) test(q);
     if (n) hand_over();
     if (lane == 0 && found) atomicAdd(&a.ctr->candidates, found);
 }
@@ -509,7 +588,7 @@ cudaError_t candgen_run(const CandgenInput& in, cudaStream_t st, int num_sms, Ca
             e = exclusive_scan_u64(ix->size_hist, in.max_len + 2, ix->scan_scratch, ix->total, st);
             if (e != cudaSuccess) return e;
             place_kernel<<<blocks, kSizeThreads, 0, st>>>(P, per, ix->size_hist, ix->probes, ix->rank);
-            token_count_kernel<<<grid_for(32ull * in.n, tb, num_sms, 8), tb, 0, st>>>(P, ix->tcnt);
+            token_count_kernel<<<grid_for((uint64_t)kSetLanes * in.n, tb, num_sms, 8), tb, 0, st>>>(P, ix->tcnt);
         }
         e = cudaMemcpyAsync(ix->toff, ix->tcnt, 8ull * (in.vocab + 1), cudaMemcpyDeviceToDevice, st);
         if (e == cudaSuccess) e = exclusive_scan_u64(ix->toff, in.vocab + 1, ix->scan_scratch, ix->total, st);
@@ -521,21 +600,34 @@ cudaError_t candgen_run(const CandgenInput& in, cudaStream_t st, int num_sms, Ca
     if (in.n) {
         e = cudaMemcpyAsync(ix->tcnt, ix->toff, 8ull * (in.vocab + 1), cudaMemcpyDeviceToDevice, st);
         if (e != cudaSuccess) return e;
-        postings_kernel<<<grid_for(32ull * in.n, tb, num_sms, 8), tb, 0, st>>>(P, ix->rank, ix->tcnt, ix->post);
+        const unsigned blocks = grid_for((uint64_t)kSetLanes * in.n, tb, num_sms, 8);
+        if (in.positional) postings_kernel<true><<<blocks, tb, 0, st>>>(P, ix->rank, ix->tcnt, ix->post);
+        else postings_kernel<false><<<blocks, tb, 0, st>>>(P, ix->rank, ix->tcnt, ix->post);
     }
     return cudaGetLastError();
 }
 
-template <int G>
+template <int G, bool POS>
 static cudaError_t launch_join(const VerifyArgs& a, const Params& P, JoinArgs J, int num_sms, cudaStream_t st) {
     constexpr size_t smem = kJoinWarps * sizeof(JoinWarp);
-    cudaError_t e = cudaFuncSetAttribute(join_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(join_kernel<G, POS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)std::max<uint64_t>(
         1, std::min<uint64_t>(((uint64_t)P.n + kJoinWarps - 1) / kJoinWarps, 4ull * num_sms));
     J.grab = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(8, P.n / (16ull * blocks * kJoinWarps)));
-    join_kernel<G><<<blocks, kJoinWarps * 32, smem, st>>>(a, P, J);
+    join_kernel<G, POS><<<blocks, kJoinWarps * 32, smem, st>>>(a, P, J);
     return cudaGetLastError();
+}
+
+template <bool POS>
+static cudaError_t launch_join(const VerifyArgs& a, const Params& P, const JoinArgs& J, int num_sms, cudaStream_t st) {
+    switch (a.single.rec_sectors[0]) {
+        case 1: return launch_join<1, POS>(a, P, J, num_sms, st);
+        case 2: return launch_join<2, POS>(a, P, J, num_sms, st);
+        case 4: return launch_join<4, POS>(a, P, J, num_sms, st);
+        case 8: return launch_join<8, POS>(a, P, J, num_sms, st);
+        default: return launch_join<0, POS>(a, P, J, num_sms, st);
+    }
 }
 
 cudaError_t join_probe(const CandgenInput& in, const CandgenIndex& ix, const VerifyArgs& a, const JoinQueue& out,
@@ -558,13 +650,7 @@ cudaError_t join_probe(const CandgenInput& in, const CandgenIndex& ix, const Ver
     J.out = out;
     cudaError_t e = cudaMemsetAsync(a.ctr, 0, sizeof(Counters), st);
     if (e != cudaSuccess) return e;
-    switch (a.single.rec_sectors[0]) {
-        case 1: e = launch_join<1>(a, P, J, num_sms, st); break;
-        case 2: e = launch_join<2>(a, P, J, num_sms, st); break;
-        case 4: e = launch_join<4>(a, P, J, num_sms, st); break;
-        case 8: e = launch_join<8>(a, P, J, num_sms, st); break;
-        default: e = launch_join<0>(a, P, J, num_sms, st); break;
-    }
+    e = in.positional ? launch_join<true>(a, P, J, num_sms, st) : launch_join<false>(a, P, J, num_sms, st);
     if (e != cudaSuccess) return e;
     queue_kernel<<<(unsigned)(2 * num_sms), kJoinWarps * 32, 0, st>>>(a, out);
     return cudaGetLastError();

@@ -250,8 +250,8 @@ cudaError_t exclusive_scan_u64(uint64_t* data, uint64_t n, uint64_t* scratch, ui
 // Self-join on the device (candgen.cu).  Scratch of the prefix index, sized by
 // the caller: size_hist max_len + 2 words, probes and rank n each, tcnt and
 // toff vocab + 1 words each, scan_scratch
-// scan_scratch_words(max(max_len + 2, vocab + 1)), total 1 word, post one
-// uint4 per index entry (known after stage 0).
+// scan_scratch_words(max(max_len + 2, vocab + 1)), total 1 word, post
+// candgen_entry_bytes per index entry (known after stage 0).
 struct CandgenIndex {
     uint64_t* size_hist;          // after stage 0: per size, the position after its last set
     uint32_t* probes;             // the sets from the largest down
@@ -260,8 +260,11 @@ struct CandgenIndex {
     uint64_t* toff;
     uint64_t* scan_scratch;
     uint64_t* total;
-    uint4* post;
+    void* post;
 };
+
+// Bytes of an index entry.
+inline size_t candgen_entry_bytes(bool positional) { return positional ? 16 : 8; }
 
 struct CandgenInput {
     const uint4* toks4;
