@@ -1277,12 +1277,13 @@ extern "C" ssj_status ssj_self_join(ssj_ctx* ctx, ssj_coll coll, uint32_t p, uin
     const uint32_t n = C.n_sets;
     CallMemory mem(ctx);
     CandgenIndex ix;
-    const uint64_t scan_n = std::max<uint64_t>((uint64_t)C.max_len + 2, (uint64_t)C.vocab + 1);
+    const uint64_t cells = candgen_cells(C.vocab);
+    const uint64_t scan_n = std::max<uint64_t>((uint64_t)C.max_len + 2, cells + 1);
     ix.size_hist = mem.get<uint64_t>((uint64_t)C.max_len + 2);
     ix.probes = mem.get<uint32_t>(n);
     ix.rank = mem.get<uint32_t>(n);
-    ix.tcnt = mem.get<uint64_t>((uint64_t)C.vocab + 1);
-    ix.toff = mem.get<uint64_t>((uint64_t)C.vocab + 1);
+    ix.tcnt = mem.get<uint64_t>(cells + 1);
+    ix.toff = mem.get<uint64_t>(cells + 1);
     ix.scan_scratch = mem.get<uint64_t>(scan_scratch_words(scan_n));
     ix.total = mem.get<uint64_t>(1);
     if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "candidate generation index");

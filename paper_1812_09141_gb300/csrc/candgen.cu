@@ -7,8 +7,8 @@
 // Steps, on one stream:
 //   1. order the sets by size (counting sort; ties in any order: the set of
 //      unordered candidate pairs does not depend on it);
-//   2. index every set's prefix: per token, the entries (position in that
-//      order, set id; for the positional bound also the token's position in
+//   2. index every set's prefix: per token and range of positions (cell), the
+//      entries (position in that order, set id; for the positional bound also the token's position in
 //      the set and the set's size), by a count / scan / scatter over the
 //      prefix tokens;
 //   3. one warp per probe walks its prefix tokens' entries, keeps those of
@@ -41,6 +41,7 @@ constexpr uint32_t kFree = 0xFFFFFFFFu;
 struct Params {
     const uint4* toks4;
     const uint2* desc;
+    uint32_t cells_log2, cell_shift;  // a token's list is cut into 1 << cells_log2 cells, by position >> cell_shift
     uint32_t n;
     uint32_t sim, p, q;     // sim: SIM_*; t = p/q
     uint32_t positional;    // apply the positional bound at the matching token
@@ -146,9 +147,16 @@ __device__ __forceinline__ void for_prefix_tokens(const Params& P, F&& f) {
     }
 }
 
-__global__ void token_count_kernel(Params P, uint64_t* tcnt) {
-    for_prefix_tokens(P, [&](uint32_t, uint32_t, uint32_t, uint32_t tok) {
-        atomicAdd(reinterpret_cast<unsigned long long*>(tcnt + tok), 1ull);
+// Cell of a token's index entries at a position.  A probe admits a range of
+// positions only (the length filter), about a sixth of them for long sets at
+// t = 0.8, so it reads the cells of that range instead of the whole list.
+__device__ __forceinline__ uint64_t cell_of(const Params& P, uint32_t tok, uint32_t pos) {
+    return ((uint64_t)tok << P.cells_log2) + (pos >> P.cell_shift);
+}
+
+__global__ void token_count_kernel(Params P, const uint32_t* rank, uint64_t* tcnt) {
+    for_prefix_tokens(P, [&](uint32_t i, uint32_t, uint32_t, uint32_t tok) {
+        atomicAdd(reinterpret_cast<unsigned long long*>(tcnt + cell_of(P, tok, rank[i])), 1ull);
     });
 }
 
@@ -175,9 +183,10 @@ __device__ __forceinline__ Entry<true> ld_entry(const Entry<true>* e) {
 template <bool POS>
 __global__ void postings_kernel(Params P, const uint32_t* rank, uint64_t* tcur, void* post) {
     for_prefix_tokens(P, [&](uint32_t i, uint32_t size, uint32_t a, uint32_t tok) {
-        const uint64_t slot = atomicAdd(reinterpret_cast<unsigned long long*>(tcur + tok), 1ull);
-        if constexpr (POS) reinterpret_cast<uint4*>(post)[slot] = make_uint4(rank[i], i, a, size);
-        else reinterpret_cast<uint2*>(post)[slot] = make_uint2(rank[i], i);
+        const uint32_t pos = rank[i];
+        const uint64_t slot = atomicAdd(reinterpret_cast<unsigned long long*>(tcur + cell_of(P, tok, pos)), 1ull);
+        if constexpr (POS) reinterpret_cast<uint4*>(post)[slot] = make_uint4(pos, i, a, size);
+        else reinterpret_cast<uint2*>(post)[slot] = make_uint2(pos, i);
     });
 }
 
@@ -202,7 +211,7 @@ __device__ __forceinline__ uint32_t mix32(uint32_t x) {
 struct JoinArgs {
     const uint32_t* probes;    // the sets in the order in which they probe: from the last position down
     const uint64_t* size_end;  // size -> position after its last set
-    const uint64_t* toff;      // token -> first index entry (n_tokens + 1)
+    const uint64_t* toff;      // cell -> first index entry (and one past the last cell)
     const void* post;          // index entries (Entry<POS>)
     uint32_t* cursor;          // next probe (from the last position down)
     uint32_t grab;             // probes per grab
@@ -307,17 +316,19 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
             }
         }
         uint32_t left = __ballot_sync(kAll, my_pl != 0);
-        // bounds of the lists of tokens k .. k + 31 of a probe, asked for ahead of their use
+        // bounds of the lists of tokens k .. k + 31 of probe p, in the cells of the positions it admits,
+        // asked for ahead of their use
         uint64_t next_start = 0, next_end = 0;
-        auto bounds = [&](uint32_t tok, bool have) {
-            next_start = have ? J.toff[tok] : 0;
-            next_end = have ? J.toff[tok + 1] : 0;
+        auto bounds = [&](uint32_t tok, bool have, int p) {
+            const uint32_t first = __shfl_sync(kAll, my_lo, p), last = P.n - 2 - (g0 + p);
+            next_start = have ? J.toff[cell_of(P, tok, first)] : 0;
+            next_end = have ? J.toff[cell_of(P, tok, last) + 1] : 0;
         };
         if (left) {
             const int p = __ffs(left) - 1;
             const uint32_t* t = reinterpret_cast<const uint32_t*>(P.toks4 + __shfl_sync(kAll, my_d.x, p));
             const bool have = (uint32_t)lane < __shfl_sync(kAll, my_pl, p);
-            bounds(have ? t[lane] : 0u, have);
+            bounds(have ? t[lane] : 0u, have, p);
         }
         while (left) {
             const int p = __ffs(left) - 1;
@@ -337,7 +348,8 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
             uint32_t hash_mask = 0;
             if (rpos - lo > kSeenBits) {
                 uint64_t e = next_end - next_start;
-                for (uint32_t k = 32 + lane; k < pl; k += 32) e += J.toff[t[k] + 1] - J.toff[t[k]];
+                for (uint32_t k = 32 + lane; k < pl; k += 32)
+                    e += J.toff[cell_of(P, t[k], rpos - 1) + 1] - J.toff[cell_of(P, t[k], lo)];
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(kAll, e, o);
                 if (e <= kSeenWords / 2) hash_mask = e <= 32 ? 63u : (2u << (31 - __clz((uint32_t)e * 2 - 1))) - 1;
@@ -423,7 +435,7 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
                         const Entry<POS>* at = locate(lane, &k_n);
                         if ((uint32_t)lane < total) en_n = ld_entry(at);
                     }
-                    bounds(tok_n, have_n);
+                    bounds(tok_n, have_n, more || again ? p : p2);
                     for (uint32_t e0 = 0; e0 < total; e0 += 32) {
                         const Entry<POS> en = en_n;
                         const uint32_t k = k_n;
@@ -574,12 +586,15 @@ cudaError_t candgen_run(const CandgenInput& in, cudaStream_t st, int num_sms, Ca
     P.p = in.p;
     P.q = in.q;
     P.positional = in.positional;
+    P.cells_log2 = candgen_cells_log2(in.vocab);
+    P.cell_shift = candgen_cell_shift(in.n, P.cells_log2);
+    const uint64_t cells = candgen_cells(in.vocab);
     cudaError_t e;
     const unsigned tb = 256;
     if (in.stage == 0) {
         // order by size, then count prefix tokens
         e = cudaMemsetAsync(ix->size_hist, 0, 8ull * (in.max_len + 2), st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(ix->tcnt, 0, 8ull * (in.vocab + 1), st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(ix->toff, 0, 8ull * (cells + 1), st);
         if (e != cudaSuccess) return e;
         if (in.n) {
             const uint32_t per = std::max<uint32_t>((in.n + 2 * (uint32_t)num_sms - 1) / (2 * (uint32_t)num_sms), 1024u);
@@ -588,18 +603,15 @@ cudaError_t candgen_run(const CandgenInput& in, cudaStream_t st, int num_sms, Ca
             e = exclusive_scan_u64(ix->size_hist, in.max_len + 2, ix->scan_scratch, ix->total, st);
             if (e != cudaSuccess) return e;
             place_kernel<<<blocks, kSizeThreads, 0, st>>>(P, per, ix->size_hist, ix->probes, ix->rank);
-            token_count_kernel<<<grid_for((uint64_t)kSetLanes * in.n, tb, num_sms, 8), tb, 0, st>>>(P, ix->tcnt);
+            token_count_kernel<<<grid_for((uint64_t)kSetLanes * in.n, tb, num_sms, 8), tb, 0, st>>>(P, ix->rank, ix->toff);
         }
-        e = cudaMemcpyAsync(ix->toff, ix->tcnt, 8ull * (in.vocab + 1), cudaMemcpyDeviceToDevice, st);
-        if (e == cudaSuccess) e = exclusive_scan_u64(ix->toff, in.vocab + 1, ix->scan_scratch, ix->total, st);
+        e = exclusive_scan_u64(ix->toff, cells + 1, ix->scan_scratch, ix->total, st, ix->tcnt);
         if (e == cudaSuccess) e = cudaMemcpyAsync(host_word, ix->total, 8, cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return e;
         return cudaStreamSynchronize(st);  // *host_word: index entries
     }
     // fill the token lists
     if (in.n) {
-        e = cudaMemcpyAsync(ix->tcnt, ix->toff, 8ull * (in.vocab + 1), cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return e;
         const unsigned blocks = grid_for((uint64_t)kSetLanes * in.n, tb, num_sms, 8);
         if (in.positional) postings_kernel<true><<<blocks, tb, 0, st>>>(P, ix->rank, ix->tcnt, ix->post);
         else postings_kernel<false><<<blocks, tb, 0, st>>>(P, ix->rank, ix->tcnt, ix->post);
@@ -640,6 +652,8 @@ cudaError_t join_probe(const CandgenInput& in, const CandgenIndex& ix, const Ver
     P.p = in.p;
     P.q = in.q;
     P.positional = in.positional;
+    P.cells_log2 = candgen_cells_log2(in.vocab);
+    P.cell_shift = candgen_cell_shift(in.n, P.cells_log2);
     JoinArgs J;
     J.probes = ix.probes;
     J.size_end = ix.size_hist;

@@ -95,9 +95,12 @@ __global__ void scan_sums(uint64_t* sums, uint64_t n, uint64_t* total) {
     if (threadIdx.x == 0) *total = carry;
 }
 
-__global__ void scan_add(uint64_t* data, uint64_t n, const uint64_t* sums) {
+__global__ void scan_add(uint64_t* data, uint64_t n, const uint64_t* sums, uint64_t* copy) {
     const uint64_t i = (uint64_t)blockIdx.x * kScanBlock + threadIdx.x;
-    if (i < n) data[i] += sums[blockIdx.x];
+    if (i >= n) return;
+    const uint64_t v = data[i] + sums[blockIdx.x];
+    data[i] = v;
+    if (copy) copy[i] = v;
 }
 
 // one warp per set: tokens to their 16-byte aligned slot, padding after
@@ -179,7 +182,7 @@ cudaError_t layout_lengths(const uint64_t* d_offs, const uint32_t* d_toks, uint3
         len_kernel<<<blocks, 256, 0, st>>>(d_offs, d_toks, n, validate, chunks, d_err);
         scan_blocks<<<(unsigned)nb, kScanBlock, 0, st>>>(chunks, n, sums);
         scan_sums<<<1, kScanBlock, 0, st>>>(sums, nb, total);
-        scan_add<<<(unsigned)nb, kScanBlock, 0, st>>>(chunks, n, sums);
+        scan_add<<<(unsigned)nb, kScanBlock, 0, st>>>(chunks, n, sums, nullptr);
     } else {
         e = cudaMemsetAsync(total, 0, sizeof(uint64_t), st);
         if (e != cudaSuccess) return e;
@@ -205,12 +208,13 @@ size_t layout_scratch_words(uint32_t n) {
 
 size_t scan_scratch_words(uint64_t n) { return (n + kScanBlock - 1) / kScanBlock + 1; }
 
-cudaError_t exclusive_scan_u64(uint64_t* data, uint64_t n, uint64_t* scratch, uint64_t* total, cudaStream_t st) {
+cudaError_t exclusive_scan_u64(uint64_t* data, uint64_t n, uint64_t* scratch, uint64_t* total, cudaStream_t st,
+                               uint64_t* copy) {
     if (n == 0) return cudaMemsetAsync(total, 0, sizeof(uint64_t), st);
     const uint64_t nb = (n + kScanBlock - 1) / kScanBlock;
     scan_blocks<<<(unsigned)nb, kScanBlock, 0, st>>>(data, n, scratch);
     scan_sums<<<1, kScanBlock, 0, st>>>(scratch, nb, total);
-    scan_add<<<(unsigned)nb, kScanBlock, 0, st>>>(data, n, scratch);
+    scan_add<<<(unsigned)nb, kScanBlock, 0, st>>>(data, n, scratch, copy);
     return cudaGetLastError();
 }
 
