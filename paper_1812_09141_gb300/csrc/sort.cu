@@ -4,9 +4,9 @@
 // The number of results is known on the device only, so the sort of up to
 // kSortTile triples an instance is queued right after the verify kernel, one
 // CTA per instance, and the host reads count and triples back at once (2,034
-// results: std::sort between two copies took about 100 us, the kernel takes
-// 6).  More results are sorted after the count has come back: tiles by the
-// same code, then passes that merge two runs each.
+// results: std::sort between two copies took about 100 us).  More results are
+// sorted after the count has come back: tiles by the same code, then passes
+// that merge two runs each.
 #include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -25,34 +25,68 @@ __device__ __forceinline__ unsigned long long key_of(const ssj_triple& t) {
     return ((unsigned long long)t.r << 32) | t.s;
 }
 
-// n <= kSortTile triples from src to dst (may be the same), by one CTA:
-// bitonic network over the next power of two in shared memory.  (Set ids are
-// below 2^31, so the padding goes last.)
-__device__ void sort_tile(const ssj_triple* src, ssj_triple* dst, uint32_t n, unsigned long long* key, uint32_t* val) {
-    uint32_t size = 2;
-    while (size < n) size <<= 1;
-    for (uint32_t i = threadIdx.x; i < size; i += blockDim.x) {
-        key[i] = i < n ? key_of(src[i]) : ~0ull;
-        val[i] = i < n ? src[i].overlap : ~0u;
-    }
-    __syncthreads();
-    for (uint32_t k = 2; k <= size; k <<= 1) {
-        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-            for (uint32_t x = threadIdx.x; x < size / 2; x += blockDim.x) {
-                const uint32_t lo = 2 * x - (x & (j - 1)), hi = lo + j;
-                const unsigned long long a = key[lo], b = key[hi];
-                if ((a > b) == ((lo & k) == 0)) {
-                    key[lo] = b;
-                    key[hi] = a;
-                    const uint32_t v = val[lo];
-                    val[lo] = val[hi];
-                    val[hi] = v;
+// n <= kSortTile triples from src to dst (may be the same), by one CTA of
+// kSortThreads: runs of 32 sorted in registers (bitonic, by shuffles), then
+// merged two by two between two buffers in shared memory, each triple finding
+// its place by a binary search of the sibling run.  (Bound by latency: 2,034
+// triples take 6 merge steps of at most 11 dependent shared-memory loads; a
+// bitonic network in shared memory needs 66 steps with a barrier each and took
+// 29 us.)  `smem` holds 2 * kSortTile keys, then as many overlaps.
+constexpr size_t kSortSmem = 2 * kSortTile * (sizeof(unsigned long long) + sizeof(uint32_t));
+
+__device__ void sort_tile(const ssj_triple* src, ssj_triple* dst, uint32_t n, unsigned long long* smem) {
+    unsigned long long *key = smem, *key2 = smem + kSortTile;
+    uint32_t *val = reinterpret_cast<uint32_t*>(smem + 2 * kSortTile), *val2 = val + kSortTile;
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint32_t i = threadIdx.x; i - lane < n; i += kSortThreads) {
+        unsigned long long k = ~0ull;  // (past the end: last; set ids are below 2^31)
+        uint32_t v = 0;
+        if (i < n) {
+            k = key_of(src[i]);
+            v = src[i].overlap;
+        }
+#pragma unroll
+        for (uint32_t size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+            for (uint32_t j = size >> 1; j > 0; j >>= 1) {
+                const unsigned long long k2 = __shfl_xor_sync(0xFFFFFFFFu, k, j);
+                const uint32_t v2 = __shfl_xor_sync(0xFFFFFFFFu, v, j);
+                // the lower lane of a pair keeps the smaller key in ascending runs
+                const bool take = ((lane & j) == 0) == ((lane & size) == 0) ? k2 < k : k2 > k;
+                if (take) {
+                    k = k2;
+                    v = v2;
                 }
             }
-            __syncthreads();
         }
+        key[i] = k;
+        val[i] = v;
     }
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+    __syncthreads();
+    for (uint32_t run = 32; run < n; run <<= 1) {
+        for (uint32_t i = threadIdx.x; i < n; i += kSortThreads) {
+            const unsigned long long k = key[i];
+            const uint32_t mine = i / run, sib = (mine ^ 1u) * run;  // first triple of the sibling run
+            const uint32_t end = min(sib + run, n);
+            uint32_t lo = min(sib, end), hi = end;
+            const bool left = (mine & 1u) == 0;
+            while (lo < hi) {  // the sibling's triples that go before: smaller ones, and for the right run's also equal ones
+                const uint32_t mid = (lo + hi) >> 1;
+                if (left ? key[mid] < k : key[mid] <= k) lo = mid + 1; else hi = mid;
+            }
+            const uint32_t to = left ? i + (lo - min(sib, end)) : sib + (i - mine * run) + (lo - sib);
+            key2[to] = k;
+            val2[to] = val[i];
+        }
+        __syncthreads();
+        unsigned long long* sk = key;
+        key = key2;
+        key2 = sk;
+        uint32_t* sv = val;
+        val = val2;
+        val2 = sv;
+    }
+    for (uint32_t i = threadIdx.x; i < n; i += kSortThreads) {
         ssj_triple t;
         t.r = (uint32_t)(key[i] >> 32);
         t.s = (uint32_t)key[i];
@@ -62,19 +96,17 @@ __device__ void sort_tile(const ssj_triple* src, ssj_triple* dst, uint32_t n, un
 }
 
 __global__ void __launch_bounds__(kSortThreads) sort_results_kernel(const Instance* table) {
-    __shared__ unsigned long long key[kSortTile];
-    __shared__ uint32_t val[kSortTile];
+    extern __shared__ unsigned long long smem[];
     const Instance& I = table[blockIdx.x];
     if (!(I.flags & VF_SORTED)) return;
     const unsigned long long n = min(*I.count, (unsigned long long)I.cap);
-    if (n >= 2 && n <= kSortTile) sort_tile(I.out, I.out, (uint32_t)n, key, val);
+    if (n >= 2 && n <= kSortTile) sort_tile(I.out, I.out, (uint32_t)n, smem);
 }
 
 __global__ void __launch_bounds__(kSortThreads) sort_tiles_kernel(const ssj_triple* src, ssj_triple* dst, uint64_t n) {
-    __shared__ unsigned long long key[kSortTile];
-    __shared__ uint32_t val[kSortTile];
+    extern __shared__ unsigned long long smem[];
     const uint64_t at = (uint64_t)blockIdx.x * kSortTile;
-    sort_tile(src + at, dst + at, (uint32_t)min((uint64_t)kSortTile, n - at), key, val);
+    sort_tile(src + at, dst + at, (uint32_t)min((uint64_t)kSortTile, n - at), smem);
 }
 
 // Runs of `run` sorted triples merged two by two from src to dst.  A CTA writes
@@ -143,9 +175,18 @@ __global__ void __launch_bounds__(256) pack_results_kernel(const Instance* table
 
 }  // namespace
 
+// The kernels' shared memory is above the default limit: raised per device
+// (again by every launch: it costs little, and no state is kept).
+template <class K>
+static cudaError_t allow_sort_smem(K kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSortSmem);
+}
+
 cudaError_t sort_results(const Instance* table, uint32_t n_inst, cudaStream_t st) {
     if (n_inst == 0) return cudaSuccess;
-    sort_results_kernel<<<n_inst, kSortThreads, 0, st>>>(table);
+    const cudaError_t e = allow_sort_smem(sort_results_kernel);
+    if (e != cudaSuccess) return e;
+    sort_results_kernel<<<n_inst, kSortThreads, kSortSmem, st>>>(table);
     return cudaGetLastError();
 }
 
@@ -161,7 +202,9 @@ cudaError_t sort_triples(ssj_triple* t, uint64_t n, ssj_triple* tmp, cudaStream_
     for (uint64_t run = kSortTile; run < n; run *= 2) ++passes;
     ssj_triple* from = (passes & 1) ? tmp : t;  // the last pass ends in t
     ssj_triple* to = (passes & 1) ? t : tmp;
-    sort_tiles_kernel<<<(unsigned)((n + kSortTile - 1) / kSortTile), kSortThreads, 0, st>>>(t, from, n);
+    const cudaError_t e = allow_sort_smem(sort_tiles_kernel);
+    if (e != cudaSuccess) return e;
+    sort_tiles_kernel<<<(unsigned)((n + kSortTile - 1) / kSortTile), kSortThreads, kSortSmem, st>>>(t, from, n);
     for (uint64_t run = kSortTile; run < n; run *= 2) {
         merge_runs_kernel<<<(unsigned)((n + kMergeTile - 1) / kMergeTile), kMergeThreads, 0, st>>>(from, to, n, run);
         std::swap(from, to);
