@@ -277,6 +277,7 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
         __syncwarp();
         n = 0;
     };
+    const Threshold th = threshold(I);
     Sector rs;        // G > 1: the probe's record
     uint32_t nr = 0;
     auto test = [&](uint32_t m) {  // the first m waiting candidates
@@ -287,10 +288,10 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
             uint32_t r_head;
             const uint32_t r = __ldg(J.probes + e.x);
             const uint32_t v = bound_of_pair<1, false>(I.s_rec[0], I.r_rec[0], e.y, r, rs, lane, &r_head);
-            pass = pass && bound_passes(I, v, r_head >> 16);
+            pass = pass && bound_passes(I, th, v, r_head >> 16);
         } else if (G > 1) {
             const uint32_t v = bound_of_pair<kG, true>(I.s_rec[0], nullptr, e.y, 0u, rs, lane);
-            pass = pass && bound_passes(I, v, nr);
+            pass = pass && bound_passes(I, th, v, nr);
         }
         const uint32_t pm = __ballot_sync(kAll, pass);
         if (pass) W.buf[n + __popc(pm & lt)] = e;

@@ -8,9 +8,9 @@
 // instructions that count their common bits, about three per four bytes.
 // Verification of 9.2e7 candidates of long sets (about 300 tokens, t = 0.6)
 // took 5.2 ms when every candidate was walked against a bitmap of its probe;
-// the test takes 1.10 ms (64 bytes per candidate, 6e9 bytes from L2) and
-// leaves 47 us of merging.  On 5.7e6 candidates of short sets (about 20
-// tokens) 55 us, leaving 18 us, instead of 195 us of merging.
+// the test takes 1.00 ms (64 bytes per candidate, 6e9 bytes from L2) and
+// leaves 50 us of verification.  On 5.7e6 candidates of short sets (about 20
+// tokens) 50 us, leaving 10 us, instead of 195 us of merging.
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -25,8 +25,10 @@ namespace {
 constexpr int kPlanThreads = 256;
 constexpr int kPlanWarps = kPlanThreads / 32;
 constexpr uint32_t kOneProbe = 64;              // candidates of a list worth rounds of their own (32: the same)
-// CTAs per SM the registers are budgeted for (64 each).  With 3 and 4 loads in flight the long sets
-// take 1.25 ms instead of 1.10, with 5 the spills cost more than the warps gain (1.32).
+// CTAs per SM the registers are budgeted for (64 each).  With 3 the long sets take 1.09 ms instead of
+// 1.00; with 5 the spills cost more than the warps gain (1.20).  Asking for the next round's records
+// before these are counted costs more registers than it hides latency (1.16 ms with 3 CTAs); more
+// candidate ids asked for ahead change nothing (2 rounds) or cost registers (4: 1.02 ms).
 constexpr int kPlanCtas = 4;
 
 // Largest k with offs[k] <= f, by the whole warp: each step narrows the range
@@ -91,6 +93,8 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
         if (f + 32 + lane < len) s_next = __ldg(cands + f + 32 + lane);
         return s;
     };
+    const Threshold th = threshold(I);
+    bool bad = false;  // a candidate id is out of range
     uint32_t f = 0;
     while (f < len && n < kPlanFlush) {
         uint32_t passed = __popc(__ballot_sync(kFull, ends <= f));  // lists of the window that end by f
@@ -115,7 +119,7 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
             for (; f < end && (end - f >= 32 || end == len) && n < kPlanFlush; f += 32) {
                 const uint32_t s = next(f);
                 const bool have = r_ok && f + lane < end, ok = have && s < s_n_sets;
-                if (have && !ok) atomicOr(err, ERR_CAND_ID);
+                bad = bad || (have && !ok);
                 bool pass = ok && !(self_join && s == r);
                 if (G == 0) {
                     if (pass && !emit_all) {
@@ -124,7 +128,7 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
                     }
                 } else {
                     const uint32_t v = bound_of_pair<kG, true>(I.s_rec[0], nullptr, ok ? s : 0u, 0u, rs, lane);
-                    pass = pass && bound_passes(I, v, nr);
+                    pass = pass && bound_passes(I, th, v, nr);
                 }
                 keep(pass, slot0 + k, s);
             }
@@ -164,7 +168,7 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
             }
             const uint32_t s = next(f);
             const bool have = r < I.r_n_sets && my < len, ok = have && s < s_n_sets;
-            if (have && !ok) atomicOr(err, ERR_CAND_ID);
+            bad = bad || (have && !ok);
             bool pass = ok && !(self_join && s == r);
             if (G == 0) {
                 if (pass && !emit_all) {
@@ -176,12 +180,13 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
                 uint32_t r_head = G > 1 ? __ldg(&I.r_rec[0][(uint64_t)rk * kG * 2].x) : 0u;
                 const uint32_t v =
                     bound_of_pair<kG, false>(I.s_rec[0], I.r_rec[0], ok ? s : 0u, rk, Sector(), lane, &r_head);
-                pass = pass && bound_passes(I, v, r_head >> 16);
+                pass = pass && bound_passes(I, th, v, r_head >> 16);
             }
             keep(pass, slot0 + k, s);
             f += 32;
         }
     }
+    if (__any_sync(kFull, bad) && lane == 0) atomicOr(err, ERR_CAND_ID);
     *n_out = n;
     return f0 + min(f, len);
 }

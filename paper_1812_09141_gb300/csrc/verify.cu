@@ -1266,18 +1266,19 @@ static void item_sizes(uint64_t n_cands, int num_sms, uint32_t* per_warp_item, u
 
 static uint64_t pair_cap(const LaunchShape& sh) { return sh.total_cands + 32ull * sh.n_tiles + 32; }
 
-// Small chunks for small batches, so that a wave of warps shares the work;
-// at least 256 candidates once block items hold several pairs, so that the
-// runs of pairs that chunk borders cut (one more work item each) fit the
-// block list (see bind_workspace).
+// Whole rounds of a wave's warps (plan kernel: 32 per SM), of chunks of at most
+// about 1024; small chunks for small batches, so that all warps share the work.
+// At least 64 once block items hold several pairs, so that the runs of pairs
+// that chunk borders cut (one more work item each) fit the item lists (see
+// bind_workspace).
 uint32_t plan_chunk(uint64_t total_cands, int num_sms) {
     uint32_t wc, bc, lc, ic;
     item_sizes(total_cands, num_sms, &wc, &bc, &lc, &ic);
-    // whole rounds of a wave's warps (plan kernel: 32 per SM), of chunks of at most about 1024
-    const uint64_t warps = 32ull * (uint64_t)num_sms, rounds = (total_cands + 1024 * warps - 1) / (1024 * warps);
-    const uint64_t per = (total_cands + warps * std::max<uint64_t>(rounds, 1) - 1) / (warps * std::max<uint64_t>(rounds, 1));
+    const uint64_t warps = 32ull * (uint64_t)num_sms;
+    const uint64_t rounds = std::max<uint64_t>((total_cands + 1024 * warps - 1) / (1024 * warps), 1);
+    const uint64_t per = (total_cands + warps * rounds - 1) / (warps * rounds);
     const uint32_t c = std::max<uint32_t>((uint32_t)((per + 31) & ~31ull), 32u);
-    return bc > 1 && c < 256 ? 256u : c;
+    return bc > 1 && c < 64 ? 64u : c;
 }
 
 LaunchShape single_shape(uint32_t n_probes, uint64_t n_cands, int num_sms) {
@@ -1294,7 +1295,7 @@ size_t workspace_bytes(const LaunchShape& sh, int num_sms) {
     uint32_t wc, bc, lc, ic;
     item_sizes(sh.total_cands, num_sms, &wc, &bc, &lc, &ic);
     const uint64_t slots = 32ull * sh.n_tiles + 1, pc = pair_cap(sh);
-    // slots * 12 + pc / 8 bytes: extra work items, see bind_workspace
+    // (the terms by probe slot and pc / 8 are room for work items, see bind_workspace)
     return align256(sizeof(Counters)) + align256(sizeof(Instance) * ((size_t)sh.n_inst + 1)) +
            align256(sizeof(uint2) * slots) + align256(sizeof(uint32_t) * slots) +
            align256(sizeof(uint32_t) * (pc / 32 + 1)) + align256(sizeof(PairRef) * pc) +
@@ -1323,15 +1324,18 @@ void bind_workspace(VerifyArgs& a, void* ws, const LaunchShape& sh, int num_sms)
     a.pair_cap = pair_cap(sh);
     a.pairs = reinterpret_cast<PairRef*>(p);
     p += align256(sizeof(PairRef) * a.pair_cap);
+    // Work items are made of runs, a probe's pairs of one chunk that are queued together: at most one
+    // per probe, one more per chunk border and one more per early flush (every kPlanFlush pairs; chunks
+    // are longer than that only in large batches).  Lane items take up to 32 pairs or more of a run,
+    // block items up to block_item_cands; neither are more than the pairs.  The lists share what the
+    // workspace holds beside the pair list, at least 48 bytes per probe and 36 (single pairs per warp
+    // and block item) to 4.6 bytes per candidate.
+    const uint64_t cuts = sh.n_chunks + sh.total_cands / kPlanFlush + 1;
+    const uint64_t lane_items = std::min<uint64_t>(sh.total_probes + cuts + sh.total_cands / 32,
+                                                   item_cap(sh.total_probes, sh.total_cands, wc));
     a.warp_items = reinterpret_cast<WorkItem*>(p);
-    a.warp_item_cap = (uint32_t)item_cap(sh.total_probes, sh.total_cands, wc);
+    a.warp_item_cap = (uint32_t)std::min<uint64_t>(lane_items, 0xFFFFFFF0ull);
     p += align256(sizeof(WorkItem) * ((size_t)a.warp_item_cap + 1));
-    // Block items take the rest: n_probes + n_cands / block_item_cands, and 12 bytes per probe slot
-    // and 1/8 byte per candidate beyond that, one item per 192 candidates: runs cut at chunk borders
-    // (chunks of 256 or more) and by early flushes (every kPlanFlush pairs of chunks above that size)
-    // are at most one per 256 candidates, or one per 480 and one per 512.  Chunks below 256 come with
-    // one pair per block item and one index item per run, at most n_cands items.  Lane items, at
-    // least one pair and up to 32 of a run, fit n_probes + n_cands / 8 the same way.
     a.block_items = reinterpret_cast<WorkItem*>(p);
     const size_t left = static_cast<char*>(ws) + workspace_bytes(sh, num_sms) - p;
     a.block_item_cap = (uint32_t)(left / sizeof(WorkItem) > 0xFFFFFFF0ull ? 0xFFFFFFF0ull : left / sizeof(WorkItem));
