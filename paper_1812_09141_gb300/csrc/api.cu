@@ -59,21 +59,19 @@ namespace {
 
 // Default of the context's index-item threshold (ssj_set_index_items).
 constexpr uint32_t kIndexMinCandsDefault = 256;
-// ssj_verify_batches runs a call as one launch per kSplitCands candidates, up to kMaxGroups
-// (on the 256-instance workload, four groups measured slower than two: 1.39e10 against
-// 1.45e10 pairs/s end to end; each launch adds its own fill and drain).
-constexpr uint64_t kSplitCands = 1ull << 24;
-constexpr uint32_t kMaxGroups = 2;
-// ...and reads inputs in pinned host memory directly over the host link (no staging copy) in
-// calls of at least this many candidates: on the 256-instance workload, 1.62e10-1.67e10 pairs/s
-// end to end against 1.09e10-1.45e10 with staged copies.
-constexpr uint64_t kDirectCands = 1ull << 25;
+// ssj_verify_batches plans a call in up to kMaxPieces pieces of whole waves of plan chunks, each as
+// soon as its candidate ids are on the device.  The host link moves 211 GB/s, to the copy engine and to
+// kernels alike; 8.1e7 candidates of 12 joins take 1.53 ms to copy and 0.8 ms to plan.  In pieces the
+// call takes 1.9 ms; in two groups of batches, copied first, 2.1; with the kernels reading all inputs
+// over the link 2.2 in pieces and 2.3 in two groups, and the same with only probe ids and offsets read
+// so (the search for a chunk's first probe is a chain of reads).
+constexpr uint32_t kMaxPieces = 16;
 // Candidates of one batch, and of one call or prepared launch: 2^40 ids are 4 TiB, beyond any
 // device's memory, and keep every workspace size computed from the count far from 64-bit wrap.
 constexpr uint64_t kMaxCands = 1ull << 40;
 // Results copied to pinned memory along with their count, before the host knows it, so that calls
 // with up to that many wait for the device once (48 KiB take about 2 us; a second wait and copy
-// take about 15): of one batch, and of a group of ssj_verify_batches.
+// take about 15): of one batch, and of all batches of ssj_verify_batches.
 constexpr uint64_t kFirstResults = 4096;
 constexpr uint64_t kPackResults = 16384;
 
@@ -173,19 +171,19 @@ struct ssj_ctx {
     void* io = nullptr;
     size_t io_bytes = 0;
     uint64_t* h_count = nullptr;  // pinned
-    uint32_t* h_err = nullptr;    // pinned, kMaxGroups words
+    uint32_t* h_err = nullptr;    // pinned
     Counters* h_ctr = nullptr;    // pinned
-    // pinned: results that come back with their count (kFirstResults; ssj_verify_batches: kPackResults
-    // a group), and ssj_verify_batches' counts and instance table
+    // pinned: results that come back with their count (kFirstResults; ssj_verify_batches:
+    // kPackResults), and ssj_verify_batches' counts and instance table
     ssj_triple* h_first = nullptr;
     uint64_t h_first_cap = 0;
     uint64_t* h_counts = nullptr;
     uint64_t h_counts_cap = 0;
     Instance* h_table = nullptr;
     uint64_t h_table_cap = 0;
-    // ssj_verify_batches: the stream and event that carry the second group's input copies
+    // ssj_verify_batches: the stream and events that carry the pieces' copies
     cudaStream_t copy_stream = nullptr;
-    cudaEvent_t copy_done[kMaxGroups] = {};
+    cudaEvent_t copy_done[kMaxPieces] = {};
     cudaEvent_t call_start = nullptr;
     Counters* last_ctr = nullptr;
     // kernel timing (SSJ_CTX_PROFILE): events around plan and verify of each launch
@@ -624,8 +622,7 @@ extern "C" ssj_status ssj_create(const ssj_config* config, ssj_ctx** out) {
         ctx->own_stream = true;
     }
     if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_count), sizeof(uint64_t)) != cudaSuccess) return SSJ_EDEVICE;
-    if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_err), kMaxGroups * sizeof(uint32_t)) != cudaSuccess)
-        return SSJ_EDEVICE;
+    if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_err), sizeof(uint32_t)) != cudaSuccess) return SSJ_EDEVICE;
     if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_ctr), sizeof(Counters)) != cudaSuccess) return SSJ_EDEVICE;
     cudaMemPoolProps props;
     memset(&props, 0, sizeof(props));
@@ -1053,8 +1050,8 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
     sh.total_probes = 0;
     sh.total_cands = 0;
     sh.n_chunks = 0;
-    const size_t packed_bytes = sizeof(ssj_triple) * kPackResults;  // a group's results for one copy
-    size_t off = align256(sizeof(uint64_t) * n_batches) + kMaxGroups * align256(packed_bytes);  // counts and these first
+    const size_t packed_bytes = sizeof(ssj_triple) * kPackResults;  // results for one copy
+    size_t off = align256(sizeof(uint64_t) * n_batches) + align256(packed_bytes);  // counts and these first
     uint64_t launch_vocab = 1;
     bool launch_force_index = false;
     const Collection* pinned = nullptr;  // the first pinned collection: its L2 window
@@ -1085,74 +1082,23 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
         const uint64_t cap = (b->flags & SSJ_COUNT_ONLY) ? 0 : std::min(caps[i], n_cands[i]);
         off += align256(sizeof(ssj_triple) * std::max<uint64_t>(cap, 1));
     }
-    // Large calls run as up to kMaxGroups launches over consecutive groups of batches with about
-    // equal candidate counts: each later group's host-to-device copies, on a second stream,
-    // overlap the earlier groups' kernels.
-    uint32_t groups = (uint32_t)std::min<uint64_t>(
-        {(uint64_t)kMaxGroups, (uint64_t)n_batches, std::max<uint64_t>(sh.total_cands / kSplitCands, 1)});
-    uint32_t gstart[kMaxGroups + 1];
-    {
-        uint32_t g = 0;
-        uint64_t acc = 0;
-        gstart[0] = 0;
-        for (uint32_t i = 0; i < n_batches && g + 1 < groups; ++i) {
-            acc += n_cands[i];
-            if (acc * groups >= (uint64_t)(g + 1) * sh.total_cands && i + 1 < n_batches) gstart[++g] = i + 1;
-        }
-        groups = g + 1;  // (a group is never empty)
-        gstart[groups] = n_batches;
-    }
-    LaunchShape shp[kMaxGroups];
-    size_t ws_off[kMaxGroups + 1];
-    ws_off[0] = 0;
-    for (uint32_t gi = 0; gi < groups; ++gi) {
-        LaunchShape& q = shp[gi];
-        q.n_inst = 0;
-        q.n_tiles = 0;
-        q.total_probes = 0;
-        q.total_cands = 0;
-        q.n_chunks = 0;
-        for (uint32_t i = gstart[gi]; i < gstart[gi + 1]; ++i) {
-            table[i].tile_base = q.n_tiles;
-            q.n_inst += 1;
-            q.n_tiles += (uint32_t)(((uint64_t)batches[i].n_probes + 31) / 32);
-            q.total_probes += batches[i].n_probes;
-            q.total_cands += n_cands[i];
-        }
-        set_chunks(table.data() + gstart[gi], q, ctx->num_sms);
-        ws_off[gi + 1] = ws_off[gi] + align256(workspace_bytes(q, ctx->num_sms));
-    }
-    const size_t ws_total = ws_off[groups];
+    set_chunks(table.data(), sh, ctx->num_sms);
     DeviceGuard g(ctx->device);
     ssj_status st = ensure_device_buffer(ctx, &ctx->io, &ctx->io_bytes, off);
     if (st != SSJ_OK) return st;
-    st = ensure_device_buffer(ctx, &ctx->ws, &ctx->ws_bytes, ws_total);
+    st = ensure_device_buffer(ctx, &ctx->ws, &ctx->ws_bytes, workspace_bytes(sh, ctx->num_sms));
     if (st != SSJ_OK) return st;
     if ((st = ensure_pinned(ctx, &ctx->h_counts, &ctx->h_counts_cap, n_batches)) != SSJ_OK ||
         (st = ensure_pinned(ctx, &ctx->h_table, &ctx->h_table_cap, n_batches)) != SSJ_OK ||
-        (st = ensure_pinned(ctx, &ctx->h_first, &ctx->h_first_cap, kMaxGroups * kPackResults)) != SSJ_OK)
+        (st = ensure_pinned(ctx, &ctx->h_first, &ctx->h_first_cap, kPackResults)) != SSJ_OK)
         return st;
     cudaStream_t s = ctx->stream;
-    cudaStream_t cs = s;  // the later groups' copies
-    if (groups > 1) {
-        if (!ctx->copy_stream) CUDA_TRY(ctx, cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
-        for (uint32_t gi = 0; gi < kMaxGroups; ++gi)
-            if (!ctx->copy_done[gi]) CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->copy_done[gi], cudaEventDisableTiming));
-        if (!ctx->call_start) CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->call_start, cudaEventDisableTiming));
-        cs = ctx->copy_stream;
-        // the copy stream starts after everything already queued on the context's stream
-        CUDA_TRY(ctx, cudaEventRecord(ctx->call_start, s));
-        CUDA_TRY(ctx, cudaStreamWaitEvent(cs, ctx->call_start, 0));
-    }
     char* base = static_cast<char*>(ctx->io);
     uint64_t* d_counts = reinterpret_cast<uint64_t*>(base);
-    char* d_packed = base + align256(sizeof(uint64_t) * n_batches);
-    for (uint32_t i = 0, gi = 0; i < n_batches; ++i) {
-        if (i == gstart[gi + 1]) {  // group gi's copies are all queued
-            if (gi > 0) CUDA_TRY(ctx, cudaEventRecord(ctx->copy_done[gi], cs));
-            ++gi;
-        }
-        const cudaStream_t cp = gi == 0 ? s : cs;
+    ssj_triple* d_packed = reinterpret_cast<ssj_triple*>(base + align256(sizeof(uint64_t) * n_batches));
+    bool any_sorted = false, any_results = false;
+    std::vector<uint32_t*> staged(n_batches, nullptr);  // device place of the candidate ids that are copied
+    for (uint32_t i = 0; i < n_batches; ++i) {
         const ssj_batch* b = &batches[i];
         char* p = base + io_off[i];
         uint32_t* d_probe = reinterpret_cast<uint32_t*>(p); p += align256(4ull * std::max<uint32_t>(b->n_probes, 1));
@@ -1160,18 +1106,15 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
         uint32_t* d_cand = reinterpret_cast<uint32_t*>(p);  p += align256(4ull * std::max<uint64_t>(n_cands[i], 1));
         // SSJ_HOST_DIRECT: pinned arrays the device can address are read by the kernels
         // themselves (over the host link), with no staging copy
-        // (calls of 2^25+ candidates read pinned inputs directly unless the batch asks for staging)
-        const bool direct = (b->flags & SSJ_HOST_DIRECT) ||
-                            (sh.total_cands >= kDirectCands && !(b->flags & SSJ_HOST_STAGED));
+        const bool direct = (b->flags & SSJ_HOST_DIRECT) != 0;
         const void* dv_probe = direct ? device_view(b->probe_ids, 4) : nullptr;
         const void* dv_offs = direct ? device_view(b->cand_offsets, 8) : nullptr;
         const void* dv_cand = direct ? device_view(b->cand_ids, 4) : nullptr;
         if (b->n_probes && !dv_probe)
-            CUDA_TRY(ctx, cudaMemcpyAsync(d_probe, b->probe_ids, 4ull * b->n_probes, cudaMemcpyHostToDevice, cp));
+            CUDA_TRY(ctx, cudaMemcpyAsync(d_probe, b->probe_ids, 4ull * b->n_probes, cudaMemcpyHostToDevice, s));
         if (b->n_probes && !dv_offs)
-            CUDA_TRY(ctx, cudaMemcpyAsync(d_offs, b->cand_offsets, 8ull * (b->n_probes + 1), cudaMemcpyHostToDevice, cp));
-        if (n_cands[i] && !dv_cand)
-            CUDA_TRY(ctx, cudaMemcpyAsync(d_cand, b->cand_ids, 4ull * n_cands[i], cudaMemcpyHostToDevice, cp));
+            CUDA_TRY(ctx, cudaMemcpyAsync(d_offs, b->cand_offsets, 8ull * (b->n_probes + 1), cudaMemcpyHostToDevice, s));
+        if (n_cands[i] && !dv_cand) staged[i] = d_cand;
         Instance& I = table[i];
         I.probe_ids = dv_probe ? static_cast<const uint32_t*>(dv_probe) : d_probe;
         I.cand_offsets = dv_offs ? static_cast<const uint64_t*>(dv_offs) : d_offs;
@@ -1179,66 +1122,97 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
         I.out = reinterpret_cast<ssj_triple*>(p);
         I.cap = (b->flags & SSJ_COUNT_ONLY) ? 0 : std::min(caps[i], n_cands[i]);
         I.count = reinterpret_cast<unsigned long long*>(d_counts + i);
+        any_sorted = any_sorted || (I.flags & VF_SORTED);
+        any_results = any_results || I.cap;
     }
-    if (groups > 1) CUDA_TRY(ctx, cudaEventRecord(ctx->copy_done[groups - 1], cs));
+    VerifyArgs a;
+    memset(&a, 0, sizeof(a));
+    apply_policy(ctx, a, launch_vocab, launch_force_index);
+    if (pinned) set_l2_window(a, *pinned);
+    bind_workspace(a, ctx->ws, sh, ctx->num_sms);
+    a.table = a.table_out;
     memcpy(ctx->h_table, table.data(), sizeof(Instance) * n_batches);
-    for (uint32_t gi = 0; gi < groups; ++gi) {
-        const uint32_t lo = gstart[gi], hi = gstart[gi + 1];
-        VerifyArgs a;
-        memset(&a, 0, sizeof(a));
-        apply_policy(ctx, a, launch_vocab, launch_force_index);
-        if (pinned) set_l2_window(a, *pinned);
-        bind_workspace(a, static_cast<char*>(ctx->ws) + ws_off[gi], shp[gi], ctx->num_sms);
-        a.table = a.table_out;
-        if (gi > 0) CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->copy_done[gi], 0));  // the group's inputs are in
-        CUDA_TRY(ctx, cudaMemcpyAsync(a.table_out, ctx->h_table + lo, sizeof(Instance) * (hi - lo),
-                                      cudaMemcpyHostToDevice, s));
-        ctx->last_ctr = a.ctr;
-        cudaError_t e = launch_verify(a, s, ctx->num_sms, ctx->block_threads, profile_events(ctx));
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "launch_verify");
-        // sorted where asked for, and the group's results packed, so that they come back in one copy
-        bool any_sorted = false, any_results = false;
-        for (uint32_t i = lo; i < hi; ++i) {
-            any_sorted = any_sorted || (table[i].flags & VF_SORTED);
-            any_results = any_results || table[i].cap;
+    CUDA_TRY(ctx, cudaMemcpyAsync(a.table_out, ctx->h_table, sizeof(Instance) * n_batches, cudaMemcpyHostToDevice, s));
+    ctx->last_ctr = a.ctr;
+    // pieces of whole waves (plan_wave chunks), each planned when its ids have come over the copy stream
+    const uint64_t wave = plan_wave(ctx->num_sms), waves = std::max<uint64_t>((sh.n_chunks + wave - 1) / wave, 1);
+    const uint64_t per_piece = wave * ((waves + kMaxPieces - 1) / kMaxPieces);
+    const uint32_t pieces = (uint32_t)std::max<uint64_t>((sh.n_chunks + per_piece - 1) / per_piece, 1);
+    cudaStream_t cs = s;
+    if (pieces > 1) {
+        if (!ctx->copy_stream) CUDA_TRY(ctx, cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking));
+        for (uint32_t k = 0; k < pieces; ++k)
+            if (!ctx->copy_done[k]) CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->copy_done[k], cudaEventDisableTiming));
+        if (!ctx->call_start) CUDA_TRY(ctx, cudaEventCreateWithFlags(&ctx->call_start, cudaEventDisableTiming));
+        cs = ctx->copy_stream;
+        // the copy stream starts after everything already queued on the context's stream
+        CUDA_TRY(ctx, cudaEventRecord(ctx->call_start, s));
+        CUDA_TRY(ctx, cudaStreamWaitEvent(cs, ctx->call_start, 0));
+    }
+    cudaEvent_t* ev = profile_events(ctx);
+    CUDA_TRY(ctx, cudaMemsetAsync(a.ctr, 0, sizeof(Counters), s));
+    if (ev) CUDA_TRY(ctx, cudaEventRecord(ev[0], s));
+    for (uint32_t k = 0, i0 = 0; k < pieces; ++k) {
+        const uint64_t c0 = k * per_piece, c1 = std::min(c0 + per_piece, sh.n_chunks);
+        for (uint32_t i = i0; i < n_batches && table[i].chunk_base < c1; ++i) {
+            const uint64_t begin = table[i].chunk_base, end = i + 1 < n_batches ? table[i + 1].chunk_base : sh.n_chunks;
+            if (end <= c0) {
+                i0 = i + 1;
+                continue;
+            }
+            if (!staged[i]) continue;
+            const uint64_t f0 = (std::max(c0, begin) - begin) * a.chunk;
+            const uint64_t f1 = std::min((std::min(c1, end) - begin) * a.chunk, n_cands[i]);
+            if (f1 > f0)
+                CUDA_TRY(ctx, cudaMemcpyAsync(staged[i] + f0, batches[i].cand_ids + f0, 4 * (f1 - f0),
+                                              cudaMemcpyHostToDevice, cs));
         }
-        ssj_triple* packed = reinterpret_cast<ssj_triple*>(d_packed + gi * align256(packed_bytes));
-        if (any_sorted) CUDA_TRY(ctx, sort_results(a.table_out, hi - lo, s));
-        if (any_results) {
-            CUDA_TRY(ctx, pack_results(a.table_out, hi - lo, packed, kPackResults, s));
-            CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_first + gi * kPackResults, packed, packed_bytes, cudaMemcpyDeviceToHost, s));
+        if (pieces > 1) {
+            CUDA_TRY(ctx, cudaEventRecord(ctx->copy_done[k], cs));
+            CUDA_TRY(ctx, cudaStreamWaitEvent(s, ctx->copy_done[k], 0));
         }
-        CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_err + gi, &a.ctr->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+        VerifyArgs piece = a;
+        piece.chunk_begin = c0;
+        piece.n_chunks = c1;
+        const cudaError_t e = launch_plan(piece, s, ctx->num_sms);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "launch_plan");
+    }
+    if (ev) CUDA_TRY(ctx, cudaEventRecord(ev[1], s));
+    const cudaError_t e = launch_merge(a, s, ctx->num_sms, ctx->block_threads);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "launch_merge");
+    if (ev) CUDA_TRY(ctx, cudaEventRecord(ev[2], s));
+    // sorted where asked for, and packed, so that all batches' results come back in one copy
+    if (any_sorted) CUDA_TRY(ctx, sort_results(a.table_out, n_batches, s));
+    if (any_results) {
+        CUDA_TRY(ctx, pack_results(a.table_out, n_batches, d_packed, kPackResults, s));
+        CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_first, d_packed, packed_bytes, cudaMemcpyDeviceToHost, s));
     }
     const uint64_t* counts = ctx->h_counts;
+    CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_err, &a.ctr->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(ctx, cudaMemcpyAsync(ctx->h_counts, d_counts, sizeof(uint64_t) * n_batches, cudaMemcpyDeviceToHost, s));
     CUDA_TRY(ctx, cudaStreamSynchronize(s));
-    uint32_t derr = 0;
-    for (uint32_t gi = 0; gi < groups; ++gi) derr |= ctx->h_err[gi];
-    if (derr) return device_check_status(ctx, derr);
+    if (*ctx->h_err) return device_check_status(ctx, *ctx->h_err);
     bool short_cap = false, waiting = false;
-    for (uint32_t gi = 0; gi < groups; ++gi) {
-        uint64_t total = 0;
-        for (uint32_t i = gstart[gi]; i < gstart[gi + 1]; ++i) {
-            n_outs[i] = counts[i];
-            if (batches[i].flags & SSJ_COUNT_ONLY) continue;
-            total += std::min(counts[i], table[i].cap);
-            short_cap = short_cap || counts[i] > caps[i];
+    uint64_t total = 0;
+    for (uint32_t i = 0; i < n_batches; ++i) {
+        n_outs[i] = counts[i];
+        if (batches[i].flags & SSJ_COUNT_ONLY) continue;
+        total += std::min(counts[i], table[i].cap);
+        short_cap = short_cap || counts[i] > caps[i];
+    }
+    const ssj_triple* from = ctx->h_first;
+    for (uint32_t i = 0; i < n_batches; ++i) {
+        if (batches[i].flags & SSJ_COUNT_ONLY) continue;
+        const uint64_t n = std::min(counts[i], table[i].cap);
+        const bool sort = (table[i].flags & VF_SORTED) && n > kSortTile;
+        if (total <= kPackResults && !sort) {
+            if (n) memcpy(outs[i], from, sizeof(ssj_triple) * n);
+        } else if (n) {
+            if (sort) CUDA_TRY(ctx, sort_in_place(ctx, table[i].out, n));
+            CUDA_TRY(ctx, cudaMemcpyAsync(outs[i], table[i].out, sizeof(ssj_triple) * n, cudaMemcpyDeviceToHost, s));
+            waiting = true;
         }
-        const ssj_triple* from = ctx->h_first + gi * kPackResults;
-        for (uint32_t i = gstart[gi]; i < gstart[gi + 1]; ++i) {
-            if (batches[i].flags & SSJ_COUNT_ONLY) continue;
-            const uint64_t n = std::min(counts[i], table[i].cap);
-            const bool sort = (table[i].flags & VF_SORTED) && n > kSortTile;
-            if (total <= kPackResults && !sort) {
-                if (n) memcpy(outs[i], from, sizeof(ssj_triple) * n);
-            } else if (n) {
-                if (sort) CUDA_TRY(ctx, sort_in_place(ctx, table[i].out, n));
-                CUDA_TRY(ctx, cudaMemcpyAsync(outs[i], table[i].out, sizeof(ssj_triple) * n, cudaMemcpyDeviceToHost, s));
-                waiting = true;
-            }
-            from += n;
-        }
+        from += n;
     }
     if (waiting) CUDA_TRY(ctx, cudaStreamSynchronize(s));
     if (short_cap) return fail(ctx, SSJ_ENOMEM, "a batch has more result pairs than its capacity (see n_outs)");

@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kPlanThreads, kPlanCtas) plan_kernel(const __g
     __shared__ PlanInst s_inst[kPlanWarps];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    if (blockIdx.x == 0) {
+    if (blockIdx.x == 0 && a.chunk_begin == 0) {
         if (!a.table && threadIdx.x == 0) a.table_out[0] = a.single;
         for (uint32_t i = threadIdx.x; i < a.n_inst; i += blockDim.x)
             *(a.table ? a.table[i].count : a.single.count) = 0ull;
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kPlanThreads, kPlanCtas) plan_kernel(const __g
     const uint32_t gwarp = blockIdx.x * kPlanWarps + warp;
     uint32_t held = 0xFFFFFFFFu;  // instance whose fields are in s_inst
     const PlanInst& I = s_inst[warp];
-    for (uint64_t c = gwarp; c < a.n_chunks; c += n_warps) {
+    for (uint64_t c = a.chunk_begin + gwarp; c < a.n_chunks; c += n_warps) {
         const uint32_t inst = a.table ? owner(a.table, a.n_inst, &Instance::chunk_base, c) : 0u;
         if (inst != held) {
             __syncwarp();
@@ -248,6 +248,7 @@ __global__ void __launch_bounds__(kPlanThreads, kPlanCtas) plan_kernel(const __g
             if (n) flush_survivors(a, I, inst, s_buf[warp], n, lane);
         }
     }
+    if (a.chunk_begin) return;  // (the first piece checks the probes)
     for (uint32_t g = n_warps - 1 - gwarp; g < a.n_tiles; g += n_warps) {
         const uint32_t inst = a.table ? owner(a.table, a.n_inst, &Instance::tile_base, g) : 0u;
         const PlanInst I = plan_inst(a.table ? a.table[inst] : a.single);
@@ -270,7 +271,8 @@ cudaError_t launch_plan(const VerifyArgs& a, cudaStream_t st, int num_sms) {
         ctas_per_sm = n;
     }
     // at most one wave; the kernel also runs for empty batches, to clear the instances' counts
-    const uint64_t units = a.n_chunks > a.n_tiles ? a.n_chunks : a.n_tiles;
+    const uint64_t chunks = a.n_chunks - a.chunk_begin, tiles = a.chunk_begin ? 0 : a.n_tiles;
+    const uint64_t units = chunks > tiles ? chunks : tiles;
     uint64_t blocks = (units + kPlanWarps - 1) / kPlanWarps;
     const uint64_t most = (uint64_t)num_sms * (uint64_t)ctas_per_sm;
     if (blocks > most) blocks = most;

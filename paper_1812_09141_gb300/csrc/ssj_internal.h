@@ -155,6 +155,7 @@ struct VerifyArgs {
     uint32_t total_probes;        // probe slots over all instances (instance-major)
     uint32_t chunk;               // candidates per plan chunk (a warp's unit of work)
     uint64_t n_chunks;            // over all instances
+    uint64_t chunk_begin;         // a plan launch of one piece: its first chunk (n_chunks: after its last)
     uint64_t total_cands;
     Counters* ctr;
     PairRef* pairs;               // pairs left to verify: short ones from the front, others from the back
@@ -197,6 +198,8 @@ struct LaunchShape {
 
 // Candidates per plan chunk of a launch, and the chunks of one instance.
 uint32_t plan_chunk(uint64_t total_cands, int num_sms);
+// Chunks that one wave of the plan kernel works on.
+inline uint64_t plan_wave(int num_sms) { return 32ull * (uint64_t)num_sms; }
 inline uint64_t chunks_of(uint64_t n_probes, uint64_t n_cands, uint32_t chunk) {
     return n_probes ? (n_cands + chunk - 1) / chunk : 0;
 }

@@ -1274,7 +1274,7 @@ static uint64_t pair_cap(const LaunchShape& sh) { return sh.total_cands + 32ull 
 uint32_t plan_chunk(uint64_t total_cands, int num_sms) {
     uint32_t wc, bc, lc, ic;
     item_sizes(total_cands, num_sms, &wc, &bc, &lc, &ic);
-    const uint64_t warps = 32ull * (uint64_t)num_sms;
+    const uint64_t warps = plan_wave(num_sms);
     const uint64_t rounds = std::max<uint64_t>((total_cands + 1024 * warps - 1) / (1024 * warps), 1);
     const uint64_t per = (total_cands + warps * rounds - 1) / (warps * rounds);
     const uint32_t c = std::max<uint32_t>((uint32_t)((per + 31) & ~31ull), 32u);
@@ -1317,6 +1317,7 @@ void bind_workspace(VerifyArgs& a, void* ws, const LaunchShape& sh, int num_sms)
     a.total_cands = sh.total_cands;
     a.chunk = plan_chunk(sh.total_cands, num_sms);
     a.n_chunks = sh.n_chunks;
+    a.chunk_begin = 0;
     a.ctr = reinterpret_cast<Counters*>(p);
     p += align256(sizeof(Counters));
     a.table_out = reinterpret_cast<Instance*>(p);
