@@ -69,6 +69,10 @@ constexpr uint32_t kMaxPieces = 16;
 // Candidates of one batch, and of one call or prepared launch: 2^40 ids are 4 TiB, beyond any
 // device's memory, and keep every workspace size computed from the count far from 64-bit wrap.
 constexpr uint64_t kMaxCands = 1ull << 40;
+// Host inputs of one batch up to this size are gathered in pinned memory and go to the device in one
+// copy that the call does not wait for: three copies from the caller's arrays and the wait for them
+// take about 25 us, gathering 128 KiB 8.
+constexpr size_t kSmallInput = 128 << 10;
 // Results copied to pinned memory along with their count, before the host knows it, so that calls
 // with up to that many wait for the device once (48 KiB take about 2 us; a second wait and copy
 // take about 15): of one batch, and of all batches of ssj_verify_batches.
@@ -131,11 +135,17 @@ struct Slot {
     uint64_t* h_offs = nullptr;
     uint32_t* h_cand = nullptr;
     uint64_t h_probe_cap = 0, h_offs_cap = 0, h_cand_cap = 0;
+    char* h_in = nullptr;           // small inputs, as they lie on the device
+    uint64_t h_in_cap = 0;
     ssj_triple* h_out = nullptr;
     uint64_t h_out_cap = 0;
     Counters* h_ctr = nullptr;
     bool busy = false;          // reserved by a ticket until ssj_results collects it
     struct Ticket* pending = nullptr;  // launched, waiting for the completion thread
+    // Wakes this slot's completion thread alone: one condition for all slots woke every thread at
+    // each submission and completion, and submissions waited about 35 us for the lock they took in
+    // turn (16 slots).
+    std::unique_ptr<std::condition_variable> wake;
     std::thread completer;
 };
 
@@ -175,6 +185,8 @@ struct ssj_ctx {
     Counters* h_ctr = nullptr;    // pinned
     // pinned: results that come back with their count (kFirstResults; ssj_verify_batches:
     // kPackResults), and ssj_verify_batches' counts and instance table
+    char* h_in = nullptr;         // pinned: small inputs, as they lie on the device
+    uint64_t h_in_cap = 0;
     ssj_triple* h_first = nullptr;
     uint64_t h_first_cap = 0;
     uint64_t* h_counts = nullptr;
@@ -193,7 +205,7 @@ struct ssj_ctx {
 
     // serving
     std::mutex mu;
-    std::condition_variable cv;
+    std::condition_variable cv;  // a ticket completed
     cudaMemPool_t pool = nullptr;
     std::vector<Slot> slots;
     std::map<uint64_t, std::unique_ptr<Ticket>> tickets;
@@ -493,6 +505,27 @@ cudaEvent_t* profile_events(ssj_ctx* ctx) {
     return evs;
 }
 
+// Places of a host batch's arrays in one device block.
+struct InputLayout {
+    size_t offs, cand, end;  // (probe ids at 0)
+    InputLayout(uint32_t n_probes, uint64_t n_cands) {
+        offs = align256(4ull * std::max<uint32_t>(n_probes, 1));
+        cand = offs + align256(8ull * (n_probes + 1));
+        end = cand + align256(4ull * std::max<uint64_t>(n_cands, 1));
+    }
+};
+
+// Gather a small batch's arrays in h (pinned) and queue their copy to base.
+cudaError_t copy_small_input(const ssj_batch* b, uint64_t n_cands, const InputLayout& at, char* h, char* base,
+                             cudaStream_t s) {
+    if (b->n_probes) {
+        memcpy(h, b->probe_ids, 4ull * b->n_probes);
+        memcpy(h + at.offs, b->cand_offsets, 8ull * (b->n_probes + 1));
+    }
+    if (n_cands) memcpy(h + at.cand, b->cand_ids, 4 * n_cands);
+    return cudaMemcpyAsync(base, h, at.cand + 4 * n_cands, cudaMemcpyHostToDevice, s);
+}
+
 void free_collection(Collection& c) {
     cudaFree(c.d_toks);
     cudaFree(c.d_desc);
@@ -634,6 +667,7 @@ extern "C" ssj_status ssj_create(const ssj_config* config, ssj_ctx** out) {
     cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &threshold);
     ctx->slots.resize(ctx->max_inflight);
     for (auto& s : ctx->slots) {
+        s.wake.reset(new std::condition_variable());
         if (cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking) != cudaSuccess) return SSJ_EDEVICE;
         // the completion threads sleep on their events instead of spinning, so that many
         // slots do not take the host cores the submitting threads need
@@ -664,7 +698,7 @@ extern "C" void ssj_destroy(ssj_ctx* ctx) {
         std::unique_lock<std::mutex> lk(ctx->mu);
         ctx->stopping = true;
     }
-    ctx->cv.notify_all();
+    for (auto& s : ctx->slots) s.wake->notify_all();
     for (auto& s : ctx->slots)
         if (s.completer.joinable()) s.completer.join();
     DeviceGuard g(ctx->device);
@@ -674,6 +708,7 @@ extern "C" void ssj_destroy(ssj_ctx* ctx) {
         cudaStreamDestroy(s.stream);
         cudaEventDestroy(s.ev);
         cudaEventDestroy(s.copied);
+        cudaFreeHost(s.h_in);
         cudaFreeHost(s.h_probe);
         cudaFreeHost(s.h_offs);
         cudaFreeHost(s.h_cand);
@@ -692,6 +727,7 @@ extern "C" void ssj_destroy(ssj_ctx* ctx) {
     cudaFreeHost(ctx->h_count);
     cudaFreeHost(ctx->h_err);
     cudaFreeHost(ctx->h_ctr);
+    cudaFreeHost(ctx->h_in);
     cudaFreeHost(ctx->h_first);
     cudaFreeHost(ctx->h_counts);
     cudaFreeHost(ctx->h_table);
@@ -996,24 +1032,27 @@ extern "C" ssj_status ssj_verify_batch(ssj_ctx* ctx, const ssj_batch* batch, ssj
         a = make_args(ctx, batch, *R, *S, n_cands);
         // device staging: probe ids, offsets, candidates, count, output
         const uint64_t out_cap = count_only ? 0 : std::min<uint64_t>(cap, n_cands);
-        size_t off = 0;
-        const size_t o_probe = off; off += align256(4ull * std::max<uint32_t>(batch->n_probes, 1));
-        const size_t o_offs = off;  off += align256(8ull * (batch->n_probes + 1));
-        const size_t o_cand = off;  off += align256(4ull * std::max<uint64_t>(n_cands, 1));
-        const size_t o_out = off;   off += align256(sizeof(ssj_triple) * std::max<uint64_t>(out_cap, 1));
-        st = ensure_device_buffer(ctx, &ctx->io, &ctx->io_bytes, off);
+        const InputLayout at(batch->n_probes, n_cands);
+        st = ensure_device_buffer(ctx, &ctx->io, &ctx->io_bytes,
+                                  at.end + align256(sizeof(ssj_triple) * std::max<uint64_t>(out_cap, 1)));
         if (st != SSJ_OK) return st;
         char* base = static_cast<char*>(ctx->io);
-        uint32_t* d_probe = reinterpret_cast<uint32_t*>(base + o_probe);
-        uint64_t* d_offs = reinterpret_cast<uint64_t*>(base + o_offs);
-        uint32_t* d_cand = reinterpret_cast<uint32_t*>(base + o_cand);
-        ssj_triple* d_out = reinterpret_cast<ssj_triple*>(base + o_out);
-        if (batch->n_probes) {
+        uint32_t* d_probe = reinterpret_cast<uint32_t*>(base);
+        uint64_t* d_offs = reinterpret_cast<uint64_t*>(base + at.offs);
+        uint32_t* d_cand = reinterpret_cast<uint32_t*>(base + at.cand);
+        ssj_triple* d_out = reinterpret_cast<ssj_triple*>(base + at.end);
+        const bool small = at.end <= kSmallInput;
+        if (small) {
+            st = ensure_pinned(ctx, &ctx->h_in, &ctx->h_in_cap, kSmallInput);
+            if (st != SSJ_OK) return st;
+            CUDA_TRY(ctx, copy_small_input(batch, n_cands, at, ctx->h_in, base, s));
+        }
+        if (batch->n_probes && !small) {
             CUDA_TRY(ctx, cudaMemcpyAsync(d_probe, batch->probe_ids, 4ull * batch->n_probes, cudaMemcpyHostToDevice, s));
             CUDA_TRY(ctx, cudaMemcpyAsync(d_offs, batch->cand_offsets, 8ull * (batch->n_probes + 1),
                                           cudaMemcpyHostToDevice, s));
         }
-        if (n_cands)
+        if (n_cands && !small)
             CUDA_TRY(ctx, cudaMemcpyAsync(d_cand, batch->cand_ids, 4ull * n_cands, cudaMemcpyHostToDevice, s));
         a.single.probe_ids = d_probe;
         a.single.cand_offsets = d_offs;
@@ -1504,7 +1543,7 @@ void completion_loop(ssj_ctx* ctx, int slot) {
         Ticket* t = nullptr;
         {
             std::unique_lock<std::mutex> lk(ctx->mu);
-            ctx->cv.wait(lk, [&] { return ctx->stopping || sl.pending != nullptr; });
+            sl.wake->wait(lk, [&] { return ctx->stopping || sl.pending != nullptr; });
             if (!sl.pending) return;  // stopping with nothing in flight
             t = sl.pending;
         }
@@ -1634,43 +1673,53 @@ extern "C" ssj_status ssj_submit(ssj_ctx* ctx, const ssj_batch* batch, uint64_t*
     char* base = static_cast<char*>(t->d_mem);
     size_t off = 0;
     if (!dev) {
-        // Inputs in pinned memory are copied straight from the caller's arrays,
-        // and the call waits for those copies before it returns; pageable
-        // inputs go through this slot's pinned staging.  Either way the caller
-        // may reuse its arrays once ssj_submit returns.
-        const uint64_t offs_n = batch->n_probes ? batch->n_probes + 1ull : 0;
-        const bool pin_probe = batch->n_probes && is_pinned(batch->probe_ids);
-        const bool pin_offs = offs_n && is_pinned(batch->cand_offsets);
-        const bool pin_cand = n_cands && is_pinned(batch->cand_ids);
-        direct_copy = pin_probe || pin_offs || pin_cand;
-        if ((!pin_probe && (st = ensure_pinned(ctx, &sl.h_probe, &sl.h_probe_cap, std::max<uint64_t>(batch->n_probes, 1))) != SSJ_OK) ||
-            (!pin_offs && (st = ensure_pinned(ctx, &sl.h_offs, &sl.h_offs_cap, batch->n_probes + 1ull)) != SSJ_OK) ||
-            (!pin_cand && (st = ensure_pinned(ctx, &sl.h_cand, &sl.h_cand_cap, std::max<uint64_t>(n_cands, 1))) != SSJ_OK)) {
-            cudaFreeAsync(t->d_mem, s);
-            return unreserve(st);
+        // Small inputs are gathered in this slot's pinned memory.  Larger ones in pinned memory are
+        // copied straight from the caller's arrays, and the call waits for those copies before it
+        // returns; pageable ones go through the slot's pinned staging.  Either way the caller may
+        // reuse its arrays once ssj_submit returns.
+        const InputLayout at(batch->n_probes, n_cands);
+        uint32_t* d_probe = reinterpret_cast<uint32_t*>(base);
+        uint64_t* d_offs = reinterpret_cast<uint64_t*>(base + at.offs);
+        uint32_t* d_cand = reinterpret_cast<uint32_t*>(base + at.cand);
+        off = at.end;
+        if (at.end <= kSmallInput) {
+            if ((st = ensure_pinned(ctx, &sl.h_in, &sl.h_in_cap, kSmallInput)) != SSJ_OK) {
+                cudaFreeAsync(t->d_mem, s);
+                return unreserve(st);
+            }
+            e = copy_small_input(batch, n_cands, at, sl.h_in, base, s);
+        } else {
+            const uint64_t offs_n = batch->n_probes ? batch->n_probes + 1ull : 0;
+            const bool pin_probe = batch->n_probes && is_pinned(batch->probe_ids);
+            const bool pin_offs = offs_n && is_pinned(batch->cand_offsets);
+            const bool pin_cand = n_cands && is_pinned(batch->cand_ids);
+            direct_copy = pin_probe || pin_offs || pin_cand;
+            if ((!pin_probe && (st = ensure_pinned(ctx, &sl.h_probe, &sl.h_probe_cap, std::max<uint64_t>(batch->n_probes, 1))) != SSJ_OK) ||
+                (!pin_offs && (st = ensure_pinned(ctx, &sl.h_offs, &sl.h_offs_cap, batch->n_probes + 1ull)) != SSJ_OK) ||
+                (!pin_cand && (st = ensure_pinned(ctx, &sl.h_cand, &sl.h_cand_cap, std::max<uint64_t>(n_cands, 1))) != SSJ_OK)) {
+                cudaFreeAsync(t->d_mem, s);
+                return unreserve(st);
+            }
+            const void* src_probe = batch->probe_ids;
+            const void* src_offs = batch->cand_offsets;
+            const void* src_cand = batch->cand_ids;
+            if (batch->n_probes && !pin_probe) {
+                staged_copy(sl.h_probe, batch->probe_ids, 4ull * batch->n_probes);
+                src_probe = sl.h_probe;
+            }
+            if (offs_n && !pin_offs) {
+                staged_copy(sl.h_offs, batch->cand_offsets, 8ull * offs_n);
+                src_offs = sl.h_offs;
+            }
+            if (n_cands && !pin_cand) {
+                staged_copy(sl.h_cand, batch->cand_ids, 4ull * n_cands);
+                src_cand = sl.h_cand;
+            }
+            if (batch->n_probes) e = cudaMemcpyAsync(d_probe, src_probe, 4ull * batch->n_probes, cudaMemcpyHostToDevice, s);
+            if (e == cudaSuccess && offs_n) e = cudaMemcpyAsync(d_offs, src_offs, 8ull * offs_n, cudaMemcpyHostToDevice, s);
+            if (e == cudaSuccess && n_cands) e = cudaMemcpyAsync(d_cand, src_cand, 4ull * n_cands, cudaMemcpyHostToDevice, s);
+            if (e == cudaSuccess && direct_copy) e = cudaEventRecord(sl.copied, s);
         }
-        const void* src_probe = batch->probe_ids;
-        const void* src_offs = batch->cand_offsets;
-        const void* src_cand = batch->cand_ids;
-        if (batch->n_probes && !pin_probe) {
-            staged_copy(sl.h_probe, batch->probe_ids, 4ull * batch->n_probes);
-            src_probe = sl.h_probe;
-        }
-        if (offs_n && !pin_offs) {
-            staged_copy(sl.h_offs, batch->cand_offsets, 8ull * offs_n);
-            src_offs = sl.h_offs;
-        }
-        if (n_cands && !pin_cand) {
-            staged_copy(sl.h_cand, batch->cand_ids, 4ull * n_cands);
-            src_cand = sl.h_cand;
-        }
-        uint32_t* d_probe = reinterpret_cast<uint32_t*>(base + off); off += align256(4ull * std::max<uint32_t>(batch->n_probes, 1));
-        uint64_t* d_offs = reinterpret_cast<uint64_t*>(base + off);  off += align256(8ull * (batch->n_probes + 1));
-        uint32_t* d_cand = reinterpret_cast<uint32_t*>(base + off);  off += align256(4ull * std::max<uint64_t>(n_cands, 1));
-        if (batch->n_probes) e = cudaMemcpyAsync(d_probe, src_probe, 4ull * batch->n_probes, cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess && offs_n) e = cudaMemcpyAsync(d_offs, src_offs, 8ull * offs_n, cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess && n_cands) e = cudaMemcpyAsync(d_cand, src_cand, 4ull * n_cands, cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess && direct_copy) e = cudaEventRecord(sl.copied, s);
         if (e != cudaSuccess) {
             cudaStreamSynchronize(s);  // no copy may still read the caller's arrays
             cudaFreeAsync(t->d_mem, s);
@@ -1720,7 +1769,7 @@ extern "C" ssj_status ssj_submit(ssj_ctx* ctx, const ssj_batch* batch, uint64_t*
     sl.pending = raw;
     *ticket = raw->id;
     lk.unlock();
-    ctx->cv.notify_all();
+    sl.wake->notify_one();
     return SSJ_OK;
 }
 
