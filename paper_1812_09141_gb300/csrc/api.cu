@@ -180,7 +180,7 @@ struct ssj_ctx {
     // device staging for synchronous host-pointer calls
     void* io = nullptr;
     size_t io_bytes = 0;
-    uint64_t* h_count = nullptr;  // pinned
+    uint64_t* h_count = nullptr;  // pinned, two words
     uint32_t* h_err = nullptr;    // pinned
     Counters* h_ctr = nullptr;    // pinned
     // pinned: results that come back with their count (kFirstResults; ssj_verify_batches:
@@ -536,6 +536,8 @@ void free_collection(Collection& c) {
 // stream: it stays in the pool (up to the pool's release threshold, the
 // serving budget) instead of being mapped and unmapped by every call (a dozen
 // cudaMalloc and cudaFree took about 1 ms), and goes back with the context.
+// An allocation from the pool still takes several microseconds: arrays whose
+// sizes are known together are carved out of one (block, then get).
 class CallMemory {
 public:
     explicit CallMemory(ssj_ctx* c) : ctx_(c) {}
@@ -544,22 +546,40 @@ public:
     }
     CallMemory(const CallMemory&) = delete;
     CallMemory& operator=(const CallMemory&) = delete;
+    // What get takes of a block for n elements.
     template <class T>
-    T* get(uint64_t n) {
+    static size_t room(uint64_t n) {
+        return align256(std::max<size_t>(n * sizeof(T), 16));
+    }
+    // One allocation for the next get calls (the rest of the last one is not used any more).
+    void block(size_t bytes) {
         void* m = nullptr;
-        if (cudaMallocFromPoolAsync(&m, std::max<size_t>(n * sizeof(T), 16), ctx_->pool, ctx_->stream) != cudaSuccess) {
+        at_ = end_ = nullptr;
+        if (cudaMallocFromPoolAsync(&m, bytes, ctx_->pool, ctx_->stream) != cudaSuccess) {
             cudaGetLastError();
             failed_ = true;
-            return nullptr;
+            return;
         }
         mem_.push_back(m);
-        return static_cast<T*>(m);
+        at_ = static_cast<char*>(m);
+        end_ = at_ + bytes;
+    }
+    template <class T>
+    T* get(uint64_t n) {
+        if (failed_) return nullptr;
+        if (room<T>(n) > (size_t)(end_ - at_)) block(room<T>(n));
+        if (failed_) return nullptr;
+        T* m = reinterpret_cast<T*>(at_);
+        at_ += room<T>(n);
+        return m;
     }
     bool ok() const { return !failed_; }
 
 private:
     ssj_ctx* ctx_;
     std::vector<void*> mem_;
+    char* at_ = nullptr;
+    char* end_ = nullptr;
     bool failed_ = false;
 };
 
@@ -654,7 +674,7 @@ extern "C" ssj_status ssj_create(const ssj_config* config, ssj_ctx** out) {
         if (cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking) != cudaSuccess) return SSJ_EDEVICE;
         ctx->own_stream = true;
     }
-    if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_count), sizeof(uint64_t)) != cudaSuccess) return SSJ_EDEVICE;
+    if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_count), 2 * sizeof(uint64_t)) != cudaSuccess) return SSJ_EDEVICE;
     if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_err), sizeof(uint32_t)) != cudaSuccess) return SSJ_EDEVICE;
     if (cudaMallocHost(reinterpret_cast<void**>(&ctx->h_ctr), sizeof(Counters)) != cudaSuccess) return SSJ_EDEVICE;
     cudaMemPoolProps props;
@@ -1292,11 +1312,15 @@ extern "C" ssj_status ssj_self_join(ssj_ctx* ctx, ssj_coll coll, uint32_t p, uin
     CandgenIndex ix;
     const uint64_t cells = candgen_cells(C.vocab);
     const uint64_t scan_n = std::max<uint64_t>((uint64_t)C.max_len + 2, cells + 1);
-    ix.size_hist = mem.get<uint64_t>((uint64_t)C.max_len + 2);
+    const uint64_t toff_at = candgen_toff_at(C.max_len);
+    mem.block(CallMemory::room<uint64_t>(toff_at + cells + 1) + 2 * CallMemory::room<uint32_t>(n) +
+              CallMemory::room<uint64_t>(cells + 1) + CallMemory::room<uint64_t>(scan_scratch_words(scan_n)) +
+              CallMemory::room<uint64_t>(1));
+    ix.size_hist = mem.get<uint64_t>(toff_at + cells + 1);
+    ix.toff = ix.size_hist + toff_at;
     ix.probes = mem.get<uint32_t>(n);
     ix.rank = mem.get<uint32_t>(n);
     ix.tcnt = mem.get<uint64_t>(cells + 1);
-    ix.toff = mem.get<uint64_t>(cells + 1);
     ix.scan_scratch = mem.get<uint64_t>(scan_scratch_words(scan_n));
     ix.total = mem.get<uint64_t>(1);
     if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "candidate generation index");
@@ -1423,16 +1447,22 @@ extern "C" ssj_status ssj_verify_groups(ssj_ctx* ctx, const ssj_group_batch* gb,
     x.q = gb->q;
     x.n_groups = gb->n_groups;
     x.n_probe_groups = gb->n_probe_groups;
+    const uint64_t scan_words = 2 * scan_scratch_words(n_entries + 1);
+    mem.block(CallMemory::room<uint64_t>((uint64_t)gb->n_groups + 1) + CallMemory::room<uint32_t>(n_members) +
+              CallMemory::room<uint32_t>(gb->n_probe_groups) +
+              CallMemory::room<uint64_t>((uint64_t)gb->n_probe_groups + 1) + CallMemory::room<uint32_t>(n_cg) +
+              CallMemory::room<uint64_t>(2 * (n_entries + 1)) + CallMemory::room<uint64_t>(n_entries) +
+              CallMemory::room<uint64_t>(scan_words) + CallMemory::room<uint64_t>(2));
     uint64_t* d_goff = mem.get<uint64_t>((uint64_t)gb->n_groups + 1);
     uint32_t* d_mem = mem.get<uint32_t>(n_members);
     uint32_t* d_pg = mem.get<uint32_t>(gb->n_probe_groups);
     uint64_t* d_coff = mem.get<uint64_t>((uint64_t)gb->n_probe_groups + 1);
     uint32_t* d_cg = mem.get<uint32_t>(n_cg);
-    x.probe_off = mem.get<uint64_t>(n_entries + 1);
-    x.pair_off = mem.get<uint64_t>(n_entries + 1);
-    x.per_probe = mem.get<uint64_t>(n_entries + 1);
-    x.scan_scratch = mem.get<uint64_t>(scan_scratch_words(n_entries + 1));
-    x.total = mem.get<uint64_t>(1);
+    x.probe_off = mem.get<uint64_t>(2 * (n_entries + 1));
+    x.pair_off = x.probe_off + n_entries + 1;
+    x.per_probe = mem.get<uint64_t>(n_entries);
+    x.scan_scratch = mem.get<uint64_t>(scan_words);
+    x.total = mem.get<uint64_t>(2);
     if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "group expansion");
     cudaError_t e = cudaMemcpyAsync(d_goff, gb->group_offsets, 8ull * (gb->n_groups + 1), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess && n_members) e = cudaMemcpyAsync(d_mem, gb->members, 4ull * n_members, cudaMemcpyHostToDevice, s);
@@ -1447,19 +1477,23 @@ extern "C" ssj_status ssj_verify_groups(ssj_ctx* ctx, const ssj_group_batch* gb,
     x.probe_groups = d_pg;
     x.cand_offsets = d_coff;
     x.cand_groups = d_cg;
-    uint64_t words[2] = {0, 0};
     x.stage = 0;
-    if (e == cudaSuccess) e = expand_groups(x, s, ctx->num_sms, words);
+    if (e == cudaSuccess) e = expand_groups(x, s, ctx->num_sms, ctx->h_count);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "group expansion (count)");
-    const uint64_t probes = words[0], pairs = words[1];
+    const uint64_t probes = ctx->h_count[0], pairs = ctx->h_count[1];
     if (n_pairs) *n_pairs = pairs;
     if (probes > 0xFFFFFFFFull) return fail(ctx, SSJ_EINVAL, "too many expanded probes");
+    const bool count_only = (gb->flags & SSJ_COUNT_ONLY) != 0;
+    const bool dev_out = (gb->flags & SSJ_DEVICE_PTRS) != 0;
+    const uint64_t out_room = count_only || dev_out ? 0 : std::max<uint64_t>(std::min<uint64_t>(cap, pairs), 1);
+    mem.block(CallMemory::room<uint32_t>(probes) + CallMemory::room<uint64_t>(probes + 1) +
+              CallMemory::room<uint32_t>(pairs) + (out_room ? CallMemory::room<ssj_triple>(out_room) : 0));
     x.probe_ids = mem.get<uint32_t>(probes);
     x.cand_offsets_out = mem.get<uint64_t>(probes + 1);
     x.cand_ids = mem.get<uint32_t>(pairs);
     if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "expanded candidates (%llu pairs)", (unsigned long long)pairs);
     x.stage = 1;
-    e = expand_groups(x, s, ctx->num_sms, words);
+    e = expand_groups(x, s, ctx->num_sms, nullptr);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "group expansion (write)");
     ssj_batch b;
     memset(&b, 0, sizeof(b));
@@ -1468,8 +1502,6 @@ extern "C" ssj_status ssj_verify_groups(ssj_ctx* ctx, const ssj_group_batch* gb,
     b.q = gb->q;
     b.n_probes = (uint32_t)probes;
     b.flags = gb->flags & ~SSJ_DEVICE_PTRS;
-    const bool count_only = (gb->flags & SSJ_COUNT_ONLY) != 0;
-    const bool dev_out = (gb->flags & SSJ_DEVICE_PTRS) != 0;
     if (probes >= (1u << 31) || pairs >= kMaxCands) return fail(ctx, SSJ_EINVAL, "too many expanded pairs");
     VerifyArgs a = make_args(ctx, &b, *R, *S, pairs);
     a.single.probe_ids = x.probe_ids;
@@ -1477,7 +1509,7 @@ extern "C" ssj_status ssj_verify_groups(ssj_ctx* ctx, const ssj_group_batch* gb,
     a.single.cand_ids = x.cand_ids;
     if (!count_only) {
         a.single.cap = dev_out ? cap : std::min<uint64_t>(cap, pairs);
-        a.single.out = dev_out ? out : mem.get<ssj_triple>(std::max<uint64_t>(a.single.cap, 1));
+        a.single.out = dev_out ? out : mem.get<ssj_triple>(out_room);
         if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "group join output");
     }
     return run_batch(ctx, a, (uint32_t)probes, pairs, dev_out || count_only ? nullptr : out, cap, n_out);

@@ -501,6 +501,7 @@ __global__ void group_count_kernel(Params P, GroupArgs G, uint64_t* n_probes, ui
     const int lane = threadIdx.x & 31;
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t n_entries = G.n_probe_groups + G.n_groups;
+    if (blockIdx.x == 0 && threadIdx.x == 0) n_probes[n_entries] = n_pairs[n_entries] = 0;  // the scans' closing entries
     for (uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n_entries; k += warps) {
         uint64_t probes = 0, pairs = 0, sum = 0;
         if (k < G.n_probe_groups) {
@@ -537,6 +538,7 @@ __global__ void group_write_kernel(GroupArgs G, const uint64_t* probe_off, const
     const int lane = threadIdx.x & 31;
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t n_entries = G.n_probe_groups + G.n_groups;
+    if (blockIdx.x == 0 && threadIdx.x == 0) cand_offsets[probe_off[n_entries]] = pair_off[n_entries];
     for (uint32_t k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < n_entries; k += warps) {
         const uint64_t p0 = probe_off[k], np = probe_off[k + 1] - p0, c0 = pair_off[k];
         if (np == 0) continue;
@@ -594,8 +596,7 @@ cudaError_t candgen_run(const CandgenInput& in, cudaStream_t st, int num_sms, Ca
     const unsigned tb = 256;
     if (in.stage == 0) {
         // order by size, then count prefix tokens
-        e = cudaMemsetAsync(ix->size_hist, 0, 8ull * (in.max_len + 2), st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(ix->toff, 0, 8ull * (cells + 1), st);
+        e = cudaMemsetAsync(ix->size_hist, 0, 8ull * (candgen_toff_at(in.max_len) + cells + 1), st);
         if (e != cudaSuccess) return e;
         if (in.n) {
             const uint32_t per = std::max<uint32_t>((in.n + 2 * (uint32_t)num_sms - 1) / (2 * (uint32_t)num_sms), 1024u);
@@ -689,29 +690,18 @@ cudaError_t expand_groups(const GroupExpand& x, cudaStream_t st, int num_sms, ui
     G.n_probe_groups = x.n_probe_groups;
     const uint64_t n_entries = (uint64_t)x.n_groups + x.n_probe_groups;
     const unsigned tb = 256;
-    cudaError_t e;
+    const unsigned blocks = grid_for(32 * (n_entries + 1), tb, num_sms, 8);
     if (x.stage == 0) {
-        e = cudaMemsetAsync(x.probe_off + n_entries, 0, 8, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(x.pair_off + n_entries, 0, 8, st);
-        if (e != cudaSuccess) return e;
-        if (n_entries)
-            group_count_kernel<<<grid_for(32 * n_entries, tb, num_sms, 8), tb, 0, st>>>(P, G, x.probe_off, x.pair_off,
-                                                                                         x.per_probe);
-        e = exclusive_scan_u64(x.probe_off, n_entries + 1, x.scan_scratch, x.total, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(host_words, x.total, 8, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = exclusive_scan_u64(x.pair_off, n_entries + 1, x.scan_scratch, x.total, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(host_words + 1, x.total, 8, cudaMemcpyDeviceToHost, st);
+        group_count_kernel<<<blocks, tb, 0, st>>>(P, G, x.probe_off, x.pair_off, x.per_probe);
+        cudaError_t e = exclusive_scan_u64(x.probe_off, n_entries + 1, x.scan_scratch, x.total, st, nullptr, 2,
+                                           x.pair_off - x.probe_off);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(host_words, x.total, 16, cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) return e;
         return cudaStreamSynchronize(st);  // host_words: expanded probes, expanded pairs
     }
-    if (n_entries)
-        group_write_kernel<<<grid_for(32 * n_entries, tb, num_sms, 8), tb, 0, st>>>(G, x.probe_off, x.pair_off,
-                                                                                     x.per_probe, x.probe_ids,
-                                                                                     x.cand_offsets_out, x.cand_ids);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    // closing offset: the total number of pairs
-    return cudaMemcpyAsync(x.cand_offsets_out + host_words[0], x.pair_off + n_entries, 8, cudaMemcpyDeviceToDevice, st);
+    group_write_kernel<<<blocks, tb, 0, st>>>(G, x.probe_off, x.pair_off, x.per_probe, x.probe_ids, x.cand_offsets_out,
+                                              x.cand_ids);
+    return cudaGetLastError();
 }
 
 }  // namespace ssj

@@ -9,7 +9,7 @@
 // Steps, all on the device after one host-to-device copy of the raw
 // offsets and tokens:
 //   1. len_kernel   - per set: length, 16-byte chunk count, sortedness check
-//   2. scan         - exclusive prefix sum of chunk counts (three kernels)
+//   2. scan         - exclusive prefix sum of chunk counts (two or three kernels)
 //   3. scatter_kernel - one warp per set copies its tokens and the padding
 //   4. record_kernel  - one warp per set: its length, signature and loss
 #include <algorithm>
@@ -22,7 +22,8 @@ namespace ssj {
 
 namespace {
 
-constexpr int kScanBlock = 1024;
+constexpr int kScanBlock = 1024;             // threads of a scan block
+constexpr int kScanTile = 4 * kScanBlock;    // and the values that it sums
 
 __global__ void len_kernel(const uint64_t* __restrict__ offs, const uint32_t* __restrict__ toks, uint32_t n,
                            int validate, uint64_t* __restrict__ chunks, uint32_t* __restrict__ err) {
@@ -67,19 +68,34 @@ __device__ uint64_t block_inclusive_scan(uint64_t v, uint64_t* sh) {
     return v;
 }
 
-// in-place exclusive scan per block; block totals to sums[blockIdx.x]
-__global__ void scan_blocks(uint64_t* data, uint64_t n, uint64_t* sums) {
+// in-place exclusive scan per tile; tile totals to sums[blockIdx.x].  blockIdx.y: the array (scanned
+// arrays lie `stride` apart).
+__global__ void __launch_bounds__(kScanBlock) scan_blocks(uint64_t* data, uint64_t n, uint64_t stride, uint64_t* sums) {
     __shared__ uint64_t sh[32];
-    const uint64_t i = (uint64_t)blockIdx.x * kScanBlock + threadIdx.x;
-    const uint64_t v = i < n ? data[i] : 0;
-    const uint64_t inc = block_inclusive_scan(v, sh);
-    if (i < n) data[i] = inc - v;
+    data += blockIdx.y * stride;
+    sums += (uint64_t)blockIdx.y * gridDim.x;
+    const uint64_t i = (uint64_t)blockIdx.x * kScanTile + 4 * threadIdx.x;
+    uint64_t v[4], sum = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        v[k] = i + k < n ? data[i + k] : 0;
+        sum += v[k];
+    }
+    const uint64_t inc = block_inclusive_scan(sum, sh);
+    uint64_t at = inc - sum;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (i + k < n) data[i + k] = at;
+        at += v[k];
+    }
     if (threadIdx.x == kScanBlock - 1) sums[blockIdx.x] = inc;
 }
 
 // exclusive scan of the block totals by one block, looping over tiles
 __global__ void scan_sums(uint64_t* sums, uint64_t n, uint64_t* total) {
     __shared__ uint64_t sh[32];
+    sums += blockIdx.y * n;
+    total += blockIdx.y;
     uint64_t carry = 0;
     for (uint64_t base = 0; base < n; base += kScanBlock) {
         const uint64_t i = base + threadIdx.x;
@@ -95,12 +111,35 @@ __global__ void scan_sums(uint64_t* sums, uint64_t n, uint64_t* total) {
     if (threadIdx.x == 0) *total = carry;
 }
 
-__global__ void scan_add(uint64_t* data, uint64_t n, const uint64_t* sums, uint64_t* copy) {
-    const uint64_t i = (uint64_t)blockIdx.x * kScanBlock + threadIdx.x;
-    if (i >= n) return;
-    const uint64_t v = data[i] + sums[blockIdx.x];
-    data[i] = v;
-    if (copy) copy[i] = v;
+// Add to a tile what the tiles before it sum to: sums[blockIdx.x] after scan_sums, or (total given)
+// the sum of the totals before it, which the block forms itself, the last one the array's total too.
+// Up to kScanBlock tiles the second way costs a load and a reduction per block in place of a launch.
+__global__ void __launch_bounds__(kScanBlock) scan_add(uint64_t* data, uint64_t n, uint64_t stride,
+                                                       const uint64_t* sums, uint64_t* total, uint64_t* copy) {
+    __shared__ uint64_t sh[32];
+    data += blockIdx.y * stride;
+    sums += (uint64_t)blockIdx.y * gridDim.x;
+    uint64_t before;
+    if (total) {
+        __shared__ uint64_t all;
+        const uint64_t inc = block_inclusive_scan(threadIdx.x < blockIdx.x ? sums[threadIdx.x] : 0, sh);
+        if (threadIdx.x == kScanBlock - 1) {
+            all = inc;
+            if (blockIdx.x == gridDim.x - 1) total[blockIdx.y] = inc + sums[blockIdx.x];
+        }
+        __syncthreads();
+        before = all;
+    } else {
+        before = sums[blockIdx.x];
+    }
+    const uint64_t i = (uint64_t)blockIdx.x * kScanTile + threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < kScanTile; k += kScanBlock) {
+        if (i + k >= n) return;
+        const uint64_t v = data[i + k] + before;
+        data[i + k] = v;
+        if (copy) copy[i + k] = v;
+    }
 }
 
 // one warp per set: tokens to their 16-byte aligned slot, padding after
@@ -167,27 +206,20 @@ cudaError_t build_records(const uint4* toks4, const uint2* desc, uint32_t n, uin
 
 // Build the padded device layout from raw device copies of offsets/tokens.
 // Returns the number of 16-byte chunks via *n_chunks (host), after a sync.
-// scratch must hold (n + 1) + ceil(n/1024) + 1 uint64 values.
+// scratch must hold layout_scratch_words(n) uint64 values.
 cudaError_t layout_lengths(const uint64_t* d_offs, const uint32_t* d_toks, uint32_t n, int validate,
                            uint64_t* d_scratch, uint32_t* d_err, uint64_t* n_chunks_host, cudaStream_t st,
                            int num_sms) {
     uint64_t* chunks = d_scratch;
-    const uint64_t nb = (n + kScanBlock - 1) / kScanBlock;
     uint64_t* sums = d_scratch + n + 1;
-    uint64_t* total = sums + nb;
+    uint64_t* total = sums + (n + kScanTile - 1) / kScanTile;
     cudaError_t e = cudaMemsetAsync(d_err, 0, sizeof(uint32_t), st);
     if (e != cudaSuccess) return e;
     if (n > 0) {
         unsigned blocks = (unsigned)std::min<uint64_t>((n + 255) / 256, (uint64_t)num_sms * 8);
         len_kernel<<<blocks, 256, 0, st>>>(d_offs, d_toks, n, validate, chunks, d_err);
-        scan_blocks<<<(unsigned)nb, kScanBlock, 0, st>>>(chunks, n, sums);
-        scan_sums<<<1, kScanBlock, 0, st>>>(sums, nb, total);
-        scan_add<<<(unsigned)nb, kScanBlock, 0, st>>>(chunks, n, sums, nullptr);
-    } else {
-        e = cudaMemsetAsync(total, 0, sizeof(uint64_t), st);
-        if (e != cudaSuccess) return e;
     }
-    e = cudaGetLastError();
+    e = exclusive_scan_u64(chunks, n, sums, total, st);
     if (e != cudaSuccess) return e;
     e = cudaMemcpyAsync(n_chunks_host, total, sizeof(uint64_t), cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return e;
@@ -203,18 +235,20 @@ cudaError_t layout_scatter(const uint64_t* d_offs, const uint32_t* d_toks, uint3
 }
 
 size_t layout_scratch_words(uint32_t n) {
-    return (size_t)n + 1 + (n + kScanBlock - 1) / kScanBlock + 1;
+    return (size_t)n + 1 + scan_scratch_words(n) + 1;
 }
 
-size_t scan_scratch_words(uint64_t n) { return (n + kScanBlock - 1) / kScanBlock + 1; }
+size_t scan_scratch_words(uint64_t n) { return (n + kScanTile - 1) / kScanTile; }
 
 cudaError_t exclusive_scan_u64(uint64_t* data, uint64_t n, uint64_t* scratch, uint64_t* total, cudaStream_t st,
-                               uint64_t* copy) {
-    if (n == 0) return cudaMemsetAsync(total, 0, sizeof(uint64_t), st);
-    const uint64_t nb = (n + kScanBlock - 1) / kScanBlock;
-    scan_blocks<<<(unsigned)nb, kScanBlock, 0, st>>>(data, n, scratch);
-    scan_sums<<<1, kScanBlock, 0, st>>>(scratch, nb, total);
-    scan_add<<<(unsigned)nb, kScanBlock, 0, st>>>(data, n, scratch, copy);
+                               uint64_t* copy, uint32_t arrays, uint64_t stride) {
+    if (n == 0) return cudaMemsetAsync(total, 0, sizeof(uint64_t) * arrays, st);
+    const uint64_t nb = scan_scratch_words(n);
+    const dim3 grid((unsigned)nb, arrays);
+    const bool sums = nb > kScanBlock;
+    scan_blocks<<<grid, kScanBlock, 0, st>>>(data, n, stride, scratch);
+    if (sums) scan_sums<<<dim3(1, arrays), kScanBlock, 0, st>>>(scratch, nb, total);
+    scan_add<<<grid, kScanBlock, 0, st>>>(data, n, stride, scratch, sums ? nullptr : total, copy);
     return cudaGetLastError();
 }
 

@@ -245,18 +245,20 @@ cudaError_t sort_triples(ssj_triple* t, uint64_t n, ssj_triple* tmp, cudaStream_
 cudaError_t build_records(const uint4* toks4, const uint2* desc, uint32_t n, uint32_t c, uint4* rec, cudaStream_t st,
                           int num_sms);
 
-// Exclusive prefix sum of n 64-bit values in place on st; *total (device)
-// receives the sum.  scratch holds scan_scratch_words(n) values.
+// Exclusive prefix sums of n 64-bit values each of `arrays` arrays, the k-th at
+// data + k * stride, in place on st; total[k] (device) receives the sum.
+// scratch holds arrays * scan_scratch_words(n) values.  copy (optional, one
+// array) receives the sums too.
 size_t scan_scratch_words(uint64_t n);
-// copy (optional) receives the sums too.
 cudaError_t exclusive_scan_u64(uint64_t* data, uint64_t n, uint64_t* scratch, uint64_t* total, cudaStream_t st,
-                               uint64_t* copy = nullptr);
+                               uint64_t* copy = nullptr, uint32_t arrays = 1, uint64_t stride = 0);
 
 // Self-join on the device (candgen.cu).  Scratch of the prefix index, sized by
-// the caller: size_hist max_len + 2 words, probes and rank n each, tcnt and
-// toff candgen_cells + 1 words each, scan_scratch
+// the caller: size_hist max_len + 2 words and toff candgen_cells + 1 words, one
+// after the other (toff_at), probes and rank n each, tcnt as toff, scan_scratch
 // scan_scratch_words(max(max_len + 2, candgen_cells + 1)), total 1 word, post
 // candgen_entry_bytes per index entry (known after stage 0).
+inline uint64_t candgen_toff_at(uint32_t max_len) { return ((uint64_t)max_len + 2 + 15) / 16 * 16; }
 struct CandgenIndex {
     uint64_t* size_hist;          // after stage 0: per size, the position after its last set
     uint32_t* probes;             // the sets from the largest down
@@ -325,9 +327,9 @@ size_t join_workspace_bytes(uint32_t n_probes, uint64_t pairs, int num_sms);
 JoinQueue bind_join_workspace(VerifyArgs& a, void* ws, uint32_t n_probes, uint64_t pairs, int num_sms);
 
 // GroupJoin expansion on the device (candgen.cu).  Entries: the probe
-// groups, then every group (pairs inside it).  probe_off / pair_off /
-// per_probe hold n_entries + 1 words; scan_scratch
-// scan_scratch_words(n_entries + 1); total one word.
+// groups, then every group (pairs inside it).  probe_off and pair_off hold
+// n_entries + 1 words each, one after the other; per_probe n_entries;
+// scan_scratch 2 * scan_scratch_words(n_entries + 1); total two words.
 struct GroupExpand {
     const uint4* toks4;
     const uint2* desc;
@@ -350,8 +352,7 @@ struct GroupExpand {
 };
 
 // Stage 0 waits and leaves (expanded probes, expanded pairs) in
-// host_words[0..1] (pinned); stage 1 enqueues the writes (host_words[0]
-// must still hold the probe count).
+// host_words[0..1] (pinned); stage 1 enqueues the writes.
 cudaError_t expand_groups(const GroupExpand& x, cudaStream_t st, int num_sms, uint64_t* host_words);
 
 // One launch of the read-bandwidth probe: `passes` sweeps over bytes (a
