@@ -5,8 +5,8 @@
 // kSortTile triples an instance is queued right after the verify kernel, one
 // CTA per instance, and the host reads count and triples back at once (2,034
 // results: std::sort between two copies took about 100 us).  More results are
-// sorted after the count has come back: tiles by the same code, then passes
-// that merge two runs each.
+// sorted after the count has come back: small tiles by the same code, one pass
+// that merges sixteen of them, then passes that merge two runs each.
 #include <algorithm>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -103,10 +103,45 @@ __global__ void __launch_bounds__(kSortThreads) sort_results_kernel(const Instan
     if (n >= 2 && n <= kSortTile) sort_tile(I.out, I.out, (uint32_t)n, smem);
 }
 
+// Of more triples, tiles of kSmallTile (one a thread: a sort of few triples in one CTA is bound by its
+// instructions, 2,034 take 17 us cold, 4,096 36).
+constexpr uint32_t kSmallTile = kSortThreads;
+constexpr uint32_t kManyRuns = 16;
+
 __global__ void __launch_bounds__(kSortThreads) sort_tiles_kernel(const ssj_triple* src, ssj_triple* dst, uint64_t n) {
     extern __shared__ unsigned long long smem[];
-    const uint64_t at = (uint64_t)blockIdx.x * kSortTile;
-    sort_tile(src + at, dst + at, (uint32_t)min((uint64_t)kSortTile, n - at), smem);
+    const uint64_t at = (uint64_t)blockIdx.x * kSmallTile;
+    sort_tile(src + at, dst + at, (uint32_t)min((uint64_t)kSmallTile, n - at), smem);
+}
+
+// kManyRuns sorted tiles merged into one run from src to dst: a triple's place is its place in its
+// tile and in each of the others, found by searches that run side by side (a warp's triples are
+// neighbours, so its loads share sectors).  7,342 triples: tiles and this pass 27 us cold; tiles
+// of 4,096 and a pass of two runs took 47.
+__global__ void __launch_bounds__(kMergeThreads) merge_tiles_kernel(const ssj_triple* src, ssj_triple* dst, uint64_t n) {
+    const uint64_t i = (uint64_t)blockIdx.x * kMergeThreads + threadIdx.x;
+    if (i >= n) return;
+    const uint64_t base = i / (kManyRuns * kSmallTile) * (kManyRuns * kSmallTile);
+    const uint32_t c = (uint32_t)(i - base) / kSmallTile;
+    const uint32_t m = (uint32_t)min((uint64_t)kManyRuns * kSmallTile, n - base);  // triples of the group
+    const ssj_triple* A = src + base;
+    const ssj_triple t = src[i];
+    const unsigned long long k = key_of(t);
+    uint32_t before[kManyRuns];
+#pragma unroll
+    for (uint32_t s = 0; s < kManyRuns; ++s) before[s] = 0;
+    for (uint32_t step = kSmallTile; step; step >>= 1) {
+#pragma unroll
+        for (uint32_t s = 0; s < kManyRuns; ++s) {
+            // smaller triples of tile s go before this one, and equal ones of an earlier tile
+            const uint32_t p = before[s] + step;
+            if (p <= kSmallTile && s * kSmallTile + p <= m && key_of(A[s * kSmallTile + p - 1]) < k + (s < c)) before[s] = p;
+        }
+    }
+    uint32_t to = (uint32_t)(i - base) - c * kSmallTile;
+#pragma unroll
+    for (uint32_t s = 0; s < kManyRuns; ++s) to += s == c ? 0u : before[s];
+    dst[base + to] = t;
 }
 
 // Runs of `run` sorted triples merged two by two from src to dst.  A CTA writes
@@ -198,14 +233,16 @@ cudaError_t pack_results(const Instance* table, uint32_t n_inst, ssj_triple* pac
 
 cudaError_t sort_triples(ssj_triple* t, uint64_t n, ssj_triple* tmp, cudaStream_t st) {
     if (n < 2) return cudaSuccess;
-    uint32_t passes = 0;
-    for (uint64_t run = kSortTile; run < n; run *= 2) ++passes;
+    uint32_t passes = 1;  // after the tiles
+    for (uint64_t run = kManyRuns * kSmallTile; run < n; run *= 2) ++passes;
     ssj_triple* from = (passes & 1) ? tmp : t;  // the last pass ends in t
     ssj_triple* to = (passes & 1) ? t : tmp;
     const cudaError_t e = allow_sort_smem(sort_tiles_kernel);
     if (e != cudaSuccess) return e;
-    sort_tiles_kernel<<<(unsigned)((n + kSortTile - 1) / kSortTile), kSortThreads, kSortSmem, st>>>(t, from, n);
-    for (uint64_t run = kSortTile; run < n; run *= 2) {
+    sort_tiles_kernel<<<(unsigned)((n + kSmallTile - 1) / kSmallTile), kSortThreads, kSortSmem, st>>>(t, from, n);
+    merge_tiles_kernel<<<(unsigned)((n + kMergeThreads - 1) / kMergeThreads), kMergeThreads, 0, st>>>(from, to, n);
+    std::swap(from, to);
+    for (uint64_t run = kManyRuns * kSmallTile; run < n; run *= 2) {
         merge_runs_kernel<<<(unsigned)((n + kMergeTile - 1) / kMergeTile), kMergeThreads, 0, st>>>(from, to, n, run);
         std::swap(from, to);
     }

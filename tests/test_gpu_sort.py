@@ -1,6 +1,7 @@
 """SSJ_SORTED: results come back sorted by (r, s) at every size where the device sort changes its way
-(one CTA's tile of 4,096, passes of two runs, odd runs) and where the results stop coming along with
-their count (4,096; 16,384 for a group of ssj_verify_batches), through every entry point.  A batch with
+(one CTA's tile of 4,096, small tiles merged by sixteen, passes of two runs, odd runs) and where the
+results stop coming along with their count (4,096; 16,384 for a group of ssj_verify_batches), through every
+entry point.  A batch with
 SSJ_EMIT_ALL lists as many results as it has pairs; repeated pairs are equal triples."""
 import numpy as np
 import pytest
@@ -12,7 +13,8 @@ from paper_1812_09141_gb300 import _build
 
 pytestmark = pytest.mark.gpu
 
-SIZES = [0, 1, 2, 3, 64, 65, 4095, 4096, 4097, 8192, 8193, 12_289, 16_385, 70_000]
+SIZES = [0, 1, 2, 3, 64, 65, 4095, 4096, 4097, 5120, 5121, 8192, 8193, 12_289, 16_383, 16_384, 16_385,
+         32_769, 70_000]
 
 
 @pytest.fixture(scope="module")
