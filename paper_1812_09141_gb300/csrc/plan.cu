@@ -97,15 +97,19 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
     bool bad = false;  // a candidate id is out of range
     uint32_t f = 0;
     while (f < len && n < kPlanFlush) {
-        uint32_t passed = __popc(__ballot_sync(kFull, ends <= f));  // lists of the window that end by f
-        while (passed == 32) {
+        // Lists of the window before the first that ends after f.  (Not the number that end by f: with
+        // offsets that are not nondecreasing, which the probe check reports, the list at that number may
+        // end before f, and no round would be made.)
+        uint32_t m = __ballot_sync(kFull, ends > f);
+        while (m == 0) {  // (list_end is beyond every f from n_probes on)
             window(kb + 32);
-            passed = __popc(__ballot_sync(kFull, ends <= f));
+            m = __ballot_sync(kFull, ends > f);
         }
-        const uint32_t end = min(__shfl_sync(kFull, ends, passed), len);
+        const uint32_t passed0 = __ffs(m) - 1;
+        const uint32_t end = min(__shfl_sync(kFull, ends, passed0), len);
         if (end - f >= kOneProbe || end == len) {
             // ---- rounds of one probe
-            const uint32_t k = kb + passed, r = __shfl_sync(kFull, ids, passed);
+            const uint32_t k = kb + passed0, r = __shfl_sync(kFull, ids, passed0);
             const bool r_ok = r < I.r_n_sets;  // (the probe check reports a bad probe id)
             const uint32_t rk = r_ok ? r : 0u;
             Sector rs;
@@ -134,6 +138,7 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
             }
         } else {
             // ---- a round of several probes
+            uint32_t passed = passed0;
             if (passed && __shfl_sync(kFull, ends, 31) <= f + 31) {  // the window may end before the round does
                 window(kb + passed);
                 passed = 0;

@@ -140,3 +140,30 @@ def test_probes_whose_candidates_all_pass(ctx, size, raw):
         _check(ctx, c, c, h, h, b, 2, 19, 20)
     finally:
         ssj.ssj_unload_collection(ctx, h)
+
+
+@pytest.mark.parametrize("mean", [1, 12, 45, 700])
+@pytest.mark.parametrize("size", [12, 300])
+def test_offsets_that_fall_back_are_an_error(ctx, mean, size):
+    """Offsets that are not nondecreasing, in batches whose chunks take several rounds: the call
+    ends with SSJ_EINVAL (every round must still move on), and a valid batch works afterwards."""
+    rng = np.random.default_rng(10 * mean + size)
+    c = _sets(rng, 100, size, 20 * size)
+    total = 1_000_000
+    offs = np.sort(rng.integers(0, total + 1, total // mean + 1)).astype(np.uint64)
+    offs[0], offs[-1] = 0, total
+    good = synth.Batch(rng.integers(0, c.n, len(offs) - 1).astype(np.uint32), offs,
+                       rng.integers(0, c.n, total).astype(np.uint32))
+    h = ssj.ssj_load_collection(ctx, c.offsets, c.tokens)
+    try:
+        for back in (1, 5, 31, 200):
+            bad = offs.copy()
+            for at in rng.integers(len(offs) // 2, len(offs) - 1, 50):
+                bad[at] = offs[int(at) - back] - 1 if back < 200 else offs[int(at)] // 2
+            assert (np.diff(bad.astype(np.int64)) < 0).any()
+            with pytest.raises(ssj.SsjError) as ei:
+                ssj.ssj_verify_batch(ctx, h, h, 3, 5, good.probe_ids, bad, good.cand_ids)
+            assert ei.value.status == ssj.SSJ_EINVAL
+        _check(ctx, c, c, h, h, good, 0, 19, 20)
+    finally:
+        ssj.ssj_unload_collection(ctx, h)
