@@ -52,9 +52,10 @@ __device__ __forceinline__ uint32_t find_probe(const uint64_t* offs, uint32_t n_
 // Candidates [f0, f1) of an instance, by one warp, 32 at a time; the pairs
 // left go to buf, *n of them, and the position up to which candidates are done
 // is returned: f1, or less when the buffer is full.  (The caller queues them:
-// a call in here would cost the loops their registers.)  The warp holds a window of 32 list ends; rounds within one probe's list keep the
-// probe's record in registers, in the others each lane finds its candidate's
-// probe in the window and reads its record.  G: sectors per record of the
+// a call in here would cost the loops their registers.)  The warp holds a
+// window of 32 list ends; rounds within one probe's list keep the probe's
+// record in registers, in the others each lane finds its candidate's probe in
+// the window and reads its record.  G: sectors per record of the
 // first level, 0 without signatures (the length filter alone).
 template <int G>
 __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0, uint64_t f1, uint2* buf,
