@@ -275,16 +275,18 @@ __device__ __noinline__ void flush_survivors(const VerifyArgs& a, const PlanInst
         *r = I.probe_ids[slot - 32u * I.tile_base];
         return probe_bin(a, I.flags, I.r_desc[*r].y, *e - *h);
     };
-    uint32_t n_long = 0;
+    uint32_t n_long = 0, n_warp = 0;
     for (uint32_t t = 0; t < n; t += 32) {
-        uint32_t h, e, r;
-        const bool is_long = t + lane < n && classify(t + lane, &h, &e, &r) != 0;
-        n_long += __popc(__ballot_sync(kFull, is_long));
+        uint32_t h, e, r, bin = 0;
+        if (t + lane < n) bin = classify(t + lane, &h, &e, &r);
+        n_long += __popc(__ballot_sync(kFull, bin != 0));
+        n_warp += __popc(__ballot_sync(kFull, bin == 1));
     }
     unsigned long long base_s = 0, base_l = 0;
     if (lane == 0) {
         if (n > n_long) base_s = atomicAdd(&a.ctr->thread_pairs, (unsigned long long)(n - n_long));
         if (n_long) base_l = atomicAdd(&a.ctr->long_pairs, (unsigned long long)n_long);
+        if (n_warp) atomicAdd(&a.ctr->warp_pairs, (unsigned long long)n_warp);
     }
     base_s = __shfl_sync(kFull, base_s, 0);
     base_l = __shfl_sync(kFull, base_l, 0);

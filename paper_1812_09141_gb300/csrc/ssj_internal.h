@@ -105,6 +105,7 @@ constexpr uint32_t kInItem = 0x80000000u;  // in s (set ids are below 2^31): a w
 struct Counters {
     unsigned long long thread_pairs;  // short pairs queued at the front of the pair list
     unsigned long long long_pairs;    // other pairs, queued at its back
+    unsigned long long warp_pairs;    // those of them that no work item covers
     unsigned long long warp_items;    // lane work items written by the plan kernel
     unsigned long long block_items;   // block work items written by the plan kernel
     uint32_t block_cursor;            // dynamic cursors of the verify kernel

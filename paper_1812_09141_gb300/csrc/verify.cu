@@ -68,7 +68,8 @@ constexpr uint32_t kWarpBBuf = kWarpWin + 16;      // s window buffer
 constexpr int kBlockD = 8;                         // merge steps per thread per window (block)
 constexpr uint32_t kBlockRCap = 4096;              // r kept whole in shared memory up to this
 constexpr uint32_t kFlatGrab = 4;                  // most 32-pair chunks taken per dynamic grab in phase 3
-constexpr uint32_t kLongGrab = 8;                  // most long pairs taken per dynamic grab in phase 2
+constexpr uint32_t kLongGrab = 8;                  // long pairs taken per dynamic grab in phase 2, about,
+constexpr uint32_t kLongScan = 256;                // and entries of their list read for them, at most
 // Up to this many queued pairs per warp of the grid, short ones too are verified one per warp, dealt
 // out statically: a thread takes about 10 us of dependent loads however few pairs there are (2,034
 // results of short sets: 10 us instead of 17 for the kernel; 48 of the tiny collection: 9 instead of
@@ -922,9 +923,14 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
     const uint32_t n_bs = (uint32_t)min(n_block, (unsigned long long)gridDim.x);
     const uint32_t free2 = n_bs * kWarps;
     const uint32_t slots2 = n_warps_total - free2;
-    // units of the pair lists: few pairs spread over the warps, many go several to a grab
-    const uint32_t long_grab = (uint32_t)max(1ull, min(n_long / (4ull * n_warps_total), (unsigned long long)kLongGrab));
-    const unsigned long long long_units = (n_long + long_grab - 1) / long_grab;
+    // Units of the pair lists: few pairs spread over the warps, many go several to a grab.  Of the long
+    // pairs, those that work items cover are passed over, 32 at a time, so a grab takes the more of them
+    // the fewer the others are (none: no units).  Where all of 1e7 pairs of 20 tokens are in index items
+    // the kernel takes 375 us; 920 with every pair of the list read by itself.
+    const unsigned long long n_lone = min(a.ctr->warp_pairs, n_long);
+    const uint32_t long_grab = (uint32_t)max(
+        1ull, min(n_long / (4ull * n_warps_total), min(kLongGrab * (n_long / max(n_lone, 1ull)), (unsigned long long)kLongScan)));
+    const unsigned long long long_units = n_lone ? (n_long + long_grab - 1) / long_grab : 0;
     const uint32_t freel = free2 + (uint32_t)min(n_warp, (unsigned long long)slots2);
     const uint32_t slotsl = n_warps_total - freel;
     const uint32_t free3 = freel + (uint32_t)min(long_units, (unsigned long long)slotsl);
@@ -1056,7 +1062,7 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
 
     // ---------------- phase 2: lane items, then long pairs, one per warp --
     const bool few = n_long + n_pairs <= (unsigned long long)kFewPairs * n_warps_total;
-    if (n_warp || n_long || (few && n_pairs)) {
+    if (n_warp || n_lone || (few && n_pairs)) {
         WarpOut wout;
         uint32_t* abuf = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(smem) + warp * kWarpSliceBytes);
         uint32_t* bbuf = abuf + kWarpABuf;
@@ -1150,7 +1156,7 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
                 if (!(pr.s & kInItem) && !verify_pair(pr)) return;  // the warp stops
             }
         } else {
-            for (uint32_t round = 0; n_long; ++round) {
+            for (uint32_t round = 0; long_units; ++round) {
                 uint32_t u = 0;
                 if (lane == 0) {
                     if (round == 0 && gwarp >= freel) u = gwarp - freel;
@@ -1160,9 +1166,17 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
                 if (u >= long_units) break;
                 const unsigned long long first = a.pair_cap - n_long + (unsigned long long)u * long_grab;
                 const unsigned long long end = min(first + long_grab, (unsigned long long)a.pair_cap);
-                for (unsigned long long m = first; m < end; ++m) {
-                    const PairRef pr = a.pairs[m];
-                    if (!(pr.s & kInItem) && !verify_pair(pr)) return;  // the warp stops
+                for (unsigned long long m = first; m < end; m += 32) {
+                    PairRef mine;
+                    mine.k = 0;
+                    mine.s = m + lane < end ? 0u : kInItem;
+                    if (m + lane < end) mine = a.pairs[m + lane];
+                    for (uint32_t left = __ballot_sync(kFull, !(mine.s & kInItem)); left; left &= left - 1) {
+                        PairRef pr;
+                        pr.k = __shfl_sync(kFull, mine.k, __ffs(left) - 1);
+                        pr.s = __shfl_sync(kFull, mine.s, __ffs(left) - 1);
+                        if (!verify_pair(pr)) return;  // the warp stops
+                    }
                 }
             }
         }
