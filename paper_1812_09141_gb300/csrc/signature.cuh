@@ -240,82 +240,128 @@ __device__ __forceinline__ uint32_t probe_bin(const VerifyArgs& a, uint32_t flag
     return key <= a.warp_max_key ? 1u : 2u;
 }
 
-// Queue the pairs that the second level leaves of the warp's n buffered ones
-// (probe slot, candidate id), in candidate order (slots ascending).  Short pairs go to the front of the pair list, the others
-// to its back, a probe's pairs side by side; lane, block and index items
-// refer to such a run, and its pairs are marked (kInItem) so that the
-// warp-per-pair phase passes over them.
-__device__ __noinline__ void flush_survivors(const VerifyArgs& a, const PlanInst& I, uint32_t inst, uint2* buf,
-                                             uint32_t n, int lane) {
-    const unsigned lt_mask = (1u << lane) - 1u;
-    switch (I.rec_sectors[1]) {
-        case 2: n = second_level<2>(I, buf, n, lane); break;
-        case 4: n = second_level<4>(I, buf, n, lane); break;
-        case 8: n = second_level<8>(I, buf, n, lane); break;
-        default: break;
+// Work items of one run: n pairs of probe r from pos on in the pair list, of
+// granularity bin (2 to 4), as items first, first + 1, ... of its list.
+__device__ __forceinline__ uint32_t item_pairs(const VerifyArgs& a, uint32_t bin) {
+    return bin == 3 ? a.lane_item_cands : (bin == 4 ? a.index_item_cands : a.block_item_cands);
+}
+__device__ __forceinline__ void write_item(const VerifyArgs& a, uint32_t bin, uint32_t inst, uint32_t r, uint32_t n,
+                                           unsigned long long pos, unsigned long long first, uint32_t it) {
+    const uint32_t per = item_pairs(a, bin);
+    if (first + it >= (bin == 3 ? a.warp_item_cap : a.block_item_cap)) {
+        atomicOr(&a.ctr->err, ERR_GUARD);
+        return;
     }
-    if (n == 0) return;
+    WorkItem wi;
+    wi.r = r;
+    wi.n = min(per, n - it * per);
+    wi.c0 = pos + (uint64_t)it * per;
+    wi.inst = inst;
+    wi.pad = bin >= 3 ? 1u : 0u;
+    (bin == 3 ? a.warp_items : a.block_items)[first + it] = wi;
+}
+
+// Queue the warp's n buffered pairs (probe slot, candidate id; n > 0) in
+// candidate order, a probe's pairs side by side.  Short pairs go to the front
+// of the pair list, the others to its back; lane, block and index items refer
+// to a run of one probe's pairs, and those pairs are marked (kInItem) so that
+// the warp-per-pair phase passes over them.
+//
+// Bound by its instructions where many pairs are left, so a buffer of one run
+// (long lists) is copied straight out, and of several runs the ends come from
+// the windows' head masks and each entry's granularity is looked up once and
+// kept.  (With two binary searches and two dependent loads per entry, twice, the
+// plan kernel took 260 us where 1e7 pairs of lists of 10,000 all pass, now 102,
+// and 178 on 5.6e6 pairs in lists of 30, all kept, now 117.)
+__device__ __noinline__ void queue_pairs(const VerifyArgs& a, const PlanInst& I, uint32_t inst, const uint2* buf,
+                                         uint32_t n, int lane) {
+    static_assert(kPlanBuf <= 16 * 32, "granularities and head masks of 16 windows");
+    const unsigned lt_mask = (1u << lane) - 1u;
     uint32_t* err = &a.ctr->err;
-    // bin of entry i and the run [h, e) of its probe's entries
-    auto classify = [&](uint32_t i, uint32_t* h, uint32_t* e, uint32_t* r) -> uint32_t {
-        const uint32_t slot = buf[i].x;
-        uint32_t lo = 0, hi = i;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (buf[mid].x < slot) lo = mid + 1; else hi = mid;
+    auto probe_of = [&](uint32_t i) -> uint32_t { return I.probe_ids[buf[i].x - 32u * I.tile_base]; };
+    // lane 0 takes room for ns short and nl long pairs (nw of them without an item); false if there is none
+    unsigned long long base_s = 0, base_l = 0;
+    auto reserve = [&](uint32_t ns, uint32_t nl, uint32_t nw) -> bool {
+        if (lane == 0) {
+            if (ns) base_s = atomicAdd(&a.ctr->thread_pairs, (unsigned long long)ns);
+            if (nl) base_l = atomicAdd(&a.ctr->long_pairs, (unsigned long long)nl);
+            if (nw) atomicAdd(&a.ctr->warp_pairs, (unsigned long long)nw);
         }
-        *h = lo;
-        lo = i + 1;
-        hi = n;
-        while (lo < hi) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (buf[mid].x <= slot) lo = mid + 1; else hi = mid;
-        }
-        *e = lo;
-        *r = I.probe_ids[slot - 32u * I.tile_base];
-        return probe_bin(a, I.flags, I.r_desc[*r].y, *e - *h);
+        base_s = __shfl_sync(kFull, base_s, 0);
+        base_l = __shfl_sync(kFull, base_l, 0);
+        // every candidate is queued at most once, so the lists never meet
+        if (base_s + ns <= a.pair_cap && base_l + nl <= a.pair_cap) return true;
+        if (lane == 0) atomicOr(err, ERR_GUARD);
+        return false;
     };
+    auto write_pair = [&](unsigned long long pos, uint2 e, uint32_t bin) {
+        if (!in_bounds(pos, a.pair_cap, err)) return;
+        PairRef pr;
+        pr.k = e.x;
+        pr.s = e.y | (bin >= 2 ? kInItem : 0u);
+        a.pairs[pos] = pr;
+    };
+    if (buf[0].x == buf[n - 1].x) {  // one run (slots ascend)
+        const uint32_t r = probe_of(0), bin = probe_bin(a, I.flags, I.r_desc[r].y, n);
+        if (!reserve(bin ? 0u : n, bin ? n : 0u, bin == 1 ? n : 0u)) return;
+        const unsigned long long pos = bin ? a.pair_cap - base_l - n : base_s;
+        for (uint32_t i = lane; i < n; i += 32) write_pair(pos + i, buf[i], bin);
+        if (bin >= 2) {
+            const uint32_t items = (n + item_pairs(a, bin) - 1) / item_pairs(a, bin);
+            unsigned long long first = 0;
+            if (lane == 0) first = atomicAdd(bin == 3 ? &a.ctr->warp_items : &a.ctr->block_items, (unsigned long long)items);
+            first = __shfl_sync(kFull, first, 0);
+            for (uint32_t it = lane; it < items; it += 32) write_item(a, bin, inst, r, n, pos, first, it);
+        }
+        __syncwarp();
+        return;
+    }
+    uint32_t heads = 0;  // lane w: the entries of window w (32 entries) that begin a run
+    for (uint32_t w = 0; 32 * w < n; ++w) {
+        const uint32_t i = 32 * w + lane;
+        const uint32_t m = __ballot_sync(kFull, i < n && (i == 0 || buf[i - 1].x != buf[i].x));
+        if (lane == (int)w) heads = m;
+    }
+    const uint32_t headed = __ballot_sync(kFull, heads != 0);  // windows with heads (the first is one)
+    // the run [h, e) of entry 32 * w + lane
+    auto run_of = [&](uint32_t w, uint32_t* h, uint32_t* e) {
+        const uint32_t m = __shfl_sync(kFull, heads, w);
+        const uint32_t earlier = (headed & ((1u << w) - 1u)) | 1u, later = headed & (kFull << w << 1);
+        const uint32_t we = 31 - __clz(earlier), wl = later ? __ffs(later) - 1 : 0u;
+        const uint32_t me = __shfl_sync(kFull, heads, we), ml = __shfl_sync(kFull, heads, wl);
+        const uint32_t upto = m & (lt_mask | 1u << lane), past = m & (kFull << lane << 1);
+        *h = upto ? 32 * w + 31 - __clz(upto) : 32 * we + 31 - __clz(me);
+        *e = past ? 32 * w + __ffs(past) - 1 : (later ? 32 * wl + __ffs(ml) - 1 : n);
+    };
+    uint64_t bins = 0;  // 3 bits a window
     uint32_t n_long = 0, n_warp = 0;
-    for (uint32_t t = 0; t < n; t += 32) {
-        uint32_t h, e, r, bin = 0;
-        if (t + lane < n) bin = classify(t + lane, &h, &e, &r);
+#pragma unroll 2
+    for (uint32_t w = 0; 32 * w < n; ++w) {
+        const uint32_t i = 32 * w + lane;
+        uint32_t h, e, bin = 0;
+        run_of(w, &h, &e);
+        if (i < n) bin = probe_bin(a, I.flags, I.r_desc[probe_of(i)].y, e - h);
+        bins |= (uint64_t)bin << (3 * w);
         n_long += __popc(__ballot_sync(kFull, bin != 0));
         n_warp += __popc(__ballot_sync(kFull, bin == 1));
     }
-    unsigned long long base_s = 0, base_l = 0;
-    if (lane == 0) {
-        if (n > n_long) base_s = atomicAdd(&a.ctr->thread_pairs, (unsigned long long)(n - n_long));
-        if (n_long) base_l = atomicAdd(&a.ctr->long_pairs, (unsigned long long)n_long);
-        if (n_warp) atomicAdd(&a.ctr->warp_pairs, (unsigned long long)n_warp);
-    }
-    base_s = __shfl_sync(kFull, base_s, 0);
-    base_l = __shfl_sync(kFull, base_l, 0);
-    // every candidate is queued at most once, so the lists never meet
-    if (base_s + (n - n_long) > a.pair_cap || base_l + n_long > a.pair_cap) {
-        if (lane == 0) atomicOr(err, ERR_GUARD);
-        return;
-    }
+    if (!reserve(n - n_long, n_long, n_warp)) return;
     unsigned long long at_s = base_s, at_l = a.pair_cap - base_l - n_long;
-    for (uint32_t t = 0; t < n; t += 32) {
-        const uint32_t i = t + lane;
-        uint32_t h = 0, e = 0, r = 0, bin = 5;
-        if (i < n) bin = classify(i, &h, &e, &r);
+    for (uint32_t w = 0; 32 * w < n; ++w) {
+        const uint32_t i = 32 * w + lane;
+        uint32_t h, e;
+        run_of(w, &h, &e);
+        const uint32_t bin = i < n ? (uint32_t)(bins >> (3 * w)) & 7u : 5u;
         const uint32_t ms = __ballot_sync(kFull, bin == 0), ml = __ballot_sync(kFull, bin >= 1 && bin <= 4);
         const unsigned long long pos = bin == 0 ? at_s + __popc(ms & lt_mask) : at_l + __popc(ml & lt_mask);
         at_s += __popc(ms);
         at_l += __popc(ml);
-        if (bin <= 4 && in_bounds(pos, a.pair_cap, err)) {
-            PairRef pr;
-            pr.k = buf[i].x;
-            pr.s = buf[i].y | (bin >= 2 ? kInItem : 0u);
-            a.pairs[pos] = pr;
-        }
+        if (bin <= 4) write_pair(pos, buf[i], bin);
         // items, by the first entry of a run
-        const bool head = i < n && i == h;
-        const uint32_t per = bin == 3 ? a.lane_item_cands : (bin == 4 ? a.index_item_cands : a.block_item_cands);
-        const uint32_t items = head && bin >= 2 ? (e - h + per - 1) / per : 0u;
-        uint32_t wn = bin == 3 ? items : 0u, bn = bin == 3 ? 0u : items;
+        const uint32_t items = i < n && i == h && bin >= 2 ? (e - h + item_pairs(a, bin) - 1) / item_pairs(a, bin) : 0u;
         if (__any_sync(kFull, items != 0)) {
+            const uint32_t r = items ? probe_of(i) : 0u;
+            const uint32_t wn = bin == 3 ? items : 0u, bn = bin == 3 ? 0u : items;
             uint32_t wincl = wn, bincl = bn;
 #pragma unroll
             for (int off = 1; off < 32; off <<= 1) {
@@ -329,23 +375,25 @@ __device__ __noinline__ void flush_survivors(const VerifyArgs& a, const PlanInst
             }
             wbase = __shfl_sync(kFull, wbase, 31) + (wincl - wn);
             bbase = __shfl_sync(kFull, bbase, 31) + (bincl - bn);
-            for (uint32_t it = 0; it < items; ++it) {
-                WorkItem wi;
-                wi.r = r;
-                wi.n = min(per, e - h - it * per);
-                wi.c0 = pos + (uint64_t)it * per;
-                wi.inst = inst;
-                wi.pad = bin >= 3 ? 1u : 0u;
-                const unsigned long long q = (bin == 3 ? wbase : bbase) + it;
-                if (q >= (bin == 3 ? a.warp_item_cap : a.block_item_cap)) {
-                    atomicOr(err, ERR_GUARD);
-                    break;
-                }
-                (bin == 3 ? a.warp_items : a.block_items)[q] = wi;
-            }
+            for (uint32_t it = 0; it < items; ++it) write_item(a, bin, inst, r, e - h, pos, bin == 3 ? wbase : bbase, it);
         }
     }
     __syncwarp();
+}
+
+// Queue what the second level leaves of the n buffered pairs.  Mostly that is
+// nothing, so only the queueing is a call (9.2e7 candidates of long sets: plan
+// kernel 961 us; 991 with a function around both, which saves its registers
+// every time).
+__device__ __forceinline__ void flush_survivors(const VerifyArgs& a, const PlanInst& I, uint32_t inst, uint2* buf,
+                                                uint32_t n, int lane) {
+    switch (I.rec_sectors[1]) {
+        case 2: n = second_level<2>(I, buf, n, lane); break;
+        case 4: n = second_level<4>(I, buf, n, lane); break;
+        case 8: n = second_level<8>(I, buf, n, lane); break;
+        default: break;
+    }
+    if (n) queue_pairs(a, I, inst, buf, n, lane);
 }
 
 }  // namespace

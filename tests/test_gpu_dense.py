@@ -39,11 +39,11 @@ def lists(n, probes, each, seed=2):
             torch.randint(0, n, (probes * each,), generator=g, device="cuda", dtype=torch.int32))
 
 
-def kernel_ms(ctx, h, b, flags, reps=9):
+def kernel_ms(ctx, h, b, flags, p=3, q=5, reps=9):
     """Medians (plan, verify) of the kernels' times, and the count."""
     times = []
     for _ in range(reps + 2):
-        n = ssj.ssj_verify_batch(ctx, h, h, 3, 5, *b, n_cands=len(b[2]),
+        n = ssj.ssj_verify_batch(ctx, h, h, p, q, *b, n_cands=len(b[2]),
                                  flags=flags | ssj.SSJ_DEVICE_PTRS | ssj.SSJ_COUNT_ONLY)
         times.append(ssj.ssj_profile_read(ctx)[1:])
     return np.median(np.array(times[2:]), axis=0), int(n)
@@ -61,5 +61,21 @@ def test_pairs_of_work_items_are_passed_over_quickly(ctx, size):
         threads, _ = kernel_ms(ctx, h, b, ssj.SSJ_FORCE_THREAD)
         assert n > 0.99 * len(b[2])
         assert items[1] < 1.9 * threads[1], (items, threads)
+    finally:
+        ssj.ssj_unload_collection(ctx, h)
+
+
+@pytest.mark.parametrize("probes,each", [(500, 10_000), (160_000, 31)])
+def test_queueing_pairs_costs_about_as_much_as_testing_them(ctx, probes, each):
+    """5e6 pairs of 20 tokens that are all queued, against as many that the signature test (a 32-byte
+    record per candidate) drops: a queued pair writes 8 bytes more, so the plan kernel takes less than
+    2.5 times as long (over three times when each pair's run was searched for twice)."""
+    h = cluster(ctx, 20, 20_000)
+    try:
+        b = lists(20_000, probes, each)
+        queued, n = kernel_ms(ctx, h, b, ssj.SSJ_EMIT_ALL)
+        dropped, left = kernel_ms(ctx, h, b, 0, 99, 100)
+        assert n > 0.99 * len(b[2]) and left < 0.01 * len(b[2])
+        assert queued[0] < 2.5 * dropped[0], (queued, dropped)
     finally:
         ssj.ssj_unload_collection(ctx, h)
