@@ -25,17 +25,18 @@ namespace {
 constexpr int kPlanThreads = 256;
 constexpr int kPlanWarps = kPlanThreads / 32;
 constexpr uint32_t kOneProbe = 64;              // candidates of a list worth rounds of their own (32: the same)
+constexpr uint32_t kWalkWindows = 4;            // windows that a round of several probes walks before it searches
 // CTAs per SM the registers are budgeted for (64 each).  With 3 the long sets take 1.09 ms instead of
 // 1.00; with 5 the spills cost more than the warps gain (1.20).  Asking for the next round's records
 // before these are counted costs more registers than it hides latency (1.16 ms with 3 CTAs); more
 // candidate ids asked for ahead change nothing (2 rounds) or cost registers (4: 1.02 ms).
 constexpr int kPlanCtas = 4;
 
-// Largest k with offs[k] <= f, by the whole warp: each step narrows the range
-// [lo, hi) of candidate answers 32-fold with one load per lane.  (Offsets that
-// are not nondecreasing give some k below n_probes.)
-__device__ __forceinline__ uint32_t find_probe(const uint64_t* offs, uint32_t n_probes, uint64_t f, int lane) {
-    uint32_t lo = 0, hi = n_probes;
+// Largest k of [lo, hi) with offs[k] <= f (lo < hi; lo, if offs[lo] is beyond
+// f), by the whole warp: each step narrows the range of candidate answers
+// 32-fold with one load per lane.  (Offsets that are not nondecreasing give
+// some k of the range.)
+__device__ __forceinline__ uint32_t find_probe(const uint64_t* offs, uint32_t lo, uint32_t hi, uint64_t f, int lane) {
     while (hi - lo > 1) {
         const uint32_t step = (hi - lo + 31) / 32;
         const uint64_t at = (uint64_t)lo + (uint64_t)step * lane;
@@ -49,6 +50,22 @@ __device__ __forceinline__ uint32_t find_probe(const uint64_t* offs, uint32_t n_
     return lo;
 }
 
+// The same by one lane for its own f, in steps that double and then a binary
+// search (it is near lo more often than not).
+__device__ __forceinline__ uint32_t find_probe_lane(const uint64_t* offs, uint32_t lo, uint32_t hi, uint64_t f) {
+    uint32_t step = 32;
+    while (step < hi - lo && __ldg(offs + lo + step) <= f) {
+        lo += step;
+        step = min(2 * step, 1u << 30);
+    }
+    hi = min(hi - lo, step) + lo;
+    while (hi - lo > 1) {
+        const uint32_t mid = lo + (hi - lo) / 2;
+        if (__ldg(offs + mid) <= f) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 // Candidates [f0, f1) of an instance, by one warp, 32 at a time; the pairs
 // left go to buf, *n of them, and the position up to which candidates are done
 // is returned: f1, or less when the buffer is full.  (The caller queues them:
@@ -57,6 +74,11 @@ __device__ __forceinline__ uint32_t find_probe(const uint64_t* offs, uint32_t n_
 // record in registers, in the others each lane finds its candidate's probe in
 // the window and reads its record.  G: sectors per record of the
 // first level, 0 without signatures (the length filter alone).
+//
+// The next list is mostly in the window or the one after it.  Beyond those the
+// warp searches for it: a batch may list any number of probes without
+// candidates, and walked window by window 1e7 probes with 1,000 candidates took
+// 6.1 ms a call (now 0.07).
 template <int G>
 __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0, uint64_t f1, uint2* buf,
                                                  uint32_t* n_out, uint32_t* err, int lane) {
@@ -67,7 +89,7 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
     const uint32_t* cands = I.cand_ids + f0;
     // lane l of the window holds probe kb + l: its id, and the end of its list relative to f0 (saturated;
     // the last probe's list ends the batch)
-    uint32_t kb = find_probe(I.cand_offsets, I.n_probes, f0, lane), ends, ids;
+    uint32_t kb = find_probe(I.cand_offsets, 0, I.n_probes, f0, lane), ends, ids;
     auto list_end = [&](uint32_t k) -> uint32_t {
         const uint64_t at = (uint64_t)k + 1 + lane;
         if (at >= I.n_probes) return 0xFFFFFFFFu;
@@ -102,8 +124,8 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
         // offsets that are not nondecreasing, which the probe check reports, the list at that number may
         // end before f, and no round would be made.)
         uint32_t m = __ballot_sync(kFull, ends > f);
-        while (m == 0) {  // (list_end is beyond every f from n_probes on)
-            window(kb + 32);
+        for (bool near = true; m == 0; near = false) {  // (kb + 32 < n_probes: the last list's end is beyond every f)
+            window(near ? kb + 32 : find_probe(I.cand_offsets, kb + 32, I.n_probes, f0 + f, lane));
             m = __ballot_sync(kFull, ends > f);
         }
         const uint32_t passed0 = __ffs(m) - 1;
@@ -156,7 +178,7 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
                 r = __shfl_sync(kFull, ids, at);
             } else {
                 k = kb;
-                for (uint32_t kw = kb, w = ends;;) {
+                for (uint32_t kw = kb, w = ends, windows = 1;; ++windows) {
                     uint32_t lo = 0;  // lists of window kw that end by my
 #pragma unroll
                     for (int step = 16; step >= 1; step >>= 1) {
@@ -167,7 +189,13 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
                     if (lo == 31 && v <= my) lo = 32;
                     if (k == kw) k = kw + lo;
                     kw += 32;
-                    if (!__any_sync(kFull, my < len && k == kw)) break;  // no lane is past this window
+                    const bool beyond = my < len && k == kw;
+                    if (!__any_sync(kFull, beyond)) break;  // no lane is past this window
+                    if (windows == kWalkWindows) {
+                        if (beyond) k = find_probe_lane(I.cand_offsets, kw, I.n_probes, f0 + my);
+                        if (f + 32 < len) window(__shfl_sync(kFull, k, 31));
+                        break;
+                    }
                     w = list_end(kw);
                 }
                 r = k < I.n_probes ? __ldg(I.probe_ids + k) : 0xFFFFFFFFu;
