@@ -461,13 +461,15 @@ void set_chunks(Instance* t, LaunchShape& sh, int num_sms) {
 // The context's granularity policy for a launch whose collections' token
 // values are all below vocab_bound; the probe bitmap of index items is sized
 // when index items are on or a batch forces them (and the values fit).
-void apply_policy(const ssj_ctx* ctx, VerifyArgs& a, uint64_t vocab_bound, bool force_index) {
+// batch_flags: all batches' flags together.
+void apply_policy(const ssj_ctx* ctx, VerifyArgs& a, uint64_t vocab_bound, uint32_t batch_flags) {
     a.thread_max_key = ctx->thread_max_key;
     a.drain_min_live = ctx->drain_min_live;
     a.lane_max_key = ctx->lane_max_key;
     a.warp_max_key = ctx->warp_max_key;
     a.index_min_cands = ctx->index_min_cands;
-    a.index_words = (ctx->index_min_cands || force_index) ? index_words_for(vocab_bound) : 0u;
+    a.index_words = (ctx->index_min_cands || (batch_flags & SSJ_FORCE_INDEX)) ? index_words_for(vocab_bound) : 0u;
+    a.force_thread = (batch_flags & SSJ_FORCE_THREAD) ? 1u : 0u;
 }
 
 // The persisting-L2 window of a pinned collection on the launch (none if c is not pinned).
@@ -486,7 +488,7 @@ VerifyArgs make_args(ssj_ctx* ctx, const ssj_batch* b, const Collection& R, cons
     memset(&a, 0, sizeof(a));
     a.single = make_instance(b, R, S, n_cands);
     a.table = nullptr;
-    apply_policy(ctx, a, vocab_bound(R, S), (b->flags & SSJ_FORCE_INDEX) != 0);
+    apply_policy(ctx, a, vocab_bound(R, S), b->flags);
     set_l2_window(a, R.l2_window ? R : S);
     return a;
 }
@@ -1112,7 +1114,7 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
     const size_t packed_bytes = sizeof(ssj_triple) * kPackResults;  // results for one copy
     size_t off = align256(sizeof(uint64_t) * n_batches) + align256(packed_bytes);  // counts and these first
     uint64_t launch_vocab = 1;
-    bool launch_force_index = false;
+    uint32_t launch_flags = 0;
     const Collection* pinned = nullptr;  // the first pinned collection: its L2 window
     for (uint32_t i = 0; i < n_batches; ++i) {
         const ssj_batch* b = &batches[i];
@@ -1126,7 +1128,7 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
         table[i] = make_instance(b, *R, *S, n_cands[i]);
         if (!pinned) pinned = R->l2_window ? R : (S->l2_window ? S : nullptr);
         launch_vocab = std::max(launch_vocab, vocab_bound(*R, *S));
-        launch_force_index = launch_force_index || (b->flags & SSJ_FORCE_INDEX) != 0;
+        launch_flags |= b->flags;
         table[i].tile_base = sh.n_tiles;
         const uint64_t tiles = ((uint64_t)b->n_probes + 31) / 32;
         if ((uint64_t)sh.n_tiles + tiles > 0x7FFFFFFull) return fail(ctx, SSJ_EINVAL, "too many probes in one call");
@@ -1186,7 +1188,7 @@ extern "C" ssj_status ssj_verify_batches(ssj_ctx* ctx, const ssj_batch* batches,
     }
     VerifyArgs a;
     memset(&a, 0, sizeof(a));
-    apply_policy(ctx, a, launch_vocab, launch_force_index);
+    apply_policy(ctx, a, launch_vocab, launch_flags);
     if (pinned) set_l2_window(a, *pinned);
     bind_workspace(a, ctx->ws, sh, ctx->num_sms);
     a.table = a.table_out;
@@ -1917,7 +1919,7 @@ struct ssj_multi {
     LaunchShape shape;
     uint32_t block_threads = 256;
     uint32_t index_words_fit = 0;  // probe bitmap words the instances' token values need (0: too many)
-    bool force_index = false;      // an instance forces index items
+    uint32_t batch_flags = 0;      // of all instances together
     void* ws = nullptr;
     std::vector<ssj_coll> colls;  // collections marked busy
     cudaStream_t capture_stream = nullptr;
@@ -1968,7 +1970,7 @@ extern "C" ssj_status ssj_multi_create(ssj_ctx* ctx, const ssj_batch* batches, u
         m->colls.push_back(b->R);
         m->colls.push_back(b->S);
         vocab = std::max(vocab, vocab_bound(*R, *S));
-        m->force_index = m->force_index || (b->flags & SSJ_FORCE_INDEX) != 0;
+        m->batch_flags |= b->flags;
         if (!pinned) pinned = R->l2_window ? R : (S->l2_window ? S : nullptr);
     }
     set_chunks(table.data(), sh, ctx->num_sms);
@@ -1977,7 +1979,7 @@ extern "C" ssj_status ssj_multi_create(ssj_ctx* ctx, const ssj_batch* batches, u
     cudaError_t e = cudaMalloc(&m->ws, bytes);
     if (e != cudaSuccess) return fail(ctx, SSJ_ENOMEM, "cudaMalloc(%zu): %s", bytes, cudaGetErrorString(e));
     memset(&m->a, 0, sizeof(m->a));
-    apply_policy(ctx, m->a, vocab, m->force_index);
+    apply_policy(ctx, m->a, vocab, m->batch_flags);
     if (pinned) set_l2_window(m->a, *pinned);
     m->index_words_fit = index_words_for(vocab);
     m->block_threads = ctx->block_threads;
@@ -2070,7 +2072,7 @@ float time_setting(ssj_ctx* ctx, const ssj_multi* m, uint32_t tmax, uint32_t lma
     a.warp_max_key = wmax;
     a.drain_min_live = dml;
     a.index_min_cands = imin;
-    a.index_words = (imin || m->force_index) ? m->index_words_fit : 0u;
+    a.index_words = (imin || (m->batch_flags & SSJ_FORCE_INDEX)) ? m->index_words_fit : 0u;
     cudaError_t e = prepare_verify(bt, a.index_words);
     if (e == cudaSuccess) e = launch_verify(a, s, ctx->num_sms, bt, nullptr);
     std::vector<float> ms;
@@ -2188,7 +2190,7 @@ extern "C" ssj_status ssj_multi_autotune(ssj_ctx* ctx, ssj_multi* m, void* strea
     m->a.warp_max_key = bw;
     m->a.drain_min_live = bd;
     m->a.index_min_cands = bi;
-    m->a.index_words = (bi || m->force_index) ? m->index_words_fit : 0u;
+    m->a.index_words = (bi || (m->batch_flags & SSJ_FORCE_INDEX)) ? m->index_words_fit : 0u;
     m->block_threads = bb;
     CUDA_TRY(ctx, prepare_verify(bb, m->a.index_words));
     if (m->exec) {

@@ -175,6 +175,7 @@ struct VerifyArgs {
     uint32_t index_min_cands;     // probes with at least this many candidates become index items (0: none)
     uint32_t index_item_cands;    // candidates per index item
     uint32_t bulk_stage;          // block and warp items stage sets by bulk copies (cp.async.bulk)
+    uint32_t force_thread;        // an instance asks for one thread per pair (VF_FORCE_THREAD)
     // host side only: an L2 access-policy window (persisting) for the verify kernel's launch, or none
     const void* l2_base;
     uint64_t l2_bytes;

@@ -27,10 +27,11 @@
 //                 Section 3.3.2; the s-side positional bound of Section
 //                 2.2.3 after every 16-byte block);
 //       phase 2 - lane items: one candidate per lane, r in the warp's shared
-//                 memory; and long pairs, or all pairs when they are few: one
-//                 warp per pair, s's tokens looked up in r, which stays in the
-//                 warp's shared memory while the next pair has the same probe
-//                 (longer probes: 32-lane merge path in windows);
+//                 memory; and long pairs, or all pairs when they are few
+//                 (few_pairs): one warp per pair, s's tokens looked up in r,
+//                 which stays in the warp's shared memory while the next pair
+//                 has the same probe (longer probes, and a forced warp
+//                 granularity: 32-lane merge path in windows);
 //       phase 3 - short pairs, one pair per thread (Alternatives A/B).
 //                 The merge compares 16-byte blocks (4 tokens of r against
 //                 4 of s, 16 compares; the block with the smaller last token
@@ -70,11 +71,6 @@ constexpr uint32_t kBlockRCap = 4096;              // r kept whole in shared mem
 constexpr uint32_t kFlatGrab = 4;                  // most 32-pair chunks taken per dynamic grab in phase 3
 constexpr uint32_t kLongGrab = 8;                  // long pairs taken per dynamic grab in phase 2, about,
 constexpr uint32_t kLongScan = 256;                // and entries of their list read for them, at most
-// Up to this many queued pairs per warp of the grid, short ones too are verified one per warp, dealt
-// out statically: a thread takes about 10 us of dependent loads however few pairs there are (2,034
-// results of short sets: 10 us instead of 17 for the kernel; 48 of the tiny collection: 9 instead of
-// 14).  At 8, 48 uneven joins take 84 us instead of 71 (long and short pairs dealt out alike).
-constexpr uint32_t kFewPairs = 2;
 constexpr uint32_t kCont = 64;                     // parked pairs per warp in phase 3
 
 // Checked build (SSJ_CHECKED): the functions that are not inlined take the
@@ -1061,7 +1057,7 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
     }
 
     // ---------------- phase 2: lane items, then long pairs, one per warp --
-    const bool few = n_long + n_pairs <= (unsigned long long)kFewPairs * n_warps_total;
+    const bool few = few_pairs(n_long, n_pairs, n_warps_total, a.force_thread);
     if (n_warp || n_lone || (few && n_pairs)) {
         WarpOut wout;
         uint32_t* abuf = reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(smem) + warp * kWarpSliceBytes);
@@ -1131,15 +1127,16 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
             const uint32_t req = required_overlap(I.sim, I.p, I.den, I.magic, nr, ns);
             uint32_t o;
             bool rej = false, failed;
-            if (nr + 4 <= kWarpRCap) {
-                if (held != pr.k + 1) {
-                    if (!stage_r(r4, nr, I.r_n_chunks - dr.x)) return false;
-                    held = pr.k + 1;
-                }
+            const bool staged = nr + 4 <= kWarpRCap;
+            if (!staged) held = 0;  // (abuf becomes a window buffer)
+            if (staged && held != pr.k + 1) {
+                if (!stage_r(r4, nr, I.r_n_chunks - dr.x)) return false;
+                held = pr.k + 1;
+            }
+            if (staged && !(I.flags & VF_FORCE_WARP)) {
                 o = warp_lookup(abuf, nr, s4, ns, lane, I.s_n_chunks - ds.x, &a.ctr->err);
-            } else {
-                held = 0;  // (abuf becomes a window buffer)
-                o = warp_merge(r4, nr, s4, ns, req, early, false, abuf, bbuf, lane, wbar, &wph, I.s_n_chunks - ds.x,
+            } else {  // r is too long, or the merge path is asked for
+                o = warp_merge(r4, nr, s4, ns, req, early, staged, abuf, bbuf, lane, wbar, &wph, I.s_n_chunks - ds.x,
                                &a.ctr->err, &failed, &rej CHK_ARGS(I.r_n_chunks - dr.x, I.s_n_chunks - ds.x, &a.ctr->err));
                 if (failed) return false;
             }
