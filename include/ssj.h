@@ -508,9 +508,10 @@ ssj_status ssj_set_granularity(ssj_ctx* ctx, uint32_t thread_max_key, uint32_t l
 /* Index items of later launches of the context (prepared launches take the
  * value at ssj_multi_create; ssj_multi_autotune tunes it per launch): a probe
  * with at least min_cands candidates left by the signature test (among those
- * that one warp of the plan kernel tests, about a thousand; values above 480
- * count as 480) is verified by a whole thread block
- * that holds the probe set r as a bitmap over the token values in shared
+ * that one warp of the plan kernel tests and buffers, up to 511 of about a
+ * thousand; values above 480 count as 480, and a quarter of the value is
+ * enough for probes beyond the one-thread-per-pair bin) is verified by a whole
+ * thread block that holds the probe set r as a bitmap over the token values in shared
  * memory (one bit per value: the launch's token values must stay below
  * 786,432, which frequency renumbering gives for vocabularies of that size;
  * otherwise the probe keeps its other granularity).  Every thread then

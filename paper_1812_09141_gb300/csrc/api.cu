@@ -57,7 +57,7 @@ struct NvtxScope {
 
 namespace {
 
-// Default of the context's index-item threshold (ssj_set_index_items).
+// Default of the context's index-item threshold (ssj_set_index_items, probe_bin).
 constexpr uint32_t kIndexMinCandsDefault = 256;
 // ssj_verify_batches plans a call in up to kMaxPieces pieces of whole waves of plan chunks, each as
 // soon as its candidate ids are on the device.  The host link moves 211 GB/s, to the copy engine and to
@@ -2120,8 +2120,8 @@ extern "C" ssj_status ssj_multi_autotune(ssj_ctx* ctx, ssj_multi* m, void* strea
                                       256 | SSJ_WIDE_REGISTERS | SSJ_BULK_STAGING,
                                       512 | SSJ_WIDE_REGISTERS | SSJ_BULK_STAGING};
     static const uint32_t kMinLive[] = {8, 12, 16, 20, 24};
-    // index-item threshold: 0 sends no probe to index items
-    static const uint32_t kIndexMin[] = {0, 32, 64, 128, 256, 512, 1024, 4096};
+    // index-item threshold: 0 sends no probe to index items (values above 480 count as 480)
+    static const uint32_t kIndexMin[] = {0, 32, 64, 128, 256, 512};
     std::map<std::tuple<uint32_t, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t>, float> seen;
     cudaError_t err = cudaSuccess;
     uint32_t bd = m->a.drain_min_live ? m->a.drain_min_live : 16;

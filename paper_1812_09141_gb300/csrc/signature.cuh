@@ -221,11 +221,19 @@ __device__ __noinline__ uint32_t second_level(const PlanInst& I, uint2* buf, uin
     return left;
 }
 
-// Granularity of a probe with |r| = nr and n candidates left: 0 thread per
+// Granularity of a run, n pairs left of a probe with |r| = nr: 0 thread per
 // pair, 1 warp per pair, 2 block per pair, 3 lane per pair with r in the
 // warp's shared memory (Alternative B; needs r to fit and enough candidates
-// to occupy the lanes), 4 index items (many candidates, when the launch's
+// to occupy the lanes), 4 an index item (many candidates, when the launch's
 // token values fit the probe bitmap).
+//
+// A list is cut into runs where a warp's candidates or its buffer end, so its
+// last run is often much shorter than the list.  Beyond the thread bin an index
+// item is the better choice from about 60 pairs on (300 tokens; 18 us an item
+// and 0.14 a pair of a CTA's time, one lane per pair 0.45) or 20 (1,500 tokens;
+// 90 and 0.6, one block per pair 5.8), within it from about 270 (60 tokens): a
+// quarter of the threshold for the former.  Lists of 1,000 pairs of 1,500 tokens
+// that all pass took 4.7 ms with one threshold for both, now 2.8.
 __device__ __forceinline__ uint32_t probe_bin(const VerifyArgs& a, uint32_t flags, uint32_t nr, uint32_t n) {
     const bool lane_ok = nr + 4 <= kWarpRCap;
     if (flags & VF_FORCE_INDEX) return a.index_words ? 4u : (lane_ok ? 3u : 1u);
@@ -233,8 +241,9 @@ __device__ __forceinline__ uint32_t probe_bin(const VerifyArgs& a, uint32_t flag
     if (flags & VF_FORCE_WARP) return 1;
     if (flags & VF_FORCE_THREAD) return 0;
     if (flags & VF_FORCE_LANE) return lane_ok ? 3u : 1u;
-    if (a.index_words && a.index_min_cands && n >= min(a.index_min_cands, kPlanFlush)) return 4;
     const uint64_t key = 2ull * nr;  // |r|+|s| at |s| = |r|
+    const uint32_t index_min = min(a.index_min_cands, kPlanFlush);
+    if (a.index_words && index_min && n >= (key <= a.thread_max_key ? index_min : max(index_min / 4, 1u))) return 4;
     if (key <= a.thread_max_key) return 0;
     if (key <= a.lane_max_key && lane_ok && n >= kLaneMinCands) return 3;
     return key <= a.warp_max_key ? 1u : 2u;
@@ -243,7 +252,7 @@ __device__ __forceinline__ uint32_t probe_bin(const VerifyArgs& a, uint32_t flag
 // Work items of one run: n pairs of probe r from pos on in the pair list, of
 // granularity bin (2 to 4), as items first, first + 1, ... of its list.
 __device__ __forceinline__ uint32_t item_pairs(const VerifyArgs& a, uint32_t bin) {
-    return bin == 3 ? a.lane_item_cands : (bin == 4 ? a.index_item_cands : a.block_item_cands);
+    return bin == 3 ? a.lane_item_cands : (bin == 4 ? kPlanBuf : a.block_item_cands);  // (an index item is a run)
 }
 __device__ __forceinline__ void write_item(const VerifyArgs& a, uint32_t bin, uint32_t inst, uint32_t r, uint32_t n,
                                            unsigned long long pos, unsigned long long first, uint32_t it) {

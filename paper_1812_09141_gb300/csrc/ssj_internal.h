@@ -144,7 +144,6 @@ constexpr uint32_t kLaneMinCands = 16;   // fewest candidates of a probe sent to
 constexpr uint32_t kWarpRCap = 1024;     // r kept whole in a warp's shared memory up to this
 constexpr uint32_t kPlanFlush = 480;     // pairs left that a plan warp queues at once
 constexpr uint32_t kIndexMaxWords = 24576;  // largest probe bitmap (32-bit words, 96 KiB): token values below 786,432
-constexpr uint32_t kIndexItemCands = 8192;  // most candidates per index item
 
 // Kernel arguments of one launch (passed by value).
 struct VerifyArgs {
@@ -172,8 +171,7 @@ struct VerifyArgs {
     uint32_t drain_min_live;      // short-pair pass 2 re-parks below this many live lanes (0: default 16)
     uint32_t index_words;         // probe bitmap words (every token value of the launch's collections below
                                   // 32 * index_words); 0: no index items
-    uint32_t index_min_cands;     // probes with at least this many candidates become index items (0: none)
-    uint32_t index_item_cands;    // candidates per index item
+    uint32_t index_min_cands;     // runs of at least this many pairs become index items (0: none; see probe_bin)
     uint32_t bulk_stage;          // block and warp items stage sets by bulk copies (cp.async.bulk)
     uint32_t force_thread;        // an instance asks for one thread per pair (VF_FORCE_THREAD)
     // host side only: an L2 access-policy window (persisting) for the verify kernel's launch, or none

@@ -1261,18 +1261,13 @@ static uint64_t item_cap(uint64_t n_probes, uint64_t n_cands, uint32_t per_item)
 // number of dynamic-scheduling atomics.  (Estimates: 32 resident warps and
 // 4 resident CTAs per SM.)
 static void item_sizes(uint64_t n_cands, int num_sms, uint32_t* per_warp_item, uint32_t* per_block_item,
-                       uint32_t* per_lane_item, uint32_t* per_index_item) {
+                       uint32_t* per_lane_item) {
     const uint64_t warps = 32ull * (uint64_t)num_sms, ctas = 4ull * (uint64_t)num_sms;
     uint64_t w = n_cands / (64 * warps), b = n_cands / (64 * ctas), l = n_cands / (8 * warps);
     *per_warp_item = (uint32_t)(w < 1 ? 1 : (w > kWarpItemCands ? kWarpItemCands : w));
     *per_block_item = (uint32_t)(b < 1 ? 1 : (b > kBlockItemCands ? kBlockItemCands : b));
     l = l < 32 ? 32 : (l > kLaneItemCands ? kLaneItemCands : l);
     *per_lane_item = (uint32_t)(l & ~31ull);
-    // index items: a few per CTA of the wave, at least one block's worth of candidates (never
-    // fewer than a block item, so the block list's capacity covers them)
-    uint64_t x = n_cands / (4 * ctas);
-    x = x < 512 ? 512 : (x > kIndexItemCands ? kIndexItemCands : x);
-    *per_index_item = (uint32_t)(x < *per_block_item ? *per_block_item : x);
 }
 
 static uint64_t pair_cap(const LaunchShape& sh) { return sh.total_cands + 32ull * sh.n_tiles + 32; }
@@ -1283,8 +1278,8 @@ static uint64_t pair_cap(const LaunchShape& sh) { return sh.total_cands + 32ull 
 // that chunk borders cut (one more work item each) fit the item lists (see
 // bind_workspace).
 uint32_t plan_chunk(uint64_t total_cands, int num_sms) {
-    uint32_t wc, bc, lc, ic;
-    item_sizes(total_cands, num_sms, &wc, &bc, &lc, &ic);
+    uint32_t wc, bc, lc;
+    item_sizes(total_cands, num_sms, &wc, &bc, &lc);
     const uint64_t warps = plan_wave(num_sms);
     const uint64_t rounds = std::max<uint64_t>((total_cands + 1024 * warps - 1) / (1024 * warps), 1);
     const uint64_t per = (total_cands + warps * rounds - 1) / (warps * rounds);
@@ -1303,8 +1298,8 @@ LaunchShape single_shape(uint32_t n_probes, uint64_t n_cands, int num_sms) {
 }
 
 size_t workspace_bytes(const LaunchShape& sh, int num_sms) {
-    uint32_t wc, bc, lc, ic;
-    item_sizes(sh.total_cands, num_sms, &wc, &bc, &lc, &ic);
+    uint32_t wc, bc, lc;
+    item_sizes(sh.total_cands, num_sms, &wc, &bc, &lc);
     const uint64_t slots = 32ull * sh.n_tiles + 1, pc = pair_cap(sh);
     // (the terms by probe slot and pc / 8 are room for work items, see bind_workspace)
     return align256(sizeof(Counters)) + align256(sizeof(Instance) * ((size_t)sh.n_inst + 1)) +
@@ -1321,7 +1316,7 @@ size_t workspace_bytes(uint32_t n_probes, uint64_t n_cands, int num_sms) {
 void bind_workspace(VerifyArgs& a, void* ws, const LaunchShape& sh, int num_sms) {
     char* p = static_cast<char*>(ws);
     uint32_t wc;
-    item_sizes(sh.total_cands, num_sms, &wc, &a.block_item_cands, &a.lane_item_cands, &a.index_item_cands);
+    item_sizes(sh.total_cands, num_sms, &wc, &a.block_item_cands, &a.lane_item_cands);
     a.n_inst = sh.n_inst;
     a.n_tiles = sh.n_tiles;
     a.total_probes = sh.total_probes;
@@ -1526,7 +1521,6 @@ JoinQueue bind_join_workspace(VerifyArgs& a, void* ws, uint32_t n_probes, uint64
     };
     a.block_item_cands = kJoinBlockCands;
     a.lane_item_cands = 32;
-    a.index_item_cands = kIndexItemCands;
     a.n_inst = 1;
     a.n_tiles = (n_probes + 31) / 32;
     a.total_probes = n_probes;

@@ -79,3 +79,18 @@ def test_queueing_pairs_costs_about_as_much_as_testing_them(ctx, probes, each):
         assert queued[0] < 2.5 * dropped[0], (queued, dropped)
     finally:
         ssj.ssj_unload_collection(ctx, h)
+
+
+def test_short_runs_of_cut_lists_of_long_sets(ctx):
+    """Lists of 1,000 pairs of 1,500 tokens that all pass: most of the runs that chunks and buffers cut
+    them into become index items as if they were asked for, so the verify kernel takes at most 1.4
+    times as long (1.7 when runs below 256 pairs were verified by a block per pair)."""
+    h = cluster(ctx, 1_500, 4_000)
+    try:
+        b = lists(4_000, 2_000, 1_000)
+        default, n = kernel_ms(ctx, h, b, 0)
+        items, m = kernel_ms(ctx, h, b, ssj.SSJ_FORCE_INDEX)
+        assert n == m > 0.99 * len(b[2])
+        assert default[1] < 1.4 * items[1], (default, items)
+    finally:
+        ssj.ssj_unload_collection(ctx, h)
