@@ -306,8 +306,10 @@ ssj_status ssj_verify_batch_noalloc(ssj_ctx* ctx, const ssj_batch* batch, ssj_tr
  * of candidates verified.  Flags: SSJ_SIM_*, SSJ_JOIN_POSITIONAL,
  * SSJ_COUNT_ONLY, SSJ_SORTED, SSJ_DEVICE_PTRS, SSJ_FORCE_*.  Token values
  * must stay below 2^30 (load with SSJ_RENUMBER_BY_FREQ, which the prefix
- * filter wants anyway).  The prefix index comes from the context's memory
- * pool, the queue of pairs is the context's workspace; a join that leaves
+ * filter wants anyway).  The prefix index comes from a memory pool of the
+ * context's, of which at most 256 MiB stay mapped after the call (until the
+ * context is destroyed; ssj_verify_groups takes its arrays from the same
+ * pool); the queue of pairs is the context's workspace; a join that leaves
  * more pairs than the queue holds is probed a second time with a larger one.
  * Errors: SSJ_EINVAL, SSJ_ENOTFOUND, SSJ_ENOMEM, SSJ_EDEVICE.
  */

@@ -78,6 +78,9 @@ constexpr size_t kSmallInput = 128 << 10;
 // take about 15): of one batch, and of all batches of ssj_verify_batches.
 constexpr uint64_t kFirstResults = 4096;
 constexpr uint64_t kPackResults = 16384;
+// Device memory that the pool of the calls' own memory keeps between them; a call that took more
+// gives the rest back before it returns.  (Self-joins of up to a million sets take 70 to 150 MB.)
+constexpr uint64_t kKeepCallMemory = 256ull << 20;
 
 struct Collection {
     uint32_t n_sets = 0;
@@ -206,7 +209,8 @@ struct ssj_ctx {
     // serving
     std::mutex mu;
     std::condition_variable cv;  // a ticket completed
-    cudaMemPool_t pool = nullptr;
+    cudaMemPool_t pool = nullptr;       // submitted batches
+    cudaMemPool_t call_pool = nullptr;  // CallMemory
     std::vector<Slot> slots;
     std::map<uint64_t, std::unique_ptr<Ticket>> tickets;
     uint64_t next_ticket = 1;
@@ -534,10 +538,10 @@ void free_collection(Collection& c) {
     for (uint4* r : c.d_rec) cudaFree(r);
 }
 
-// Device memory of one call, from the context's pool in the order of its
-// stream: it stays in the pool (up to the pool's release threshold, the
-// serving budget) instead of being mapped and unmapped by every call (a dozen
-// cudaMalloc and cudaFree took about 1 ms), and goes back with the context.
+// Device memory of one call, from a pool of the context's in the order of its
+// stream: up to kKeepCallMemory stays in the pool instead of being mapped and
+// unmapped by every call (a dozen cudaMalloc and cudaFree took about 1 ms), and
+// goes back with the context.
 // An allocation from the pool still takes several microseconds: arrays whose
 // sizes are known together are carved out of one (block, then get).
 class CallMemory {
@@ -545,6 +549,12 @@ public:
     explicit CallMemory(ssj_ctx* c) : ctx_(c) {}
     ~CallMemory() {
         for (void* m : mem_) cudaFreeAsync(m, ctx_->stream);
+        uint64_t held = 0;
+        if (cudaMemPoolGetAttribute(ctx_->call_pool, cudaMemPoolAttrReservedMemCurrent, &held) != cudaSuccess ||
+            held <= kKeepCallMemory)
+            return;
+        cudaStreamSynchronize(ctx_->stream);
+        cudaMemPoolTrimTo(ctx_->call_pool, kKeepCallMemory);
     }
     CallMemory(const CallMemory&) = delete;
     CallMemory& operator=(const CallMemory&) = delete;
@@ -557,7 +567,7 @@ public:
     void block(size_t bytes) {
         void* m = nullptr;
         at_ = end_ = nullptr;
-        if (cudaMallocFromPoolAsync(&m, bytes, ctx_->pool, ctx_->stream) != cudaSuccess) {
+        if (cudaMallocFromPoolAsync(&m, bytes, ctx_->call_pool, ctx_->stream) != cudaSuccess) {
             cudaGetLastError();
             failed_ = true;
             return;
@@ -687,6 +697,9 @@ extern "C" ssj_status ssj_create(const ssj_config* config, ssj_ctx** out) {
     if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess) return SSJ_EDEVICE;
     uint64_t threshold = ctx->budget;
     cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &threshold);
+    if (cudaMemPoolCreate(&ctx->call_pool, &props) != cudaSuccess) return SSJ_EDEVICE;
+    threshold = kKeepCallMemory;
+    cudaMemPoolSetAttribute(ctx->call_pool, cudaMemPoolAttrReleaseThreshold, &threshold);
     ctx->slots.resize(ctx->max_inflight);
     for (auto& s : ctx->slots) {
         s.wake.reset(new std::condition_variable());
@@ -760,6 +773,7 @@ extern "C" void ssj_destroy(ssj_ctx* ctx) {
 
     for (cudaEvent_t ev : ctx->prof_ev) cudaEventDestroy(ev);
     if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+    if (ctx->call_pool) cudaMemPoolDestroy(ctx->call_pool);
     if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
     delete ctx;
 }
