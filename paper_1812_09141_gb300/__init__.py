@@ -16,8 +16,8 @@ from dataclasses import dataclass
 import numpy as np
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
-# SSJ_LIBRARY=checked loads the checked build (every kernel index tested, an
-# out-of-bounds one reported as device error bit 4 instead of faulting).
+# SSJ_LIBRARY=checked loads the checked build (the verification kernels test their
+# indexes; an out-of-bounds one is reported as device error bit 4 instead of faulting).
 LIB_PATH = os.path.join(_HERE, "libssj_checked.so" if os.environ.get("SSJ_LIBRARY") == "checked" else "libssj.so")
 
 # status codes

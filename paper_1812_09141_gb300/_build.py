@@ -1,7 +1,7 @@
 """Build libssj.so in-tree with nvcc for sm_103a (GB300), and its checked
-twin libssj_checked.so (-DSSJ_CHECKED: every index of the plan and verify
-kernels is tested against its array's extent; a bad one sets an error bit
-instead of faulting), which tests load with SSJ_LIBRARY=checked.
+twin libssj_checked.so (-DSSJ_CHECKED: the plan, verify, join and queue
+kernels test their indexes against the arrays' extents; a bad one sets an
+error bit instead of faulting), which tests load with SSJ_LIBRARY=checked.
 
 Each translation unit is compiled to an object in parallel, then linked
 into one shared library next to this file.  A stamp of the sources and

@@ -1354,7 +1354,7 @@ extern "C" ssj_status ssj_self_join(ssj_ctx* ctx, ssj_coll coll, uint32_t p, uin
     in.stage = 0;
     cudaError_t e = candgen_run(in, s, ctx->num_sms, &ix, ctx->h_count);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "candidate generation (index)");
-    const uint64_t entries = *ctx->h_count;
+    const uint64_t entries = ix.entries = *ctx->h_count;
     ix.post = mem.get<char>(candgen_entry_bytes(in.positional != 0) * entries);
     if (!mem.ok()) return fail(ctx, SSJ_ENOMEM, "prefix index of %llu entries", (unsigned long long)entries);
     in.stage = 1;

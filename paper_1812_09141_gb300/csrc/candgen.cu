@@ -170,12 +170,12 @@ template <>
 struct Entry<true> {
     uint32_t rank, id, at, size;
 };
-__device__ __forceinline__ Entry<false> ld_entry(const Entry<false>* e) {
-    const uint2 x = __ldg(reinterpret_cast<const uint2*>(e));
+__device__ __forceinline__ Entry<false> ld_entry(const Entry<false>* post, uint64_t e, uint64_t n, uint32_t* err) {
+    const uint2 x = ld_at(reinterpret_cast<const uint2*>(post), e, n, err);
     return {x.x, x.y};
 }
-__device__ __forceinline__ Entry<true> ld_entry(const Entry<true>* e) {
-    const uint4 x = __ldg(reinterpret_cast<const uint4*>(e));
+__device__ __forceinline__ Entry<true> ld_entry(const Entry<true>* post, uint64_t e, uint64_t n, uint32_t* err) {
+    const uint4 x = ld_at(reinterpret_cast<const uint4*>(post), e, n, err);
     return {x.x, x.y, x.z, x.w};
 }
 
@@ -213,6 +213,7 @@ struct JoinArgs {
     const uint64_t* size_end;  // size -> position after its last set
     const uint64_t* toff;      // cell -> first index entry (and one past the last cell)
     const void* post;          // index entries (Entry<POS>)
+    uint64_t sizes, cells, entries;  // of size_end, toff (without the closing one) and post
     uint32_t* cursor;          // next probe (from the last position down)
     uint32_t grab;             // probes per grab
     JoinQueue out;             // pairs left
@@ -258,6 +259,12 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
     __syncthreads();
     const PlanInst& I = s_inst;
     const Entry<POS>* post = static_cast<const Entry<POS>*>(J.post);
+    uint32_t* err = &a.ctr->err;
+    const uint32_t* all_tokens = reinterpret_cast<const uint32_t*>(P.toks4);
+    auto token = [&](uint32_t first_block, uint32_t k) -> uint32_t {
+        return ld_at(all_tokens, 4ull * first_block + k, 4ull * a.single.r_n_chunks, err);
+    };
+    auto cell_start = [&](uint64_t c) -> uint64_t { return ld_at(J.toff, c, J.cells + 1, err); };
     unsigned long long found = 0;  // candidates (warp-uniform)
     uint32_t n = 0, q = 0;         // pairs in buf, candidates waiting for the test (warp-uniform)
     auto hand_over = [&]() {       // buf as one run
@@ -286,15 +293,15 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
         bool pass = (uint32_t)lane < m;
         if (G == 1) {
             uint32_t r_head;
-            const uint32_t r = __ldg(J.probes + e.x);
-            const uint32_t v = bound_of_pair<1, false>(I.s_rec[0], I.r_rec[0], e.y, r, rs, lane, &r_head);
+            const uint32_t r = ld_at(J.probes, e.x, P.n, err);
+            const uint32_t v = bound_of_pair<1, false>(I.s_rec[0], I.r_rec[0], e.y, r, rs, lane, P.n, P.n, err, &r_head);
             pass = pass && bound_passes(I, th, v, r_head >> 16);
         } else if (G > 1) {
-            const uint32_t v = bound_of_pair<kG, true>(I.s_rec[0], nullptr, e.y, 0u, rs, lane);
+            const uint32_t v = bound_of_pair<kG, true>(I.s_rec[0], nullptr, e.y, 0u, rs, lane, P.n, 0u, err);
             pass = pass && bound_passes(I, th, v, nr);
         }
         const uint32_t pm = __ballot_sync(kAll, pass);
-        if (pass) W.buf[n + __popc(pm & lt)] = e;
+        if (pass && in_bounds(n + __popc(pm & lt), kJoinRun, err)) W.buf[n + __popc(pm & lt)] = e;
         n += __popc(pm);
         __syncwarp();
     };
@@ -308,11 +315,11 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
         uint32_t my_r = 0, my_pl = 0, my_lo = 0;
         uint2 my_d = make_uint2(0u, 0u);
         if ((uint32_t)lane < probes) {
-            my_r = J.probes[g0 + lane];
-            my_d = P.desc[my_r];
+            my_r = ld_at(J.probes, g0 + lane, P.n, err);
+            my_d = ld_at(P.desc, my_r, P.n, err);
             my_pl = prefix_len(P, my_d.y);
             if (my_pl) {
-                my_lo = (uint32_t)J.size_end[min_overlap(P, my_d.y) - 1];  // (at least 1, at most the size)
+                my_lo = (uint32_t)ld_at(J.size_end, min_overlap(P, my_d.y) - 1, J.sizes, err);  // (at least 1, at most the size)
                 if (my_lo >= P.n - 1 - (g0 + lane)) my_pl = 0;
             }
         }
@@ -322,14 +329,14 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
         uint64_t next_start = 0, next_end = 0;
         auto bounds = [&](uint32_t tok, bool have, int p) {
             const uint32_t first = __shfl_sync(kAll, my_lo, p), last = P.n - 2 - (g0 + p);
-            next_start = have ? J.toff[cell_of(P, tok, first)] : 0;
-            next_end = have ? J.toff[cell_of(P, tok, last) + 1] : 0;
+            next_start = have ? cell_start(cell_of(P, tok, first)) : 0;
+            next_end = have ? cell_start(cell_of(P, tok, last) + 1) : 0;
         };
         if (left) {
             const int p = __ffs(left) - 1;
-            const uint32_t* t = reinterpret_cast<const uint32_t*>(P.toks4 + __shfl_sync(kAll, my_d.x, p));
+            const uint32_t t = __shfl_sync(kAll, my_d.x, p);
             const bool have = (uint32_t)lane < __shfl_sync(kAll, my_pl, p);
-            bounds(have ? t[lane] : 0u, have, p);
+            bounds(have ? token(t, lane) : 0u, have, p);
         }
         while (left) {
             const int p = __ffs(left) - 1;
@@ -338,19 +345,18 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
             const uint32_t g = g0 + p, rpos = P.n - 1 - g, lo = __shfl_sync(kAll, my_lo, p);
             const uint32_t L = __shfl_sync(kAll, my_d.y, p), pl = __shfl_sync(kAll, my_pl, p);
             const uint32_t pl2 = left ? __shfl_sync(kAll, my_pl, p2) : 0u;
-            const uint32_t* t = reinterpret_cast<const uint32_t*>(P.toks4 + __shfl_sync(kAll, my_d.x, p));
-            const uint32_t* t2 = reinterpret_cast<const uint32_t*>(P.toks4 + __shfl_sync(kAll, my_d.x, p2));
+            const uint32_t t = __shfl_sync(kAll, my_d.x, p), t2 = __shfl_sync(kAll, my_d.x, p2);  // first blocks
             if (G > 1) {
                 const uint32_t r = __shfl_sync(kAll, my_r, p);
-                rs = ld_sector(I.r_rec[0] + ((uint64_t)r * kG + lane % kG) * 2);
-                nr = __ldg(&I.r_rec[0][(uint64_t)r * kG * 2].x) >> 16;
+                rs = ld_sector(I.r_rec[0], (uint64_t)r * kG + lane % kG, (uint64_t)P.n * kG, err);
+                nr = ld_header(I.r_rec[0], r, kG, P.n, err) >> 16;
             }
             // entries in all, if the positions are more than the bitmap holds
             uint32_t hash_mask = 0;
             if (rpos - lo > kSeenBits) {
                 uint64_t e = next_end - next_start;
                 for (uint32_t k = 32 + lane; k < pl; k += 32)
-                    e += J.toff[cell_of(P, t[k], rpos - 1) + 1] - J.toff[cell_of(P, t[k], lo)];
+                    e += cell_start(cell_of(P, token(t, k), rpos - 1) + 1) - cell_start(cell_of(P, token(t, k), lo));
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(kAll, e, o);
                 if (e <= kSeenWords / 2) hash_mask = e <= 32 ? 63u : (2u << (31 - __clz((uint32_t)e * 2 - 1))) - 1;
@@ -375,12 +381,12 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
                             }
                         } else {
                             const uint32_t b = en.rank - w0, bit = 1u << (b & 31u);
-                            is_new = (atomicOr(W.seen + (b >> 5), bit) & bit) == 0;
+                            is_new = in_bounds(b >> 5, kSeenWords, err) && (atomicOr(W.seen + (b >> 5), bit) & bit) == 0;
                         }
                     }
                     const uint32_t m = __ballot_sync(kAll, is_new);
                     if (m == 0) return;
-                    if (is_new) W.fresh[q + __popc(m & lt)] = make_uint2(g, en.id);
+                    if (is_new && in_bounds(q + __popc(m & lt), 64, err)) W.fresh[q + __popc(m & lt)] = make_uint2(g, en.id);
                     q += __popc(m);
                     found += __popc(m);
                     __syncwarp();
@@ -399,7 +405,7 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
                     const bool more = k0 + 32 < pl, again = !more && w1 < rpos;
                     const uint32_t kn = more ? k0 + 32 + lane : (uint32_t)lane;
                     const bool have_n = kn < (more || again ? pl : pl2);
-                    const uint32_t tok_n = have_n ? (more || again ? t : t2)[kn] : 0u;
+                    const uint32_t tok_n = have_n ? token(more || again ? t : t2, kn) : 0u;
                     // lists that do not add up in 32 bits, one by one
                     uint32_t longs = __ballot_sync(kAll, len >= kLongList);
                     while (longs) {
@@ -408,7 +414,7 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
                         const uint64_t e0 = __shfl_sync(kAll, start, src), e1 = e0 + __shfl_sync(kAll, len, src);
                         for (uint64_t e = e0; e < e1; e += 32) {
                             const bool have = e + lane < e1;
-                            take(have, ld_entry(post + (have ? e + lane : e)), k0 + src);
+                            take(have, ld_entry(post, have ? e + lane : e, J.entries, err), k0 + src);
                         }
                     }
                     const uint32_t mine = len >= kLongList ? 0u : (uint32_t)len;
@@ -420,7 +426,7 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
                     }
                     const uint32_t total = __shfl_sync(kAll, incl, 31);
                     const uint64_t base = start - (incl - mine);  // entry e of the one list is base + e of its token
-                    auto locate = [&](uint32_t e, uint32_t* k) -> const Entry<POS>* {
+                    auto locate = [&](uint32_t e, uint32_t* k) -> uint64_t {
                         uint32_t x = 0;  // tokens whose entries end by e
 #pragma unroll
                         for (int step = 16; step >= 1; step >>= 1) {
@@ -428,13 +434,13 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
                             if (v <= e) x += step;
                         }
                         *k = x;
-                        return post + (__shfl_sync(kAll, base, x) + e);
+                        return __shfl_sync(kAll, base, x) + e;
                     };
                     Entry<POS> en_n = {};
                     uint32_t k_n = 0;
                     if (total) {
-                        const Entry<POS>* at = locate(lane, &k_n);
-                        if ((uint32_t)lane < total) en_n = ld_entry(at);
+                        const uint64_t at = locate(lane, &k_n);
+                        if ((uint32_t)lane < total) en_n = ld_entry(post, at, J.entries, err);
                     }
                     bounds(tok_n, have_n, more || again ? p : p2);
                     for (uint32_t e0 = 0; e0 < total; e0 += 32) {
@@ -442,8 +448,8 @@ __global__ void __launch_bounds__(kJoinWarps * 32, 4) join_kernel(const __grid_c
                         const uint32_t k = k_n;
                         if (e0 + 32 < total) {
                             const uint32_t e = e0 + 32 + lane;
-                            const Entry<POS>* at = locate(e, &k_n);
-                            if (e < total) en_n = ld_entry(at);
+                            const uint64_t at = locate(e, &k_n);
+                            if (e < total) en_n = ld_entry(post, at, J.entries, err);
                         }
                         take(e0 + lane < total, en, k0 + k);
                     }
@@ -473,7 +479,8 @@ __global__ void __launch_bounds__(kJoinWarps * 32) queue_kernel(const __grid_con
     for (unsigned long long b = blockIdx.x * kJoinWarps + warp; b < runs; b += gridDim.x * kJoinWarps) {
         const ulonglong2 run = Q.runs[b];
         const uint32_t n = min((uint32_t)run.y, kJoinRun);
-        for (uint32_t k = lane; k < n; k += 32) s_buf[warp][k] = Q.pairs[run.x + k];
+        for (uint32_t k = lane; k < n; k += 32)
+            s_buf[warp][k] = in_bounds(run.x + k, Q.pair_cap, &a.ctr->err) ? Q.pairs[run.x + k] : make_uint2(0u, 0u);
         __syncwarp();
         flush_survivors(a, s_inst, 0, s_buf[warp], n, lane);
         __syncwarp();
@@ -661,6 +668,9 @@ cudaError_t join_probe(const CandgenInput& in, const CandgenIndex& ix, const Ver
     J.size_end = ix.size_hist;
     J.toff = ix.toff;
     J.post = ix.post;
+    J.sizes = (uint64_t)in.max_len + 2;
+    J.cells = candgen_cells(in.vocab);
+    J.entries = ix.entries;
     J.cursor = &a.ctr->probe_cursor;
     J.grab = 1;
     J.out = out;

@@ -36,11 +36,13 @@ constexpr int kPlanCtas = 4;
 // f), by the whole warp: each step narrows the range of candidate answers
 // 32-fold with one load per lane.  (Offsets that are not nondecreasing give
 // some k of the range.)
-__device__ __forceinline__ uint32_t find_probe(const uint64_t* offs, uint32_t lo, uint32_t hi, uint64_t f, int lane) {
+__device__ __forceinline__ uint32_t find_probe(const uint64_t* offs, uint32_t lo, uint32_t hi, uint64_t f, uint32_t* err,
+                                               int lane) {
+    const uint32_t n = hi;
     while (hi - lo > 1) {
         const uint32_t step = (hi - lo + 31) / 32;
         const uint64_t at = (uint64_t)lo + (uint64_t)step * lane;
-        const bool le = lane == 0 || (at < hi && __ldg(offs + at) <= f);
+        const bool le = lane == 0 || (at < hi && ld_at(offs, at, n, err) <= f);
         const uint32_t m = __ballot_sync(kFull, le);
         const uint32_t last = 31 - __clz(m);
         const uint64_t end = (uint64_t)lo + (uint64_t)step * (last + 1);
@@ -52,16 +54,18 @@ __device__ __forceinline__ uint32_t find_probe(const uint64_t* offs, uint32_t lo
 
 // The same by one lane for its own f, in steps that double and then a binary
 // search (it is near lo more often than not).
-__device__ __forceinline__ uint32_t find_probe_lane(const uint64_t* offs, uint32_t lo, uint32_t hi, uint64_t f) {
+__device__ __forceinline__ uint32_t find_probe_lane(const uint64_t* offs, uint32_t lo, uint32_t hi, uint64_t f,
+                                                    uint32_t* err) {
+    const uint32_t n = hi;
     uint32_t step = 32;
-    while (step < hi - lo && __ldg(offs + lo + step) <= f) {
+    while (step < hi - lo && ld_at(offs, lo + step, n, err) <= f) {
         lo += step;
         step = min(2 * step, 1u << 30);
     }
     hi = min(hi - lo, step) + lo;
     while (hi - lo > 1) {
         const uint32_t mid = lo + (hi - lo) / 2;
-        if (__ldg(offs + mid) <= f) lo = mid; else hi = mid;
+        if (ld_at(offs, mid, n, err) <= f) lo = mid; else hi = mid;
     }
     return lo;
 }
@@ -87,19 +91,20 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
     const bool emit_all = (I.flags & VF_EMIT_ALL) != 0, self_join = (I.flags & VF_SELF_JOIN) != 0;
     const uint32_t len = (uint32_t)(f1 - f0), slot0 = 32u * I.tile_base, s_n_sets = I.s_n_sets;
     const uint32_t* cands = I.cand_ids + f0;
+    auto cand = [&](uint32_t at) -> uint32_t { return ld_at(cands, at, I.n_cands - f0, err); };
     // lane l of the window holds probe kb + l: its id, and the end of its list relative to f0 (saturated;
     // the last probe's list ends the batch)
-    uint32_t kb = find_probe(I.cand_offsets, 0, I.n_probes, f0, lane), ends, ids;
+    uint32_t kb = find_probe(I.cand_offsets, 0, I.n_probes, f0, err, lane), ends, ids;
     auto list_end = [&](uint32_t k) -> uint32_t {
         const uint64_t at = (uint64_t)k + 1 + lane;
         if (at >= I.n_probes) return 0xFFFFFFFFu;
-        const uint64_t v = __ldg(I.cand_offsets + at);
+        const uint64_t v = ld_at(I.cand_offsets, at, I.n_probes + 1ull, err);
         return v <= f0 ? 0u : (uint32_t)min(v - f0, (uint64_t)0xFFFFFFFFu);
     };
     auto window = [&](uint32_t k) {
         kb = k;
         ends = list_end(k);
-        ids = (uint64_t)k + lane < I.n_probes ? __ldg(I.probe_ids + k + lane) : 0xFFFFFFFFu;
+        ids = (uint64_t)k + lane < I.n_probes ? ld_at(I.probe_ids, (uint64_t)k + lane, I.n_probes, err) : 0xFFFFFFFFu;
     };
     window(kb);
     uint32_t n = 0;  // buffered pairs (warp-uniform)
@@ -110,10 +115,10 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
         if (pass && in_bounds(q, kPlanBuf, err)) buf[q] = make_uint2(slot, s);
         n += __popc(m);
     };
-    uint32_t s_next = (uint32_t)lane < len ? __ldg(cands + lane) : 0u;  // the lane's candidate of the next round
+    uint32_t s_next = (uint32_t)lane < len ? cand(lane) : 0u;  // the lane's candidate of the next round
     auto next = [&](uint32_t f) -> uint32_t {  // the round at f's candidate; asks for the one after
         const uint32_t s = s_next;
-        if (f + 32 + lane < len) s_next = __ldg(cands + f + 32 + lane);
+        if (f + 32 + lane < len) s_next = cand(f + 32 + lane);
         return s;
     };
     const Threshold th = threshold(I);
@@ -125,7 +130,7 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
         // end before f, and no round would be made.)
         uint32_t m = __ballot_sync(kFull, ends > f);
         for (bool near = true; m == 0; near = false) {  // (kb + 32 < n_probes: the last list's end is beyond every f)
-            window(near ? kb + 32 : find_probe(I.cand_offsets, kb + 32, I.n_probes, f0 + f, lane));
+            window(near ? kb + 32 : find_probe(I.cand_offsets, kb + 32, I.n_probes, f0 + f, err, lane));
             m = __ballot_sync(kFull, ends > f);
         }
         const uint32_t passed0 = __ffs(m) - 1;
@@ -138,10 +143,10 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
             Sector rs;
             uint32_t nr;
             if (G == 0) {
-                nr = r_ok ? I.r_desc[rk].y : 0u;
+                nr = r_ok ? ld_at(I.r_desc, rk, I.r_n_sets, err).y : 0u;
             } else {
-                rs = ld_sector(I.r_rec[0] + ((uint64_t)rk * kG + lane % kG) * 2);
-                nr = __ldg(&I.r_rec[0][(uint64_t)rk * kG * 2].x) >> 16;
+                rs = ld_sector(I.r_rec[0], (uint64_t)rk * kG + lane % kG, (uint64_t)I.r_n_sets * kG, err);
+                nr = ld_header(I.r_rec[0], rk, kG, I.r_n_sets, err) >> 16;
             }
             for (; f < end && (end - f >= 32 || end == len) && n < kPlanFlush; f += 32) {
                 const uint32_t s = next(f);
@@ -150,11 +155,11 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
                 bool pass = ok && !(self_join && s == r);
                 if (G == 0) {
                     if (pass && !emit_all) {
-                        const uint32_t ns = I.s_desc[s].y;
+                        const uint32_t ns = ld_at(I.s_desc, s, s_n_sets, err).y;
                         pass = overlap_passes(I, min(nr, ns), nr, ns);
                     }
                 } else {
-                    const uint32_t v = bound_of_pair<kG, true>(I.s_rec[0], nullptr, ok ? s : 0u, 0u, rs, lane);
+                    const uint32_t v = bound_of_pair<kG, true>(I.s_rec[0], nullptr, ok ? s : 0u, 0u, rs, lane, s_n_sets, 0u, err);
                     pass = pass && bound_passes(I, th, v, nr);
                 }
                 keep(pass, slot0 + k, s);
@@ -192,13 +197,13 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
                     const bool beyond = my < len && k == kw;
                     if (!__any_sync(kFull, beyond)) break;  // no lane is past this window
                     if (windows == kWalkWindows) {
-                        if (beyond) k = find_probe_lane(I.cand_offsets, kw, I.n_probes, f0 + my);
+                        if (beyond) k = find_probe_lane(I.cand_offsets, kw, I.n_probes, f0 + my, err);
                         if (f + 32 < len) window(__shfl_sync(kFull, k, 31));
                         break;
                     }
                     w = list_end(kw);
                 }
-                r = k < I.n_probes ? __ldg(I.probe_ids + k) : 0xFFFFFFFFu;
+                r = k < I.n_probes ? ld_at(I.probe_ids, k, I.n_probes, err) : 0xFFFFFFFFu;
             }
             const uint32_t s = next(f);
             const bool have = r < I.r_n_sets && my < len, ok = have && s < s_n_sets;
@@ -206,14 +211,14 @@ __device__ __forceinline__ uint64_t filter_chunk(const PlanInst& I, uint64_t f0,
             bool pass = ok && !(self_join && s == r);
             if (G == 0) {
                 if (pass && !emit_all) {
-                    const uint32_t nr = I.r_desc[r].y, ns = I.s_desc[s].y;
+                    const uint32_t nr = ld_at(I.r_desc, r, I.r_n_sets, err).y, ns = ld_at(I.s_desc, s, s_n_sets, err).y;
                     pass = overlap_passes(I, min(nr, ns), nr, ns);
                 }
             } else {
                 const uint32_t rk = r < I.r_n_sets ? r : 0u;
-                uint32_t r_head = G > 1 ? __ldg(&I.r_rec[0][(uint64_t)rk * kG * 2].x) : 0u;
-                const uint32_t v =
-                    bound_of_pair<kG, false>(I.s_rec[0], I.r_rec[0], ok ? s : 0u, rk, Sector(), lane, &r_head);
+                uint32_t r_head = G > 1 ? ld_header(I.r_rec[0], rk, kG, I.r_n_sets, err) : 0u;
+                const uint32_t v = bound_of_pair<kG, false>(I.s_rec[0], I.r_rec[0], ok ? s : 0u, rk, Sector(), lane, s_n_sets,
+                                                            I.r_n_sets, err, &r_head);
                 pass = pass && bound_passes(I, th, v, r_head >> 16);
             }
             keep(pass, slot0 + k, s);
@@ -288,10 +293,11 @@ __global__ void __launch_bounds__(kPlanThreads, kPlanCtas) plan_kernel(const __g
         const PlanInst I = plan_inst(a.table ? a.table[inst] : a.single);
         const uint32_t k = 32u * (g - I.tile_base) + (uint32_t)lane;
         if (k < I.n_probes) {
-            const uint64_t c0 = I.cand_offsets[k], c1 = I.cand_offsets[k + 1];
+            const uint64_t n_offs = I.n_probes + 1ull;
+            const uint64_t c0 = ld_at(I.cand_offsets, k, n_offs, &a.ctr->err), c1 = ld_at(I.cand_offsets, k + 1, n_offs, &a.ctr->err);
             if ((k == 0 && c0 != 0) || (k + 1 == I.n_probes && c1 != I.n_cands) || c1 < c0 || c1 > I.n_cands)
                 atomicOr(&a.ctr->err, ERR_OFFSETS);
-            else if (c1 > c0 && I.probe_ids[k] >= I.r_n_sets)
+            else if (c1 > c0 && ld_at(I.probe_ids, k, I.n_probes, &a.ctr->err) >= I.r_n_sets)
                 atomicOr(&a.ctr->err, ERR_PROBE_ID);
         }
     }

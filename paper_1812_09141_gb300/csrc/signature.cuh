@@ -88,12 +88,19 @@ struct Sector {
     uint32_t w[8];
 };
 
-__device__ __forceinline__ Sector ld_sector(const uint4* p) {
-    Sector x;
+// Sector i of an array of n.
+__device__ __forceinline__ Sector ld_sector(const uint4* rec, uint64_t i, uint64_t n, uint32_t* err) {
+    Sector x = {};
+    if (!in_bounds(i, n, err)) return x;
     asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=r"(x.w[0]), "=r"(x.w[1]), "=r"(x.w[2]), "=r"(x.w[3]), "=r"(x.w[4]), "=r"(x.w[5]), "=r"(x.w[6]), "=r"(x.w[7])
-        : "l"(p));
+        : "l"(rec + 2 * i));
     return x;
+}
+
+// Header of set r's record, of n sets' records of `sectors` each.
+__device__ __forceinline__ uint32_t ld_header(const uint4* rec, uint32_t r, uint32_t sectors, uint32_t n, uint32_t* err) {
+    return ld_at(reinterpret_cast<const uint32_t*>(rec), (uint64_t)r * sectors * 8, (uint64_t)n * sectors * 8, err);
 }
 
 // Common bits of two sectors, the first word only where `first` has bits:
@@ -137,9 +144,11 @@ __device__ __forceinline__ uint32_t sum_of_group(uint32_t (&part)[G], uint32_t s
 // lane and load: with 128-byte records 90% of the L1's wavefronts and twice
 // the time); the partial counts of the group's G pairs are then summed across
 // it.  kSame: every lane's probe is the one whose sector of this lane is rs.
+// s_n, r_n: sets of both collections (bounds of the checked build).
 template <int G, bool kSame>
 __device__ __forceinline__ uint32_t bound_of_pair(const uint4* s_rec, const uint4* r_rec, uint32_t s, uint32_t r,
-                                                  const Sector& rs, int lane, uint32_t* r_head = nullptr) {
+                                                  const Sector& rs, int lane, uint32_t s_n, uint32_t r_n, uint32_t* err,
+                                                  uint32_t* r_head = nullptr) {
     const uint32_t sub = lane % G;
     const uint32_t first = sub == 0 ? 0u : kFull;  // the first sector's first word is the header
     constexpr int kBatch = G < kSectors ? G : kSectors;  // loads in flight
@@ -150,7 +159,7 @@ __device__ __forceinline__ uint32_t bound_of_pair(const uint4* s_rec, const uint
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
             const uint32_t sj = G == 1 ? s : __shfl_sync(kFull, s, b + i, G);
-            x[i] = ld_sector(s_rec + ((uint64_t)sj * G + sub) * 2);
+            x[i] = ld_sector(s_rec, (uint64_t)sj * G + sub, (uint64_t)s_n * G, err);
         }
 #pragma unroll
         for (int i = 0; i < kBatch; ++i) {
@@ -160,7 +169,7 @@ __device__ __forceinline__ uint32_t bound_of_pair(const uint4* s_rec, const uint
                 hr = rs.w[0];
             } else {
                 const uint32_t rj = G == 1 ? r : __shfl_sync(kFull, r, b + i, G);
-                const Sector y = ld_sector(r_rec + ((uint64_t)rj * G + sub) * 2);
+                const Sector y = ld_sector(r_rec, (uint64_t)rj * G + sub, (uint64_t)r_n * G, err);
                 part[b + i] = common_bits(x[i], y, first);
                 hr = y.w[0];
                 if (G == 1) *r_head = hr;
@@ -202,19 +211,19 @@ __device__ __forceinline__ bool bound_passes(const PlanInst& I, const Threshold&
 // Second level: the n buffered pairs tested with the long records; the ones
 // left stay in the buffer, in order.  Returns their number.
 template <int G>
-__device__ __noinline__ uint32_t second_level(const PlanInst& I, uint2* buf, uint32_t n, int lane) {
+__device__ __noinline__ uint32_t second_level(const PlanInst& I, uint2* buf, uint32_t n, uint32_t* err, int lane) {
     const unsigned lt_mask = (1u << lane) - 1u;
     const Threshold th = threshold(I);
     uint32_t left = 0;
     for (uint32_t t = 0; t < n; t += 32) {
         const bool have = t + lane < n;
         const uint2 e = buf[have ? t + lane : t];
-        const uint32_t r = __ldg(I.probe_ids + (e.x - 32u * I.tile_base));
-        const uint32_t r_head = __ldg(&I.r_rec[1][(uint64_t)r * G * 2].x);
-        const uint32_t v = bound_of_pair<G, false>(I.s_rec[1], I.r_rec[1], e.y, r, Sector(), lane);
+        const uint32_t r = ld_at(I.probe_ids, e.x - 32u * I.tile_base, I.n_probes, err);
+        const uint32_t r_head = ld_header(I.r_rec[1], r, G, I.r_n_sets, err);
+        const uint32_t v = bound_of_pair<G, false>(I.s_rec[1], I.r_rec[1], e.y, r, Sector(), lane, I.s_n_sets, I.r_n_sets, err);
         const bool pass = have && bound_passes(I, th, v, r_head >> 16);
         const uint32_t m = __ballot_sync(kFull, pass);  // (every lane has read its entry)
-        if (pass) buf[left + __popc(m & lt_mask)] = e;
+        if (pass && in_bounds(left + __popc(m & lt_mask), n, err)) buf[left + __popc(m & lt_mask)] = e;
         left += __popc(m);
         __syncwarp();
     }
@@ -287,7 +296,8 @@ __device__ __noinline__ void queue_pairs(const VerifyArgs& a, const PlanInst& I,
     static_assert(kPlanBuf <= 16 * 32, "granularities and head masks of 16 windows");
     const unsigned lt_mask = (1u << lane) - 1u;
     uint32_t* err = &a.ctr->err;
-    auto probe_of = [&](uint32_t i) -> uint32_t { return I.probe_ids[buf[i].x - 32u * I.tile_base]; };
+    auto probe_of = [&](uint32_t i) -> uint32_t { return ld_at(I.probe_ids, buf[i].x - 32u * I.tile_base, I.n_probes, err); };
+    auto size_of = [&](uint32_t r) -> uint32_t { return ld_at(I.r_desc, r, I.r_n_sets, err).y; };
     // lane 0 takes room for ns short and nl long pairs (nw of them without an item); false if there is none
     unsigned long long base_s = 0, base_l = 0;
     auto reserve = [&](uint32_t ns, uint32_t nl, uint32_t nw) -> bool {
@@ -311,7 +321,7 @@ __device__ __noinline__ void queue_pairs(const VerifyArgs& a, const PlanInst& I,
         a.pairs[pos] = pr;
     };
     if (buf[0].x == buf[n - 1].x) {  // one run (slots ascend)
-        const uint32_t r = probe_of(0), bin = probe_bin(a, I.flags, I.r_desc[r].y, n);
+        const uint32_t r = probe_of(0), bin = probe_bin(a, I.flags, size_of(r), n);
         if (!reserve(bin ? 0u : n, bin ? n : 0u, bin == 1 ? n : 0u)) return;
         const unsigned long long pos = bin ? a.pair_cap - base_l - n : base_s;
         for (uint32_t i = lane; i < n; i += 32) write_pair(pos + i, buf[i], bin);
@@ -349,7 +359,7 @@ __device__ __noinline__ void queue_pairs(const VerifyArgs& a, const PlanInst& I,
         const uint32_t i = 32 * w + lane;
         uint32_t h, e, bin = 0;
         run_of(w, &h, &e);
-        if (i < n) bin = probe_bin(a, I.flags, I.r_desc[probe_of(i)].y, e - h);
+        if (i < n) bin = probe_bin(a, I.flags, size_of(probe_of(i)), e - h);
         bins |= (uint64_t)bin << (3 * w);
         n_long += __popc(__ballot_sync(kFull, bin != 0));
         n_warp += __popc(__ballot_sync(kFull, bin == 1));
@@ -397,9 +407,9 @@ __device__ __noinline__ void queue_pairs(const VerifyArgs& a, const PlanInst& I,
 __device__ __forceinline__ void flush_survivors(const VerifyArgs& a, const PlanInst& I, uint32_t inst, uint2* buf,
                                                 uint32_t n, int lane) {
     switch (I.rec_sectors[1]) {
-        case 2: n = second_level<2>(I, buf, n, lane); break;
-        case 4: n = second_level<4>(I, buf, n, lane); break;
-        case 8: n = second_level<8>(I, buf, n, lane); break;
+        case 2: n = second_level<2>(I, buf, n, &a.ctr->err, lane); break;
+        case 4: n = second_level<4>(I, buf, n, &a.ctr->err, lane); break;
+        case 8: n = second_level<8>(I, buf, n, &a.ctr->err, lane); break;
         default: break;
     }
     if (n) queue_pairs(a, I, inst, buf, n, lane);

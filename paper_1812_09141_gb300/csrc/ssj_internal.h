@@ -127,10 +127,13 @@ enum : uint32_t {
     ERR_BOUNDS = 16u, // checked build (SSJ_CHECKED): an index was out of bounds; the access was skipped
 };
 
-// The checked build (-DSSJ_CHECKED, libssj_checked.so) tests every index of
-// the plan and verify kernels against its array's extent before the access;
-// an index out of bounds sets ERR_BOUNDS and the access is skipped (a load
-// reads zeros), so a bug shows as an error status, never as a fault.
+// The checked build (-DSSJ_CHECKED, libssj_checked.so) tests the indexes with
+// which the plan, verify, join and queue kernels read the batch, the
+// collections, their records, the index and the pair lists, and write their
+// buffers and lists, against each array's extent before the access; an index
+// out of bounds sets ERR_BOUNDS and the access is skipped (a load reads zeros),
+// so a bug shows as an error status, never as a fault.  (Not the kernels that
+// lay a collection out, build its index, expand groups, scan and sort.)
 #ifdef SSJ_CHECKED
 constexpr bool kChecked = true;
 #else
@@ -268,6 +271,7 @@ struct CandgenIndex {
     uint64_t* scan_scratch;
     uint64_t* total;
     void* post;
+    uint64_t entries;             // index entries (after stage 0)
 };
 
 // A token's index entries are kept in cells by position: as many (a power of

@@ -318,22 +318,22 @@ __device__ __forceinline__ void lane_merge(const uint32_t* A, uint32_t rw, const
 __device__ __forceinline__ uint32_t warp_lookup(const uint32_t* R, uint32_t nr, const uint4* __restrict__ s4,
                                                 uint32_t ns, int lane, uint64_t slim, uint32_t* err) {
     uint32_t c = 0;
+    auto r_at = [&](uint32_t p) -> uint32_t { return in_bounds(p, nr, err) ? R[p] : 0u; };
     if (nr) {
         for (uint32_t b = lane; b < (ns + 3) >> 2; b += 32) {
             const uint4 x = ld_block(s4, b, slim, err);
             uint32_t p0 = 0, p1 = 0, p2 = 0, p3 = 0;  // first token of r not below x's, among the last n
             for (uint32_t n = nr; n > 1;) {
                 const uint32_t half = n >> 1;
-                const uint32_t* m = R + half - 1;
-                p0 += m[p0] < x.x ? half : 0u;
-                p1 += m[p1] < x.y ? half : 0u;
-                p2 += m[p2] < x.z ? half : 0u;
-                p3 += m[p3] < x.w ? half : 0u;
+                p0 += r_at(p0 + half - 1) < x.x ? half : 0u;
+                p1 += r_at(p1 + half - 1) < x.y ? half : 0u;
+                p2 += r_at(p2 + half - 1) < x.z ? half : 0u;
+                p3 += r_at(p3 + half - 1) < x.w ? half : 0u;
                 n -= half;
             }
             const uint32_t valid = ns - 4 * b;  // (the tokens past s's end repeat its last one)
-            c += (R[p0] == x.x ? 1u : 0u) + (valid > 1 && R[p1] == x.y ? 1u : 0u) +
-                 (valid > 2 && R[p2] == x.z ? 1u : 0u) + (valid > 3 && R[p3] == x.w ? 1u : 0u);
+            c += (r_at(p0) == x.x ? 1u : 0u) + (valid > 1 && r_at(p1) == x.y ? 1u : 0u) +
+                 (valid > 2 && r_at(p2) == x.z ? 1u : 0u) + (valid > 3 && r_at(p3) == x.w ? 1u : 0u);
         }
     }
     return __reduce_add_sync(kFull, c);
@@ -621,7 +621,7 @@ __device__ __noinline__ void lane_item(const Instance& I, const WorkItem& wi, co
             const uint32_t my = cursor + __popc(idle & lt_mask);
             if (!active && my < wi.n) {
                 const uint32_t s = run[my].s & ~kInItem;
-                const uint2 ds = I.s_desc[s];
+                const uint2 ds = ld_at(I.s_desc, s, I.s_n_sets, err);
                 active = true;
                 s_id = s;
                 ns = ds.y;
@@ -759,7 +759,7 @@ __device__ __noinline__ void index_item(const Instance& I, const WorkItem& wi, c
     // r's last token (the padding repeats it in the last block's last lane)
     const uint32_t rmax = nr ? ld_block(r4, (nr - 1) >> 2, rlim, err).w : 0u;
     if (32u * (uint32_t)warp < wi.n) {  // warp-uniform: the first batch's descriptors
-        if (p_ok) p_desc = I.s_desc[p_id];
+        if (p_ok) p_desc = ld_at(I.s_desc, p_id, I.s_n_sets, err);
         pstage = 2;
     }
     __syncthreads();
@@ -816,7 +816,7 @@ __device__ __noinline__ void index_item(const Instance& I, const WorkItem& wi, c
         // ---- preparation (a batch queued here makes room for the next one to be taken in the
         // same step, so a batch is taken every second round)
         if (pstage == 1) {
-            if (p_ok) p_desc = I.s_desc[p_id];
+            if (p_ok) p_desc = ld_at(I.s_desc, p_id, I.s_n_sets, err);
             pstage = 2;
         } else {
             if (pstage == 2) {
@@ -985,7 +985,7 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
             // thread 0: stage candidate m's s if it fits a buffer
             auto prefetch = [&](uint32_t m) -> uint32_t {
                 if (m >= bi.n || !in_bounds(bi.c0 + m, a.pair_cap, &a.ctr->err)) return 0u;
-                const uint2 dx = I.s_desc[a.pairs[bi.c0 + m].s & ~kInItem];
+                const uint2 dx = ld_at(I.s_desc, a.pairs[bi.c0 + m].s & ~kInItem, I.s_n_sets, &a.ctr->err);
                 if (dx.y == 0 || dx.y + 4 > kBlockWin + 16) return 0u;
                 bulk_stage(sbuf[m & 1], I.s_toks4 + dx.x, 0u, (dx.y + 3) >> 2, I.s_n_chunks - dx.x,
                            (kBlockWin + 16) / 4, &bsm.bar[1 + (m & 1)], &a.ctr->err);
@@ -1027,7 +1027,7 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
                 }
                 if (!in_bounds(bi.c0 + m, a.pair_cap, &a.ctr->err)) break;
                 const uint32_t s = a.pairs[bi.c0 + m].s & ~kInItem;
-                const uint2 ds = I.s_desc[s];
+                const uint2 ds = ld_at(I.s_desc, s, I.s_n_sets, &a.ctr->err);
                 const uint32_t ns = ds.y;
                 const uint32_t req = required_overlap(I.sim, I.p, I.den, I.magic, nr, ns);
                 bool rej;
@@ -1149,7 +1149,9 @@ __global__ void __launch_bounds__(BT, MINB) verify_kernel(VerifyArgs a) {
         if (few) {  // neighbouring pairs on different SMs
             for (unsigned long long u = (unsigned long long)warp * gridDim.x + blockIdx.x; u < n_long + n_pairs;
                  u += n_warps_total) {
-                const PairRef pr = a.pairs[u < n_long ? a.pair_cap - n_long + u : u - n_long];
+                const unsigned long long at = u < n_long ? a.pair_cap - n_long + u : u - n_long;
+                if (!in_bounds(at, a.pair_cap, &a.ctr->err)) continue;  // (uniform over the warp)
+                const PairRef pr = a.pairs[at];
                 if (!(pr.s & kInItem) && !verify_pair(pr)) return;  // the warp stops
             }
         } else {
