@@ -97,13 +97,6 @@ struct Collection {
     uint32_t busy = 0;           // submitted batches not yet collected
     size_t l2_window = 0;        // SSJ_PIN_L2: bytes of the token array kept in the persisting L2 set-aside
     float l2_hit_ratio = 0.f;    // share of the window the set-aside holds
-    DevColl dev() const {
-        DevColl d;
-        d.toks4 = reinterpret_cast<const uint4*>(d_toks);
-        d.desc = d_desc;
-        d.n_sets = n_sets;
-        return d;
-    }
 };
 
 enum class TicketState { kRunning, kDone, kFailed };
@@ -1544,7 +1537,6 @@ uint64_t batch_device_bytes(uint32_t n_probes, uint64_t n_cands, bool count_only
         b += align256(8ull * (n_probes + 1));
         b += align256(4ull * std::max<uint64_t>(n_cands, 1));
     }
-    b += 256;  // count
     b += align256(workspace_bytes(n_probes, n_cands, num_sms));
     if (!count_only) b += align256(sizeof(ssj_triple) * std::max<uint64_t>(n_cands, 1));
     return b;
@@ -1781,7 +1773,6 @@ extern "C" ssj_status ssj_submit(ssj_ctx* ctx, const ssj_batch* batch, uint64_t*
         a.single.cand_offsets = batch->cand_offsets;
         a.single.cand_ids = batch->cand_ids;
     }
-    off += 256;
     void* ws = base + off;
     const size_t ws_bytes = align256(workspace_bytes(batch->n_probes, n_cands, ctx->num_sms));
     off += ws_bytes;

@@ -199,6 +199,7 @@ __device__ __forceinline__ bool position_ok(const Params& P, const Entry<true>& 
     return ub >= pair_required(P, L, e.size);
 }
 
+// The 32-bit finaliser of MurmurHash3 (Appleby).
 __device__ __forceinline__ uint32_t mix32(uint32_t x) {
     x ^= x >> 16;
     x *= 0x85ebca6bu;

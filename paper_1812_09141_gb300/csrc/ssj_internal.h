@@ -9,15 +9,6 @@
 
 namespace ssj {
 
-// Device layout of one collection (Section 3.3.1, Fig. datasetslayout):
-// tokens linearised with every set starting on a 16-byte boundary so that
-// sets are read with 128-bit loads; desc[i] = (first 16-byte chunk, length).
-struct DevColl {
-    const uint4* toks4;
-    const uint2* desc;
-    uint32_t n_sets;
-};
-
 enum : uint32_t {
     VF_COUNT_ONLY = 1u,
     VF_EMIT_ALL = 2u,
