@@ -4,13 +4,15 @@
 //
 // What bounds it: the records gathered from L2 (32 to 256 bytes a candidate,
 // by the collections' set sizes, instead of the tokens the merge would read:
-// 4 bytes each, of both sets, up to the positional filter's stop) and the
-// instructions that count their common bits, about three per four bytes.
+// 4 bytes each, of both sets, up to the positional filter's stop).  On long
+// sets their loads take 75% of the L1 data pipe's wavefronts and half of a
+// warp's waiting is for them; the issue slots are busy 58% of the time with
+// counting common bits (about three instructions per four bytes), L2 40%.
 // Verification of 9.2e7 candidates of long sets (about 300 tokens, t = 0.6)
 // took 5.2 ms when every candidate was walked against a bitmap of its probe;
-// the test takes 1.00 ms (64 bytes per candidate, 6e9 bytes from L2) and
+// the test takes 0.95 ms (64 bytes per candidate, 6e9 bytes from L2) and
 // leaves 50 us of verification.  On 5.7e6 candidates of short sets (about 20
-// tokens) 50 us, leaving 10 us, instead of 195 us of merging.
+// tokens) 48 us, leaving 10 us, instead of 195 us of merging.
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -26,10 +28,10 @@ constexpr int kPlanThreads = 256;
 constexpr int kPlanWarps = kPlanThreads / 32;
 constexpr uint32_t kOneProbe = 64;              // candidates of a list worth rounds of their own (32: the same)
 constexpr uint32_t kWalkWindows = 4;            // windows that a round of several probes walks before it searches
-// CTAs per SM the registers are budgeted for (64 each).  With 3 the long sets take 1.09 ms instead of
+// CTAs per SM the registers are budgeted for (64 each).  With 3 the long sets took 1.09 ms instead of
 // 1.00; with 5 the spills cost more than the warps gain (1.20).  Asking for the next round's records
-// before these are counted costs more registers than it hides latency (1.16 ms with 3 CTAs); more
-// candidate ids asked for ahead change nothing (2 rounds) or cost registers (4: 1.02 ms).
+// before these are counted cost more registers than it hid latency (1.16 ms with 3 CTAs); more
+// candidate ids asked for ahead changed nothing (2 rounds) or cost registers (4: 1.02 ms).
 constexpr int kPlanCtas = 4;
 
 // Largest k of [lo, hi) with offs[k] <= f (lo < hi; lo, if offs[lo] is beyond
