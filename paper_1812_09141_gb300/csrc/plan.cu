@@ -13,6 +13,7 @@
 // the test takes 0.95 ms (64 bytes per candidate, 6e9 bytes from L2) and
 // leaves 50 us of verification.  On 5.7e6 candidates of short sets (about 20
 // tokens) 48 us, leaving 10 us, instead of 195 us of merging.
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -306,11 +307,14 @@ __global__ void __launch_bounds__(kPlanThreads, kPlanCtas) plan_kernel(const __g
 }
 
 cudaError_t launch_plan(const VerifyArgs& a, cudaStream_t st, int num_sms) {
-    static int ctas_per_sm = 0;  // resident CTAs per SM (same value from every thread)
+    // resident CTAs per SM: the same value from every thread that submits (all devices are alike)
+    static std::atomic<int> cached{0};
+    int ctas_per_sm = cached.load(std::memory_order_relaxed);
     if (ctas_per_sm == 0) {
-        int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, plan_kernel, kPlanThreads, 0) != cudaSuccess || n < 1) n = 4;
-        ctas_per_sm = n;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas_per_sm, plan_kernel, kPlanThreads, 0) != cudaSuccess ||
+            ctas_per_sm < 1)
+            ctas_per_sm = kPlanCtas;
+        cached.store(ctas_per_sm, std::memory_order_relaxed);
     }
     // at most one wave; the kernel also runs for empty batches, to clear the instances' counts
     const uint64_t chunks = a.n_chunks - a.chunk_begin, tiles = a.chunk_begin ? 0 : a.n_tiles;
