@@ -243,6 +243,8 @@ __device__ __noinline__ uint32_t second_level(const PlanInst& I, uint2* buf, uin
 // 90 and 0.6, one block per pair 5.8), within it from about 270 (60 tokens): a
 // quarter of the threshold for the former.  Lists of 1,000 pairs of 1,500 tokens
 // that all pass took 4.7 ms with one threshold for both, now 2.8.
+// (The line holds with the largest bitmaps: 780,000 token values, lists of 130
+// pairs of 300 tokens 1.29 ms, 1.48 with the full threshold.)
 __device__ __forceinline__ uint32_t probe_bin(const VerifyArgs& a, uint32_t flags, uint32_t nr, uint32_t n) {
     const bool lane_ok = nr + 4 <= kWarpRCap;
     if (flags & VF_FORCE_INDEX) return a.index_words ? 4u : (lane_ok ? 3u : 1u);
